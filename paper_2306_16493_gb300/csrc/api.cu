@@ -322,6 +322,22 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
             }
             c->gsf32.release();
         }
+        // factorised Re->k sum: R_e index of every point of its bounding cube (a set that holds a
+        // vector twice is left to the direct sum)
+        c->re_cube_ok = false;
+        if (c->fac_re_r >= 0) {
+            const int r = c->fac_re_r, Dc = 2 * r + 1;
+            std::vector<int> cube((size_t)Dc * Dc * Dc, -1);
+            bool twice = false;
+            for (int k = 0; k < nRe; ++k) {
+                int &at = cube[((size_t)(s->Re[3 * k] + r) * Dc + (s->Re[3 * k + 1] + r)) * Dc + (s->Re[3 * k + 2] + r)];
+                twice |= at >= 0;
+                at = k;
+            }
+            upload(c->re_cube, cube.data(), cube.size(), c->stream);
+            EPWI_CUDA(cudaStreamSynchronize(c->stream));   // cube is freed on return
+            c->re_cube_ok = !twice;
+        }
         // |ghat(k)[rp][mu][i][n]| <= sum_Re sum_j |w g| (|V_jn| <= 1): scale fp16 operands so
         // that this bound maps to 2^14 (no overflow, full mantissa for the split).
         std::vector<double> rp_bound(nRp, 0.0);

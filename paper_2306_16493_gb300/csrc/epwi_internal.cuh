@@ -174,6 +174,11 @@ struct epwi_ctx {
     int fac_re_r = -1, fac_rp_r = -1;
     DevBuf fac_Hc, fac_Pc;         // double2 [Dc^3][W W], [Dc^3][Nm Nm]
     DevBuf fac_T, fac_U;           // stage outputs (see eigs.cu)
+    // factorised Re->k sum (kstage.cuh)
+    bool re_cube_ok = false;       // re_cube is valid (R_e within |n| <= 6, no vector twice)
+    DevBuf re_cube;                // int [Dc^3]: R_e index of each bounding-cube point, -1 if absent
+    DevBuf ks_T;                   // stage outputs T1, T2
+    DevBuf col_buf;                // (k2, k3) columns of a k-point list
     // band velocities: with vel_defer (set by epwi_eigs) the eigensolve leaves them out and
     // they are formed from the kept electron stage output fac_Uel for the k-points that need
     // them: those of each new window, or every point on request (ensure_velocities)
@@ -227,7 +232,8 @@ struct epwi_ctx {
                          &tc_n32, &tc_hw32, &tc_err, &tc_meta, &is_pairs, &is_w,
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
                          &ib_kpos, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
-                         &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel};
+                         &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
+                         &re_cube, &ks_T, &col_buf};
         for (DevBuf *b : all) b->release();
         mlp_free(mlp);
     }

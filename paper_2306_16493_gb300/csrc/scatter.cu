@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "epwi_internal.cuh"
+#include "kstage.cuh"
 #include "scatter.cuh"
 
 namespace {
@@ -230,7 +231,17 @@ void launch_fp64_scatter(const ScatterArgs &sa, int64_t ntiles, cudaStream_t st)
     }
 }
 
-void fp64_restage(const RestageArgs &ra, int W, cudaStream_t st) {
+struct Fp64Store {
+    double2 *out;
+    int64_t nrow;
+    __device__ __forceinline__ void operator()(int64_t s, int row, double2 v) const { out[s * nrow + row] = v; }
+};
+
+void fp64_restage(epwi_ctx *c, const RestageArgs &ra, int W, cudaStream_t st) {
+    if (kstage_pays(c, ra.nkp_all, ra.nrow, true)) {
+        kstage_run<double2>(c, ra, ra.gw64, ra.ph64, ra.V64, Fp64Store{ra.ghat64, ra.nrow});
+        return;
+    }
     if (W == 1) launch_fp64_pair<1, 0>(ra, ScatterArgs{}, 0, st);
     else if (W == 4) launch_fp64_pair<4, 0>(ra, ScatterArgs{}, 0, st);
     else if (W == 8) launch_fp64_pair<8, 0>(ra, ScatterArgs{}, 0, st);
@@ -321,6 +332,7 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, double *g
     ra.V64 = c->V.as<double2>();
     ra.V32 = c->V32.as<float2>();
     ra.nkp = (int)nkpc;
+    ra.nkp_all = ws.nkp;
     ra.kpts = ws.kpts + cv.kp0;
     ra.kp_state = ws.kp_state + cv.kp0;
     ra.s_base = cv.s_base;
@@ -335,7 +347,7 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, double *g
     cudaEventRecord(tm.re.e[0], c->stream);
     if (sf) sf_restage(c, ra);
     else if (tc) tc_restage(c, ra);
-    else fp64_restage(ra, W, c->stream);
+    else fp64_restage(c, ra, W, c->stream);
     cudaEventRecord(tm.re.e[1], c->stream);
     // Rp->q + rotations + delta sum
     ScatterArgs sa;

@@ -25,6 +25,8 @@ struct RestageArgs {
     void *ghat_raw;                       // split-precision output (layout of the TC kernel)
     int precision;
     int64_t nstates_chunk;                // states of the chunk
+    int64_t nkp_all;                      // k-points of the whole work set: the Re->k kernel is chosen
+                                          // by it, so that results do not depend on the chunking
 };
 
 struct ScatterArgs {

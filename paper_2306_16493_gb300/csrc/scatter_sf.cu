@@ -28,6 +28,7 @@
 #include <algorithm>
 
 #include "epwi_internal.cuh"
+#include "kstage.cuh"
 #include "scatter.cuh"
 #include "sieve.cuh"
 
@@ -147,6 +148,13 @@ __global__ void __launch_bounds__(256) k_restage_f32_kb(RestageArgs a, float2 *_
         }
     }
 }
+
+// The value of (state, row) in the fp32 mode's layout.
+struct SfStore {
+    float2 *out;
+    int64_t nrow;
+    __device__ __forceinline__ void operator()(int64_t s, int row, float2 v) const { out[s * nrow + row] = v; }
+};
 
 // g'(Re, f1 f2 f3) = (T x T x T) g(Re, cube): along each axis, form 0 is R = 0, form 2R-1 is
 // v[R] + v[-R] and form 2R is i (v[R] - v[-R]).  cube[c] is the index of the R_p vector at
@@ -767,6 +775,10 @@ void sf_restage(epwi_ctx *c, const RestageArgs &ra_in) {
     ra.nrow = Dc * Dc * Dc * c->nm * c->nw;
     const int W = ra.W;
     float2 *out = static_cast<float2 *>(ra.ghat_raw);
+    if (kstage_pays(c, ra.nkp_all, ra.nrow, false)) {
+        kstage_run<float2>(c, ra, c->gsf32.as<float2>(), c->ph32.as<float2>(), c->V32.as<float2>(), SfStore{out, ra.nrow});
+        return;
+    }
     auto go = [&](auto kern, int KG) {
         dim3 grid((ra.nrow + 127) / 128, (unsigned)((ra.nkp + KG - 1) / KG));
         const size_t sm = sizeof(float2) * KG * ra.nRe;

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "kstage.cuh"
 #include "scatter.cuh"
 #include "tc_ptx.cuh"
 
@@ -181,19 +182,40 @@ __host__ __device__ __forceinline__ uint32_t cm_off(int c, int k) {
     return (uint32_t)(((c >> 3) * 4 + (k * ES) / 16) * 128 + (c & 7) * 16 + (k * ES) % 16);
 }
 
+// Writes the value of (state, row) into the B image below: scaled, split into hi + lo.
+template <class Op, int NMW>
+struct ImgStore {
+    uint8_t *img;
+    int64_t ns;
+    float scale;
+    __device__ __forceinline__ void operator()(int64_t s, int row, float2 o) const {
+        constexpr int ES = Op::kBytes;
+        constexpr int KC = 64 / ES;
+        constexpr uint32_t BLK = (NMW + 15) / 16 * 16 * 64;
+        const int rp = row / NMW, c = row - rp * NMW;
+        const int ch = rp / KC, kk = rp - ch * KC;
+        uint32_t w6[6];
+        split2f<Op>(o.x * scale, w6[0], w6[2]);
+        split2f<Op>(o.y * scale, w6[1], w6[3]);
+        const uint32_t sign = ES == 4 ? 0x80000000u : 0x8000u;
+        w6[4] = w6[1] ^ sign;
+        w6[5] = w6[3] ^ sign;
+#pragma unroll
+        for (int arr = 0; arr < 6; ++arr) {
+            uint8_t *dst = img + ((size_t)(ch * 6 + arr) * ns + s) * BLK + cm_off<ES>(c, kk);
+            if constexpr (ES == 4) *reinterpret_cast<uint32_t *>(dst) = w6[arr];
+            else *reinterpret_cast<uint16_t *>(dst) = (uint16_t)w6[arr];
+        }
+    }
+};
+
 // Re->k stage for the split-precision path.  ghat(k)[rp][mu][i][n] = sum_j [sum_Re e^{ik.Re}
 // gw32] V32_jn is accumulated in FP32, scaled by 2^e, split into hi + lo and written as the
 // B operand image of the tensor-core kernel:
 //   img[ch][arr][state][NMWP rows][64 bytes]  (arr: Br_hi, Bi_hi, Br_lo, Bi_lo, -Bi_hi, -Bi_lo),
 // row = mu*W + i (rows NMW..NMWP-1 and K beyond nRp stay zero), K = rp - ch*KC.
 template <class Op, int W, int NM, int KG>
-__global__ void __launch_bounds__(128) k_restage_tc(RestageArgs a, uint8_t *__restrict__ img,
-                                                    int64_t ns, float scale) {
-    constexpr int ES = Op::kBytes;
-    constexpr int KC = 64 / ES;
-    constexpr int NMW = NM * W;
-    constexpr int NMWP = (NMW + 15) / 16 * 16;
-    constexpr uint32_t BLK = NMWP * 64;
+__global__ void __launch_bounds__(128) k_restage_tc(RestageArgs a, ImgStore<Op, NM * W> store) {
     extern __shared__ float2 Pf[];   // [KG][nRe]
     const int kg0 = blockIdx.y * KG;
     for (int idx = threadIdx.x; idx < KG * a.nRe; idx += blockDim.x) {
@@ -227,9 +249,6 @@ __global__ void __launch_bounds__(128) k_restage_tc(RestageArgs a, uint8_t *__re
             for (int j = 0; j < W; ++j) acc[kk][j] = cfmaf(p, gv[j], acc[kk][j]);
         }
     }
-    const int rp = row / NMW, c = row - rp * NMW;
-    const int ch = rp / KC, kk = rp - ch * KC;
-    const uint32_t eoff = cm_off<ES>(c, kk);
 #pragma unroll
     for (int q = 0; q < KG; ++q) {
         if (kg0 + q >= a.nkp) break;
@@ -242,18 +261,7 @@ __global__ void __launch_bounds__(128) k_restage_tc(RestageArgs a, uint8_t *__re
             float2 o = make_float2(0.f, 0.f);
 #pragma unroll
             for (int j = 0; j < W; ++j) o = cfmaf(acc[q][j], Vk[j * W + lo + np], o);
-            uint32_t w6[6];
-            split2f<Op>(o.x * scale, w6[0], w6[2]);
-            split2f<Op>(o.y * scale, w6[1], w6[3]);
-            const uint32_t sign = ES == 4 ? 0x80000000u : 0x8000u;
-            w6[4] = w6[1] ^ sign;
-            w6[5] = w6[3] ^ sign;
-#pragma unroll
-            for (int arr = 0; arr < 6; ++arr) {
-                uint8_t *dst = img + ((size_t)(ch * 6 + arr) * ns + (s0 + np)) * BLK + eoff;
-                if constexpr (ES == 4) *reinterpret_cast<uint32_t *>(dst) = w6[arr];
-                else *reinterpret_cast<uint16_t *>(dst) = (uint16_t)w6[arr];
-            }
+            store(s0 + np, row, o);
         }
     }
 }
@@ -1119,12 +1127,17 @@ void restage_tc_launch(epwi_ctx *c, const RestageArgs &ra) {
     uint8_t *img = static_cast<uint8_t *>(ra.ghat_raw);
     EPWI_CUDA(cudaMemsetAsync(img, 0, tc_state_bytes(c) * (size_t)ra.nstates_chunk, c->stream));
     const int e = (Op::kFmt == 0 && !Op::kTF32) ? c->tc_scale_exp : 0;
+    const ImgStore<Op, NM * W> store{img, ra.nstates_chunk, std::ldexp(1.0f, e)};
+    if (kstage_pays(c, ra.nkp_all, ra.nrow, false)) {
+        kstage_run<float2>(c, ra, ra.gw32, c->ph32.as<float2>(), c->V32.as<float2>(), store);
+        return;
+    }
     dim3 grid((ra.nrow + 127) / 128, (unsigned)((ra.nkp + KG - 1) / KG));
     const size_t sm = sizeof(float2) * KG * ra.nRe;
     auto kern = k_restage_tc<Op, W, NM, KG>;
     if (sm > 48 * 1024)
         EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    kern<<<grid, 128, sm, c->stream>>>(ra, img, ra.nstates_chunk, std::ldexp(1.0f, e));
+    kern<<<grid, 128, sm, c->stream>>>(ra, store);
     EPWI_CHECK_LAUNCH();
 }
 
