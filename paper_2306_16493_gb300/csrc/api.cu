@@ -313,14 +313,20 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
             c->gcube_ready = false;
             c->gcube32.release();
             c->h_rp_cube.clear();
+            c->rp_twice = false;
             if (r <= 6) {
                 const int Dc = 2 * r + 1;
                 c->h_rp_cube.assign((size_t)Dc * Dc * Dc, -1);
-                for (int k = 0; k < nRp; ++k)
-                    c->h_rp_cube[((size_t)(s->Rp[3 * k] + r) * Dc + (s->Rp[3 * k + 1] + r)) * Dc +
-                                 (s->Rp[3 * k + 2] + r)] = k;
+                for (int k = 0; k < nRp; ++k) {
+                    int &at = c->h_rp_cube[((size_t)(s->Rp[3 * k] + r) * Dc + (s->Rp[3 * k + 1] + r)) * Dc +
+                                           (s->Rp[3 * k + 2] + r)];
+                    c->rp_twice |= at >= 0;
+                    at = k;
+                }
             }
             c->gsf32.release();
+            c->gsf64.release();
+            c->sf_g64_ready = false;
         }
         // factorised Re->k sum: R_e index of every point of its bounding cube (a set that holds a
         // vector twice is left to the direct sum)

@@ -164,6 +164,9 @@ struct epwi_ctx {
     std::vector<int> h_rp_cube;    // fp32 mode: R_p index of each bounding-cube point, -1 if absent
     DevBuf gsf32;                  // fp32 mode: g' [Re][cube forms][Nm][W][W] (+-R recombined)
     bool sf_g_ready = false;       // gsf32 built for the current system
+    DevBuf gsf64;                  // FP64 mode: the same in FP64
+    bool sf_g64_ready = false;
+    bool rp_twice = false;         // R_p holds a vector twice (no FP64 cube form)
     DevBuf sf_Vt32;                // fp32 mode: float2 [m][Nk][i], columns of V band-major
     DevBuf sf_ef;                  // fp32 mode: float2 [m][Nk]: (eps - mu, f), band-major
     DevBuf sf_uS, sf_wn;           // fp32 mode: float2 [mu nu][Nq] u(q), [nu][Nq] (hbar omega, N)
@@ -233,7 +236,7 @@ struct epwi_ctx {
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
                          &ib_kpos, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
                          &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
-                         &re_cube, &ks_T, &col_buf};
+                         &re_cube, &ks_T, &col_buf, &gsf64};
         for (DevBuf *b : all) b->release();
         mlp_free(mlp);
     }

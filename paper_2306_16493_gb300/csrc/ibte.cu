@@ -310,8 +310,8 @@ void ibte_prepare(epwi_ctx *c, WorkSet &ws) {
     const size_t eb = fp64 ? sizeof(double) : sizeof(float);
     const size_t gam_bytes = eb * (size_t)(nent + 1);
     c->ib_gam.ensure(gam_bytes);
-    // the fp32 mode writes only the bands it does not skip (the others are exactly zero)
-    if (c->opt.precision == EPWI_FP32) EPWI_CUDA(cudaMemsetAsync(c->ib_gam.p, 0, gam_bytes, c->stream));
+    // the sum-factorised kernels write only the bands they do not skip (the others are exactly zero)
+    if (c->opt.precision == EPWI_FP32 || fp64) EPWI_CUDA(cudaMemsetAsync(c->ib_gam.p, 0, gam_bytes, c->stream));
     c->ib_stats.n_entries = nent;
     c->ib_stats.entry_bytes = (int32_t)eb;
     ws.pairs_dev = c->ib_pairs.as<int>();

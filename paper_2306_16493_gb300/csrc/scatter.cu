@@ -289,19 +289,20 @@ struct StageTimers {
 };
 
 // Tiles, Re->k, Rp->q with rotations and the delta sum, and the reduction of one chunk.
-int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, double *g2out, double *tout,
+int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, bool sf64, double *g2out, double *tout,
                   int tstride, StageTimers &tm) {
     const int W = c->nw, Nm = c->nm;
     const bool sf = c->opt.precision == EPWI_FP32;
     const bool tc = !sf && c->opt.precision != EPWI_FP64;
     const int nRp = tc ? tc_rp_count(c) : c->nRp;           // the split modes' view of R_p
-    const int64_t nrow = (int64_t)nRp * Nm * W;
+    // the cube forms of R_p (sum-factorised FP64), else the set itself
+    const int64_t nrow = sf64 ? (int64_t)(sf64_state_bytes(c) / sizeof(double2)) : (int64_t)nRp * Nm * W;
     const size_t state_bytes = sf ? sf_state_bytes(c) : tc ? tc_state_bytes(c) : sizeof(double2) * nrow;
     GridInfo g = make_grid_info(c);
     const int64_t nkpc = cv.kp1 - cv.kp0;
-    // tiles (the fp32 mode works per (k-point, band) instead)
+    // tiles (the sum-factorised kernels work per (k-point, band) instead)
     int64_t nt = 0;
-    if (!sf) {
+    if (!sf && !sf64) {
         c->kp_tile.ensure(sizeof(int64_t) * (nkpc + 1));
         c->scan_tmp.ensure(sizeof(int64_t) * (nkpc + 1));
         k_tiles_count<<<(unsigned)((nkpc + 255) / 256), 256, 0, c->stream>>>(
@@ -325,7 +326,7 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, double *g
     ra.nRp = nRp;
     ra.nrow = (int)nrow;
     ra.Re = c->Re.as<int>();
-    ra.gw64 = c->gw64.as<double2>();
+    ra.gw64 = sf64 ? c->gsf64.as<double2>() : c->gw64.as<double2>();
     ra.gw32 = (tc && c->rp_cube_r < 0) ? c->gcube32.as<float2>() : c->gw32.as<float2>();
     ra.ph64 = c->ph64.as<double2>();
     ra.ph32 = c->ph32.as<float2>();
@@ -405,13 +406,15 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, double *g
         sf_scatter(c, sa, nkpc, cv.kp_pairs, cv.p_off, hks);
     } else if (tc) {
         tc_scatter(c, sa, nt);
+    } else if (sf64) {
+        sf64_scatter(c, sa, nkpc, cv.kp_pairs, cv.p_off);
     } else {
         fp64_scatter(sa, nt, c->stream);
     }
     cudaEventRecord(tm.sc.e[1], c->stream);
-    // reduce (the fp32 mode wrote 1/tau already)
+    // reduce (the sum-factorised kernels wrote 1/tau already)
     cudaEventRecord(tm.red.e[0], c->stream);
-    if (!sf && !g2out && !tout && nkpc > 0) {
+    if (!sf && !sf64 && !g2out && !tout && nkpc > 0) {
         const double pref = 2.0 * epc::kPi / epc::kHbarEVs / (double)c->nk /
                             (sqrt(epc::kPi) * c->eta);
         k_reduce_tiles<<<(unsigned)((nkpc + 127) / 128), 128, 0, c->stream>>>(
@@ -449,12 +452,17 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
         sf_prepare(c);
     }
     if (tc) tc_prepare(c);
+    // Sum-factorised FP64 rates: needs pair lists in the sieve's order (filled here, or for the
+    // Gamma capture) and the window's bands, without weights or per-pair outputs
+    const bool sf64 = !sf && !tc && !g2out && !tout && !ws.pair_w && ws.ovr_nsel < 0 && (!ws.pairs_dev || ws.gam64) &&
+                      sf64_ok(c);
+    if (sf64) sf64_prepare(c);
     // chunk limits: pairs and Re->k output size
-    // pair lists per chunk: 2^32 q indices (16 GiB) in the fp32 mode, whose launches are one
+    // pair lists per chunk: 2^32 q indices (16 GiB) for the sum-factorised kernels, whose launches are one
     // CTA per state and need thousands of states per chunk to fill the GPU on large grids (200^3:
     // ~1.8 M pairs per state); 2^27 otherwise
-    const int64_t max_pairs = int64_t(1) << (sf ? 32 : 27);
-    const size_t state_bytes = sf ? sf_state_bytes(c) : tc ? tc_state_bytes(c) : sizeof(double2) * nrow;
+    const int64_t max_pairs = int64_t(1) << (sf || sf64 ? 32 : 27);
+    const size_t state_bytes = sf ? sf_state_bytes(c) : sf64 ? sf64_state_bytes(c) : tc ? tc_state_bytes(c) : sizeof(double2) * nrow;
     const int64_t max_states = std::max<int64_t>(1, (int64_t)((size_t(3) << 30) / state_bytes));
     const int64_t kp_cap = c->opt.kpoint_chunk > 0 ? c->opt.kpoint_chunk : (int64_t)1 << 40;
     StageTimers tm;
@@ -481,7 +489,7 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
             sieve_fill_chunk(c, kp0, kp1, c->pairs.as<int>());
             cv.pairs = c->pairs.as<int>();
         }
-        ntiles_total += run_chunk(c, ws, cv, g2out, tout, tstride, tm);
+        ntiles_total += run_chunk(c, ws, cv, sf64, g2out, tout, tstride, tm);
         ++nchunks;
         kp0 = kp1;
     }

@@ -112,5 +112,11 @@ size_t sf_state_bytes(const epwi_ctx *c);
 void sf_check(const epwi_ctx *c);
 void sf_prepare(epwi_ctx *c);
 void sf_restage(epwi_ctx *c, const RestageArgs &ra);
+// FP64 mode, sieved rates (scatter_sf64.cu): whether the system and grid have a kernel, g' in
+// FP64, bytes of ghat' per state, rates of a chunk
+bool sf64_ok(const epwi_ctx *c);
+void sf64_prepare(epwi_ctx *c);
+size_t sf64_state_bytes(const epwi_ctx *c);
+void sf64_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off);
 void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off,
                 const std::vector<int64_t> &h_kp_state_chunk);

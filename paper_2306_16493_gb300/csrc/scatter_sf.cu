@@ -30,12 +30,11 @@
 #include "epwi_internal.cuh"
 #include "kstage.cuh"
 #include "scatter.cuh"
+#include "scatter_sf.cuh"
 #include "sieve.cuh"
 
 namespace {
 
-constexpr int kSfThreads = 256;
-constexpr int kSfWarps = kSfThreads / 32;
 
 // Re->k in FP32: ghat32[state][row] = sum_j [sum_Re w e^{ik.Re} g(Re)[row][j]] V_{j, lo+n}(k),
 // row = (cube form, mu, i); one thread per row, KG k-points per block row.
@@ -158,10 +157,12 @@ struct SfStore {
 
 // g'(Re, f1 f2 f3) = (T x T x T) g(Re, cube): along each axis, form 0 is R = 0, form 2R-1 is
 // v[R] + v[-R] and form 2R is i (v[R] - v[-R]).  cube[c] is the index of the R_p vector at
-// cube point c, or -1 (zero weight).  One thread per output element; FP64 sums, FP32 output.
+// cube point c, or -1 (zero weight).  One thread per output element; FP64 sums, output in FP32
+// or FP64.
+template <class C2>
 __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, const int *__restrict__ cube,
                                const double2 *__restrict__ g64, const float2 *__restrict__ g32,
-                               float2 *__restrict__ out) {
+                               C2 *__restrict__ out) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n) return;
     const int e = (int)(idx % rowlen);              // (mu, i, j) within the (Re, form) block
@@ -202,7 +203,11 @@ __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, c
                 const double2 v = g64 ? g64[gi] : make_double2(g32[gi].x, g32[gi].y);
                 s = cadd(s, cmul(cmul(cmul(cv[0][x], cv[1][y]), cv[2][z]), v));
             }
-    out[idx] = make_float2((float)s.x, (float)s.y);
+    using R = decltype(C2::x);
+    C2 o;
+    o.x = (R)s.x;
+    o.y = (R)s.y;
+    out[idx] = o;
 }
 
 // Band-major tables of the k+q side (FP32): Vb[m][k][i] = V[k][i][m] and
@@ -239,24 +244,6 @@ __global__ void k_band_major_ef(int64_t nk, int W, const float *__restrict__ ere
     ef[idx] = make_float2(erel[k * W + m], f32[k * W + m]);
 }
 
-// Division by a divisor fixed at launch (x < 2^31): q = (umulhi(x, m) + x) >> l with
-// l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1 (Granlund & Montgomery, PLDI 1994).
-struct FDiv {
-    uint32_t d, m, l;
-};
-FDiv make_fdiv(uint32_t d) {
-    FDiv f;
-    f.d = d;
-    uint32_t l = 0;
-    while ((uint64_t(1) << l) < d) ++l;
-    f.l = l;
-    f.m = (uint32_t)(((uint64_t(1) << 32) * ((uint64_t(1) << l) - d)) / d + 1);
-    return f;
-}
-__device__ __forceinline__ int fdiv(int x, const FDiv &f) {
-    return (int)((__umulhi((uint32_t)x, f.m) + (uint32_t)x) >> f.l);
-}
-
 struct SfArgs {
     GridInfo g;
     int nplane;                     // N2 N3
@@ -285,31 +272,6 @@ struct SfArgs {
     float *gam;                     // Gamma capture (iterative BTE) or nullptr: row n of each
     const int64_t *goff;            // pair's block, block start goff[chunk pair]
 };
-
-// first position in [lo, hi) whose key is >= key (keys ascending)
-template <typename F>
-__device__ __forceinline__ int64_t lower_bound(int64_t lo, int64_t hi, int64_t key, F keyof) {
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (keyof(mid) < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// Shared-memory layout of k_scatter_sf (float2 units first, then floats, then ints).
-struct SfSmem {
-    size_t y, u, cs, ints, bytes;
-};
-__host__ __device__ inline SfSmem sf_smem_layout(int D, int X, int jq, int N1, int N2, int N3, int njg, int pbmax) {
-    SfSmem s;
-    s.y = (size_t)D * D * jq * X;                          // float2: Y of one q2 group
-    s.u = (size_t)kSfWarps * D * jq * X;                   // float2: U of one run per warp
-    s.cs = (size_t)(N1 + N2 + N3) * (D - 1);               // float: (cos, sin) per R >= 1
-    s.ints = (size_t)kSieveBlock + 2 * (size_t)N1 * njg + (size_t)N1 + (size_t)pbmax + 1 + 4;
-    s.bytes = sizeof(float2) * (s.y + s.u) + sizeof(float) * s.cs + sizeof(int) * s.ints;
-    return s;
-}
 
 template <int W, int NM, int RC, bool GAM>
 __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfArgs a) {
@@ -672,25 +634,6 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
     }
 }
 
-struct SfPlan {
-    int jq, njg, pbmax;
-    size_t smem;
-};
-
-// q2 values per group (jq): Y of one group and one run's U per warp within budgets that keep
-// two or more CTAs per SM.
-SfPlan sf_plan(int D, int X, int q2max, int N1, int N2, int N3) {
-    const size_t ybudget = 40 * 1024, ubudget = 36 * 1024;
-    SfPlan p;
-    const size_t per_j = sizeof(float2) * D * X;
-    const int jmax = std::max(1, std::min({q2max, (int)(ybudget / (per_j * D)), (int)(ubudget / (per_j * kSfWarps))}));
-    p.njg = (q2max + jmax - 1) / jmax;             // groups of equal size
-    p.jq = (q2max + p.njg - 1) / p.njg;
-    p.pbmax = (N2 * N3 + kSieveBlock - 1) / kSieveBlock;
-    p.smem = sf_smem_layout(D, X, p.jq, N1, N2, N3, p.njg, p.pbmax).bytes;
-    return p;
-}
-
 template <int W, int NM, int RC, bool GAM>
 void launch_sf_t(epwi_ctx *c, const SfArgs &a, int nitems, size_t sm) {
     EPWI_REQUIRE(sm <= 200 * 1024, EPWI_EUNSUPPORTED,
@@ -707,11 +650,6 @@ template <int W, int NM, int RC>
 void launch_sf(epwi_ctx *c, const SfArgs &a, int nitems, size_t sm) {
     if (a.gam) launch_sf_t<W, NM, RC, true>(c, a, nitems, sm);
     else launch_sf_t<W, NM, RC, false>(c, a, nitems, sm);
-}
-
-bool sf_shape_built(int W, int NM, int r) {
-    return (W == 4 && NM == 3 && r >= 1 && r <= 3) || (W == 1 && NM == 3 && r >= 1 && r <= 2) ||
-           (W == 8 && NM == 6 && r >= 1 && r <= 3);
 }
 
 }  // namespace
@@ -731,23 +669,35 @@ void sf_check(const epwi_ctx *c) {
     EPWI_REQUIRE(c->ng[0] * 2 <= 4096 && c->ng[2] <= 0xffff, EPWI_EUNSUPPORTED, "fp32 mode: grid too large");
 }
 
+// g' in the recombined cube forms (once per system).
+template <class C2>
+static void build_gsf(epwi_ctx *c, DevBuf &out) {
+    const int Dc = 2 * c->sf_r + 1, rowlen = c->nm * c->nw * c->nw;
+    const int64_t n = (int64_t)c->nRe * Dc * Dc * Dc * rowlen;
+    DevBuf cube;
+    upload_ints(c, cube, c->h_rp_cube);
+    out.ensure(sizeof(C2) * n);
+    k_sf_transform<C2><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
+        n, c->nRp, Dc, c->sf_r, rowlen, cube.as<int>(), c->keep_g64 ? c->gw64.as<double2>() : nullptr,
+        c->gw32.as<float2>(), out.as<C2>());
+    EPWI_CHECK_LAUNCH();
+    EPWI_CUDA(cudaStreamSynchronize(c->stream));   // cube is released next
+    cube.release();
+}
+
+void sf64_prepare(epwi_ctx *c) {
+    if (c->sf_g64_ready) return;
+    build_gsf<double2>(c, c->gsf64);
+    c->sf_g64_ready = true;
+}
+
 // Builds what the fp32 mode reads besides the eigen-tables: g' (cube embedding and the +-R
 // recombination of the R_p axes, once per system) and the band-major FP32 V and (eps - mu, f)
 // tables (per rates call).
 void sf_prepare(epwi_ctx *c) {
     const int W = c->nw, NM = c->nm;
-    const int Dc = 2 * c->sf_r + 1;
     if (!c->sf_g_ready) {
-        const int rowlen = NM * W * W;
-        const int64_t n = (int64_t)c->nRe * Dc * Dc * Dc * rowlen;
-        DevBuf cube;
-        upload_ints(c, cube, c->h_rp_cube);
-        c->gsf32.ensure(sizeof(float2) * n);
-        k_sf_transform<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
-            n, c->nRp, Dc, c->sf_r, rowlen, cube.as<int>(), c->keep_g64 ? c->gw64.as<double2>() : nullptr,
-            c->gw32.as<float2>(), c->gsf32.as<float2>());
-        EPWI_CHECK_LAUNCH();
-        EPWI_CUDA(cudaStreamSynchronize(c->stream));   // cube is freed on return
+        build_gsf<float2>(c, c->gsf32);
         c->sf_g_ready = true;
     }
     const int64_t nv = c->nk * W * W, ne = c->nk * W;
@@ -807,12 +757,7 @@ void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *
     SfArgs a;
     a.g = sa.g;
     a.nplane = sa.g.n2 * sa.g.n3;
-    int q2max = 1;
-    for (int64_t pb = 0; pb * kSieveBlock < a.nplane; ++pb) {
-        const int64_t c0 = pb * kSieveBlock, c1 = std::min<int64_t>(a.nplane, c0 + kSieveBlock) - 1;
-        q2max = std::max<int>(q2max, (int)(c1 / sa.g.n3 - c0 / sa.g.n3 + 1));
-    }
-    const SfPlan plan = sf_plan(D, X, q2max, sa.g.n1, sa.g.n2, sa.g.n3);
+    const SfPlan plan = sf_plan(D, X, sf_q2max(sa.g.n2, sa.g.n3), sa.g.n1, sa.g.n2, sa.g.n3);
     EPWI_REQUIRE((int64_t)sa.g.n1 * plan.njg <= 8192 && plan.pbmax <= 8192, EPWI_EUNSUPPORTED,
                  "fp32 mode: too many runs or plane blocks");
     a.jq = plan.jq;
