@@ -10,6 +10,7 @@
 #include <cstdlib>
 
 #include "epwi_internal.cuh"
+#include "kstage.cuh"
 #include "sieve.cuh"
 
 namespace {
@@ -405,6 +406,159 @@ __global__ void __launch_bounds__(256, 3) k_sieve_count_fast(SieveArgs a, const 
     if (threadIdx.x == 0) counts[blockIdx.x] = tot;
 }
 
+// k_sieve_count_fast (decisions, counts, mask layout) for many window k-points: one CTA takes a
+// (k2, k3) column of k-points and TB consecutive (q2, q3) combinations p.  The point k+q of the
+// column's k-points at the same p and axis-1 index b1 is the same grid point, so its energies
+// are loaded once for all of them (q1 = b1 - k1); the largest mode energies of the N1 values
+// of q1 stay in shared memory.  Per k-point the table of energies is otherwise streamed through
+// L2 once (20 bytes per candidate), which bound the per-k-point kernel; here the arithmetic
+// does.  A whole b1 is passed over when no lane of the warp has a band within the largest reach
+// of any window energy of the column.  Candidates inside the FP32 margin are collected per b1
+// and decided exactly (pair_valid_tail) after the others.
+constexpr int kColSlots = 16;                    // k-points of a column per pass
+
+__host__ __device__ constexpr size_t sieve_cols_smem(int N1, int TB) {
+    return sizeof(float) * (size_t)N1 * TB + sizeof(uint32_t) * kColSlots * ((size_t)N1 * (TB / 32) + 1);
+}
+
+template <int WT, int NMT, int TB>
+__global__ void __launch_bounds__(TB) k_sieve_count_cols(SieveArgs a, ColumnSet cs, const int *__restrict__ kpts,
+                                                         const int *__restrict__ lo, const int *__restrict__ cnt,
+                                                         unsigned long long *__restrict__ counts,
+                                                         uint32_t *__restrict__ mask, int64_t words_per_kp) {
+    constexpr int NWB = TB / 32;                 // mask words of one q1 written by this CTA
+    constexpr int V4 = WT / 4;
+    extern __shared__ float hms[];               // [N1][TB] hwmax(q1, p), -3e38 where nothing is kept
+    __shared__ float4 rec[kColSlots];            // e_0, e_1, k1, band count (0 for padding)
+    __shared__ float en32[kColSlots][WT];
+    __shared__ double en[kColSlots][WT];
+    __shared__ int s_kp[kColSlots];
+    const int N1 = a.g.n1, N2 = a.g.n2, N3 = a.g.n3, nplane = N2 * N3;
+    const int MS = N1 * NWB + 1;                 // odd row stride: lanes (k-points) on distinct banks
+    uint32_t *mst = reinterpret_cast<uint32_t *>(hms + (size_t)N1 * TB);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int col = blockIdx.x, cid = cs.id[col], k3 = cid / N2, k2 = cid - k3 * N2;
+    const int p = blockIdx.y * TB + tid;
+    const bool inb = p < nplane;
+    const int kqp = inb ? (int)plane_kq(a.g, k2, k3, p) : 0;
+    float hmx = -3.0e38f;
+    for (int q1 = 0; q1 < N1; ++q1) {
+        float h = inb ? a.hwmax32[(int64_t)q1 * nplane + p] : -1.f;
+        if (h < 0.f) h = -3.0e38f;
+        hms[q1 * TB + tid] = h;                  // read back by this thread only
+        hmx = fmaxf(hmx, h);
+    }
+    const float rej = a.ceta32 + a.delta32, acc = a.ceta32 - a.delta32;
+    const float hm_fast = a.ceta32 - 2.f * a.delta32;
+    const float4 *eq = reinterpret_cast<const float4 *>(a.eps32) + (size_t)kqp * V4;
+    const size_t rowv = (size_t)nplane * V4;
+    const int p0 = cs.start[col], p1 = cs.start[col + 1];
+    const int pbi = (int)(((int64_t)blockIdx.y * TB) / kSieveBlock);
+    const int w0 = (int)(((int64_t)blockIdx.y * TB) % kSieveBlock) / 32;   // first mask word within 8
+    for (int b = p0; b < p1; b += kColSlots) {
+        const int nb = min(kColSlots, p1 - b), nbp = (nb + 3) & ~3;
+        __syncthreads();                         // rec, mst of the previous pass are consumed
+        if (tid < kColSlots) {
+            float4 r = make_float4(3.0e38f, 3.0e38f, __int_as_float(0), __int_as_float(1));
+            if (tid < nb) {
+                const int kp = cs.kp[b + tid], ik = kpts[kp], ns = cnt[ik];
+                s_kp[tid] = kp;
+                for (int n = 0; n < ns; ++n) {
+                    en[tid][n] = a.eps[(int64_t)ik * WT + lo[ik] + n];
+                    en32[tid][n] = a.eps32[(int64_t)ik * WT + lo[ik] + n];
+                }
+                r = make_float4(en32[tid][0], ns > 1 ? en32[tid][1] : 3.0e38f, __int_as_float(ik / nplane),
+                                __int_as_float(ns));
+            }
+            rec[tid] = r;
+        }
+        __syncthreads();
+        float elo = 3.0e38f, ehi = -3.0e38f;     // window energies of the pass (bands ascend)
+        for (int x = 0; x < nb; ++x) {
+            elo = fminf(elo, en32[x][0]);
+            ehi = fmaxf(ehi, en32[x][__float_as_int(rec[x].w) - 1]);
+        }
+        // |e_n - e_m| <= hm + rej needs e_m in [elo - lim, ehi + lim]; the pad covers FP32 rounding
+        const float lim = hmx + rej + 1e-4f;
+        elo -= lim;
+        ehi += lim;
+        int c = 0;                               // lane x: kept pairs of k-point x
+        float4 nx[V4];
+#pragma unroll
+        for (int v = 0; v < V4; ++v) nx[v] = eq[v];
+        for (int b1 = 0; b1 < N1; ++b1) {
+            float em[WT];
+#pragma unroll
+            for (int v = 0; v < V4; ++v) {
+                em[4 * v] = nx[v].x; em[4 * v + 1] = nx[v].y; em[4 * v + 2] = nx[v].z; em[4 * v + 3] = nx[v].w;
+            }
+            if (b1 + 1 < N1) {
+#pragma unroll
+                for (int v = 0; v < V4; ++v) nx[v] = eq[(b1 + 1) * rowv + v];
+            }
+            bool in = false;
+#pragma unroll
+            for (int m = 0; m < WT; ++m) in |= (em[m] >= elo) & (em[m] <= ehi);
+            uint32_t mine = 0u, amb = 0u;
+            if (__any_sync(0xffffffffu, in)) {
+#pragma unroll 4
+                for (int x = 0; x < nbp; ++x) {
+                    const float4 r = rec[x];
+                    int q1 = b1 - __float_as_int(r.z);
+                    if (q1 < 0) q1 += N1;
+                    const float hm = hms[q1 * TB + tid];
+                    float d = fabsf(r.x - em[0]);
+#pragma unroll
+                    for (int m = 1; m < WT; ++m) d = fminf(d, fabsf(r.x - em[m]));
+                    const int ns = __float_as_int(r.w);
+                    if (ns > 1) {                // uniform over the block
+#pragma unroll
+                        for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(r.y - em[m]));
+                        for (int n = 2; n < ns; ++n) {
+                            const float e = en32[x][n];
+#pragma unroll
+                            for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(e - em[m]));
+                        }
+                    }
+                    const bool near = d <= hm + rej;
+                    const bool sure = (hm <= hm_fast) & (d <= hm + acc);
+                    const uint32_t bits = __ballot_sync(0xffffffffu, near & sure);
+                    if (lane == x) mine = bits;
+                    amb |= (near & !sure ? 1u : 0u) << x;
+                }
+                uint32_t any = __reduce_or_sync(0xffffffffu, amb);
+                while (any) {
+                    const int x = __ffs(any) - 1;
+                    any &= any - 1;
+                    int q1 = b1 - __float_as_int(rec[x].z);
+                    if (q1 < 0) q1 += N1;
+                    bool v = false;
+                    if ((amb >> x) & 1u)
+                        v = pair_valid_tail<WT, NMT>(a, __float_as_int(rec[x].w), en[x], en32[x],
+                                                     (int64_t)q1 * nplane + p, (int64_t)b1 * nplane + kqp,
+                                                     hms[q1 * TB + tid], em);
+                    const uint32_t bits = __ballot_sync(0xffffffffu, v);
+                    if (lane == x) mine |= bits;
+                }
+            }
+            if (lane < nb) {
+                int q1 = b1 - __float_as_int(rec[lane].z);
+                if (q1 < 0) q1 += N1;
+                mst[lane * MS + q1 * NWB + wid] = mine;
+                c += __popc(mine);
+            }
+        }
+        if (lane < nb && c) atomicAdd(&counts[s_kp[lane]], (unsigned long long)c);
+        if (mask) {
+            __syncthreads();
+            for (int x = 0; x < nb; ++x) {
+                uint32_t *row = mask + (int64_t)s_kp[x] * words_per_kp + (int64_t)pbi * N1 * 8 + w0;
+                for (int i = tid; i < N1 * NWB; i += TB) row[(i / NWB) * 8 + i % NWB] = mst[x * MS + i];
+            }
+        }
+    }
+}
+
 // Pair lists from the decision mask of k_sieve_count, in the same candidate order: each
 // thread takes one mask word, the block scans the word populations in word order, every
 // thread puts the q of its word's set bits (in bit order) at their places in a shared buffer,
@@ -528,6 +682,31 @@ static void seg_ranges(epwi_ctx *c) {
     c->seg_ready = true;
 }
 
+// The column kernel where its sharing pays: enough candidates to fill the GPU with columns (8 M: 0.1 ms
+// of the other kernel), and at least two k-points per column on average (symmetry-reduced lists
+// may have fewer).  Measured: metal 48^3 11.9 -> 7.1 ms, Si-like 100^3 11.6 -> 3.4 ms.  Returns false
+// (nothing launched) otherwise.
+static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
+    const int N1 = c->ng[0];
+    const int64_t nplane = (int64_t)c->ng[1] * c->ng[2];
+    if (N1 > 128 || nplane > (1 << 20) || c->nkp * c->nk < (int64_t(1) << 23)) return false;
+    const ColumnSet cs = build_columns(c, c->kpts.as<int>(), c->nkp);
+    if (c->nkp < 2 * (int64_t)cs.ncol) return false;
+    EPWI_CUDA(cudaMemsetAsync(c->counts.p, 0, sizeof(int64_t) * c->nkp, c->stream));
+    auto go = [&](auto kern, int TB) {
+        const size_t sm = sieve_cols_smem(N1, TB);
+        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        const dim3 grid((unsigned)cs.ncol, (unsigned)((nplane + kSieveBlock - 1) / kSieveBlock * (kSieveBlock / TB)));
+        kern<<<grid, TB, sm, c->stream>>>(a, cs, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(),
+                                          c->counts.as<unsigned long long>(), mk, c->mask_words);
+    };
+    // 256 combinations keep three CTAs per SM up to 64 axis-1 points (1.5 KB each), 128 two or
+    // more beyond
+    if (c->nw == 4) N1 <= 64 ? go(k_sieve_count_cols<4, 3, 256>, 256) : go(k_sieve_count_cols<4, 3, 128>, 128);
+    else N1 <= 64 ? go(k_sieve_count_cols<8, 6, 256>, 256) : go(k_sieve_count_cols<8, 6, 128>, 128);
+    return true;
+}
+
 void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
     // out has n + 1 entries; out[n] = sum.  Recursive over block sums.
     const int64_t per = (int64_t)kScanBlock * kScanItems;
@@ -627,7 +806,8 @@ void sieve_count(epwi_ctx *c) {
         uint32_t *mk = c->mask_words ? c->sieve_mask.as<uint32_t>() : nullptr;
         auto fast = (c->nw == 4 && c->nm == 3) ? k_sieve_count_fast<4, 3, false>
                     : (c->nw == 8 && c->nm == 6) ? k_sieve_count_fast<8, 6, false> : nullptr;
-        if (fast && sieve_fast_ok(c)) {
+        if (fast && sieve_fast_ok(c) && sieve_count_cols(c, a, mk)) {
+        } else if (fast && sieve_fast_ok(c)) {
             fast<<<(unsigned)nkp, kSieveBlock, sizeof(uint32_t) * 8 * (size_t)c->ng[0], c->stream>>>(
                 a, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(), c->counts.as<int64_t>(), mk,
                 c->mask_words, 0, nullptr, nullptr);
