@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("name,grid,half,eta", [
-    ("al_like", (18, 17, 19), 0.3, 0.02),         # two plane blocks, the second one partial
-    ("al_like", (18, 17, 19), 0.5, 0.002),        # c eta below the phonon energies: exact per-mode test
+    ("al_like", (18, 15, 20), 0.3, 0.02),         # two plane blocks, the second one partial
+    ("al_like", (18, 15, 20), 0.5, 0.002),        # c eta below the phonon energies: exact per-mode test
     ("al_like", (48, 10, 11), 1.5, 0.01),         # up to 48 k-points per column: three passes, several bands
     ("al_like", (70, 9, 9), 0.4, 0.02),           # beyond 64 axis-1 points: 128 threads
     ("si_like", (20, 15, 16), 2.0, 0.01),         # eight bands
