@@ -1,8 +1,14 @@
 // Interpolated electrons and phonons on the full grid (Sec. II B, Eqs. 4-6; Sec. III A
-// preprocessing): H(k) and D(q) Fourier sums with exact integer phase reduction, FP64
-// cyclic complex Jacobi, band velocities and phonon displacement vectors.
+// preprocessing): H(k) and D(q) Fourier sums with exact integer phase reduction, Jacobi
+// eigensolvers with FP64 results (jacobi.cuh), band velocities and phonon displacement vectors.
 //
-// One thread owns one grid point.  Each point is diagonalised once (Nk + Nq solves); the
+// One thread owns one grid point (matrices of up to 8 rows; a warp beyond).  The FP64 units
+// bind: per point the kernels form only the upper triangle of the Hermitian sums, and the
+// launches use small blocks on small grids so that every SM's FP64 unit has work.  Measured on one
+// GB300 against plain FP64 Jacobi sweeps (FP64 sweeps after an FP32 start for 8 and 6 rows), all
+// eigensolves and velocities of a step: Si-like 100^3 (8 and 6 rows) 65 -> 40.5 ms, metal 48^3 (4 and
+// 3 rows) 2.9 -> 0.96 ms, tiny 8^3 0.57 -> 0.20 ms; seven systems of up to 24 rows one after the other
+// 15 -> 7.5 ms.  Each point is diagonalised once (Nk + Nq solves); the
 // scattering loops gather V(k+q), u(q) from these tables instead of re-diagonalising per
 // pair.
 #include <algorithm>
@@ -95,7 +101,7 @@ __global__ void k_fac_axis2(int D, int rc, int N2, int N3, int s2, int L, int E,
 
 // The axis-2 stage output U[s][n1][k2 k3][e] of a factorised build (sources s = 0, 1, 2).
 struct FacDesc {
-    const double2 *U;
+    const double2 *U = nullptr;      // NULL: direct sums over the R-set
     int D, rc;
     int64_t plane;                   // N2 N3
 };
@@ -103,10 +109,11 @@ struct Lattice {
     double a[3][3];                  // rows a_1, a_2, a_3 (A)
 };
 
-// Electrons: eps (ascending), V (columns), velocities, FP32 copies.  FAC: H(k) and dH/dk from
-// the factorised stages (fac, lattice rows lat) instead of direct sums over the R-set.
-template <int WMAX, bool FAC>
-__global__ void __launch_bounds__(128) k_eig_el(GridInfo g, int64_t nk, int W, int nR,
+// Electrons: eps (ascending), V (columns), velocities, FP32 copies.
+// fac.U given: H(k) from the factorised stages (and no velocities); otherwise direct sums, with the
+// velocities of every point when do_vel is set.
+template <int WMAX, bool FIXED>
+__global__ void __launch_bounds__(128) k_eig_el(GridInfo g, int64_t nk, int W_, int nR,
                                                 const int *__restrict__ R,
                                                 const double *__restrict__ Rcart,
                                                 const double2 *__restrict__ Hw,
@@ -118,126 +125,139 @@ __global__ void __launch_bounds__(128) k_eig_el(GridInfo g, int64_t nk, int W, i
                                                 FacDesc fac, Lattice lat, int do_vel) {
     int64_t ik = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ik >= nk) return;
+    const int W = FIXED ? WMAX : W_;
+    constexpr int U = WMAX <= 4 ? WMAX : 1;
     int i1, i2, i3;
     grid_coords(g, ik, i1, i2, i3);
     const int a1 = (int)((int64_t)i1 * g.s1 % g.L), a2 = (int)((int64_t)i2 * g.s2 % g.L),
               a3 = (int)((int64_t)i3 * g.s3 % g.L);
-    double2 A[WMAX * WMAX], Vm[WMAX * WMAX];
+    double2 A[WMAX * WMAX], Vm[WMAX * WMAX];      // A: upper triangle
     const int WW = W * W;
     const int64_t pp = (int64_t)i2 * g.n3 + i3;   // (k2, k3) of this point (factorised build)
-    for (int e = 0; e < WW; ++e) A[e] = make_double2(0, 0);
-    if constexpr (FAC) {
-        for (int j = 0; j < fac.D; ++j) {
-            const double2 p = axis_ph(ph, j - fac.rc, a1, g.L);
-            const double2 *u = fac.U + ((int64_t)j * fac.plane + pp) * WW;
-            for (int e = 0; e < WW; ++e) A[e] = cfma(p, u[e], A[e]);
-        }
+#pragma unroll U
+    for (int i = 0; i < W; ++i)
+#pragma unroll U
+        for (int j = i; j < W; ++j) A[i * WMAX + j] = make_double2(0, 0);
+    auto add = [&](double2 p, const double2 *h) {
+#pragma unroll U
+        for (int i = 0; i < W; ++i)
+#pragma unroll U
+            for (int j = i; j < W; ++j) A[i * WMAX + j] = cfma(p, h[i * W + j], A[i * WMAX + j]);
+    };
+    if (fac.U) {
+        for (int j = 0; j < fac.D; ++j)
+            add(axis_ph(ph, j - fac.rc, a1, g.L), fac.U + ((int64_t)j * fac.plane + pp) * WW);
     } else {
-        for (int r = 0; r < nR; ++r) {
-            const double2 p = ph[phase_index(a1, a2, a3, R[3 * r], R[3 * r + 1], R[3 * r + 2], g.L)];
-            const double2 *h = Hw + (size_t)r * WW;
-            for (int e = 0; e < WW; ++e) A[e] = cfma(p, h[e], A[e]);
-        }
+        for (int r = 0; r < nR; ++r)
+            add(ph[phase_index(a1, a2, a3, R[3 * r], R[3 * r + 1], R[3 * r + 2], g.L)], Hw + (size_t)r * WW);
     }
     double w[WMAX];
-    // FP64 results either way; the mixed solver where the FP64 Jacobi binds (8 x 8)
-    int ok = WMAX >= 8 ? jacobi_hermitian_mixed<WMAX>(A, Vm, W, w) : jacobi_hermitian<WMAX>(A, Vm, W, w);
-    if (!ok) atomicAdd(flag, 1);
+    if (!eig_hermitian<WMAX>(A, Vm, W, w)) atomicAdd(flag, 1);
+#pragma unroll U
     for (int n = 0; n < W; ++n) {
         eps[ik * W + n] = w[n];
         eps32[ik * W + n] = (float)w[n];
     }
-    for (int e = 0; e < WW; ++e) {
-        Vout[ik * WW + e] = Vm[e];
-        V32[ik * WW + e] = make_float2((float)Vm[e].x, (float)Vm[e].y);
-    }
+#pragma unroll U
+    for (int i = 0; i < W; ++i)
+#pragma unroll U
+        for (int j = 0; j < W; ++j) {
+            const double2 v = Vm[i * WMAX + j];
+            Vout[ik * WW + i * W + j] = v;
+            V32[ik * WW + i * W + j] = make_float2((float)v.x, (float)v.y);
+        }
     if (!do_vel) return;                 // velocities later, for the k-points that need them
-    // v_n,a = (1/hbar) Re[V^dag (sum_R w_R i R_a e^{ik.R} H(R)) V]_nn, one axis at a time
+    // v_n,a = (1/hbar) Re[V^dag (sum_R w_R i R_a e^{ik.R} H(R)) V]_nn, one axis at a time (direct
+    // sums: the factorised build leaves the velocities to k_vel_fac)
     for (int ax = 0; ax < 3; ++ax) {
-        for (int e = 0; e < WW; ++e) A[e] = make_double2(0, 0);
-        if constexpr (FAC) {
-            // i R_a = i (n1 A_1a + n2 A_2a + n3 A_3a): U_0 weighted by n1, U_1 (n2 sums), U_2 (n3 sums)
-            const int64_t src = (int64_t)fac.D * fac.plane * WW;
-            for (int j = 0; j < fac.D; ++j) {
-                const int n1 = j - fac.rc;
-                const double2 p = axis_ph(ph, n1, a1, g.L);
-                const double2 ip = make_double2(-p.y, p.x);   // i e1
-                const double c0 = n1 * lat.a[0][ax], c1 = lat.a[1][ax], c2 = lat.a[2][ax];
-                const double2 *u = fac.U + ((int64_t)j * fac.plane + pp) * WW;
-                for (int e = 0; e < WW; ++e) {
-                    const double2 sr = make_double2(c0 * u[e].x + c1 * u[src + e].x + c2 * u[2 * src + e].x,
-                                                    c0 * u[e].y + c1 * u[src + e].y + c2 * u[2 * src + e].y);
-                    A[e] = cfma(ip, sr, A[e]);
-                }
-            }
-        } else {
-            for (int r = 0; r < nR; ++r) {
-                const double2 p = ph[phase_index(a1, a2, a3, R[3 * r], R[3 * r + 1], R[3 * r + 2], g.L)];
-                const double ra = Rcart[3 * r + ax];
-                const double2 ip = make_double2(-ra * p.y, ra * p.x);   // i R_a e^{ik.R}
-                const double2 *h = Hw + (size_t)r * WW;
-                for (int e = 0; e < WW; ++e) A[e] = cfma(ip, h[e], A[e]);
-            }
+        for (int i = 0; i < W; ++i)
+            for (int j = i; j < W; ++j) A[i * WMAX + j] = make_double2(0, 0);
+        for (int r = 0; r < nR; ++r) {
+            const double2 p = ph[phase_index(a1, a2, a3, R[3 * r], R[3 * r + 1], R[3 * r + 2], g.L)];
+            const double ra = Rcart[3 * r + ax];
+            add(make_double2(-ra * p.y, ra * p.x), Hw + (size_t)r * WW);   // i R_a e^{ik.R}
         }
         for (int n = 0; n < W; ++n) {
             double acc = 0;
             for (int i = 0; i < W; ++i) {
-                double2 t = make_double2(0, 0);
-                for (int j = 0; j < W; ++j) t = cfma(A[i * W + j], Vm[j * W + n], t);
-                acc += Vm[i * W + n].x * t.x + Vm[i * W + n].y * t.y;   // Re(conj(V_in) t)
+                const double2 vi = Vm[i * WMAX + n];
+                acc = fma(A[i * WMAX + i].x, fma(vi.x, vi.x, vi.y * vi.y), acc);
+                for (int j = i + 1; j < W; ++j) {
+                    const double2 c = cmulc(vi, Vm[j * WMAX + n]);
+                    acc = fma(2.0, fma(A[i * WMAX + j].x, c.x, -A[i * WMAX + j].y * c.y), acc);
+                }
             }
             vel[(ik * W + n) * 3 + ax] = acc / epc::kHbarEVs * 1e-10;
         }
     }
 }
 
-// Band velocities from the factorised stages and the stored eigenvectors (the velocity part of
-// k_eig_el<WMAX, true>, same arithmetic), for the grid points with win_n > 0 (every point when
-// win_n is NULL).
-template <int WMAX>
-__global__ void __launch_bounds__(128) k_vel_fac(GridInfo g, int64_t nk, int W, const int *__restrict__ win_n,
+// Band velocities from the factorised stages and the stored eigenvectors for the grid points with
+// win_n > 0 (every point when win_n is NULL): with S_b(k) = sum_R n_b e^{ik.R} H(R) from the three
+// sources, dH/dk_a = i sum_b A_ba S_b, so the expectation values of the Hermitian i S_b are taken
+// once per lattice axis b and combined at the end.
+template <int WMAX, bool FIXED>
+__global__ void __launch_bounds__(128) k_vel_fac(GridInfo g, int64_t nk, int W_, const int *__restrict__ win_n,
                                                  const double2 *__restrict__ ph, const double2 *__restrict__ Vin,
                                                  double *__restrict__ vel, FacDesc fac, Lattice lat) {
     const int64_t ik = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ik >= nk || (win_n && win_n[ik] == 0)) return;
+    const int W = FIXED ? WMAX : W_;
+    constexpr int U = WMAX <= 4 ? WMAX : 1;
     int i1, i2, i3;
     grid_coords(g, ik, i1, i2, i3);
     const int a1 = (int)((int64_t)i1 * g.s1 % g.L);
     const int WW = W * W;
     const int64_t pp = (int64_t)i2 * g.n3 + i3;
-    double2 A[WMAX * WMAX], Vm[WMAX * WMAX];
-    for (int e = 0; e < WW; ++e) Vm[e] = Vin[ik * WW + e];
     const int64_t src = (int64_t)fac.D * fac.plane * WW;
-    for (int ax = 0; ax < 3; ++ax) {
-        for (int e = 0; e < WW; ++e) A[e] = make_double2(0, 0);
-        for (int j = 0; j < fac.D; ++j) {
-            const int n1 = j - fac.rc;
+    const double2 *V = Vin + ik * WW;
+    double ex[3][WMAX];                           // <n| i S_b |n>
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        double2 M[WMAX * WMAX];                   // upper triangle of i S_b
+#pragma unroll U
+        for (int i = 0; i < W; ++i)
+#pragma unroll U
+            for (int j = i; j < W; ++j) M[i * WMAX + j] = make_double2(0, 0);
+        for (int d = 0; d < fac.D; ++d) {
+            const int n1 = d - fac.rc;
             const double2 p = axis_ph(ph, n1, a1, g.L);
-            const double2 ip = make_double2(-p.y, p.x);   // i e1
-            const double c0 = n1 * lat.a[0][ax], c1 = lat.a[1][ax], c2 = lat.a[2][ax];
-            const double2 *u = fac.U + ((int64_t)j * fac.plane + pp) * WW;
-            for (int e = 0; e < WW; ++e) {
-                const double2 sr = make_double2(c0 * u[e].x + c1 * u[src + e].x + c2 * u[2 * src + e].x,
-                                                c0 * u[e].y + c1 * u[src + e].y + c2 * u[2 * src + e].y);
-                A[e] = cfma(ip, sr, A[e]);
-            }
+            const double s = b == 0 ? (double)n1 : 1.0;                    // the axis-1 weight is applied here
+            const double2 ip = make_double2(-s * p.y, s * p.x);            // i n_1 e1 or i e1
+            const double2 *u = fac.U + b * src + ((int64_t)d * fac.plane + pp) * WW;
+#pragma unroll U
+            for (int i = 0; i < W; ++i)
+#pragma unroll U
+                for (int j = i; j < W; ++j) M[i * WMAX + j] = cfma(ip, u[i * W + j], M[i * WMAX + j]);
         }
+#pragma unroll U
         for (int n = 0; n < W; ++n) {
             double acc = 0;
+#pragma unroll U
             for (int i = 0; i < W; ++i) {
-                double2 t = make_double2(0, 0);
-                for (int j = 0; j < W; ++j) t = cfma(A[i * W + j], Vm[j * W + n], t);
-                acc += Vm[i * W + n].x * t.x + Vm[i * W + n].y * t.y;   // Re(conj(V_in) t)
+                const double2 vi = V[i * W + n];
+                acc = fma(M[i * WMAX + i].x, fma(vi.x, vi.x, vi.y * vi.y), acc);
+#pragma unroll U
+                for (int j = i + 1; j < W; ++j) {
+                    const double2 c = cmulc(vi, V[j * W + n]);             // conj(v_i) v_j
+                    acc = fma(2.0, fma(M[i * WMAX + j].x, c.x, -M[i * WMAX + j].y * c.y), acc);
+                }
             }
-            vel[(ik * W + n) * 3 + ax] = acc / epc::kHbarEVs * 1e-10;
+            ex[b][n] = acc;
         }
     }
+#pragma unroll U
+    for (int n = 0; n < W; ++n)
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax)
+            vel[(ik * W + n) * 3 + ax] =
+                (lat.a[0][ax] * ex[0][n] + lat.a[1][ax] * ex[1][n] + lat.a[2][ax] * ex[2][n]) * (1e-10 / epc::kHbarEVs);
 }
 
-// Phonons: hbar*omega, u = e (hbar^2 / (2 m hbar omega))^{1/2}, FP32 copies.  FAC: D(q) from
-// the factorised stages.
-template <int NMAX, bool FAC>
-__global__ void __launch_bounds__(128) k_eig_ph(GridInfo g, int64_t nq, int Nm, int nR,
+// Phonons: hbar*omega, u = e (hbar^2 / (2 m hbar omega))^{1/2}, FP32 copies; D(q) from the
+// factorised stages when fac.U is given.
+template <int NMAX, bool FIXED>
+__global__ void __launch_bounds__(128) k_eig_ph(GridInfo g, int64_t nq, int Nm_, int nR,
                                                 const int *__restrict__ R,
                                                 const double *__restrict__ Phiw,
                                                 const double *__restrict__ mode_mass,
@@ -249,34 +269,45 @@ __global__ void __launch_bounds__(128) k_eig_ph(GridInfo g, int64_t nq, int Nm, 
                                                 FacDesc fac) {
     int64_t iq = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (iq >= nq) return;
+    const int Nm = FIXED ? NMAX : Nm_;
+    constexpr int U = NMAX <= 4 ? NMAX : 1;
     int i1, i2, i3;
     grid_coords(g, iq, i1, i2, i3);
     const int a1 = (int)((int64_t)i1 * g.s1 % g.L), a2 = (int)((int64_t)i2 * g.s2 % g.L),
               a3 = (int)((int64_t)i3 * g.s3 % g.L);
-    double2 A[NMAX * NMAX], E[NMAX * NMAX];
+    double2 A[NMAX * NMAX], E[NMAX * NMAX];       // A: upper triangle
     const int MM = Nm * Nm;
-    for (int e = 0; e < MM; ++e) A[e] = make_double2(0, 0);
-    if constexpr (FAC) {
+#pragma unroll U
+    for (int i = 0; i < Nm; ++i)
+#pragma unroll U
+        for (int j = i; j < Nm; ++j) A[i * NMAX + j] = make_double2(0, 0);
+    if (fac.U) {
         const int64_t pp = (int64_t)i2 * g.n3 + i3;
-        for (int j = 0; j < fac.D; ++j) {
-            const double2 p = axis_ph(ph, j - fac.rc, a1, g.L);
-            const double2 *u = fac.U + ((int64_t)j * fac.plane + pp) * MM;
-            for (int e = 0; e < MM; ++e) A[e] = cfma(p, u[e], A[e]);
+        for (int d = 0; d < fac.D; ++d) {
+            const double2 p = axis_ph(ph, d - fac.rc, a1, g.L);
+            const double2 *u = fac.U + ((int64_t)d * fac.plane + pp) * MM;
+#pragma unroll U
+            for (int i = 0; i < Nm; ++i)
+#pragma unroll U
+                for (int j = i; j < Nm; ++j) A[i * NMAX + j] = cfma(p, u[i * Nm + j], A[i * NMAX + j]);
         }
     } else {
         for (int r = 0; r < nR; ++r) {
             const double2 p = ph[phase_index(a1, a2, a3, R[3 * r], R[3 * r + 1], R[3 * r + 2], g.L)];
             const double *f = Phiw + (size_t)r * MM;
-            for (int e = 0; e < MM; ++e) {
-                A[e].x = fma(p.x, f[e], A[e].x);
-                A[e].y = fma(p.y, f[e], A[e].y);
-            }
+#pragma unroll U
+            for (int i = 0; i < Nm; ++i)
+#pragma unroll U
+                for (int j = i; j < Nm; ++j) {
+                    A[i * NMAX + j].x = fma(p.x, f[i * Nm + j], A[i * NMAX + j].x);
+                    A[i * NMAX + j].y = fma(p.y, f[i * Nm + j], A[i * NMAX + j].y);
+                }
         }
     }
     double lam[NMAX];
-    int ok = NMAX >= 6 ? jacobi_hermitian_mixed<NMAX>(A, E, Nm, lam) : jacobi_hermitian<NMAX>(A, E, Nm, lam);
-    if (!ok) atomicAdd(flag, 1);
+    if (!eig_hermitian<NMAX>(A, E, Nm, lam)) atomicAdd(flag, 1);
     float wmax = -1.f;
+#pragma unroll U
     for (int nu = 0; nu < Nm; ++nu) {
         const double l = lam[nu];
         const double w = (l >= 0 ? 1.0 : -1.0) * sqrt(fabs(l) * epc::kHbar2AmuA2);
@@ -284,9 +315,14 @@ __global__ void __launch_bounds__(128) k_eig_ph(GridInfo g, int64_t nq, int Nm, 
         const bool keep = w >= omega_min;
         hw32[iq * Nm + nu] = keep ? (float)w : -1.0f;
         if (keep) wmax = fmaxf(wmax, (float)w);
+        double amp = 0, mass = -1;                // one root and division per atom
+#pragma unroll U
         for (int m = 0; m < Nm; ++m) {
-            double amp = keep ? sqrt(epc::kHbar2AmuA2 / (2.0 * mode_mass[m] * w)) : 0.0;
-            double2 v = make_double2(E[m * Nm + nu].x * amp, E[m * Nm + nu].y * amp);
+            if (mode_mass[m] != mass) {
+                mass = mode_mass[m];
+                amp = keep ? sqrt(epc::kHbar2AmuA2 / (2.0 * mass * w)) : 0.0;
+            }
+            const double2 v = make_double2(E[m * NMAX + nu].x * amp, E[m * NMAX + nu].y * amp);
             uout[iq * MM + m * Nm + nu] = v;
             u32[iq * MM + m * Nm + nu] = make_float2((float)v.x, (float)v.y);
         }
@@ -362,7 +398,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_eig_el_warp(
         }
     }
     __syncwarp();
-    const int ok = jacobi_hermitian_warp(S.A, S.V, W, ld, S.w, S.rot, S.perm);
+    const int ok = eig_hermitian_warp(S.A, S.V, W, ld, S.w, S.rot, S.perm);
     if (lane == 0 && !ok) atomicAdd(flag, 1);
     if (lane < W) {
         eps[ik * W + lane] = S.w[lane];
@@ -455,7 +491,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_eig_ph_warp(
         }
     }
     __syncwarp();
-    const int ok = jacobi_hermitian_warp(S.A, S.V, Nm, ld, S.w, S.rot, S.perm);
+    const int ok = eig_hermitian_warp(S.A, S.V, Nm, ld, S.w, S.rot, S.perm);
     if (lane == 0 && !ok) atomicAdd(flag, 1);
     // lane = mode nu
     float wmax = -1.f;
@@ -521,6 +557,27 @@ void set_smem_once(K kern, size_t bytes) {
     }
 }
 
+// Threads per block of the thread-per-point kernels: an SM's FP64 unit takes 16 clocks per warp
+// instruction, so a grid's points are spread over all SMs first (32-thread blocks up to 128 points
+// per SM, 64 up to 256).
+static int eig_block(int64_t nk) { return nk <= 152 * 128 ? 32 : nk <= 152 * 256 ? 64 : 128; }
+
+// Velocities of the points with win > 0 (all: NULL) from the electron stage output f.
+static void launch_vel(epwi_ctx *c, const FacDesc &f, const Lattice &lat, const int *win) {
+    const int W = c->nw;
+    const GridInfo g = make_grid_info(c);
+    const int bs = eig_block(win ? c->nk / 2 : c->nk);
+    const unsigned nb = (unsigned)((c->nk + bs - 1) / bs);
+#define VEL_ARGS g, c->nk, W, win, c->ph64.as<double2>(), c->V.as<double2>(), c->vel.as<double>(), f, lat
+    if (W == 1) k_vel_fac<1, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+    else if (W == 4) k_vel_fac<4, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+    else if (W < 4) k_vel_fac<4, false><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+    else if (W == 8) k_vel_fac<8, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+    else k_vel_fac<8, false><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+#undef VEL_ARGS
+    EPWI_CHECK_LAUNCH();
+}
+
 void launch_eigs(epwi_ctx *c) {
     const int64_t nk = c->nk;
     const int W = c->nw, Nm = c->nm;
@@ -537,7 +594,7 @@ void launch_eigs(epwi_ctx *c) {
     c->eig_flag.ensure(sizeof(int) * 2);
     EPWI_CUDA(cudaMemsetAsync(c->eig_flag.p, 0, sizeof(int) * 2, c->stream));
     GridInfo g = make_grid_info(c);
-    const int bs = 128;
+    const int bs = eig_block(nk);
     const unsigned nb = (unsigned)((nk + bs - 1) / bs);
     const int64_t plane = (int64_t)g.n2 * g.n3;
     // factorised build: axis-3 and axis-2 stages into fac_U (sources 0..nsrc-1), axis 1 in the
@@ -602,22 +659,26 @@ void launch_eigs(epwi_ctx *c) {
     }
     FacDesc fe{}, fp{};
     if (fac_el) fe = fac_stages(c->fac_Hc, c->fac_re_r, W * W, true, defer ? c->fac_Uel : c->fac_U);
-    const int do_vel = defer ? 0 : 1;
     c->vel_state = defer ? 0 : 2;
 #define EL_ARGS                                                                              \
     g, nk, W, c->nRe, c->Re.as<int>(), c->Rcart.as<double>(), c->Hw.as<double2>(),            \
         c->ph64.as<double2>(), c->eps.as<double>(), c->eps32.as<float>(), c->V.as<double2>(), \
         c->V32.as<float2>(), c->vel.as<double>(), c->eig_flag.as<int>()
     const unsigned nbw = (unsigned)((nk + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    if (W <= 1) {
-        if (fac_el) k_eig_el<1, true><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, do_vel);
-        else k_eig_el<1, false><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, 1);
-    } else if (W <= 4) {
-        if (fac_el) k_eig_el<4, true><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, do_vel);
-        else k_eig_el<4, false><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, 1);
-    } else if (W <= 8) {
-        if (fac_el) k_eig_el<8, true><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, do_vel);
-        else k_eig_el<8, false><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, 1);
+#define EL_LAUNCH(N, FIXED)                                                                  \
+    do {                                                                                     \
+        k_eig_el<N, FIXED><<<nb, bs, 0, c->stream>>>(EL_ARGS, fe, lat, fac_el ? 0 : 1);      \
+    } while (0)
+    if (W == 1) {
+        EL_LAUNCH(1, true);
+    } else if (W == 4) {
+        EL_LAUNCH(4, true);
+    } else if (W < 4) {
+        EL_LAUNCH(4, false);
+    } else if (W == 8) {
+        EL_LAUNCH(8, true);
+    } else if (W < 8) {
+        EL_LAUNCH(8, false);
     } else {
         const size_t sm = warp_scratch_bytes(W);
         if (fac_el) {
@@ -628,8 +689,10 @@ void launch_eigs(epwi_ctx *c) {
             k_eig_el_warp<false><<<nbw, 32 * kWarpsPerBlock, sm, c->stream>>>(EL_ARGS, fe, lat);
         }
     }
+#undef EL_LAUNCH
 #undef EL_ARGS
     EPWI_CHECK_LAUNCH();
+    if (fac_el && W <= 8 && !defer) launch_vel(c, fe, lat, nullptr);   // before the phonon stages reuse fac_U
 #define PH_ARGS                                                                             \
     g, nk, Nm, c->nRp, c->Rp.as<int>(), c->Phiw.as<double>(), c->mode_mass.as<double>(),     \
         c->ph64.as<double2>(), c->opt.omega_min_eV, c->hw.as<double>(), c->hwmax32.as<float>(), \
@@ -637,12 +700,10 @@ void launch_eigs(epwi_ctx *c) {
         c->u.as<double2>(), c->u32.as<float2>(), c->eig_flag.as<int>() + 1
     // the electron kernel above has read fac_U; the phonon stages reuse the buffers (same stream)
     if (fac_ph) fp = fac_stages(c->fac_Pc, c->fac_rp_r, Nm * Nm, false, c->fac_U);
-    if (Nm <= 3) {
-        if (fac_ph) k_eig_ph<3, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
-        else k_eig_ph<3, false><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
-    } else if (Nm <= 6) {
-        if (fac_ph) k_eig_ph<6, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
-        else k_eig_ph<6, false><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
+    if (Nm == 3) {
+        k_eig_ph<3, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
+    } else if (Nm == 6) {
+        k_eig_ph<6, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
     } else {
         const size_t sm = warp_scratch_bytes(Nm);
         if (fac_ph) {
@@ -659,7 +720,6 @@ void launch_eigs(epwi_ctx *c) {
 
 void ensure_velocities(epwi_ctx *c, bool all) {
     if (c->vel_state == 2 || (!all && c->vel_state == 1)) return;
-    const int W = c->nw;
     GridInfo g = make_grid_info(c);
     FacDesc f;
     f.U = c->fac_Uel.as<double2>();
@@ -669,12 +729,6 @@ void ensure_velocities(epwi_ctx *c, bool all) {
     Lattice lat;
     for (int i = 0; i < 9; ++i) lat.a[i / 3][i % 3] = c->lattice[i];
     const int *win = all ? nullptr : c->win_n.as<int>();
-    const unsigned nb = (unsigned)((c->nk + 127) / 128);
-#define VEL_ARGS g, c->nk, W, win, c->ph64.as<double2>(), c->V.as<double2>(), c->vel.as<double>(), f, lat
-    if (W <= 1) k_vel_fac<1><<<nb, 128, 0, c->stream>>>(VEL_ARGS);
-    else if (W <= 4) k_vel_fac<4><<<nb, 128, 0, c->stream>>>(VEL_ARGS);
-    else k_vel_fac<8><<<nb, 128, 0, c->stream>>>(VEL_ARGS);
-#undef VEL_ARGS
-    EPWI_CHECK_LAUNCH();
+    launch_vel(c, f, lat, win);
     c->vel_state = all ? 2 : 1;
 }
