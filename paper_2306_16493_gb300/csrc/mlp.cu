@@ -221,14 +221,46 @@ __global__ void __launch_bounds__(256) k_wgrad(int64_t n, const float *__restric
     }
 }
 
-// out[i] = sum over slices s (in order) of part[s * len + i]
-__global__ void k_reduce_slices(int64_t len, int nslices, const float *__restrict__ part,
-                                float *__restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len) return;
+// out[i] = sum over slices s of part[s * len + i].  A block owns 32 elements and splits the slices
+// over its eight warps (contiguous ranges, four running sums per lane for loads in flight); the
+// partial sums are added in a fixed order.  (One thread per element walking every slice, and one
+// thread adding all rows of db4, took 2.5 of the 3.4 ms of a 65536-row gradient.)
+__global__ void __launch_bounds__(256) k_reduce_slices(int64_t len, int64_t nslices, const float *__restrict__ part,
+                                                       float *__restrict__ out) {
+    __shared__ float sm[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    const int64_t per = (nslices + 7) / 8, k0 = per * wid, k1 = min(nslices, k0 + per);
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    if (i < len) {
+        int64_t k = k0;
+        for (; k + 4 <= k1; k += 4)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[j] += part[(k + j) * len + i];
+        for (; k < k1; ++k) s[0] += part[k * len + i];
+    }
+    sm[wid][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+    __syncthreads();
+    if (wid == 0 && i < len) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += sm[w][lane];
+        out[i] = t;
+    }
+}
+
+// out[0] = sum of x[0 .. n-1]: one block, strided sums per thread, then a fixed tree.
+__global__ void __launch_bounds__(1024) k_sum_all(int64_t n, const float *__restrict__ x, float *__restrict__ out) {
+    __shared__ float sm[32];
     float s = 0.f;
-    for (int k = 0; k < nslices; ++k) s += part[(int64_t)k * len + i];
-    out[i] = s;
+    for (int64_t i = threadIdx.x; i < n; i += 1024) s += x[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = sm[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) out[0] = s;
+    }
 }
 
 // bf16 copy of the master weights (round to nearest even)
@@ -391,10 +423,9 @@ void weight_grad(epwi_ctx *c, int64_t n, const float *D, const float *X, int64_t
     k_wgrad<K><<<(unsigned)nsl, 256, 0, c->stream>>>(n, D, X, part, partb);
     EPWI_CHECK_LAUNCH();
     float *g = s.grad.as<float>();
-    k_reduce_slices<<<(unsigned)((kHid * K + 255) / 256), 256, 0, c->stream>>>(kHid * K, nsl, part,
-                                                                              g + oW);
+    k_reduce_slices<<<(unsigned)((kHid * K + 31) / 32), 256, 0, c->stream>>>(kHid * K, nsl, part, g + oW);
     EPWI_CHECK_LAUNCH();
-    k_reduce_slices<<<1, kHid, 0, c->stream>>>(kHid, nsl, partb, g + ob);
+    k_reduce_slices<<<kHid / 32, 256, 0, c->stream>>>(kHid, nsl, partb, g + ob);
     EPWI_CHECK_LAUNCH();
 }
 
@@ -460,10 +491,9 @@ double mlp_loss_grad(epwi_ctx *c, int64_t n, const float *X, const float *Y, boo
         // sum over the slice of h3[r][c] dy[r]
         k_wgrad<1><<<(unsigned)nsl, 256, 0, c->stream>>>(n, a.H3, a.dy, part, partb);
         EPWI_CHECK_LAUNCH();
-        k_reduce_slices<<<1, kHid, 0, c->stream>>>(kHid, nsl, part, g + ow4);
+        k_reduce_slices<<<kHid / 32, 256, 0, c->stream>>>(kHid, nsl, part, g + ow4);
         EPWI_CHECK_LAUNCH();
-        // db4: the slice reduction with one element per "slice" sums dy in row order
-        k_reduce_slices<<<1, 32, 0, c->stream>>>(1, (int)n, a.dy, g + ob4);
+        k_sum_all<<<1, 1024, 0, c->stream>>>(n, a.dy, g + ob4);
         EPWI_CHECK_LAUNCH();
     }
     weight_grad<kHid>(c, n, a.D3, a.H2, oW3, ob3);
