@@ -125,31 +125,38 @@ __global__ void k_normalise(int64_t n, float shift, float inv_scale, float *__re
 }
 
 // ------------------------------------------------------------------ proposal
-struct PropArgs {
-    GridInfo g;
-    int W, Nm, s;                 // s = cell stride
-    int c2, c3;                   // cells per axis 2, 3
-    int64_t ncell;
-    const int *st_k, *st_n;
-    const double *eps;
-    double mu;
-};
-
-// Features of proposal rows r0 .. r0+n-1 of the chunk's states starting at global state s0;
-// row = (state * ncell + cell) * Nm + nu.
-__global__ void k_prop_features(PropArgs a, int64_t s0, int64_t r0, int64_t n,
-                                float *__restrict__ X) {
+// The network inputs of the proposal rows (state, cell, mode) depend on the state, on one cell
+// index per axis or on the mode only: tables of make_features' values, each formed in FP64 and
+// rounded once.  (One row of nine FP64 divisions per (state, cell, mode) kept the FP64 units
+// busy for as long as the network itself took.)
+__global__ void k_prop_states(int64_t ns, GridInfo g, int W, int Nm, int64_t s0, const int *__restrict__ st_k,
+                              const int *__restrict__ st_n, const double *__restrict__ eps, double mu,
+                              float *__restrict__ out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int64_t r = r0 + j;
-    const int nu = (int)(r % a.Nm);
-    const int64_t sc = r / a.Nm;
-    const int64_t cell = sc % a.ncell;
-    const int64_t st = s0 + sc / a.ncell;
-    const int ik = a.st_k[st], bn = a.st_n[st];
-    const int c3 = (int)(cell % a.c3), c2 = (int)((cell / a.c3) % a.c2), c1 = (int)(cell / ((int64_t)a.c3 * a.c2));
-    const int64_t iq = grid_index(a.g, a.s * c1, a.s * c2, a.s * c3);
-    make_features(a.g, ik, iq, a.eps[(int64_t)ik * a.W + bn] - a.mu, bn, nu, a.W, a.Nm, X + j * kIn);
+    if (j >= ns) return;
+    const int ik = st_k[s0 + j], bn = st_n[s0 + j];
+    float x[kIn];
+    make_features(g, ik, 0, eps[(int64_t)ik * W + bn] - mu, bn, 0, W, Nm, x);
+    float *o = out + j * 5;
+    o[0] = x[0];
+    o[1] = x[1];
+    o[2] = x[2];
+    o[3] = x[6];
+    o[4] = x[7];
+}
+
+__global__ void k_prop_tables(GridInfo g, int s, int c1, int c2, int c3, int Nm, float *__restrict__ tab) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= c1 + c2 + c3 + Nm) return;
+    float x[kIn];
+    if (e >= c1 + c2 + c3) {
+        make_features(g, 0, 0, 0.0, 0, e - c1 - c2 - c3, 1, Nm, x);
+        tab[e] = x[8];
+        return;
+    }
+    const int ax = e < c1 ? 0 : e < c1 + c2 ? 1 : 2, i = s * (e - (ax > 0 ? c1 : 0) - (ax > 1 ? c2 : 0));
+    make_features(g, 0, grid_index(g, ax == 0 ? i : 0, ax == 1 ? i : 0, ax == 2 ? i : 0), 0.0, 0, 0, 1, Nm, x);
+    tab[e] = x[3 + ax];
 }
 
 // logit[(row0 / Nm) + j] = log sum_nu exp(scale * yhat) over the Nm rows of each (state, cell).
@@ -306,43 +313,56 @@ __device__ __forceinline__ bool keep_draw(const SampleArgs &a, int ik, int nsel,
     return pair_valid(a.sv, nsel, en, en32, q, kplusq(a.g, ik, q));
 }
 
-__global__ void __launch_bounds__(256) k_is_count(SampleArgs a, int64_t *__restrict__ out) {
-    __shared__ int64_t sm[33];
+// Kept draws of each chunk k-point (one block each): their number, and one bit per q (word
+// q / 32) for the fill.
+__global__ void __launch_bounds__(256) k_is_count(SampleArgs a, int64_t words, int64_t *__restrict__ out,
+                                                  uint32_t *__restrict__ kept) {
     __shared__ double en[epc::kMaxW];
     __shared__ float en32[epc::kMaxW];
+    __shared__ int s_n;
     const int ik = a.kpts[blockIdx.x];
     const int nsel = a.win_n[ik];
+    if (threadIdx.x == 0) s_n = 0;
     load_window(a.sv, ik, a.win_lo[ik], nsel, en, en32);
     const int *cn = a.counts + (int64_t)blockIdx.x * a.nq;
-    int64_t c = 0;
-    for (int64_t q = threadIdx.x; q < a.nq; q += blockDim.x)
-        c += cn[q] > 0 && keep_draw(a, ik, nsel, en, en32, q);
-    int64_t tot;
-    block_excl_scan_i64(c, sm, tot);
-    if (threadIdx.x == 0) out[blockIdx.x] = tot;
+    const int lane = threadIdx.x & 31;
+    int c = 0;
+    for (int64_t w = threadIdx.x >> 5; w < words; w += 8) {
+        const int64_t q = w * 32 + lane;
+        const bool k = q < a.nq && cn[q] > 0 && keep_draw(a, ik, nsel, en, en32, q);
+        const uint32_t bits = __ballot_sync(0xffffffffu, k);
+        if (lane == 0) kept[blockIdx.x * words + w] = bits;
+        c += __popc(bits);
+    }
+    if (lane == 0 && c) atomicAdd(&s_n, c);
+    __syncthreads();
+    if (threadIdx.x == 0) out[blockIdx.x] = s_n;
 }
 
-// Ordered compaction of the drawn q of each chunk k-point (one block each) with their
-// weights c / (S p(q)).
-__global__ void __launch_bounds__(256) k_is_fill(SampleArgs a, const int64_t *__restrict__ off,
-                                                 int *__restrict__ pairs, double *__restrict__ w) {
+// Ordered compaction of the kept draws of each chunk k-point (one block each) with their weights
+// c / (S p(q)): every thread takes a contiguous range of the k-point's words and one scan of the
+// ranges' populations places them.
+__global__ void __launch_bounds__(256) k_is_fill(SampleArgs a, int64_t words, const uint32_t *__restrict__ kept,
+                                                 const int64_t *__restrict__ off, int *__restrict__ pairs,
+                                                 double *__restrict__ w) {
     __shared__ int64_t sm[33];
-    __shared__ double en[epc::kMaxW];
-    __shared__ float en32[epc::kMaxW];
     const int64_t kpl = blockIdx.x;
     const int ik = a.kpts[kpl];
     const int nwin = a.win_n[ik];
-    load_window(a.sv, ik, a.win_lo[ik], nwin, en, en32);
     const int64_t st0 = a.kp_state[kpl] - a.s_base;
     const int *cn = a.counts + kpl * a.nq;
-    int64_t base = off[kpl];
+    const uint32_t *kw = kept + kpl * words;
     const double inv_s3 = 1.0 / ((double)a.s * a.s * a.s);
-    for (int64_t q0 = 0; q0 < a.nq; q0 += blockDim.x) {
-        const int64_t q = q0 + threadIdx.x;
-        const int cnt = q < a.nq && cn[q] > 0 && keep_draw(a, ik, nwin, en, en32, q) ? cn[q] : 0;
-        int64_t tot;
-        const int64_t ex = block_excl_scan_i64(cnt > 0, sm, tot);
-        if (cnt > 0) {
+    const int64_t per = (words + blockDim.x - 1) / blockDim.x;
+    const int64_t w0 = min(words, per * threadIdx.x), w1 = min(words, w0 + per);
+    int64_t n = 0, tot;
+    for (int64_t x = w0; x < w1; ++x) n += __popc(kw[x]);
+    int64_t o = off[kpl] + block_excl_scan_i64(n, sm, tot);
+    for (int64_t x = w0; x < w1; ++x) {
+        uint32_t bits = kw[x];
+        while (bits) {
+            const int64_t q = x * 32 + __ffs(bits) - 1;
+            bits &= bits - 1;
             double p = 1.0 / (double)a.nq;
             if (a.cdf) {
                 int i1, i2, i3;
@@ -359,10 +379,10 @@ __global__ void __launch_bounds__(256) k_is_fill(SampleArgs a, const int64_t *__
                 }
                 p = pm / nwin;
             }
-            pairs[base + ex] = (int)q;
-            w[base + ex] = (double)cnt / ((double)a.S * p);
+            pairs[o] = (int)q;
+            w[o] = (double)cn[q] / ((double)a.S * p);
+            ++o;
         }
-        base += tot;
     }
 }
 
@@ -581,19 +601,18 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
     int64_t kpc = std::max<int64_t>(1, (int64_t(1) << 30) / (4 * nq));
     if (learned) kpc = std::min<int64_t>(kpc, std::max<int64_t>(1, (int64_t(1) << 31) / (12 * ncell * max_w)));
     kpc = std::min<int64_t>(kpc, std::max<int64_t>(1, (int64_t(1) << 30) / std::max<int64_t>(1, S)));
-    DevBuf counts, cdf, tot, logit, xb, yb, cnt, off;
+    DevBuf counts, cdf, tot, logit, fs, tab, yb, cnt, off, kept;
     std::vector<DevBuf> chunk_pairs, chunk_w;
     std::vector<int64_t> kp_off(nkp + 1, 0);
     double flops = 0;
     float ms_prop = 0;
     auto cleanup = [&] {
-        counts.release(); cdf.release(); tot.release(); logit.release(); xb.release();
-        yb.release(); cnt.release(); off.release();
+        counts.release(); cdf.release(); tot.release(); logit.release(); fs.release();
+        tab.release(); yb.release(); cnt.release(); off.release(); kept.release();
         for (auto &b : chunk_pairs) b.release();
         for (auto &b : chunk_w) b.release();
     };
     try {
-        const int64_t rows_per_batch = (((int64_t)1 << 22) / c->nm) * c->nm;
         for (int64_t kp0 = 0; kp0 < nkp; kp0 += kpc) {
             const int64_t kp1 = std::min(nkp, kp0 + kpc), nkc = kp1 - kp0;
             const int64_t s0 = h_state[kp0], nsc = h_state[kp1] - s0;
@@ -623,31 +642,33 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
                 logit.ensure(sizeof(float) * nsc * ncell);
                 cdf.ensure(sizeof(double) * nsc * ncell);
                 tot.ensure(sizeof(double) * (nsc + 1));
-                xb.ensure(sizeof(float) * rows_per_batch * kIn);
-                yb.ensure(sizeof(float) * rows_per_batch);
-                PropArgs pa;
-                pa.g = g;
-                pa.W = c->nw;
-                pa.Nm = c->nm;
-                pa.s = s;
-                pa.c2 = c2;
-                pa.c3 = c3;
-                pa.ncell = ncell;
-                pa.st_k = c->st_k.as<int>();
-                pa.st_n = c->st_n.as<int>();
-                pa.eps = c->eps.as<double>();
-                pa.mu = mu;
-                const int64_t rows = nsc * ncell * c->nm;
-                for (int64_t r0 = 0; r0 < rows; r0 += rows_per_batch) {
-                    const int64_t nr = std::min(rows_per_batch, rows - r0);
-                    k_prop_features<<<(unsigned)((nr + 255) / 256), 256, 0, st>>>(pa, s0, r0, nr,
-                                                                                   xb.as<float>());
-                    EPWI_CHECK_LAUNCH();
-                    mlp_forward_fast(c, nr, xb.as<float>(), yb.as<float>());
-                    const int64_t ng = nr / c->nm;
+                const int64_t per_state = ncell * c->nm, rows = nsc * per_state;
+                // whole states per launch, at most 2^28 rows (1 GiB of outputs)
+                const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nsc, (int64_t(1) << 28) / per_state));
+                EPWI_REQUIRE(per_state < (int64_t(1) << 31), EPWI_EUNSUPPORTED, "too many cells and modes");
+                yb.ensure(sizeof(float) * batch * per_state);
+                fs.ensure(sizeof(float) * 5 * nsc);
+                tab.ensure(sizeof(float) * (c1 + c2 + c3 + c->nm));
+                k_prop_states<<<(unsigned)((nsc + 127) / 128), 128, 0, st>>>(nsc, g, c->nw, c->nm, s0, c->st_k.as<int>(),
+                                                                           c->st_n.as<int>(), c->eps.as<double>(), mu,
+                                                                           fs.as<float>());
+                EPWI_CHECK_LAUNCH();
+                k_prop_tables<<<(unsigned)((c1 + c2 + c3 + c->nm + 127) / 128), 128, 0, st>>>(g, s, c1, c2, c3, c->nm,
+                                                                                            tab.as<float>());
+                EPWI_CHECK_LAUNCH();
+                PropRows pr;
+                pr.Nm = c->nm;
+                pr.ncell = (int)ncell;
+                pr.c1 = c1;
+                pr.c2 = c2;
+                pr.c3 = c3;
+                pr.tab = tab.as<float>();
+                for (int64_t b0 = 0; b0 < nsc; b0 += batch) {
+                    const int64_t nb = std::min(batch, nsc - b0), ng = nb * ncell;
+                    pr.state = fs.as<float>() + 5 * b0;
+                    mlp_forward_fast(c, nb * per_state, nullptr, yb.as<float>(), &pr);
                     k_prop_lse<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(
-                        ng, c->nm, (float)c->mlp->out_scale, yb.as<float>(),
-                        logit.as<float>() + r0 / c->nm);
+                        ng, c->nm, (float)c->mlp->out_scale, yb.as<float>(), logit.as<float>() + b0 * ncell);
                     EPWI_CHECK_LAUNCH();
                 }
                 flops += 2.0 * (double)rows * (kIn * kHid + 2.0 * kHid * kHid + kHid);
@@ -674,7 +695,9 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
             }
             cnt.ensure(sizeof(int64_t) * (nkc + 1));
             off.ensure(sizeof(int64_t) * (nkc + 1));
-            k_is_count<<<(unsigned)nkc, 256, 0, st>>>(sa, cnt.as<int64_t>());
+            const int64_t words = (nq + 31) / 32;
+            kept.ensure(sizeof(uint32_t) * nkc * words);
+            k_is_count<<<(unsigned)nkc, 256, 0, st>>>(sa, words, cnt.as<int64_t>(), kept.as<uint32_t>());
             EPWI_CHECK_LAUNCH();
             int64_t npc = 0;
             scan_exclusive_i64(c, cnt.as<int64_t>(), off.as<int64_t>(), nkc, &npc);
@@ -684,8 +707,8 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
             chunk_w.emplace_back();
             chunk_pairs.back().ensure(sizeof(int) * (npc + 1));
             chunk_w.back().ensure(sizeof(double) * (npc + 1));
-            k_is_fill<<<(unsigned)nkc, 256, 0, st>>>(sa, off.as<int64_t>(), chunk_pairs.back().as<int>(),
-                                                     chunk_w.back().as<double>());
+            k_is_fill<<<(unsigned)nkc, 256, 0, st>>>(sa, words, kept.as<uint32_t>(), off.as<int64_t>(),
+                                                     chunk_pairs.back().as<int>(), chunk_w.back().as<double>());
             EPWI_CHECK_LAUNCH();
             EPWI_CUDA(cudaStreamSynchronize(st));
         }

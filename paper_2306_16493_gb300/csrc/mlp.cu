@@ -524,11 +524,12 @@ double mlp_dataset_loss(epwi_ctx *c) {
     return 0.5 * t / (double)n;
 }
 
-void mlp_forward_fast(epwi_ctx *c, int64_t n, const float *X, float *y) {
+void mlp_forward_fast(epwi_ctx *c, int64_t n, const float *X, float *y, const PropRows *pr) {
     MlpState &s = state(c);
     s.err.ensure(sizeof(int));
     EPWI_CUDA(cudaMemsetAsync(s.err.p, 0, sizeof(int), c->stream));
-    mlp_forward_tc(c, n, X, y, s.err.as<int>());
+    if (pr) mlp_proposal_tc(c, n, *pr, y, s.err.as<int>());
+    else mlp_forward_tc(c, n, X, y, s.err.as<int>());
     int h = 0;
     EPWI_CUDA(cudaMemcpyAsync(&h, s.err.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     EPWI_CUDA(cudaStreamSynchronize(c->stream));

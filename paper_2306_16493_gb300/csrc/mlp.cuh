@@ -68,10 +68,19 @@ double mlp_loss_grad(epwi_ctx *c, int64_t n, const float *X, const float *Y,
                      bool want_loss = true);
 double mlp_dataset_loss(epwi_ctx *c);
 void mlp_train_graph(epwi_ctx *c, const std::vector<StepParams> &steps, int64_t B);
+// Rows (state, cell, mode) of the proposal, mode fastest: inputs put together in the kernel.
+struct PropRows {
+    int Nm = 1, ncell = 1, c1 = 1, c2 = 1, c3 = 1;   // modes, cells, cells per axis
+    const float *state = nullptr;     // [state][5]: k coordinates, energy, band inputs
+    const float *tab = nullptr;       // [c1 + c2 + c3 + Nm]: q coordinate of each cell index, mode input
+};
+
 // mlp_tc.cu: the same forward pass on the tensor cores (BF16 activations between layers)
-int mlp_forward_tc(epwi_ctx *c, int64_t n, const float *X, float *y, int *err_dev);
-// tensor-core forward with its error check (throws EPWI_ETIMEOUT)
-void mlp_forward_fast(epwi_ctx *c, int64_t n, const float *X, float *y);
+void mlp_forward_tc(epwi_ctx *c, int64_t n, const float *X, float *y, int *err_dev);
+// the same for the n < 2^31 proposal rows of pr
+void mlp_proposal_tc(epwi_ctx *c, int64_t n, const PropRows &pr, float *y, int *err_dev);
+// tensor-core forward with its error check (throws EPWI_ETIMEOUT): X or pr gives the rows
+void mlp_forward_fast(epwi_ctx *c, int64_t n, const float *X, float *y, const PropRows *pr = nullptr);
 
 // learned.cu
 void mlp_train(epwi_ctx *c, double T, double mu, double eta, double emin, double emax,
