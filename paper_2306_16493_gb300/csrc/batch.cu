@@ -541,6 +541,9 @@ struct epwi_batch {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    // branches of the captured step (see plan): used during the capture only
+    std::vector<cudaStream_t> branch;
+    std::vector<cudaEvent_t> branch_ev;      // fork, then one join per branch
     epwi_batch_stats stats{};
 
     void drop_graph() {
@@ -553,6 +556,8 @@ struct epwi_batch {
         drop_graph();
         for (auto &e : ev)
             if (e) cudaEventDestroy(e);
+        for (auto &e : branch_ev) cudaEventDestroy(e);
+        for (auto &s : branch) cudaStreamDestroy(s);
         for (auto &b : pairs) b.release();
         for (auto &b : ghat) b.release();
         DevBuf *all[] = {&d_sys, &d_items, &d_order, &d_counter, &d_part, &d_state_item,
@@ -628,15 +633,62 @@ void restage(epwi_batch *b, int s) {
     }
 }
 
-// The per-system work that precedes the persistent kernel in every step.
-void system_prologue(epwi_batch *b, int s) {
+// The per-system work that precedes the persistent kernel in every step: tables, eigensolves and
+// pair lists on stream st, then the Re->k stage (its scratch is shared by the systems).
+void system_prologue(epwi_batch *b, int s, cudaStream_t st) {
     epwi_ctx *c = b->sys[s];
+    struct Swap {
+        epwi_ctx *c;
+        cudaStream_t saved;
+        ~Swap() { c->stream = saved; }
+    } sw{c, c->stream};
+    c->stream = st;
     launch_phase_tables(c);
     launch_eigs(c);
     occupation_tables(c);
     tc_tables(c);
     sieve_fill_chunk(c, 0, c->nkp, b->pairs[s].as<int>());
-    restage(b, s);
+}
+
+// The eigensolves of a batch's small grids leave most of the GPU idle one after the other (a few
+// hundred matrices of FP64 latency each), so the captured step runs the systems' first stages on
+// up to kBranches parallel branches; every buffer they touch belongs to one system.  The Re->k
+// stages follow in line.
+constexpr int kBranches = 8;
+
+void capture_prologues(epwi_batch *b) {
+    const int ns = (int)b->sys.size(), nb = std::min(kBranches, ns);
+    while ((int)b->branch.size() < nb) {
+        cudaStream_t s = nullptr;
+        EPWI_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        b->branch.push_back(s);
+    }
+    while ((int)b->branch_ev.size() < nb + 1) {
+        cudaEvent_t e = nullptr;
+        EPWI_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        b->branch_ev.push_back(e);
+    }
+    EPWI_CUDA(cudaEventRecord(b->branch_ev[0], b->stream));
+    for (int i = 0; i < nb; ++i) EPWI_CUDA(cudaStreamWaitEvent(b->branch[i], b->branch_ev[0], 0));
+    // largest eigensolves first, each to the branch with the least work so far
+    std::vector<int> order(ns);
+    std::iota(order.begin(), order.end(), 0);
+    std::vector<double> work(ns), load(nb, 0.0);
+    for (int s = 0; s < ns; ++s) {
+        const epwi_ctx *c = b->sys[s];
+        work[s] = (double)c->nk * (std::pow((double)c->nw, 3) + std::pow((double)c->nm, 3));
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return work[x] > work[y]; });
+    for (int s : order) {
+        const int i = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        load[i] += work[s];
+        system_prologue(b, s, b->branch[i]);
+    }
+    for (int i = 0; i < nb; ++i) {
+        EPWI_CUDA(cudaEventRecord(b->branch_ev[i + 1], b->branch[i]));
+        EPWI_CUDA(cudaStreamWaitEvent(b->stream, b->branch_ev[i + 1], 0));
+    }
+    for (int s = 0; s < ns; ++s) restage(b, s);
 }
 
 // Items of system s in (k-point, band, q block) order, with their states' item offsets.
@@ -920,7 +972,7 @@ void plan(epwi_batch *b, bool tune) {
     // capture the step
     EPWI_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
     try {
-        for (int s = 0; s < ns; ++s) system_prologue(b, s);
+        capture_prologues(b);
         EPWI_CUDA(cudaMemsetAsync(b->d_counter.p, 0, sizeof(int), st));
         // external event records become graph nodes (a plain record inside a capture does not)
         EPWI_CUDA(cudaEventRecordWithFlags(b->ev[2], st, cudaEventRecordExternal));
