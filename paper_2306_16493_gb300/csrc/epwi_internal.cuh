@@ -203,6 +203,7 @@ struct epwi_ctx {
     DevBuf is_w;                   // double weight count / (S p(q)) per sampled pair
     DevBuf is_kp_pairs;            // int64 [nkp+1] pair offsets of the sampled pairs
     std::vector<int64_t> h_is_kp_pairs;
+    DevBuf is_ws[10];              // workspaces of the draws (learned.cu)
 
     // iterative BTE: Gamma in pair blocks, mean free paths
     bool have_ibte = false;
@@ -238,6 +239,7 @@ struct epwi_ctx {
                          &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
                          &re_cube, &ks_T, &col_buf, &gsf64};
         for (DevBuf *b : all) b->release();
+        for (DevBuf &b : is_ws) b.release();
         mlp_free(mlp);
     }
 };

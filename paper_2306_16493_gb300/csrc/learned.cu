@@ -229,6 +229,7 @@ struct SampleArgs {
     int64_t ncell, nq;
     int64_t S;                     // draws per k-point
     double alpha;
+    uint64_t alpha53;              // (h >> 11) < alpha53 is u53(h) < alpha
     uint64_t seed;
     const int *kpts;               // chunk k-points
     const int64_t *kp_state;       // global state offsets of the chunk k-points
@@ -244,34 +245,36 @@ __device__ __forceinline__ uint64_t draw_key(uint64_t seed, int ik, int64_t s) {
                  0xd1b54a32d192ed03ull * (uint64_t)(s + 1));
 }
 
+// One draw per thread.  The FP64 unit is slow here (1/64 of the FP32 rate) and a draw needs it for
+// one product only: the comparisons of non-negative doubles are made on their bit patterns, and
+// uniforms are compared with alpha, or scaled by a power of two, as the integers they come from.
 __global__ void k_is_sample(SampleArgs a, int64_t nkpc) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nkpc * a.S) return;
-    const int64_t kpl = t / a.S, s = t % a.S;
+    const int64_t kpl = t / a.S, s = t - kpl * a.S;
     const int ik = a.kpts[kpl];
     const uint64_t key = draw_key(a.seed, ik, s);
-    const double u0 = u53(mix64(key + 1)), u1 = u53(mix64(key + 2)), u2 = u53(mix64(key + 3)),
-                 u3 = u53(mix64(key + 4));
+    const uint64_t h1 = mix64(key + 2) >> 11, h2 = mix64(key + 3);
     int64_t iq;
-    if (u1 < a.alpha || !a.cdf) {
-        iq = min((int64_t)(u2 * (double)a.nq), a.nq - 1);
+    if (h1 < a.alpha53 || !a.cdf) {
+        iq = min((int64_t)(u53(h2) * (double)a.nq), a.nq - 1);
     } else {
         const int nwin = a.win_n[ik];
-        const int b = min((int)(u0 * nwin), nwin - 1);
+        const int b = nwin > 1 ? min((int)(u53(mix64(key + 1)) * nwin), nwin - 1) : 0;
         const int64_t st = a.kp_state[kpl] - a.s_base + b;
-        const double *cd = a.cdf + st * a.ncell;
-        const double target = u2 * a.tot[st];
-        int64_t lo = 0, hi = a.ncell - 1;               // first c with cdf[c] > target
+        const long long *cd = reinterpret_cast<const long long *>(a.cdf + st * a.ncell);
+        const long long target = __double_as_longlong(u53(h2) * a.tot[st]);
+        int lo = 0, hi = (int)a.ncell - 1;              // first c with cdf[c] > target
         while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
+            const int mid = (lo + hi) >> 1;
             if (cd[mid] > target) hi = mid;
             else lo = mid + 1;
         }
-        const int64_t cell = lo;
-        const int c3 = (int)(cell % a.c3), c2 = (int)((cell / a.c3) % a.c2),
-                  c1 = (int)(cell / ((int64_t)a.c3 * a.c2));
+        const int cell = lo;
+        const int c12 = cell / a.c3, c3 = cell - c12 * a.c3, c1 = c12 / a.c2, c2 = c12 - c1 * a.c2;
         const int s3 = a.s * a.s * a.s;
-        const int o = min((int)(u3 * s3), s3 - 1);
+        const uint64_t h3 = mix64(key + 4);
+        const int o = (s3 & (s3 - 1)) == 0 ? (int)((h3 >> 11) >> (53 - (__ffs(s3) - 1))) : min((int)(u53(h3) * s3), s3 - 1);
         const int o1 = o / (a.s * a.s), o2 = (o / a.s) % a.s, o3 = o % a.s;
         const int h = a.s / 2;
         const int i1 = (a.s * c1 - h + o1 + a.g.n1) % a.g.n1;
@@ -308,13 +311,16 @@ __device__ __forceinline__ int64_t block_excl_scan_i64(int64_t v, int64_t *sm, i
 }
 
 // A drawn q is evaluated when the sieve keeps (k, q); otherwise every term t(k, q) is zero.
+template <int WT, int NMT>
 __device__ __forceinline__ bool keep_draw(const SampleArgs &a, int ik, int nsel, const double *en,
                                           const float *en32, int64_t q) {
-    return pair_valid(a.sv, nsel, en, en32, q, kplusq(a.g, ik, q));
+    if constexpr (WT > 0) return pair_valid_t<WT, NMT>(a.sv, nsel, en, en32, q, kplusq(a.g, ik, q));
+    else return pair_valid(a.sv, nsel, en, en32, q, kplusq(a.g, ik, q));
 }
 
 // Kept draws of each chunk k-point (one block each): their number, and one bit per q (word
 // q / 32) for the fill.
+template <int WT, int NMT>
 __global__ void __launch_bounds__(256) k_is_count(SampleArgs a, int64_t words, int64_t *__restrict__ out,
                                                   uint32_t *__restrict__ kept) {
     __shared__ double en[epc::kMaxW];
@@ -329,7 +335,7 @@ __global__ void __launch_bounds__(256) k_is_count(SampleArgs a, int64_t words, i
     int c = 0;
     for (int64_t w = threadIdx.x >> 5; w < words; w += 8) {
         const int64_t q = w * 32 + lane;
-        const bool k = q < a.nq && cn[q] > 0 && keep_draw(a, ik, nsel, en, en32, q);
+        const bool k = q < a.nq && cn[q] > 0 && keep_draw<WT, NMT>(a, ik, nsel, en, en32, q);
         const uint32_t bits = __ballot_sync(0xffffffffu, k);
         if (lane == 0) kept[blockIdx.x * words + w] = bits;
         c += __popc(bits);
@@ -601,14 +607,18 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
     int64_t kpc = std::max<int64_t>(1, (int64_t(1) << 30) / (4 * nq));
     if (learned) kpc = std::min<int64_t>(kpc, std::max<int64_t>(1, (int64_t(1) << 31) / (12 * ncell * max_w)));
     kpc = std::min<int64_t>(kpc, std::max<int64_t>(1, (int64_t(1) << 30) / std::max<int64_t>(1, S)));
-    DevBuf counts, cdf, tot, logit, fs, tab, yb, cnt, off, kept;
+    // workspaces of a chunk: kept in the context up to 4 GiB
+    DevBuf &counts = c->is_ws[0], &cdf = c->is_ws[1], &tot = c->is_ws[2], &logit = c->is_ws[3], &fs = c->is_ws[4],
+           &tab = c->is_ws[5], &yb = c->is_ws[6], &cnt = c->is_ws[7], &off = c->is_ws[8], &kept = c->is_ws[9];
     std::vector<DevBuf> chunk_pairs, chunk_w;
     std::vector<int64_t> kp_off(nkp + 1, 0);
     double flops = 0;
     float ms_prop = 0;
     auto cleanup = [&] {
-        counts.release(); cdf.release(); tot.release(); logit.release(); fs.release();
-        tab.release(); yb.release(); cnt.release(); off.release(); kept.release();
+        size_t held = 0;
+        for (auto &b : c->is_ws) held += b.bytes;
+        if (held > (size_t(4) << 30))
+            for (auto &b : c->is_ws) b.release();
         for (auto &b : chunk_pairs) b.release();
         for (auto &b : chunk_w) b.release();
     };
@@ -625,6 +635,7 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
             sa.nq = nq;
             sa.S = S;
             sa.alpha = learned ? alpha : 1.0;
+            sa.alpha53 = (uint64_t)std::ceil(std::ldexp(sa.alpha, 53));
             sa.seed = seed;
             sa.kpts = c->kpts.as<int>() + kp0;
             sa.kp_state = c->kp_state.as<int64_t>() + kp0;
@@ -697,25 +708,33 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
             off.ensure(sizeof(int64_t) * (nkc + 1));
             const int64_t words = (nq + 31) / 32;
             kept.ensure(sizeof(uint32_t) * nkc * words);
-            k_is_count<<<(unsigned)nkc, 256, 0, st>>>(sa, words, cnt.as<int64_t>(), kept.as<uint32_t>());
+            auto count = c->nw == 4 && c->nm == 3   ? k_is_count<4, 3>
+                         : c->nw == 8 && c->nm == 6 ? k_is_count<8, 6>
+                                                    : k_is_count<0, 0>;
+            count<<<(unsigned)nkc, 256, 0, st>>>(sa, words, cnt.as<int64_t>(), kept.as<uint32_t>());
             EPWI_CHECK_LAUNCH();
             int64_t npc = 0;
             scan_exclusive_i64(c, cnt.as<int64_t>(), off.as<int64_t>(), nkc, &npc);
             std::vector<int64_t> ho = download_vec<int64_t>(off, (size_t)nkc + 1, st);
             for (int64_t k = 0; k < nkc; ++k) kp_off[kp0 + k + 1] = kp_off[kp0] + ho[k + 1];
-            chunk_pairs.emplace_back();
-            chunk_w.emplace_back();
-            chunk_pairs.back().ensure(sizeof(int) * (npc + 1));
-            chunk_w.back().ensure(sizeof(double) * (npc + 1));
+            // one chunk writes the final lists; several are put together below
+            const bool one = kp0 == 0 && kp1 == nkp;
+            if (!one) {
+                chunk_pairs.emplace_back();
+                chunk_w.emplace_back();
+            }
+            DevBuf &dp = one ? c->is_pairs : chunk_pairs.back(), &dw = one ? c->is_w : chunk_w.back();
+            dp.ensure(sizeof(int) * (npc + 1));
+            dw.ensure(sizeof(double) * (npc + 1));
             k_is_fill<<<(unsigned)nkc, 256, 0, st>>>(sa, words, kept.as<uint32_t>(), off.as<int64_t>(),
-                                                     chunk_pairs.back().as<int>(), chunk_w.back().as<double>());
+                                                     dp.as<int>(), dw.as<double>());
             EPWI_CHECK_LAUNCH();
             EPWI_CUDA(cudaStreamSynchronize(st));
         }
         const int64_t npairs = kp_off[nkp];
         c->is_pairs.ensure(sizeof(int) * (npairs + 1));
         c->is_w.ensure(sizeof(double) * (npairs + 1));
-        {
+        if (!chunk_pairs.empty()) {
             int64_t k = 0;
             for (size_t ci = 0; ci < chunk_pairs.size(); ++ci) {
                 const int64_t kp0 = (int64_t)ci * kpc, kp1 = std::min(nkp, kp0 + kpc);
