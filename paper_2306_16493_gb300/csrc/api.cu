@@ -448,7 +448,7 @@ epwi_status epwi_carrier_density(epwi_ctx *c, double T, double mu, int32_t nv, d
     return guard(c, [&] {
         require_eigs(c);
         EPWI_REQUIRE(T > 0 && n && nv >= 0 && nv < c->nw, EPWI_EINVAL, "bad argument");
-        *n = carrier_density(c, T, mu, nv);
+        *n = carrier_density(c, T, mu, nv, -HUGE_VAL);
     });
 }
 
@@ -457,14 +457,15 @@ epwi_status epwi_find_mu(epwi_ctx *c, double T, double n_c, int32_t nv, double *
         require_eigs(c);
         EPWI_REQUIRE(T > 0 && n_c > 0 && mu_out && nv >= 0 && nv < c->nw, EPWI_EINVAL, "bad argument");
         const double *e = c->eps.as<double>();
-        double lo = device_reduce_minmax(c, e, c->nk, c->nw, nv, false) - 3.0;
+        const double emin = device_reduce_minmax(c, e, c->nk, c->nw, nv, false);
+        double lo = emin - 3.0;
         double hi = device_reduce_minmax(c, e, c->nk, c->nw, c->nw - 1, true) + 3.0;
         // n(mu) is increasing and nearly exponential below the band edge, so the root of
         // h(mu) = ln n(mu) - ln n_c is bracketed and found by regula falsi with the Illinois
         // modification (a retained end's h is halved), falling back to bisection where h is not
         // finite (n underflowed); stop at the same residual as a bisection: |n - n_c| <= 1e-13 n_c.
         auto h = [&](double mu, double &n) {
-            n = carrier_density(c, T, mu, nv);
+            n = carrier_density(c, T, mu, nv, emin);
             return n > 0 ? std::log(n / n_c) : -HUGE_VAL;
         };
         double nlo, nhi;

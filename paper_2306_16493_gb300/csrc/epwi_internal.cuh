@@ -344,7 +344,8 @@ void sym_expand(epwi_ctx *c);
 void sieve_count(epwi_ctx *c);
 void occupation_tables(epwi_ctx *c);
 void run_scatter(epwi_ctx *c);
-double carrier_density(epwi_ctx *c, double T, double mu, int n_valence);
+// emin: the lowest energy of band n_valence (or -infinity where it is not known: no cut)
+double carrier_density(epwi_ctx *c, double T, double mu, int n_valence, double emin);
 void conductivity(epwi_ctx *c, double sigma[9]);
 void transport_moments(epwi_ctx *c, double m[3][9]);
 void transport_moments_F(epwi_ctx *c, const double *F, double m[3][9]);

@@ -2,6 +2,9 @@
 // sigma (Eq. 12 with F = v tau), conduction-electron density for the chemical potential
 // (Sec. III A), band extrema.  All reductions are two-pass with a fixed block count and a
 // fixed tree order, so results are bitwise reproducible for a given input size.
+#include <algorithm>
+#include <cmath>
+
 #include "epwi_internal.cuh"
 #include "scatter.cuh"
 
@@ -141,21 +144,24 @@ __global__ void __launch_bounds__(kRedThreads) k_final_sum(int nb, const double 
         for (int j = 0; j < NV; ++j) out[j] = v[j];
 }
 
+// Partial sums of f over the bands n >= nv.  Energies above ecut add nothing at FP64 (see
+// carrier_density); the bands of a point ascend, so its later ones are passed over as well.  (Every
+// band of every point took an FP64 exponential and division: 286 us per density at Si-like 100^3,
+// 18 densities per chemical potential.)
 __global__ void __launch_bounds__(kRedThreads) k_density_part(int64_t nk, int W, int nv,
                                                               const double *__restrict__ eps,
-                                                              double mu, double kT,
+                                                              double mu, double kT, double ecut,
                                                               double *__restrict__ part) {
     __shared__ double sm[kRedThreads];
-    const int nc = W - nv;
-    const int64_t n = nk * nc;
-    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t b0 = per * blockIdx.x, b1 = min(n, b0 + per);
+    const int64_t per = (nk + gridDim.x - 1) / gridDim.x;
+    const int64_t b0 = per * blockIdx.x, b1 = min(nk, b0 + per);
     double v[1] = {0};
-    for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-        const int64_t k = i / nc;
-        const int b = nv + (int)(i % nc);
-        v[0] += fermi(eps[k * W + b], mu, kT);
-    }
+    for (int64_t k = b0 + threadIdx.x; k < b1; k += blockDim.x)
+        for (int b = nv; b < W; ++b) {
+            const double e = eps[k * W + b];
+            if (!(e <= ecut)) break;
+            v[0] += fermi(e, mu, kT);
+        }
     block_sum<1>(v, sm);
     if (threadIdx.x == 0) part[blockIdx.x] = v[0];
 }
@@ -236,14 +242,16 @@ double device_reduce_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t str
     return want_max ? h[1] : h[0];
 }
 
-double carrier_density(epwi_ctx *c, double T, double mu, int nv) {
+double carrier_density(epwi_ctx *c, double T, double mu, int nv, double emin) {
     const int64_t n = c->nk * (c->nw - nv);
-    const int nb = red_blocks(n);
+    const int nb = red_blocks(c->nk);
     c->red_tmp.ensure(sizeof(double) * (nb + 16));
     double *part = c->red_tmp.as<double>();
     double *out = part + nb;
-    k_density_part<<<nb, kRedThreads, 0, c->stream>>>(c->nk, c->nw, nv, c->eps.as<double>(), mu,
-                                                      epc::kKbEVK * T, part);
+    const double kT = epc::kKbEVK * T;
+    // n f(e) below e^-46 = 1e-20 of the lowest band's f at emin (or of 1/2 above it): under the rounding
+    const double ecut = std::isfinite(emin) ? std::max(emin, mu) + kT * (std::log((double)n) + 46.0) : HUGE_VAL;
+    k_density_part<<<nb, kRedThreads, 0, c->stream>>>(c->nk, c->nw, nv, c->eps.as<double>(), mu, kT, ecut, part);
     EPWI_CHECK_LAUNCH();
     k_final_sum<1><<<1, kRedThreads, 0, c->stream>>>(nb, part, out);
     EPWI_CHECK_LAUNCH();
