@@ -130,6 +130,7 @@ epwi_status epwi_create(epwi_ctx **out, const epwi_options *opt) {
         EPWI_REQUIRE(c->device >= 0 && c->device < n, EPWI_EINVAL, "no such CUDA device");
         EPWI_CUDA(cudaSetDevice(c->device));
         EPWI_CUDA(cudaFree(nullptr));   // create the primary context now
+        EPWI_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
     });
     if (st != EPWI_OK) {
         delete c;
@@ -407,6 +408,9 @@ epwi_status epwi_eigs(epwi_ctx *c, const int32_t kgrid[3], const int32_t qgrid[3
         launch_eigs(c);
         cudaEventRecord(e1, c->stream);
         int flag[2];
+        double range[2];
+        EPWI_CUDA(cudaMemcpyAsync(range, device_minmax(c, c->eps.as<double>(), nk * c->nw, 1, 0), sizeof(range),
+                                  cudaMemcpyDeviceToHost, c->stream));
         EPWI_CUDA(cudaMemcpyAsync(flag, c->eig_flag.p, sizeof(flag), cudaMemcpyDeviceToHost, c->stream));
         EPWI_CUDA(cudaStreamSynchronize(c->stream));
         cudaEventElapsedTime(&c->ms_eigs, e0, e1);
@@ -415,11 +419,9 @@ epwi_status epwi_eigs(epwi_ctx *c, const int32_t kgrid[3], const int32_t qgrid[3
         EPWI_REQUIRE(flag[0] == 0 && flag[1] == 0, EPWI_ENUMERIC,
                      "Jacobi did not converge on " + std::to_string(flag[0]) + " H(k) and " +
                          std::to_string(flag[1]) + " D(q) matrices");
-        {
-            const double lo = device_reduce_minmax(c, c->eps.as<double>(), nk * c->nw, 1, 0, false);
-            const double hi = device_reduce_minmax(c, c->eps.as<double>(), nk * c->nw, 1, 0, true);
-            c->eabs_max = std::max(std::fabs(lo), std::fabs(hi));
-        }
+        c->eps_min = range[0];
+        c->eps_max = range[1];
+        c->eabs_max = std::max(std::fabs(range[0]), std::fabs(range[1]));
         c->have_eigs = true;
     });
 }
@@ -427,10 +429,8 @@ epwi_status epwi_eigs(epwi_ctx *c, const int32_t kgrid[3], const int32_t qgrid[3
 epwi_status epwi_band_range(epwi_ctx *c, double *emin, double *emax) {
     return guard(c, [&] {
         require_eigs(c);
-        const double *e = c->eps.as<double>();
-        const int64_t n = c->nk * c->nw;
-        if (emin) *emin = device_reduce_minmax(c, e, n, 1, 0, false);
-        if (emax) *emax = device_reduce_minmax(c, e, n, 1, 0, true);
+        if (emin) *emin = c->eps_min;
+        if (emax) *emax = c->eps_max;
     });
 }
 
@@ -518,7 +518,7 @@ WorkSet begin_rates(epwi_ctx *c, double T, double mu, double eta, double emin, d
     std::memset(&c->stats, 0, sizeof(c->stats));
     c->stats.precision = c->opt.precision;
     c->stats.ms_eigs = c->ms_eigs;
-    EPWI_CUDA(cudaDeviceGetAttribute(&c->stats.sm_count, cudaDevAttrMultiProcessorCount, c->device));
+    c->stats.sm_count = c->sm_count;
     // window and sieve (ms_sieve); the window's deferred band velocities count as eigensolve
     // work (ms_eigs)
     cudaEvent_t ev[4];
@@ -527,11 +527,11 @@ WorkSet begin_rates(epwi_ctx *c, double T, double mu, double eta, double emin, d
     if (sym) sym_prepare(c);                 // representatives of the stars; invariance check
     build_window(c, sym ? c->sym_rep.as<int>() : nullptr);
     cudaEventRecord(ev[1], c->stream);
-    ensure_velocities(c, false);
+    if (!sym) ensure_velocities(c, false);   // sym_expand forms those of every window state
     cudaEventRecord(ev[2], c->stream);
     sieve_count(c);
     cudaEventRecord(ev[3], c->stream);
-    EPWI_CUDA(cudaStreamSynchronize(c->stream));
+    EPWI_CUDA(cudaEventSynchronize(ev[3]));
     float ms_w = 0, ms_v = 0, ms_s = 0;
     cudaEventElapsedTime(&ms_w, ev[0], ev[1]);
     cudaEventElapsedTime(&ms_v, ev[1], ev[2]);
@@ -548,10 +548,7 @@ WorkSet begin_rates(epwi_ctx *c, double T, double mu, double eta, double emin, d
     ws.kp_state = c->kp_state.as<int64_t>();
     ws.kp_pairs = c->kp_pairs.as<int64_t>();
     ws.h_kp_pairs = c->h_kp_pairs;
-    ws.h_kp_state.resize(c->nkp + 1);
-    EPWI_CUDA(cudaMemcpyAsync(ws.h_kp_state.data(), c->kp_state.p, sizeof(int64_t) * (c->nkp + 1),
-                              cudaMemcpyDeviceToHost, c->stream));
-    EPWI_CUDA(cudaStreamSynchronize(c->stream));
+    ws.h_kp_state = c->h_kp_state;
     return ws;
 }
 

@@ -84,6 +84,7 @@ struct epwi_ctx {
     cudaStream_t stream = nullptr;
     std::string err;
     int device = 0;
+    int sm_count = 0;
 
     // system (after epwi_setup)
     bool have_sys = false;
@@ -115,6 +116,7 @@ struct epwi_ctx {
     DevBuf hw;                     // double [Nq][Nm] eV (dropped modes keep their value)
     DevBuf hwmax32;                // float [Nq] largest kept mode energy, -1 if none
     DevBuf hw32;                   // float [Nq][Nm] mode energy, -1 for dropped modes
+    double eps_min = 0, eps_max = 0;   // band extrema of the grid
     double eabs_max = 0;           // max |eps| over the grid (FP32 error bounds)
     DevBuf u;                      // double2 [Nq][Nm][Nm] A (row mu, column nu), 0 if dropped
     DevBuf u32;                    // float2 [Nq][Nm][Nm]
@@ -135,7 +137,7 @@ struct epwi_ctx {
     DevBuf st_k, st_n;             // int32 [nstates]
     DevBuf focc;                   // double [Nk][W] Fermi-Dirac
     DevBuf nocc;                   // double [Nq][Nm] Bose-Einstein (0 for dropped modes)
-    std::vector<int64_t> h_kp_pairs;
+    std::vector<int64_t> h_kp_pairs, h_kp_state;   // host copies of kp_pairs, kp_state (sieve_count)
     epwi_stats stats{};
 
     // scratch
@@ -144,7 +146,8 @@ struct epwi_ctx {
     DevBuf tiles;                  // int4 per tile {kp_local, pair_begin, pair_end, 0}
     DevBuf tile_part;              // double [tile][W] partial sums
     DevBuf kp_tile;                // int64 [chunk kp + 1]
-    DevBuf scan_tmp;               // scan workspace
+    DevBuf scan_tmp;               // scan input / output
+    DevBuf scan_ws;                // block sums of long scans
     DevBuf red_tmp;                // reduction workspace
     DevBuf counts;                 // int64 per kp
 
@@ -182,6 +185,7 @@ struct epwi_ctx {
     DevBuf re_cube;                // int [Dc^3]: R_e index of each bounding-cube point, -1 if absent
     DevBuf ks_T;                   // stage outputs T1, T2
     DevBuf col_buf;                // (k2, k3) columns of a k-point list
+    int win_ncol = 0, win_nk3 = 0; // columns and distinct k3 of the current window (0: not counted)
     // band velocities: with vel_defer (set by epwi_eigs) the eigensolve leaves them out and
     // they are formed from the kept electron stage output fac_Uel for the k-points that need
     // them: those of each new window, or every point on request (ensure_velocities)
@@ -232,7 +236,7 @@ struct epwi_ctx {
                          &eps, &eps32, &V, &V32, &vel, &hw, &hwmax32, &hw32, &u, &u32, &eig_flag,
                          &kpts, &win_lo, &win_n, &kp_state, &kp_pairs, &inv_tau, &st_k,
                          &st_n, &focc, &nocc, &pairs, &ghat, &tiles, &tile_part, &kp_tile,
-                         &scan_tmp, &red_tmp, &counts, &tc_ptab, &tc_erel, &tc_f32,
+                         &scan_tmp, &scan_ws, &red_tmp, &counts, &tc_ptab, &tc_erel, &tc_f32,
                          &tc_n32, &tc_hw32, &tc_err, &tc_meta, &is_pairs, &is_w,
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
                          &ib_kpos, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
@@ -332,6 +336,9 @@ void ensure_velocities(epwi_ctx *c, bool all);
 void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total);
 double device_reduce_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t stride, int64_t off,
                             bool want_max);
+// The same without the copy to the host: {min, max} in device memory (valid until the next
+// reduction on the context).
+const double *device_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t stride, int64_t off);
 // Window of the current rates call: lo/count per k from eps, then the lists of k-points and
 // states.  rep (optional, symmetry): only k-points that represent their star take part.
 void build_window(epwi_ctx *c, const int *rep = nullptr);

@@ -76,6 +76,28 @@ __global__ void k_scan_apply(const int64_t *in, int64_t n, const int64_t *boff, 
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) out[n] = run;
 }
 
+// The whole scan in one block (short inputs: one launch instead of four).
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(const int64_t *in, int64_t n, int64_t *out) {
+    __shared__ int64_t sm[33];
+    int64_t carry = 0;
+    for (int64_t base = 0; base < n; base += kScanBlock * kScanItems) {
+        const int64_t i0 = base + threadIdx.x * kScanItems;
+        int64_t v[kScanItems], s = 0;
+        for (int i = 0; i < kScanItems; ++i) {
+            v[i] = i0 + i < n ? in[i0 + i] : 0;
+            s += v[i];
+        }
+        int64_t tot;
+        int64_t run = carry + block_excl_scan(s, sm, tot);
+        for (int i = 0; i < kScanItems; ++i) {
+            if (i0 + i < n) out[i0 + i] = run;
+            run += v[i];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) out[n] = carry;
+}
+
 // ------------------------------------------------------------------- window / k_eff
 __global__ void k_window(int64_t nk, int W, const double *__restrict__ eps, double emin,
                          double emax, int *__restrict__ lo, int *__restrict__ cnt) {
@@ -94,30 +116,29 @@ __device__ __forceinline__ bool window_kpoint(int64_t k, const int *cnt, const i
     return cnt[k] > 0 && (!rep || rep[k] == (int)k);
 }
 
+// k-points and states of each grid point, packed in one word (k-points above bit 36: a grid has
+// fewer than 2^31 points of at most 24 bands), so that one scan places both.
+constexpr int kStateBits = 36;
 __global__ void k_window_flags(int64_t nk, const int *__restrict__ cnt, const int *__restrict__ rep,
                                int64_t *__restrict__ flag) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nk) flag[k] = window_kpoint(k, cnt, rep) ? 1 : 0;
+    if (k < nk) flag[k] = window_kpoint(k, cnt, rep) ? ((int64_t)1 << kStateBits) + cnt[k] : 0;
 }
 
-__global__ void k_compact_kpts(int64_t nk, const int64_t *__restrict__ pos,
-                               const int *__restrict__ cnt, const int *__restrict__ rep, int *__restrict__ kpts,
-                               int64_t *__restrict__ nsel) {
+// The k-point list, first states (with the total at the end) and states of the window.
+__global__ void k_compact_kpts(int64_t nk, const int64_t *__restrict__ pos, const int *__restrict__ cnt,
+                               const int *__restrict__ rep, const int *__restrict__ lo, int *__restrict__ kpts,
+                               int64_t *__restrict__ kp_state, int *__restrict__ st_k, int *__restrict__ st_n) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t low = ((int64_t)1 << kStateBits) - 1;
+    if (k == 0) kp_state[pos[nk] >> kStateBits] = pos[nk] & low;
     if (k >= nk || !window_kpoint(k, cnt, rep)) return;
-    kpts[pos[k]] = (int)k;
-    nsel[pos[k]] = cnt[k];
-}
-
-__global__ void k_states(int64_t nkp, const int *__restrict__ kpts, const int *__restrict__ lo,
-                         const int64_t *__restrict__ soff, int *__restrict__ st_k,
-                         int *__restrict__ st_n) {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nkp) return;
-    const int k = kpts[p];
-    for (int64_t s = soff[p]; s < soff[p + 1]; ++s) {
-        st_k[s] = k;
-        st_n[s] = lo[k] + (int)(s - soff[p]);
+    const int64_t p = pos[k] >> kStateBits, s0 = pos[k] & low;
+    kpts[p] = (int)k;
+    kp_state[p] = s0;
+    for (int n = 0; n < cnt[k]; ++n) {
+        st_k[s0 + n] = (int)k;
+        st_n[s0 + n] = lo[k] + n;
     }
 }
 
@@ -691,6 +712,8 @@ static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
     const int64_t nplane = (int64_t)c->ng[1] * c->ng[2];
     if (N1 > 128 || nplane > (1 << 20) || c->nkp * c->nk < (int64_t(1) << 23)) return false;
     const ColumnSet cs = build_columns(c, c->kpts.as<int>(), c->nkp);
+    c->win_ncol = cs.ncol;
+    c->win_nk3 = cs.nk3;
     if (c->nkp < 2 * (int64_t)cs.ncol) return false;
     EPWI_CUDA(cudaMemsetAsync(c->counts.p, 0, sizeof(int64_t) * c->nkp, c->stream));
     auto go = [&](auto kern, int TB) {
@@ -707,42 +730,42 @@ static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
     return true;
 }
 
-void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
-    // out has n + 1 entries; out[n] = sum.  Recursive over block sums.
+static void scan_levels(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int level, int64_t level_off) {
     const int64_t per = (int64_t)kScanBlock * kScanItems;
     const int64_t nb = (n + per - 1) / per;
+    // up to 16 blocks' worth in one block; the block sums of longer inputs go to the context's
+    // workspace, level by level (nb + 1 sums and offsets each)
+    if (nb <= 16) {
+        k_scan_one<<<1, kScanBlock, 0, c->stream>>>(in, n, out);
+        EPWI_CHECK_LAUNCH();
+    } else {
+        if (level == 0) {
+            int64_t need = 0;
+            for (int64_t m = nb; m > 16; m = (m + per - 1) / per) need += 2 * (m + 1);
+            c->scan_ws.ensure(sizeof(int64_t) * (need + 2 * 17 + 2));
+            level_off = 0;
+        }
+        int64_t *bs = c->scan_ws.as<int64_t>() + level_off, *bo = bs + nb + 1;
+        k_scan_blocks<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bs);
+        EPWI_CHECK_LAUNCH();
+        scan_levels(c, bs, bo, nb, level + 1, level_off + 2 * (nb + 1));
+        k_scan_apply<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bo, out);
+        EPWI_CHECK_LAUNCH();
+    }
+}
+
+void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
+    // out has n + 1 entries; out[n] = sum
     if (n == 0) {
         EPWI_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), c->stream));
         if (total) *total = 0;
         return;
     }
-    DevBuf bs, bo;
-    bs.ensure(sizeof(int64_t) * (nb + 1));
-    bo.ensure(sizeof(int64_t) * (nb + 1));
-    try {
-        k_scan_blocks<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bs.as<int64_t>());
-        EPWI_CHECK_LAUNCH();
-        if (nb > 1) {
-            scan_exclusive_i64(c, bs.as<int64_t>(), bo.as<int64_t>(), nb, nullptr);
-        } else {
-            EPWI_CUDA(cudaMemsetAsync(bo.p, 0, sizeof(int64_t), c->stream));
-        }
-        k_scan_apply<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bo.as<int64_t>(), out);
-        EPWI_CHECK_LAUNCH();
-        if (total) {
-            EPWI_CUDA(cudaMemcpyAsync(total, out + n, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                                      c->stream));
-            EPWI_CUDA(cudaStreamSynchronize(c->stream));
-        } else {
-            EPWI_CUDA(cudaStreamSynchronize(c->stream));   // bs/bo are freed on return
-        }
-    } catch (...) {
-        bs.release();
-        bo.release();
-        throw;
+    scan_levels(c, in, out, n, 0, 0);
+    if (total) {
+        EPWI_CUDA(cudaMemcpyAsync(total, out + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+        EPWI_CUDA(cudaStreamSynchronize(c->stream));
     }
-    bs.release();
-    bo.release();
 }
 
 void build_window(epwi_ctx *c, const int *rep) {
@@ -765,27 +788,21 @@ void window_lists(epwi_ctx *c, const int *rep) {
     const unsigned nb = (unsigned)((nk + 255) / 256);
     k_window_flags<<<nb, 256, 0, c->stream>>>(nk, c->win_n.as<int>(), rep, c->counts.as<int64_t>());
     EPWI_CHECK_LAUNCH();
-    int64_t nkp = 0;
-    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->scan_tmp.as<int64_t>(), nk, &nkp);
+    int64_t tot = 0;
+    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->scan_tmp.as<int64_t>(), nk, &tot);
+    const int64_t nkp = tot >> kStateBits, nst = tot & (((int64_t)1 << kStateBits) - 1);
     c->nkp = nkp;
+    c->nstates = nst;
+    c->win_ncol = c->win_nk3 = 0;
     c->kpts.ensure(sizeof(int) * (nkp + 1));
     c->kp_state.ensure(sizeof(int64_t) * (nkp + 1));
-    // reuse counts as the per-kp band count
-    k_compact_kpts<<<nb, 256, 0, c->stream>>>(nk, c->scan_tmp.as<int64_t>(), c->win_n.as<int>(), rep,
-                                             c->kpts.as<int>(), c->counts.as<int64_t>());
-    EPWI_CHECK_LAUNCH();
-    int64_t nst = 0;
-    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->kp_state.as<int64_t>(), nkp, &nst);
-    c->nstates = nst;
     c->st_k.ensure(sizeof(int) * (nst + 1));
     c->st_n.ensure(sizeof(int) * (nst + 1));
     c->inv_tau.ensure(sizeof(double) * (nst + 1));
-    if (nkp > 0) {
-        k_states<<<(unsigned)((nkp + 255) / 256), 256, 0, c->stream>>>(
-            nkp, c->kpts.as<int>(), c->win_lo.as<int>(), c->kp_state.as<int64_t>(),
-            c->st_k.as<int>(), c->st_n.as<int>());
-        EPWI_CHECK_LAUNCH();
-    }
+    k_compact_kpts<<<nb, 256, 0, c->stream>>>(nk, c->scan_tmp.as<int64_t>(), c->win_n.as<int>(), rep, c->win_lo.as<int>(),
+                                             c->kpts.as<int>(), c->kp_state.as<int64_t>(), c->st_k.as<int>(),
+                                             c->st_n.as<int>());
+    EPWI_CHECK_LAUNCH();
 }
 
 void sieve_count(epwi_ctx *c) {
@@ -819,13 +836,15 @@ void sieve_count(epwi_ctx *c) {
         }
         EPWI_CHECK_LAUNCH();
     }
-    int64_t np = 0;
-    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->kp_pairs.as<int64_t>(), nkp, &np);
-    c->npairs = np;
+    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->kp_pairs.as<int64_t>(), nkp, nullptr);
     c->h_kp_pairs.resize(nkp + 1);
+    c->h_kp_state.resize(nkp + 1);
     EPWI_CUDA(cudaMemcpyAsync(c->h_kp_pairs.data(), c->kp_pairs.p, sizeof(int64_t) * (nkp + 1),
                               cudaMemcpyDeviceToHost, c->stream));
+    EPWI_CUDA(cudaMemcpyAsync(c->h_kp_state.data(), c->kp_state.p, sizeof(int64_t) * (nkp + 1),
+                              cudaMemcpyDeviceToHost, c->stream));
     EPWI_CUDA(cudaStreamSynchronize(c->stream));
+    c->npairs = c->h_kp_pairs[nkp];
 }
 
 void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs) {

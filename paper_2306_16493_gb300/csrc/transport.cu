@@ -194,15 +194,31 @@ __global__ void __launch_bounds__(kRedThreads) k_minmax_part(const double *__res
     }
 }
 
-__global__ void k_minmax_final(int nb, const double *__restrict__ part, double *__restrict__ out) {
-    if (threadIdx.x != 0) return;
+__global__ void __launch_bounds__(kRedThreads) k_minmax_final(int nb, const double *__restrict__ part,
+                                                              double *__restrict__ out) {
+    __shared__ double smn[kRedThreads / 32], smx[kRedThreads / 32];
     double mn = INFINITY, mx = -INFINITY;
-    for (int b = 0; b < nb; ++b) {
+    for (int b = threadIdx.x; b < nb; b += kRedThreads) {
         mn = fmin(mn, part[2 * b]);
         mx = fmax(mx, part[2 * b + 1]);
     }
-    out[0] = mn;
-    out[1] = mx;
+    for (int o = 16; o > 0; o >>= 1) {
+        mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        smn[threadIdx.x >> 5] = mn;
+        smx[threadIdx.x >> 5] = mx;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kRedThreads / 32; ++w) {
+            mn = fmin(mn, smn[w]);
+            mx = fmax(mx, smx[w]);
+        }
+        out[0] = mn;
+        out[1] = mx;
+    }
 }
 
 int red_blocks(int64_t n) {
@@ -226,18 +242,22 @@ void occupation_tables(epwi_ctx *c) {
     if (c->opt.precision != EPWI_FP64) tc_tables(c);
 }
 
-double device_reduce_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t stride, int64_t off,
-                            bool want_max) {
+const double *device_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t stride, int64_t off) {
     const int nb = red_blocks(n);
     c->red_tmp.ensure(sizeof(double) * (2 * nb + 16));
     double *part = c->red_tmp.as<double>();
     double *out = part + 2 * nb;
     k_minmax_part<<<nb, kRedThreads, 0, c->stream>>>(x, n, stride, off, part);
     EPWI_CHECK_LAUNCH();
-    k_minmax_final<<<1, 32, 0, c->stream>>>(nb, part, out);
+    k_minmax_final<<<1, kRedThreads, 0, c->stream>>>(nb, part, out);
     EPWI_CHECK_LAUNCH();
+    return out;
+}
+
+double device_reduce_minmax(epwi_ctx *c, const double *x, int64_t n, int64_t stride, int64_t off,
+                            bool want_max) {
     double h[2];
-    EPWI_CUDA(cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    EPWI_CUDA(cudaMemcpyAsync(h, device_minmax(c, x, n, stride, off), sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     EPWI_CUDA(cudaStreamSynchronize(c->stream));
     return want_max ? h[1] : h[0];
 }
