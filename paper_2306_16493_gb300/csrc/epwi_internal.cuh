@@ -212,7 +212,7 @@ struct epwi_ctx {
     // iterative BTE: Gamma in pair blocks, mean free paths
     bool have_ibte = false;
     DevBuf ib_pairs;               // int32 q index per pair (all k-points of the window; capture only)
-    DevBuf ib_goff;                // int64 [npairs + 1] first Gamma entry of each pair (capture only)
+    DevBuf ib_goff;                // uint32 [npairs] first Gamma entry of each pair, from its k-point's first
     DevBuf ib_col;                 // uint32 per Gamma entry: (final state << 5) | band of k (step only)
     DevBuf ib_ent;                 // int64 [nkp + 1] first Gamma entry of each window k-point
 
@@ -225,7 +225,7 @@ struct epwi_ctx {
     double hw_max = 0;             // largest mode energy on the grid
     bool sym_used = false;         // the last rates call computed representatives only
     DevBuf ib_gam;                 // double (FP64 path) or float: per pair [n][m in window(k+q)]
-    DevBuf ib_kpos;                // int32 [Nk] window k-point of each grid point, -1 outside
+    DevBuf ib_pt;                  // uint32 [Nk] (first window state << 5) | window bands of each grid point
     DevBuf ib_F0, ib_F, ib_Fn;     // double [nstates][3] m: v tau, current and next iterate
     DevBuf ib_F32, ib_Fn32;        // float4 [nstates]: FP32 copies of ib_F, ib_Fn (split paths)
     DevBuf ib_red;                 // uint64 [2]: bit patterns of max |dF| and max |F|
@@ -239,7 +239,7 @@ struct epwi_ctx {
                          &scan_tmp, &scan_ws, &red_tmp, &counts, &tc_ptab, &tc_erel, &tc_f32,
                          &tc_n32, &tc_hw32, &tc_err, &tc_meta, &is_pairs, &is_w,
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
-                         &ib_kpos, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
+                         &ib_pt, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
                          &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
                          &re_cube, &ks_T, &col_buf, &gsf64};
         for (DevBuf *b : all) b->release();

@@ -2,17 +2,19 @@
 //
 // Gamma storage: the sieved pairs of the window in pair order (k-point major, as the sieve
 // writes them), and for every pair (k, q) one block Gamma[n][m] over the window bands n of k
-// and m of k+q, blocks back to back.  goff[pair] is the first entry of a pair's block.  The
+// and m of k+q, blocks back to back.  A pair's block starts at its k-point's first entry, ent[k], plus
+// the pair's 32-bit offset goff[pair].  The
 // value stored is sum_nu |g|^2 [(N + f_m) e^{-x+^2/eta^2} + (1 + N - f_m) e^{-x-^2/eta^2}] (eV^2),
 // the summand of Eq. 10 without its constant 2 pi / (hbar N_q sqrt(pi) eta), which the step
 // applies once per state.
 //
-// After the capture every Gamma entry gets a 4-byte column word: the index of its final state
+// Every Gamma entry has a 4-byte column word (written before the capture, with the offsets, in one
+// pass over the pairs): the index of its final state
 // (k+q, m) in the window's state list and the band n of k, (s << 5) | n.  The step is then a
 // sparse product over entries, Gamma_e F_s accumulated into the row of band n of k: it reads one
 // column word and one value per entry, gathers F at s, and needs no grid arithmetic or table
 // lookups.  The pair list and the per-pair block offsets serve only the capture and are freed
-// afterwards, so the resident index is the column word per entry plus 8 bytes per k-point
+// afterwards when they are large, so the resident index is the column word per entry plus 8 bytes per k-point
 // (half the bytes of FP64 Gamma, equal to those of FP32 Gamma).
 //
 // Step: one block per window k-point, its entries split into eight contiguous warp ranges;
@@ -30,6 +32,8 @@
 
 #include "epwi_internal.cuh"
 #include "scatter.cuh"
+#include "scatter_sf.cuh"
+#include "sieve.cuh"
 
 namespace {
 
@@ -38,45 +42,92 @@ constexpr int kIbWarps = kIbThreads / 32;
 constexpr int kIbMaxBands = 8;  // bands of k accumulated in registers at a time (at most)
 constexpr int kIbUnroll = 4;    // entries per lane whose loads are issued together
 
-__global__ void k_ib_kpos(int64_t nkp, const int *__restrict__ kpts, int *__restrict__ kpos) {
+// Per grid point: its first window state << 5 | window bands (0 bands outside the window).
+__global__ void k_ib_points(int64_t nkp, const int *__restrict__ kpts, const int64_t *__restrict__ kp_state,
+                            unsigned *__restrict__ pt) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < nkp) kpos[kpts[p]] = (int)p;
+    if (p < nkp) pt[kpts[p]] = (unsigned)kp_state[p] << 5 | (unsigned)(kp_state[p + 1] - kp_state[p]);
 }
 
-// sizes[pair] = n_window(k) x n_window(k+q); one block per window k-point
-__global__ void k_ib_sizes(GridInfo g, const int *__restrict__ kpts, const int *__restrict__ win_n,
-                           const int64_t *__restrict__ kp_pairs, const int *__restrict__ pairs,
-                           int64_t *__restrict__ sizes) {
-    const int kp = blockIdx.x;
-    const int ik = kpts[kp];
-    const int nsel = win_n[ik];
-    for (int64_t p = kp_pairs[kp] + threadIdx.x; p < kp_pairs[kp + 1]; p += blockDim.x)
-        sizes[p] = (int64_t)nsel * win_n[kplusq(g, ik, pairs[p])];
-}
-
-// Column words of the Gamma entries: entry goff[p] + n nw + j of pair p = (k, q) gets
-// ((s + j) << 5) | n, s the first window state of k+q, j its band, n the band of k; and the
-// first entry of every window k-point (ent[nkp] = the entry count).  One block per k-point.
-__global__ void k_ib_columns(GridInfo g, int64_t nkp, const int *__restrict__ kpts, const int *__restrict__ win_n,
-                             const int *__restrict__ kpos, const int64_t *__restrict__ kp_state,
-                             const int64_t *__restrict__ kp_pairs, const int *__restrict__ pairs,
-                             const int64_t *__restrict__ goff, unsigned *__restrict__ col,
-                             int64_t *__restrict__ ent) {
-    const int kp = blockIdx.x;
-    const int ik = kpts[kp];
-    const int nsel = win_n[ik];
-    for (int64_t p = kp_pairs[kp] + threadIdx.x; p < kp_pairs[kp + 1]; p += blockDim.x) {
-        const int64_t ikq = kplusq(g, ik, pairs[p]);
-        const int nw = win_n[ikq];
-        if (nw == 0) continue;
-        const unsigned sb = (unsigned)kp_state[kpos[ikq]];
-        unsigned *c = col + goff[p];
-        for (int n = 0; n < nsel; ++n)
-            for (int j = 0; j < nw; ++j) c[n * nw + j] = ((sb + (unsigned)j) << 5) | (unsigned)n;
+// k+q of the pairs of one k-point, with the divisions by launch constants.
+struct IbGrid {
+    GridInfo g;
+    FDiv fplane, fn3;
+    int k1, k2, k3;
+    __device__ __forceinline__ void at(int ik) { grid_coords(g, ik, k1, k2, k3); }
+    __device__ __forceinline__ int64_t kq(int q) const {
+        const int i1 = fdiv(q, fplane), r = q - i1 * (int)fplane.d, i2 = fdiv(r, fn3), i3 = r - i2 * g.n3;
+        int b1 = k1 + i1, b2 = k2 + i2, b3 = k3 + i3;
+        if (b1 >= g.n1) b1 -= g.n1;
+        if (b2 >= g.n2) b2 -= g.n2;
+        if (b3 >= g.n3) b3 -= g.n3;
+        return grid_index(g, b1, b2, b3);
     }
-    if (threadIdx.x == 0) {
-        ent[kp] = goff[kp_pairs[kp]];
-        if (kp == nkp - 1) ent[nkp] = goff[kp_pairs[nkp]];
+};
+
+// Gamma entries of every window k-point: n_window(k) times the sum of n_window(k+q) over its
+// pairs.  One block per k-point.
+__global__ void __launch_bounds__(kIbThreads) k_ib_entries(IbGrid g, const int *__restrict__ kpts,
+                                                           const unsigned *__restrict__ pt,
+                                                           const int64_t *__restrict__ kp_pairs,
+                                                           const int *__restrict__ pairs, int64_t *__restrict__ n_ent) {
+    __shared__ unsigned long long tot;
+    const int kp = blockIdx.x, ik = kpts[kp];
+    g.at(ik);
+    if (threadIdx.x == 0) tot = 0;
+    __syncthreads();
+    unsigned n = 0;
+    for (int64_t p = kp_pairs[kp] + threadIdx.x; p < kp_pairs[kp + 1]; p += kIbThreads) n += pt[g.kq(pairs[p])] & 31u;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&tot, (unsigned long long)n);
+    __syncthreads();
+    if (threadIdx.x == 0) n_ent[kp] = (int64_t)tot * (pt[ik] & 31u);
+}
+
+// Block offsets of the pairs, relative to their k-point's first entry, and the column words of the
+// entries: entry ent[kp] + goff[p] + n nw + j of pair p = (k, q) gets ((s + j) << 5) | n, s the
+// first window state of k+q, j its band, n the band of k.  One block per k-point; a block scan
+// per 256 pairs, in pair order.
+__global__ void __launch_bounds__(kIbThreads) k_ib_index(IbGrid g, const int *__restrict__ kpts,
+                                                         const unsigned *__restrict__ pt,
+                                                         const int64_t *__restrict__ kp_pairs,
+                                                         const int *__restrict__ pairs, const int64_t *__restrict__ ent,
+                                                         uint32_t *__restrict__ goff, unsigned *__restrict__ col) {
+    __shared__ unsigned sm[2][kIbWarps];
+    const int kp = blockIdx.x, ik = kpts[kp];
+    g.at(ik);
+    const unsigned nsel = pt[ik] & 31u;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t p1 = kp_pairs[kp + 1];
+    unsigned *c0 = col + ent[kp];
+    unsigned base = 0;
+    int buf = 0;
+    for (int64_t p0 = kp_pairs[kp]; p0 < p1; p0 += kIbThreads, buf ^= 1) {
+        const int64_t p = p0 + threadIdx.x;
+        const unsigned w = p < p1 ? pt[g.kq(pairs[p])] : 0u;
+        const unsigned nw = w & 31u, size = nsel * nw;
+        unsigned x = size;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) sm[buf][wid] = x;
+        __syncthreads();                          // two buffers: one barrier per step
+        unsigned before = base, tot = 0;
+#pragma unroll
+        for (int v = 0; v < kIbWarps; ++v) {
+            const unsigned y = sm[buf][v];
+            if (v < wid) before += y;
+            tot += y;
+        }
+        const unsigned off = before + x - size;
+        base += tot;
+        if (p < p1) {
+            goff[p] = off;
+            for (unsigned n = 0; n < nsel; ++n)
+                for (unsigned j = 0; j < nw; ++j) c0[off + n * nw + j] = (((w >> 5) + j) << 5) | n;
+        }
     }
 }
 
@@ -111,8 +162,13 @@ struct StepArgs {
     const float4 *Fin32;                  // FP32 copy of Fin (split paths), w unused
     float4 *Fout32;
     double pref;                          // 2 pi / (hbar N_q sqrt(pi) eta), s^-1 per eV^2
-    unsigned long long *red;              // [2] max |dF|, max |F| as bit patterns
+    unsigned long long *red;              // [2] max |dF|, max |F| of this step as bit patterns
+    const unsigned long long *red_prev;   // the same of the step before, or nullptr
+    double tol;
 };
+
+// The stop rule of the iteration; with it met the steps queued behind do nothing.
+__host__ __device__ inline bool ib_done(double dmax, double fmax_, double tol) { return dmax <= tol * fmax_; }
 
 // Accumulation type of the lane and warp sums: FP64 with FP64 Gamma; FP32 with FP32 Gamma
 // (GB300 issues FP64 at 1/64 of the FP32 rate, so FP64 sums would bind the split paths on
@@ -189,6 +245,14 @@ template <typename GT, int NB>
 __global__ void __launch_bounds__(kIbThreads, NB <= 4 ? 4 : 2) k_ib_step(StepArgs<GT> a) {
     using AT = typename Acc<GT>::T;
     __shared__ AT part[kIbWarps][NB][3];
+    if (a.red_prev) {
+        // a step that met the stop rule marks the next one's maxima with NaN patterns, and so on
+        const unsigned long long d = a.red_prev[0], f = a.red_prev[1];
+        if (d == ~0ull || ib_done(__longlong_as_double((long long)d), __longlong_as_double((long long)f), a.tol)) {
+            if (threadIdx.x == 0) a.red[0] = ~0ull;
+            return;
+        }
+    }
     const int kp = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int ik = a.kpts[kp];
@@ -247,7 +311,8 @@ __global__ void __launch_bounds__(kIbThreads, NB <= 4 ? 4 : 2) k_ib_step(StepArg
 }
 
 template <typename GT>
-void launch_step(epwi_ctx *c, const double *Fin, double *Fout, const float4 *Fin32, float4 *Fout32) {
+void launch_step(epwi_ctx *c, const double *Fin, double *Fout, const float4 *Fin32, float4 *Fout32,
+                 unsigned long long *red, const unsigned long long *red_prev, double tol) {
     StepArgs<GT> a;
     a.kpts = c->kpts.as<int>();
     a.win_n = c->win_n.as<int>();
@@ -262,7 +327,9 @@ void launch_step(epwi_ctx *c, const double *Fin, double *Fout, const float4 *Fin
     a.Fin32 = Fin32;
     a.Fout32 = Fout32;
     a.pref = 2.0 * epc::kPi / epc::kHbarEVs / (double)c->nk / (sqrt(epc::kPi) * c->eta);
-    a.red = c->ib_red.as<unsigned long long>();
+    a.red = red;
+    a.red_prev = red_prev;
+    a.tol = tol;
     // band group: the smallest of 1, 2, 4, 8 covering the bands (wider windows loop)
     const unsigned grid = (unsigned)c->nkp;
     if (c->nw <= 1) k_ib_step<GT, 1><<<grid, kIbThreads, 0, c->stream>>>(a);
@@ -281,31 +348,40 @@ void ibte_prepare(epwi_ctx *c, WorkSet &ws) {
     const bool fp64 = c->opt.precision == EPWI_FP64;
     c->ib_pairs.ensure(sizeof(int) * (npairs + 1));
     sieve_fill_chunk(c, 0, nkp, c->ib_pairs.as<int>());
-    c->ib_kpos.ensure(sizeof(int) * c->nk);
-    EPWI_CUDA(cudaMemsetAsync(c->ib_kpos.p, 0xff, sizeof(int) * c->nk, c->stream));
+    EPWI_REQUIRE(c->nstates < (int64_t(1) << 27), EPWI_EUNSUPPORTED, "iterative BTE needs fewer than 2^27 states");
+    c->ib_pt.ensure(sizeof(unsigned) * c->nk);
+    EPWI_CUDA(cudaMemsetAsync(c->ib_pt.p, 0, sizeof(unsigned) * c->nk, c->stream));
+    c->ib_goff.ensure(sizeof(uint32_t) * (npairs + 1));
+    c->ib_ent.ensure(sizeof(int64_t) * (nkp + 1));
+    c->counts.ensure(sizeof(int64_t) * (nkp + 1));
+    IbGrid g;
+    g.g = make_grid_info(c);
+    g.fplane = make_fdiv((uint32_t)(g.g.n2 * g.g.n3));
+    g.fn3 = make_fdiv((uint32_t)g.g.n3);
+    g.k1 = g.k2 = g.k3 = 0;
     if (nkp > 0) {
-        k_ib_kpos<<<(unsigned)((nkp + 255) / 256), 256, 0, c->stream>>>(nkp, c->kpts.as<int>(),
-                                                                      c->ib_kpos.as<int>());
+        k_ib_points<<<(unsigned)((nkp + 255) / 256), 256, 0, c->stream>>>(nkp, c->kpts.as<int>(),
+                                                                        c->kp_state.as<int64_t>(), c->ib_pt.as<unsigned>());
+        EPWI_CHECK_LAUNCH();
+        k_ib_entries<<<(unsigned)nkp, kIbThreads, 0, c->stream>>>(g, c->kpts.as<int>(), c->ib_pt.as<unsigned>(),
+                                                                 c->kp_pairs.as<int64_t>(), c->ib_pairs.as<int>(),
+                                                                 c->counts.as<int64_t>());
         EPWI_CHECK_LAUNCH();
     }
-    c->ib_goff.ensure(sizeof(int64_t) * (npairs + 1));
-    int64_t nent = 0;
-    {
-        DevBuf sizes;
-        try {
-            sizes.ensure(sizeof(int64_t) * (npairs + 1));
-            if (nkp > 0) {
-                k_ib_sizes<<<(unsigned)nkp, 256, 0, c->stream>>>(
-                    make_grid_info(c), c->kpts.as<int>(), c->win_n.as<int>(), c->kp_pairs.as<int64_t>(),
-                    c->ib_pairs.as<int>(), sizes.as<int64_t>());
-                EPWI_CHECK_LAUNCH();
-            }
-            scan_exclusive_i64(c, sizes.as<int64_t>(), c->ib_goff.as<int64_t>(), npairs, &nent);
-        } catch (...) {
-            sizes.release();
-            throw;
-        }
-        sizes.release();
+    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->ib_ent.as<int64_t>(), nkp, nullptr);
+    std::vector<int64_t> h_ent(nkp + 1);
+    EPWI_CUDA(cudaMemcpyAsync(h_ent.data(), c->ib_ent.p, sizeof(int64_t) * (nkp + 1), cudaMemcpyDeviceToHost, c->stream));
+    EPWI_CUDA(cudaStreamSynchronize(c->stream));
+    const int64_t nent = h_ent[nkp];
+    for (int64_t p = 0; p < nkp; ++p)
+        EPWI_REQUIRE(h_ent[p + 1] - h_ent[p] < (int64_t(1) << 32), EPWI_EUNSUPPORTED,
+                     "iterative BTE: more than 2^32 couplings of one k-point");
+    c->ib_col.ensure(sizeof(unsigned) * (nent + 1));
+    if (nkp > 0) {
+        k_ib_index<<<(unsigned)nkp, kIbThreads, 0, c->stream>>>(
+            g, c->kpts.as<int>(), c->ib_pt.as<unsigned>(), c->kp_pairs.as<int64_t>(), c->ib_pairs.as<int>(),
+            c->ib_ent.as<int64_t>(), c->ib_goff.as<uint32_t>(), c->ib_col.as<unsigned>());
+        EPWI_CHECK_LAUNCH();
     }
     const size_t eb = fp64 ? sizeof(double) : sizeof(float);
     const size_t gam_bytes = eb * (size_t)(nent + 1);
@@ -315,7 +391,8 @@ void ibte_prepare(epwi_ctx *c, WorkSet &ws) {
     c->ib_stats.n_entries = nent;
     c->ib_stats.entry_bytes = (int32_t)eb;
     ws.pairs_dev = c->ib_pairs.as<int>();
-    ws.goff = c->ib_goff.as<int64_t>();
+    ws.goff = c->ib_goff.as<uint32_t>();
+    ws.gent = c->ib_ent.as<int64_t>();
     if (fp64) ws.gam64 = c->ib_gam.as<double>();
     else ws.gam32 = c->ib_gam.as<float>();
 }
@@ -331,65 +408,69 @@ void ibte_iterate(epwi_ctx *c, int max_iter, double tol) {
         c->ib_F32.ensure(sizeof(float4) * (ns + 1));
         c->ib_Fn32.ensure(sizeof(float4) * (ns + 1));
     }
-    c->ib_red.ensure(sizeof(unsigned long long) * 2);
-    // the step's index: one column word per Gamma entry and the first entry of every k-point;
-    // the pair list and per-pair offsets are needed only by the capture and are freed here
-    EPWI_REQUIRE(ns < (int64_t(1) << 27), EPWI_EUNSUPPORTED, "iterative BTE needs fewer than 2^27 states");
-    const int64_t nkp = c->nkp, nent = c->ib_stats.n_entries;
-    c->ib_ent.ensure(sizeof(int64_t) * (nkp + 1));
-    c->ib_col.ensure(sizeof(unsigned) * (nent + 1));
-    if (nkp > 0) {
-        k_ib_columns<<<(unsigned)nkp, 256, 0, c->stream>>>(
-            make_grid_info(c), nkp, c->kpts.as<int>(), c->win_n.as<int>(), c->ib_kpos.as<int>(),
-            c->kp_state.as<int64_t>(), c->kp_pairs.as<int64_t>(), c->ib_pairs.as<int>(), c->ib_goff.as<int64_t>(),
-            c->ib_col.as<unsigned>(), c->ib_ent.as<int64_t>());
-        EPWI_CHECK_LAUNCH();
+    const int64_t nent = c->ib_stats.n_entries, nkp = c->nkp;
+    // the pair list and the offsets served the capture; up to 4 GiB of them stay for the next call
+    if (c->ib_goff.bytes + c->ib_pairs.bytes > (size_t(4) << 30)) {
+        EPWI_CUDA(cudaStreamSynchronize(c->stream));
+        c->ib_goff.release();
+        c->ib_pairs.release();
     }
-    EPWI_CUDA(cudaStreamSynchronize(c->stream));
-    c->ib_goff.release();
-    c->ib_pairs.release();
     if (ns > 0) {
         k_ib_f0<<<(unsigned)((ns + 255) / 256), 256, 0, c->stream>>>(
             ns, c->nw, c->st_k.as<int>(), c->st_n.as<int>(), c->inv_tau.as<double>(), c->vel.as<double>(),
             c->ib_F0.as<double>(), c->ib_F.as<double>(), fp64 ? nullptr : c->ib_F32.as<float4>());
         EPWI_CHECK_LAUNCH();
     }
+    // Steps are queued kQueue at a time; each looks at the maxima of the one before and does nothing
+    // once the stop rule is met, so the host reads the maxima only once per kQueue steps.
+    constexpr int kQueue = 8;
+    c->ib_red.ensure(sizeof(unsigned long long) * 2 * (kQueue + 1));
+    unsigned long long *red = c->ib_red.as<unsigned long long>();   // slot 0: last step of the queue before
     cudaEvent_t e0, e1;
     EPWI_CUDA(cudaEventCreate(&e0));
     EPWI_CUDA(cudaEventCreate(&e1));
-    unsigned long long *h = nullptr;
     auto cleanup = [&] {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        if (h) cudaFreeHost(h);
     };
     int it = 0;
     double change = 0, ms_steps = 0;
     try {
-        EPWI_CUDA(cudaMallocHost(&h, sizeof(unsigned long long) * 2));
-        for (it = 0; it < max_iter && c->nkp > 0;) {
-            EPWI_CUDA(cudaMemsetAsync(c->ib_red.p, 0, sizeof(unsigned long long) * 2, c->stream));
+        bool done = false;
+        while (!done && it < max_iter && nkp > 0) {
+            const int n = std::min(kQueue, max_iter - it);
+            EPWI_CUDA(cudaMemsetAsync(red, 0, sizeof(unsigned long long) * 2 * (kQueue + 1), c->stream));
             EPWI_CUDA(cudaEventRecord(e0, c->stream));
-            if (fp64) launch_step<double>(c, c->ib_F.as<double>(), c->ib_Fn.as<double>(), nullptr, nullptr);
-            else launch_step<float>(c, c->ib_F.as<double>(), c->ib_Fn.as<double>(), c->ib_F32.as<float4>(),
-                                    c->ib_Fn32.as<float4>());
+            double *F[2] = {c->ib_F.as<double>(), c->ib_Fn.as<double>()};
+            float4 *F32[2] = {c->ib_F32.as<float4>(), c->ib_Fn32.as<float4>()};
+            for (int i = 0; i < n; ++i) {
+                unsigned long long *r = red + 2 * (i + 1), *rp = i ? red + 2 * i : nullptr;
+                if (fp64) launch_step<double>(c, F[i & 1], F[~i & 1], nullptr, nullptr, r, rp, tol);
+                else launch_step<float>(c, F[i & 1], F[~i & 1], F32[i & 1], F32[~i & 1], r, rp, tol);
+            }
             EPWI_CUDA(cudaEventRecord(e1, c->stream));
-            EPWI_CUDA(cudaMemcpyAsync(h, c->ib_red.p, sizeof(unsigned long long) * 2, cudaMemcpyDeviceToHost,
-                                      c->stream));
+            unsigned long long h[2 * (kQueue + 1)];
+            EPWI_CUDA(cudaMemcpyAsync(h, red, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
             EPWI_CUDA(cudaStreamSynchronize(c->stream));
             float ms = 0;
             EPWI_CUDA(cudaEventElapsedTime(&ms, e0, e1));
             ms_steps += ms;
-            ++it;
-            std::swap(c->ib_F, c->ib_Fn);
-            std::swap(c->ib_F32, c->ib_Fn32);
-            double dmax, fmax_;
-            std::memcpy(&dmax, &h[0], sizeof(double));
-            std::memcpy(&fmax_, &h[1], sizeof(double));
-            EPWI_REQUIRE(std::isfinite(dmax) && std::isfinite(fmax_), EPWI_ENUMERIC,
-                         "non-finite mean free path in the iteration");
-            change = fmax_ > 0 ? dmax / fmax_ : 0.0;
-            if (dmax <= tol * fmax_) break;
+            int ran = 0;                                  // steps of this queue that did their work
+            for (int i = 0; i < n && !done; ++i) {
+                double dmax, fmax_;
+                std::memcpy(&dmax, &h[2 * (i + 1)], sizeof(double));
+                std::memcpy(&fmax_, &h[2 * (i + 1) + 1], sizeof(double));
+                EPWI_REQUIRE(std::isfinite(dmax) && std::isfinite(fmax_), EPWI_ENUMERIC,
+                             "non-finite mean free path in the iteration");
+                ++ran;
+                change = fmax_ > 0 ? dmax / fmax_ : 0.0;
+                done = ib_done(dmax, fmax_, tol);
+            }
+            it += ran;
+            if (ran & 1) {                                // the newest iterate is in Fn
+                std::swap(c->ib_F, c->ib_Fn);
+                std::swap(c->ib_F32, c->ib_Fn32);
+            }
         }
     } catch (...) {
         cleanup();

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(128) k_scatter_fp64(ScatterArgs a) {
                     gm += g2 * term;
                 }
                 if (!TERMS && a.gam64 && m >= lokq && m < lokq + nwkq)
-                    a.gam64[a.goff[pair] + (int64_t)np * nwkq + (m - lokq)] = gm;
+                    a.gam64[a.gent[kpl] + a.goff[pair] + (int64_t)np * nwkq + (m - lokq)] = gm;
             }
         }
         if (TERMS) {
@@ -391,6 +391,7 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, bool sf64
     sa.gam32 = ws.gam32;
     sa.gam64 = ws.gam64;
     sa.goff = ws.goff ? ws.goff + cv.g_base : nullptr;
+    sa.gent = ws.gent ? ws.gent + cv.kp0 : nullptr;
     sa.precision = c->opt.precision;
     sa.nstates_chunk = cv.ns;
     sa.nsel_max = 1;

@@ -61,7 +61,8 @@ struct ScatterArgs {
     int tstride;
     float *gam32;                         // Gamma capture (split paths) or nullptr
     double *gam64;                        // Gamma capture (FP64 path) or nullptr
-    const int64_t *goff;                  // chunk pair -> first Gamma entry (with a capture)
+    const uint32_t *goff;                 // with a capture: chunk pair -> first Gamma entry, relative to
+    const int64_t *gent;                  // its k-point's first, gent[chunk k-point]
     int precision;
     int nsel_max;                         // largest band window of the chunk
     int64_t nstates_chunk;                // states of the chunk
@@ -77,10 +78,11 @@ struct WorkSet {
     const double *pair_w = nullptr;       // per pair weight of pairs_dev (FP64 path only)
     // Gamma capture of the iterative BTE (rates mode): for every pair, the block
     // [n in window(k)][m in window(k+q)] of sum_nu |g|^2 [occupation x exp] starting at
-    // goff[pair] (global pair index), in gam64 (FP64 path) or gam32 (split paths)
+    // gent[k-point] + goff[pair] (global indices), in gam64 (FP64 path) or gam32 (split paths)
     float *gam32 = nullptr;
     double *gam64 = nullptr;
-    const int64_t *goff = nullptr;
+    const uint32_t *goff = nullptr;
+    const int64_t *gent = nullptr;
     int ovr_lo = -1, ovr_nsel = -1;
 };
 

@@ -270,7 +270,8 @@ struct SfArgs {
     double *inv_tau;
     const int2 *items;              // {chunk kp, band}
     float *gam;                     // Gamma capture (iterative BTE) or nullptr: row n of each
-    const int64_t *goff;            // pair's block, block start goff[chunk pair]
+    const uint32_t *goff;           // pair's block, block start gent[kp] + goff[chunk pair]
+    const int64_t *gent;
 };
 
 template <int W, int NM, int RC, bool GAM>
@@ -502,7 +503,7 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
                     if constexpr (GAM) {
                         lokq = __ldg(a.win_lo + ikq);
                         nwkq = __ldg(a.win_n + ikq);
-                        grow = a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
+                        grow = a.gent[kp] + a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
                     }
                     const float2 *uq = a.uS + q;                     // element e at uq[e * nk]
                     // small shapes: G (every column) once per pair, shared by its bands
@@ -801,6 +802,7 @@ void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *
     a.items = c->sf_items.as<int2>();
     a.gam = sa.gam32;
     a.goff = sa.goff;
+    a.gent = sa.gent;
     const int ni = (int)items.size();
     const size_t sm = plan.smem;
     if (W == 4 && NM == 3 && r == 1) launch_sf<4, 3, 1>(c, a, ni, sm);

@@ -40,7 +40,8 @@ struct Sf64Args {
     double *inv_tau;
     int nkp;
     double *gam;                    // Gamma capture or nullptr (see scatter_sf.cu)
-    const int64_t *goff;
+    const uint32_t *goff;
+    const int64_t *gent;
 };
 
 // One CTA per (k-point, band): blockIdx.x runs over the chunk's states; the k-point is found in
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
                     if constexpr (GAM) {
                         lokq = __ldg(a.win_lo + ikq);
                         nwkq = __ldg(a.win_n + ikq);
-                        grow = a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
+                        grow = a.gent[kp] + a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
                     }
                     constexpr bool kPreG = X <= 12;   // G kept for all bands of the pair
                     auto column = [&](int x) {
@@ -342,6 +343,7 @@ void sf64_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t
     a.nkp = (int)nkp;
     a.gam = sa.gam64;
     a.goff = sa.goff;
+    a.gent = sa.gent;
     const int64_t ns = sa.nstates_chunk;
     if (ns <= 0) return;
     if (W == 4 && r == 1) launch<4, 3, 1>(c, a, ns, plan.smem);

@@ -814,7 +814,7 @@ __global__ void __maxnreg__(168) k_scatter_tc(TcArgs a) {
                 if (active) {
                     lokq = __ldg(s.win_lo + ikq);
                     nwkq = __ldg(s.win_n + ikq);
-                    goffp = s.goff[pair];
+                    goffp = s.gent[m.kpl] + s.goff[pair];
                 }
             }
             if (tile + 1 < t_end)
