@@ -133,6 +133,7 @@ struct epwi_ctx {
     DevBuf kp_pairs;               // int64 [nkp+1] pair offsets
     DevBuf sieve_mask;             // uint32 [nkp][mask_words]: sieve decisions of the count
     int64_t mask_words = 0;        // words per k-point (0: no mask, the fill re-evaluates)
+    DevBuf chunk_mask, chunk_counts;   // decisions of one chunk where there is no mask (sieve_mask_chunk)
     DevBuf inv_tau;                // double [nstates]
     DevBuf st_k, st_n;             // int32 [nstates]
     DevBuf focc;                   // double [Nk][W] Fermi-Dirac
@@ -142,6 +143,7 @@ struct epwi_ctx {
 
     // scratch
     DevBuf pairs;                  // int32 q index per pair of the chunk
+    DevBuf runs;                   // int32 run tables of the chunk's k-points (sieve.cuh)
     DevBuf ghat;                   // per-chunk Re->k output
     DevBuf tiles;                  // int4 per tile {kp_local, pair_begin, pair_end, 0}
     DevBuf tile_part;              // double [tile][W] partial sums
@@ -162,7 +164,6 @@ struct epwi_ctx {
     DevBuf tc_err;                 // int: timed-out waits in the tensor-core kernel
     DevBuf tc_meta;                // per-tile metadata of the tensor-core kernel
     DevBuf tc_arows;               // gathered-A mode: split phase rows of every grid point
-    DevBuf sf_items;               // fp32 mode: (k-point, band) work items of a chunk
     int sf_r = 0;                  // fp32 mode: half-width of the bounding cube of R_p
     std::vector<int> h_rp_cube;    // fp32 mode: R_p index of each bounding-cube point, -1 if absent
     DevBuf gsf32;                  // fp32 mode: g' [Re][cube forms][Nm][W][W] (+-R recombined)
@@ -170,9 +171,8 @@ struct epwi_ctx {
     DevBuf gsf64;                  // FP64 mode: the same in FP64
     bool sf_g64_ready = false;
     bool rp_twice = false;         // R_p holds a vector twice (no FP64 cube form)
-    DevBuf sf_Vt32;                // fp32 mode: float2 [m][Nk][i], columns of V band-major
-    DevBuf sf_ef;                  // fp32 mode: float2 [m][Nk]: (eps - mu, f), band-major
-    DevBuf sf_uS, sf_wn;           // fp32 mode: float2 [mu nu][Nq] u(q), [nu][Nq] (hbar omega, N)
+    DevBuf sf_kqt, sf_qt;          // fp32 mode: gather tables of the k+q and q sides (scatter_sf.cu)
+    DevBuf sf_coef;                // fp32 mode: cos and sin of the axes' phases
     DevBuf gcube32;                // split modes, R_p not a cube: weighted g in the bounding cube
     bool gcube_ready = false;      // gcube32 built for the current system
     // factorised H(k) / D(q) builds: weighted H and Phi/sqrt(m m) embedded in the bounding cubes
@@ -235,12 +235,12 @@ struct epwi_ctx {
         DevBuf *all[] = {&Re, &Rp, &Rcart, &Hw, &Phiw, &mode_mass, &gw64, &gw32, &ph64, &ph32,
                          &eps, &eps32, &V, &V32, &vel, &hw, &hwmax32, &hw32, &u, &u32, &eig_flag,
                          &kpts, &win_lo, &win_n, &kp_state, &kp_pairs, &inv_tau, &st_k,
-                         &st_n, &focc, &nocc, &pairs, &ghat, &tiles, &tile_part, &kp_tile,
+                         &st_n, &focc, &nocc, &pairs, &runs, &ghat, &tiles, &tile_part, &kp_tile,
                          &scan_tmp, &scan_ws, &red_tmp, &counts, &tc_ptab, &tc_erel, &tc_f32,
                          &tc_n32, &tc_hw32, &tc_err, &tc_meta, &is_pairs, &is_w,
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
-                         &ib_pt, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &sf_items, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
-                         &gsf32, &sf_Vt32, &sf_ef, &sf_uS, &sf_wn, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
+                         &ib_pt, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
+                         &gsf32, &sf_kqt, &sf_qt, &sf_coef, &chunk_mask, &chunk_counts, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
                          &re_cube, &ks_T, &col_buf, &gsf64};
         for (DevBuf *b : all) b->release();
         for (DevBuf &b : is_ws) b.release();

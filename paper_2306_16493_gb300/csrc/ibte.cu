@@ -347,7 +347,10 @@ void ibte_prepare(epwi_ctx *c, WorkSet &ws) {
     const int64_t nkp = c->nkp, npairs = c->npairs;
     const bool fp64 = c->opt.precision == EPWI_FP64;
     c->ib_pairs.ensure(sizeof(int) * (npairs + 1));
-    sieve_fill_chunk(c, 0, nkp, c->ib_pairs.as<int>());
+    const int64_t rstride = run_stride(make_grid_info(c));
+    c->runs.ensure(sizeof(int) * (nkp * rstride + 1));
+    sieve_fill_chunk(c, 0, nkp, c->ib_pairs.as<int>(), c->runs.as<int>());
+    ws.runs_dev = c->runs.as<int>();
     EPWI_REQUIRE(c->nstates < (int64_t(1) << 27), EPWI_EUNSUPPORTED, "iterative BTE needs fewer than 2^27 states");
     c->ib_pt.ensure(sizeof(unsigned) * c->nk);
     EPWI_CUDA(cudaMemsetAsync(c->ib_pt.p, 0, sizeof(unsigned) * c->nk, c->stream));

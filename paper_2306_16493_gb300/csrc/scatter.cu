@@ -15,6 +15,7 @@
 #include "epwi_internal.cuh"
 #include "kstage.cuh"
 #include "scatter.cuh"
+#include "sieve.cuh"
 
 namespace {
 
@@ -264,8 +265,6 @@ struct Ev {
 
 }  // namespace
 
-void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs);
-
 // Processes the work set ws (k-points with their pair lists) chunk by chunk.  In rates mode
 // it writes inv_tau for every state of the work set; in g2 mode (g2out != nullptr) it writes
 // |g|^2 per pair instead.
@@ -276,7 +275,8 @@ namespace {
 // local pair of kp), its global pair index base and its states.
 struct ChunkView {
     int64_t kp0, kp1;
-    const int *pairs;
+    const int *pairs, *runs;
+    const uint32_t *mask;                 // sum-factorised kernels
     const int64_t *kp_pairs;
     int64_t p_off;
     int64_t np;
@@ -369,6 +369,9 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, bool sf64
     sa.ovr_lo = ws.ovr_lo;
     sa.ovr_nsel = ws.ovr_nsel;
     sa.pairs = cv.pairs;
+    sa.runs = cv.runs;
+    sa.mask = cv.mask;
+    sa.mask_words = sieve_words(c);
     sa.ghat64 = c->ghat.as<double2>();
     sa.ghat_raw = c->ghat.p;
     sa.V64 = c->V.as<double2>();
@@ -403,8 +406,7 @@ int64_t run_chunk(epwi_ctx *c, const WorkSet &ws, const ChunkView &cv, bool sf64
     }
     cudaEventRecord(tm.sc.e[0], c->stream);
     if (sf) {
-        std::vector<int64_t> hks(ws.h_kp_state.begin() + cv.kp0, ws.h_kp_state.begin() + cv.kp1 + 1);
-        sf_scatter(c, sa, nkpc, cv.kp_pairs, cv.p_off, hks);
+        sf_scatter(c, sa, nkpc, cv.kp_pairs, cv.p_off);
     } else if (tc) {
         tc_scatter(c, sa, nt);
     } else if (sf64) {
@@ -455,17 +457,17 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
     if (tc) tc_prepare(c);
     // Sum-factorised FP64 rates: needs pair lists in the sieve's order (filled here, or for the
     // Gamma capture) and the window's bands, without weights or per-pair outputs
-    const bool sf64 = !sf && !tc && !g2out && !tout && !ws.pair_w && ws.ovr_nsel < 0 && (!ws.pairs_dev || ws.gam64) &&
+    const bool sf64 = !sf && !tc && !g2out && !tout && !ws.pair_w && ws.ovr_nsel < 0 && (!ws.pairs_dev || ws.runs_dev) &&
                       sf64_ok(c);
     if (sf64) sf64_prepare(c);
-    // chunk limits: pairs and Re->k output size
-    // pair lists per chunk: 2^32 q indices (16 GiB) for the sum-factorised kernels, whose launches are one
-    // CTA per state and need thousands of states per chunk to fill the GPU on large grids (200^3:
-    // ~1.8 M pairs per state); 2^27 otherwise
-    const int64_t max_pairs = int64_t(1) << (sf || sf64 ? 32 : 27);
+    // chunk limits: Re->k output size, and the pair lists (2^27 q indices) or, in the sum-factorised
+    // kernels, the decision mask where it is evaluated per chunk (2 GiB)
+    const int64_t max_pairs = sf || sf64 ? (int64_t)1 << 62 : int64_t(1) << 27;
     const size_t state_bytes = sf ? sf_state_bytes(c) : sf64 ? sf64_state_bytes(c) : tc ? tc_state_bytes(c) : sizeof(double2) * nrow;
     const int64_t max_states = std::max<int64_t>(1, (int64_t)((size_t(3) << 30) / state_bytes));
-    const int64_t kp_cap = c->opt.kpoint_chunk > 0 ? c->opt.kpoint_chunk : (int64_t)1 << 40;
+    const int64_t mask_cap = (sf || sf64) && !c->mask_words ? std::max<int64_t>(1, (int64_t(1) << 29) / sieve_words(c)) : (int64_t)1 << 40;
+    const int64_t kp_cap = std::min(mask_cap, c->opt.kpoint_chunk > 0 ? (int64_t)c->opt.kpoint_chunk : (int64_t)1 << 40);
+    const int64_t rstride = run_stride(make_grid_info(c));
     StageTimers tm;
     int64_t kp0 = 0, nchunks = 0, ntiles_total = 0;
     while (kp0 < ws.nkp) {
@@ -485,7 +487,11 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
         cv.kp_pairs = ws.kp_pairs + kp0;
         cudaEventRecord(tm.fill.e[0], c->stream);
         cv.pairs = ws.pairs_dev ? ws.pairs_dev + cv.p_off : nullptr;
-        if (!cv.pairs) {
+        cv.runs = ws.runs_dev ? ws.runs_dev + kp0 * rstride : nullptr;
+        cv.mask = nullptr;
+        if (sf || sf64) {
+            cv.mask = sieve_mask_chunk(c, kp0, kp1);     // the kernels read the decisions themselves
+        } else if (!cv.pairs) {
             c->pairs.ensure(sizeof(int) * (cv.np + 1));
             sieve_fill_chunk(c, kp0, kp1, c->pairs.as<int>());
             cv.pairs = c->pairs.as<int>();

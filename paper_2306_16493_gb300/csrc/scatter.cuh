@@ -42,6 +42,9 @@ struct ScatterArgs {
     const int *win_lo, *win_n;
     int ovr_lo, ovr_nsel;
     const int *pairs;                     // chunk pair list: q index
+    const uint32_t *mask;                 // sieve decisions of the chunk's k-points (sum-factorised kernels):
+    int64_t mask_words;                   // words per k-point
+    const int *runs;                      // run tables of the chunk's k-points (with a capture)
     const double2 *ghat64;
     const void *ghat_raw;
     const double2 *V64;
@@ -75,6 +78,7 @@ struct WorkSet {
     const int64_t *kp_pairs = nullptr;
     std::vector<int64_t> h_kp_state, h_kp_pairs;
     const int *pairs_dev = nullptr;       // all pairs, or nullptr: sieve fill per chunk
+    const int *runs_dev = nullptr;        // run tables of all k-points (pairs_dev in the sieve's order)
     const double *pair_w = nullptr;       // per pair weight of pairs_dev (FP64 path only)
     // Gamma capture of the iterative BTE (rates mode): for every pair, the block
     // [n in window(k)][m in window(k+q)] of sum_nu |g|^2 [occupation x exp] starting at
@@ -91,7 +95,12 @@ struct WorkSet {
 // band and mode, tout[(pair * tstride + np) * Nm + nu].
 void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout = nullptr,
                      int tstride = 0);
-void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs);
+// Pair lists of window k-points kp0 .. kp1-1 and, when runs is given, their run tables (sieve.cuh).
+void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs, int *runs = nullptr);
+// Decision mask of window k-points kp0 .. kp1-1 (the mask of the count, or evaluated again into a
+// chunk buffer) and its words per k-point.
+int64_t sieve_words(const epwi_ctx *c);
+const uint32_t *sieve_mask_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1);
 
 // split-precision (tcgen05) path
 size_t tc_state_bytes(const epwi_ctx *c);
@@ -120,5 +129,4 @@ bool sf64_ok(const epwi_ctx *c);
 void sf64_prepare(epwi_ctx *c);
 size_t sf64_state_bytes(const epwi_ctx *c);
 void sf64_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off);
-void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off,
-                const std::vector<int64_t> &h_kp_state_chunk);
+void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off);

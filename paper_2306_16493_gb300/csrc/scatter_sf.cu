@@ -11,20 +11,29 @@
 // of 4).  The recombination acts on the R_p index only, so it commutes with the Re->k sum and
 // the U^dag(k) rotation and is applied to g(Re, Rp) itself (k_sf_transform).
 //
-// The sieve lists the pairs of a k-point in plane blocks pb of 256 consecutive (q2, q3)
-// combinations, then by q1, then by combination.  For the state (k, n) of one CTA:
+// The sieve decides the pairs of a k-point in plane blocks pb of 256 consecutive (q2, q3)
+// combinations, by q1 (8 mask words a run).  For the state (k, n) of one CTA:
 //   Y[f1][f3][j]  = sum_f2 c2(q2_j)[f2] ghat'[f1][f2][f3]    per plane block and group of q2 values j
 //   U[f3][j]      = sum_f1 c1(q1)[f1]  Y[f1][f3][j]           per run (plane block, q1, q2 group)
 //   G             = sum_f3 c3(q3)[f3]  U[f3][j(q)]            per pair
 // with ghat' = (g' P^el) U^dag(k) from the FP32 Re->k stage, every column (mu, i) at once.
-// U is built for a batch of runs by the whole CTA; then every thread takes pairs of the batch
-// from one flat list.  Per pair, each lane loops over the final bands m that have a mode within
-// c eta of either energy shell (others add exactly zero), and for each band streams the modes
-// mu: h = sum_i conj(V_im(k+q)) G[mu][i], g_nu += h u_mu,nu(q); then |g|^2 and the two delta
-// terms, in FP32.  With a Gamma capture (iterative BTE) the CTA also writes its band's row of
-// every pair's Gamma block (rows of bands out of range stay at the zero the buffer was cleared
-// to).  Lane sums are FP32 within a batch, FP64 across batches, and the CTA adds its threads
-// in a fixed order, so the result is deterministic and independent of k-point chunking.
+// A warp takes the two runs q1 and N1 - q1 of a group: U = E +- O from one pass over Y, their mask
+// words expanded to a list of combinations in shared memory, then 32 pairs at a time.  Per pair,
+// the final bands m that have a mode within c eta of either energy shell count (others add
+// exactly zero); a lane does its first one, further ones go to a list that is worked off 32 at a
+// time.  Per band the modes mu are streamed: h = sum_i conj(V_im(k+q)) G[mu][i], g_nu += h u_mu,nu(q); then
+// |g|^2 and the two delta terms, in FP32.  With a Gamma capture (iterative BTE) the CTA also writes
+// its band's row of every pair's Gamma block (rows of bands out of range stay at the zero the
+// buffer was cleared to), a pair's place in the list being its run's first plus its rank there.  Lane
+// sums are FP32 within an item (the two runs), FP64 across items, added in a fixed order, so the
+// result is deterministic and independent of k-point chunking.
+//
+// Bound by the instructions and gathers of the pairs (k_kq_table, k_q_table: tiles of 64 grid points, so
+// that the 32 neighbouring points of a warp share cache lines).  Reading the mask directly needs no pair
+// lists (4 bytes per pair written and read twice) and no search for the runs in them.  Measured on
+// one GB300, Al-like 48^3 (1.26 G pairs), list fill and this kernel together: 57.1 ms with a run per
+// warp pass, 50.7 ms with both runs from one pass and the runs' bounds from a table, 49.3 ms from the
+// mask; 20 x 27 x 45 (61 M pairs) 4.6, 3.4 and 3.3 ms.
 #include <algorithm>
 
 #include "epwi_internal.cuh"
@@ -34,7 +43,6 @@
 #include "sieve.cuh"
 
 namespace {
-
 
 // Re->k in FP32: ghat32[state][row] = sum_j [sum_Re w e^{ik.Re} g(Re)[row][j]] V_{j, lo+n}(k),
 // row = (cube form, mu, i); one thread per row, KG k-points per block row.
@@ -171,26 +179,14 @@ __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, c
     const int cf = (int)(t % D3);
     const int64_t re = t / D3;
     const int f[3] = {cf / (Dc * Dc), (cf / Dc) % Dc, cf % Dc};
-    int Rv[3][2], nt[3];
-    double2 cv[3][2];
+    int Rv[3][2], nt[3], pw[3][2];                  // terms per axis: R, and the power of i
     for (int a = 0; a < 3; ++a) {
-        if (f[a] == 0) {
-            nt[a] = 1;
-            Rv[a][0] = 0;
-            cv[a][0] = make_double2(1, 0);
-        } else {
-            const int R = (f[a] + 1) / 2;
-            nt[a] = 2;
-            Rv[a][0] = R;
-            Rv[a][1] = -R;
-            if (f[a] & 1) {
-                cv[a][0] = make_double2(1, 0);
-                cv[a][1] = make_double2(1, 0);
-            } else {
-                cv[a][0] = make_double2(0, 1);
-                cv[a][1] = make_double2(0, -1);
-            }
-        }
+        const int R = (f[a] + 1) / 2, even = f[a] && !(f[a] & 1);
+        nt[a] = f[a] ? 2 : 1;
+        Rv[a][0] = R;
+        Rv[a][1] = -R;
+        pw[a][0] = even ? 1 : 0;                    // i v[R]
+        pw[a][1] = even ? 3 : 0;                    // -i v[-R]
     }
     double2 s = make_double2(0, 0);
     for (int x = 0; x < nt[0]; ++x)
@@ -201,7 +197,10 @@ __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, c
                 if (rp < 0) continue;
                 const size_t gi = ((size_t)re * nRp + rp) * rowlen + e;
                 const double2 v = g64 ? g64[gi] : make_double2(g32[gi].x, g32[gi].y);
-                s = cadd(s, cmul(cmul(cmul(cv[0][x], cv[1][y]), cv[2][z]), v));
+                const int p = (pw[0][x] + pw[1][y] + pw[2][z]) & 3;     // s += i^p v
+                const double px = p & 1 ? v.y : v.x, py = p & 1 ? v.x : v.y;
+                s.x += p == 1 || p == 2 ? -px : px;
+                s.y += p & 2 ? -py : py;
             }
     using R = decltype(C2::x);
     C2 o;
@@ -210,69 +209,98 @@ __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, c
     out[idx] = o;
 }
 
-// Band-major tables of the k+q side (FP32): Vb[m][k][i] = V[k][i][m] and
-// EF[m][k] = (eps_mk - mu, f_mk), so that lanes on consecutive k+q points and one band m read
-// contiguous memory.
-__global__ void k_band_major_v(int64_t nk, int W, const float2 *__restrict__ V, float2 *__restrict__ Vb) {
+// Gather tables (FP32) in blocks of 64 grid points, one row of 64 per element, so that lanes on
+// nearby points read contiguous memory and one address serves every element of a point (the rows
+// lie at fixed distances).
+// k+q side, [k / 64][m]: W / 2 rows of two V_im(k) each (odd W: W rows of one), then one row of
+// (eps_mk - mu, f_mk).  q side, [q / 64]: N_m^2 rows of u_mu,nu(q), then N_m rows of
+// (hbar omega, N).  Sizes in float2.
+constexpr int kTb = 64;
+__host__ __device__ constexpr int kq_block(int W) { return kTb * (W + 1); }
+__host__ __device__ constexpr int q_block(int NM) { return kTb * (NM * NM + NM); }
+
+__global__ void k_kq_table(int64_t nk, int W, const float2 *__restrict__ V, const float *__restrict__ erel,
+                           const float *__restrict__ f32, float2 *__restrict__ out) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nk * W * W) return;
-    const int i = (int)(idx % W);
-    const int64_t t = idx / W;
-    const int64_t k = t % nk;
-    const int m = (int)(t / nk);
-    Vb[idx] = V[k * W * W + i * W + m];
+    const int64_t k = idx / W;
+    const int m = (int)(idx % W);
+    if (k >= nk) return;
+    float2 *o = out + ((k / kTb) * W + m) * kq_block(W);
+    const int x = (int)(k % kTb), w = W % 2 ? 1 : 2;
+    for (int i = 0; i < W; ++i) o[(i / w) * (kTb * w) + x * w + i % w] = V[k * W * W + i * W + m];
+    o[kTb * W + x] = make_float2(erel[idx], f32[idx]);
 }
 
-// Structure-of-arrays tables of the q side (FP32): uS[mu nu][q] = u_mu,nu(q) and
-// wn[nu][q] = (hbar omega, N), so that lanes on consecutive q read contiguous memory.
-__global__ void k_soa_q(int64_t nq, int NM, const float2 *__restrict__ u, const float *__restrict__ hw,
-                        const float *__restrict__ n, float2 *__restrict__ uS, float2 *__restrict__ wn) {
+__global__ void k_q_table(int64_t nq, int NM, const float2 *__restrict__ u, const float *__restrict__ hw,
+                          const float *__restrict__ n, float2 *__restrict__ out) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nq * NM * NM) return;
     const int64_t q = idx % nq;
     const int e = (int)(idx / nq);
-    uS[idx] = u[q * NM * NM + e];
-    if (e < NM) wn[idx] = make_float2(hw[q * NM + e], n[q * NM + e]);
-}
-
-__global__ void k_band_major_ef(int64_t nk, int W, const float *__restrict__ erel, const float *__restrict__ f32,
-                                float2 *__restrict__ ef) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nk * W) return;
-    const int64_t k = idx % nk;
-    const int m = (int)(idx / nk);
-    ef[idx] = make_float2(erel[k * W + m], f32[k * W + m]);
+    if (e >= NM * NM + NM) return;
+    float2 v;
+    if (e < NM * NM) v = u[q * NM * NM + e];
+    else v = make_float2(hw[q * NM + e - NM * NM], n[q * NM + e - NM * NM]);
+    out[(q / kTb) * q_block(NM) + e * kTb + q % kTb] = v;
 }
 
 struct SfArgs {
     GridInfo g;
     int nplane;                     // N2 N3
-    FDiv fplane, fjq;               // division by N2 N3 and by jq
+    FDiv fn3, fper;                 // division by N3 and by the columns of a group (jq X / 2 or jq X)
     int jq;                         // q2 values per group (Y and the U buffers hold one group)
     int njg;                        // groups per plane block (over the largest block)
     int pbmax;                      // plane blocks
-    const float2 *ph32;             // e^{2 pi i m / L}
+    const float *coef;              // [N1 + N2 + N3][D - 1] cos, sin of theta R (k_sf_coef)
     const float2 *ghat;             // [state - s_base][D^3 forms][N_m][W]
     const int *kpts, *win_lo, *win_n;
     const int64_t *kp_state;        // chunk k-points' first states (global)
     int64_t s_base;
-    const int64_t *kp_pairs;        // chunk-local pair offsets, minus p_off
-    int64_t p_off;
-    const int *pairs;               // chunk pair list: q index
-    const float2 *Vb32, *u32;       // Vb32[m][k][i]: band-major columns of V
-    const float2 *ef;               // [m][k]: (eps - mu, f), band-major
-    const float2 *uS;               // [mu nu][q]: u(q), structure of arrays
-    const float2 *wn;               // [nu][q]: (hbar omega, N), structure of arrays
-    int64_t nk;
-    const float *erel, *f32, *n32, *hw32, *hwmax32;
+    const uint32_t *mask;           // sieve decisions of the chunk's k-points (rows of mask_words)
+    int64_t mask_words;
+    const float2 *kqt, *qt;         // gather tables (k_kq_table, k_q_table)
+    const float *erel, *hwmax32;
     float ceta32, inv_eta32;
     double pref;                    // 2 pi / (hbar N_q sqrt(pi) eta)
     double *inv_tau;
-    const int2 *items;              // {chunk kp, band}
+    int nkp;                        // k-points of the chunk
     float *gam;                     // Gamma capture (iterative BTE) or nullptr: row n of each
     const uint32_t *goff;           // pair's block, block start gent[kp] + goff[chunk pair]
     const int64_t *gent;
+    const int64_t *kp_pairs;        // with a capture: chunk-local pair offsets, minus p_off, and the
+    int64_t p_off;                  // run tables (sieve.cuh), which place a pair in the list
+    const int *runs;
+    int64_t run_stride;
 };
+
+template <int NF>
+__device__ __forceinline__ void load_coef(const float *p, float (&c)[NF]) {
+    if constexpr (NF == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(p);
+        c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+    } else {
+#pragma unroll
+        for (int f = 0; f < NF; f += 2) {
+            const float2 v = *reinterpret_cast<const float2 *>(p + f);
+            c[f] = v.x;
+            c[f + 1] = v.y;
+        }
+    }
+}
+
+template <int NF>
+__device__ __forceinline__ void load_coef_g(const float *__restrict__ p, float (&c)[NF]) {
+    if constexpr (NF == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+        c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+    } else {
+#pragma unroll
+        for (int f = 0; f < NF; f += 2) {
+            const float2 v = __ldg(reinterpret_cast<const float2 *>(p + f));
+            c[f] = v.x;
+            c[f + 1] = v.y;
+        }
+    }
+}
 
 template <int W, int NM, int RC, bool GAM>
 __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfArgs a) {
@@ -281,117 +309,146 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
     constexpr int X = NM * W;                    // columns (mu, i)
     constexpr bool V2 = (W % 2) == 0;            // rows of W float2 are 16-byte aligned
     constexpr int kMuUnroll = NM <= 3 ? NM : 1;  // wide systems: one mode row at a time (registers)
-    constexpr bool kPreG = X <= 12 && X % 2 == 0;  // G of a pair kept in registers for its bands
     extern __shared__ __align__(16) float2 sm[];
-    const int N1 = a.g.n1, N2 = a.g.n2, N3 = a.g.n3, L = a.g.L;
+    const int N1 = a.g.n1, N2 = a.g.n2, N3 = a.g.n3;
     const int JQ = a.jq, NJG = a.njg;
-    const SfSmem lay = sf_smem_layout(D, X, JQ, N1, N2, N3, NJG, a.pbmax);
+    const SfSmem lay = sf_smem_layout(D, X, W, JQ, N1, N3, NJG, a.pbmax, sizeof(float));
     float2 *Y = sm;                              // [D f1][D f3][JQ][X]
-    float *CS = reinterpret_cast<float *>(Y + lay.y + lay.u);   // [N1 + N2 + N3][NF]: cos, sin of theta R
-    int *cq = reinterpret_cast<int *>(CS + lay.cs);     // [256]: (j << 16) | q3 of combination t
-    int *ss = cq + kSieveBlock;                  // [N1 NJG]: segment start (relative), -1 if none
-    int *se = ss + N1 * NJG;                     // [N1 NJG]: segment end
-    int *gl = se + N1 * NJG;                     // [N1]: runs (q1) of the current group
-    int *pbs = gl + N1;                          // [pbmax + 1]: first pair of each plane block
-    int *nglist = pbs + a.pbmax + 1;             // [1]
-    __shared__ double wsum[kSfWarps];
-    const int2 item = a.items[blockIdx.x];
-    const int kp = item.x, n = item.y;
+    float *CS3 = reinterpret_cast<float *>(Y + lay.y + lay.u);  // [N3][NF]: axis-3 coefficients
+    const int nh = N1 / 2 + 1;
+    float *rs = CS3 + lay.cs;                           // [nh]: sums of the current group's items
+    int *gl = reinterpret_cast<int *>(rs + lay.rs);     // [nh]: the items, (q1, N1 - q1)
+    int *nglist = gl + nh;                              // [2]: items of the group, next one to take
+    uint32_t *flags = reinterpret_cast<uint32_t *>(nglist + 2);      // bit pb NJG + jg: the group has pairs
+    uint8_t *clist = reinterpret_cast<uint8_t *>(flags + lay.flags) + (threadIdx.x >> 5) * kSieveBlock;
+    uint16_t *left = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(flags + lay.flags) + kSfWarps * kSieveBlock) +
+                     (threadIdx.x >> 5) * 32 * W;       // see below
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    float2 *Uw = Y + lay.y + (size_t)wid * D * JQ * X;   // this warp's run: [D f3][JQ][X]
+    const int ustride = D * JQ * X;
+    float2 *Uw = Y + lay.y + (size_t)wid * 2 * ustride;  // this warp's two runs: [2][D f3][JQ][X]
+    const int64_t s = a.s_base + blockIdx.x;     // global state
+    // its k-point: the last one whose first state is <= s (every listed k-point has a state)
+    const int kp = (int)lower_bound(0, a.nkp, s + 1, [&](int64_t p) { return a.kp_state[p + 1]; });
+    const int n = (int)(s - a.kp_state[kp]);
     const int ik = a.kpts[kp];
     const int lo = a.win_lo[ik];
-    const int64_t s = a.kp_state[kp] + n;        // global state
     const float2 *gs = a.ghat + (size_t)(s - a.s_base) * D * D * D * X;
-    // cos / sin tables of the three axes (exact integer reduction of x R onto the L roots)
-    for (int e = tid; e < (N1 + N2 + N3) * RC; e += kSfThreads) {
-        const int R = e % RC + 1, x = e / RC;
-        int xx, st;
-        if (x < N1) { xx = x; st = a.g.s1; }
-        else if (x < N1 + N2) { xx = x - N1; st = a.g.s2; }
-        else { xx = x - N1 - N2; st = a.g.s3; }
-        const int t = (int)(((int64_t)xx * st % L) * R % L);
-        const float2 v = a.ph32[t];
-        CS[x * NF + 2 * (R - 1)] = v.x;
-        CS[x * NF + 2 * (R - 1) + 1] = v.y;
-    }
-    const float *CS1 = CS, *CS2 = CS + N1 * NF, *CS3 = CS + (N1 + N2) * NF;
+    const float *CS1 = a.coef, *CS2 = CS1 + N1 * NF;
+    for (int e = tid; e < N3 * NF; e += kSfThreads) CS3[e] = CS2[N2 * NF + e];
     const int nplane = a.nplane;
     const int pb_n = (nplane + kSieveBlock - 1) / kSieveBlock;
-    const int64_t P0 = a.kp_pairs[kp] - a.p_off, P1 = a.kp_pairs[kp + 1] - a.p_off;
-    const int *pl = a.pairs + P0;                // this k-point's pairs, relative index
-    const int np = (int)(P1 - P0);
-    // first pair of every plane block (the list is ordered by plane block)
-    for (int pb = tid; pb <= pb_n; pb += kSfThreads)
-        pbs[pb] = (int)lower_bound(0, np, pb, [&](int64_t p) {
-            const int q = pl[p];
-            return (int64_t)((q - fdiv(q, a.fplane) * nplane) / kSieveBlock);
-        });
+    const uint32_t *mrow = a.mask + (int64_t)kp * a.mask_words;   // [pb][q1][8 words]
+    // groups with pairs: every thread takes runs (pb, q1) and marks the groups of their set bits
+    for (int e = tid; e < (int)lay.flags; e += kSfThreads) flags[e] = 0u;
+    __syncthreads();
+    for (int r = tid; r < pb_n * N1; r += kSfThreads) {
+        const uint4 *w4 = reinterpret_cast<const uint4 *>(mrow) + 2 * (int64_t)r;
+        const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
+        const uint32_t w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        const int pb = r / N1;
+        if (NJG == 1) {
+            if (w[0] | w[1] | w[2] | w[3] | w[4] | w[5] | w[6] | w[7]) atomicOr(flags + (pb >> 5), 1u << (pb & 31));
+            continue;
+        }
+        const int q2lo = fdiv(pb * kSieveBlock, a.fn3);
+        int seen = -1;                           // last group marked
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            uint32_t b = w[x];
+            while (b) {
+                const int c = x * 32 + __ffs(b) - 1;
+                const int jg = (fdiv(pb * kSieveBlock + c, a.fn3) - q2lo) / JQ;
+                if (jg != seen) {
+                    const int f = pb * NJG + jg;
+                    atomicOr(flags + (f >> 5), 1u << (f & 31));
+                    seen = jg;
+                }
+                // on to the group's end
+                const int end = (q2lo + (jg + 1) * JQ) * N3 - pb * kSieveBlock - x * 32;
+                b = end < 32 ? b & ~((1u << end) - 1u) : 0u;
+            }
+        }
+    }
     int k1, k2, k3;
     grid_coords(a.g, ik, k1, k2, k3);
     const float en = a.erel[(int64_t)ik * W + lo + n];
     const float ceta = a.ceta32, ieta = a.inv_eta32;
-    double acc = 0;                              // this warp's run sums (lane 0)
+    double acc = 0;                              // warp 0: sums of the items lane, lane + 32, ...
     __syncthreads();
     for (int pb = 0; pb < pb_n; ++pb) {
-        const int seg0 = pbs[pb], nseg = pbs[pb + 1] - seg0;   // the plane block's pairs
-        if (nseg == 0) continue;
-        const int *pp = pl + seg0;
         const int c_lo = pb * kSieveBlock, c_hi = min(nplane, c_lo + kSieveBlock) - 1;
-        const int q2lo = c_lo / N3, nq2 = c_hi / N3 - q2lo + 1;
+        const int q2lo = fdiv(c_lo, a.fn3), nq2 = fdiv(c_hi, a.fn3) - q2lo + 1;
         const int njg = (nq2 + JQ - 1) / JQ;
-        for (int t = tid; t < kSieveBlock; t += kSfThreads) {
-            const int c = c_lo + t, q2 = c / N3;
-            cq[t] = ((q2 - q2lo) << 16) | (c - q2 * N3);
-        }
-        for (int t = tid; t < N1 * NJG; t += kSfThreads) ss[t] = -1;
-        __syncthreads();
-        // segments: the block's pairs are ordered by q1, then by combination (so by q2 group);
-        // key = q1 NJG + group, neighbours' keys by shuffle
-        auto keyof = [&](int t) -> int {
-            const int q = pp[t];
-            const int q1 = fdiv(q, a.fplane);
-            const int j = cq[q - q1 * nplane - c_lo] >> 16;
-            return q1 * NJG + fdiv(j, a.fjq);
-        };
-        for (int t0 = wid * 32; t0 < nseg; t0 += kSfThreads) {
-            const int t = t0 + lane;
-            const bool on = t < nseg;
-            const int key = on ? keyof(t) : -1;
-            int kprev = __shfl_up_sync(0xffffffffu, key, 1);
-            int knext = __shfl_down_sync(0xffffffffu, key, 1);
-            if (lane == 0 && t > 0 && on) kprev = keyof(t - 1);
-            if (lane == 31 && t + 1 < nseg) knext = keyof(t + 1);
-            if (on) {
-                if (t == 0 || kprev != key) ss[key] = t;
-                if (t == nseg - 1 || knext != key) se[key] = t + 1;
-            }
-        }
-        __syncthreads();
+        const uint32_t *mpb = mrow + (int64_t)pb * N1 * 8;
         for (int jg = 0; jg < njg; ++jg) {
+            const int fl = pb * NJG + jg;
+            if (!((flags[fl >> 5] >> (fl & 31)) & 1u)) continue;
             const int j0 = jg * JQ, jn = min(JQ, nq2 - j0);
-            // the group's non-empty runs, in q1 order (warp 0)
+            // combinations [r0, r1) of the plane block belong to the group
+            const int r0 = max(0, (q2lo + j0) * N3 - c_lo), r1 = min(kSieveBlock, (q2lo + j0 + jn) * N3 - c_lo);
+            // bits of word x (of 8) inside the group
+            auto in_group = [&](int x) -> uint32_t {
+                const int a0 = min(max(r0 - 32 * x, 0), 32), a1 = min(max(r1 - 32 * x, 0), 32);
+                const uint32_t lo_m = a0 < 32 ? ~0u << a0 : 0u, hi_m = a1 < 32 ? ~(~0u << a1) : ~0u;
+                return lo_m & hi_m;
+            };
+            // the group's items {q1, N1 - q1} with pairs (warp 0): the two-run ones first
             if (wid == 0) {
                 int cnt = 0;
-                for (int q0 = 0; q0 < N1; q0 += 32) {
-                    const int q1 = q0 + lane;
-                    const bool on = q1 < N1 && ss[q1 * NJG + jg] >= 0;
+                const int n2 = (N1 - 1) / 2;                     // items with two runs
+                auto filled = [&](int q1) {
+                    const uint4 *w4 = reinterpret_cast<const uint4 *>(mpb) + 2 * q1;
+                    const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
+                    if (NJG == 1) return (u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w) != 0u;
+                    return ((u.x & in_group(0)) | (u.y & in_group(1)) | (u.z & in_group(2)) | (u.w & in_group(3)) |
+                            (v.x & in_group(4)) | (v.y & in_group(5)) | (v.z & in_group(6)) | (v.w & in_group(7))) != 0u;
+                };
+                for (int h0 = 0; h0 < nh; h0 += 32) {
+                    const int h = h0 + lane;                     // 1 .. n2, then 0, then N1 / 2
+                    const int q1 = h < n2 ? h + 1 : h == n2 ? 0 : h;
+                    const bool on = h < nh && (filled(q1) || (h < n2 && filled(N1 - q1)));
                     const unsigned b = __ballot_sync(0xffffffffu, on);
                     if (on) gl[cnt + __popc(b & ((1u << lane) - 1u))] = q1;
                     cnt += __popc(b);
                 }
-                if (lane == 0) *nglist = cnt;
+                if (lane == 0) {
+                    nglist[0] = cnt;
+                    nglist[1] = 0;
+                }
             }
-            // Y of this group's q2 values (all threads), read from ghat' (L1 / L2)
-            {
-                const int per = jn * X;                 // (jj, col) of one (f1, f3)
-                for (int e = tid; e < D * D * per; e += kSfThreads) {
-                    const int r13 = e / per, e2 = e - r13 * per;
+            // Y of this group's q2 values (all threads), read from ghat' (L1 / L2): two columns per
+            // thread and step; the index is taken apart by a launch constant and compile-time ones
+            if constexpr (X % 2 == 0) {
+                const int per4 = JQ * (X / 2);
+                for (int e = tid; e < D * D * per4; e += kSfThreads) {
+                    const int r13 = fdiv(e, a.fper), e2 = e - r13 * per4;
+                    const int jj = e2 / (X / 2), col2 = e2 - jj * (X / 2);
+                    if (jj >= jn) continue;
+                    const int f1 = r13 / D, f3 = r13 - f1 * D;
+                    float c2[NF];
+                    load_coef_g<NF>(CS2 + (q2lo + j0 + jj) * NF, c2);
+                    const float4 *src = reinterpret_cast<const float4 *>(gs + ((f1 * D) * D + f3) * X) + col2;
+                    float4 v = __ldg(src);                   // form f2 = 0
+#pragma unroll
+                    for (int f2 = 1; f2 < D; ++f2) {
+                        const float c = c2[f2 - 1];
+                        const float4 w = __ldg(src + f2 * D * X / 2);
+                        v.x = fmaf(c, w.x, v.x);
+                        v.y = fmaf(c, w.y, v.y);
+                        v.z = fmaf(c, w.z, v.z);
+                        v.w = fmaf(c, w.w, v.w);
+                    }
+                    reinterpret_cast<float4 *>(Y)[e] = v;    // [r13][jj][col], rows of JQ X
+                }
+            } else {
+                for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
+                    const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
                     const int jj = e2 / X, col = e2 - jj * X;
-                    const int f3 = r13 % D, f1 = r13 / D;
+                    if (jj >= jn) continue;
+                    const int f1 = r13 / D, f3 = r13 - f1 * D;
                     const float *c2 = CS2 + (q2lo + j0 + jj) * NF;
                     const float2 *src = gs + ((f1 * D) * D + f3) * X + col;
-                    float2 v = __ldg(src);                   // form f2 = 0
+                    float2 v = __ldg(src);
 #pragma unroll
                     for (int f2 = 1; f2 < D; ++f2) {
                         const float c = c2[f2 - 1];
@@ -399,20 +456,47 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
                         v.x = fmaf(c, w.x, v.x);
                         v.y = fmaf(c, w.y, v.y);
                     }
-                    Y[(r13 * JQ + jj) * X + col] = v;
+                    Y[e] = v;
                 }
             }
             __syncthreads();
-            const int ng = *nglist;
-            // runs round-robin over the warps (a fixed assignment keeps the sums deterministic)
-            for (int r = wid; r < ng; r += kSfWarps) {
+            const int ng = nglist[0];
+            // items are taken from a counter; each writes its own sum, so the result does not
+            // depend on which warp takes it
+            while (true) {
+                int r = 0;
+                if (lane == 0) r = atomicAdd(nglist + 1, 1);
+                r = __shfl_sync(0xffffffffu, r, 0);
+                if (r >= ng) break;
                 const int q1 = gl[r];
-                const int t0 = ss[q1 * NJG + jg], t1 = se[q1 * NJG + jg];
-                // U of the run: for each form f3, the contiguous (jj, col) row of Y
+                const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
+                // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
+                const int wx = lane & 7;
+                uint32_t word = 0u;
+                if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
+                int skip = 0;                                    // pairs of the run in earlier groups (capture)
+                if (NJG > 1) {
+                    if constexpr (GAM) skip = __popc(word & (r0 > 32 * wx + 31 ? ~0u : r0 > 32 * wx ? ~(~0u << (r0 - 32 * wx)) : 0u));
+                    word &= in_group(wx);
+                }
+                int npc = __popc(word);
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    npc += __shfl_xor_sync(0xffffffffu, npc, o);
+                    if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
+                }
+                const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
+                int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
+                if constexpr (GAM) {
+                    const int *ru = a.runs + (int64_t)kp * a.run_stride + pb * N1;
+                    t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
+                    t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
+                }
+                // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
+                // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
                 {
                     float c1[NF];
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) c1[f] = CS1[q1 * NF + f];
+                    load_coef_g<NF>(CS1 + q1 * NF, c1);
                     if constexpr (X % 2 == 0) {
                         // (f3, e2) over D rows of per4 float4, walked as one list by the lanes
                         const int per4 = jn * X / 2;
@@ -424,17 +508,23 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
                             }
                             if (f3 >= D) break;
                             const float4 *src = reinterpret_cast<const float4 *>(Y + (size_t)f3 * JQ * X) + e2;
-                            float4 v = src[0];
+                            float4 v = src[0], o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                            for (int f1 = 1; f1 < D; ++f1) {
-                                const float c = c1[f1 - 1];
-                                const float4 w = src[f1 * D * JQ * X / 2];
-                                v.x = fmaf(c, w.x, v.x);
-                                v.y = fmaf(c, w.y, v.y);
-                                v.z = fmaf(c, w.z, v.z);
-                                v.w = fmaf(c, w.w, v.w);
+                            for (int R = 1; R <= RC; ++R) {
+                                const float cc = c1[2 * R - 2], cs = c1[2 * R - 1];
+                                const float4 w = src[(2 * R - 1) * D * JQ * X / 2], z = src[2 * R * D * JQ * X / 2];
+                                v.x = fmaf(cc, w.x, v.x);
+                                v.y = fmaf(cc, w.y, v.y);
+                                v.z = fmaf(cc, w.z, v.z);
+                                v.w = fmaf(cc, w.w, v.w);
+                                o.x = fmaf(cs, z.x, o.x);
+                                o.y = fmaf(cs, z.y, o.y);
+                                o.z = fmaf(cs, z.z, o.z);
+                                o.w = fmaf(cs, z.w, o.w);
                             }
-                            reinterpret_cast<float4 *>(Uw + (size_t)f3 * JQ * X)[e2] = v;
+                            float4 *dst = reinterpret_cast<float4 *>(Uw + (size_t)f3 * JQ * X) + e2;
+                            dst[0] = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+                            dst[ustride / 2] = make_float4(v.x - o.x, v.y - o.y, v.z - o.z, v.w - o.w);
                             e2 += 32;
                         }
                     } else {
@@ -444,201 +534,230 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
                             const float2 *src = Y + (size_t)f3 * JQ * X;
                             float2 *dst = Uw + (size_t)f3 * JQ * X;
                             for (int e = lane; e < per; e += 32) {
-                                float2 v = src[e];
+                                float2 v = src[e], o = make_float2(0.f, 0.f);
 #pragma unroll
-                                for (int f1 = 1; f1 < D; ++f1) {
-                                    const float c = c1[f1 - 1];
-                                    const float2 w = src[e + f1 * D * JQ * X];
-                                    v.x = fmaf(c, w.x, v.x);
-                                    v.y = fmaf(c, w.y, v.y);
+                                for (int R = 1; R <= RC; ++R) {
+                                    const float2 w = src[e + (2 * R - 1) * D * JQ * X], z = src[e + 2 * R * D * JQ * X];
+                                    v.x = fmaf(c1[2 * R - 2], w.x, v.x);
+                                    v.y = fmaf(c1[2 * R - 2], w.y, v.y);
+                                    o.x = fmaf(c1[2 * R - 1], z.x, o.x);
+                                    o.y = fmaf(c1[2 * R - 1], z.y, o.y);
                                 }
-                                dst[e] = v;
+                                dst[e] = make_float2(v.x + o.x, v.y + o.y);
+                                dst[e + ustride] = make_float2(v.x - o.x, v.y - o.y);
                             }
                         }
                     }
                 }
-                __syncwarp();
                 float rate = 0.f;
-                int b1 = k1 + q1;
-                if (b1 >= N1) b1 -= N1;
-                const int qbase = q1 * nplane + c_lo;
-                for (int t = t0 + lane; t < t1; t += 32) {
-                    const int q = pp[t];
-                    const int jq = cq[q - qbase];
-                    const int j = jq >> 16, q3 = jq & 0xffff;
-                    int b2 = k2 + q2lo + j, b3 = k3 + q3;
-                    if (b2 >= N2) b2 -= N2;
-                    if (b3 >= N3) b3 -= N3;
-                    const int ikq = (b1 * N2 + b2) * N3 + b3;   // nk W^2 < 2^31 (checked on the host)
-                    // final bands within the largest kept mode energy + c eta of e_nk (a superset
-                    // of the bands with a mode inside c eta of either shell; the others add zero)
-                    const float lim = __ldg(a.hwmax32 + q) + ceta + 1e-5f;
-                    float emr[W];
-                    if constexpr (W % 4 == 0) {
-#pragma unroll
-                        for (int m4 = 0; m4 < W / 4; ++m4) {
-                            const float4 e4 = __ldg(reinterpret_cast<const float4 *>(a.erel + ikq * W) + m4);
-                            emr[4 * m4] = e4.x; emr[4 * m4 + 1] = e4.y; emr[4 * m4 + 2] = e4.z; emr[4 * m4 + 3] = e4.w;
+                int b1a = k1 + q1, b1b = k1 + q1b;
+                if (b1a >= N1) b1a -= N1;
+                if (b1b >= N1) b1b -= N1;
+                // The pairs of both runs as one list of combinations (one run at a time where both hold
+                // more than a plane block's worth), 32 at a time, each lane with the first final band
+                // within reach of its pair.  The few further bands are kept in a list of the
+                // warp, (pair, band), and worked off 32 at a time as well: one lane with two bands
+                // would otherwise hold up the other 31 for a second pass over the band.
+                const int parts = na + nb <= kSieveBlock ? 1 : 2;
+                for (int part = 0; part < parts; ++part) {
+                    const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
+                    __syncwarp();                                    // Uw is complete, clist is consumed
+                    {
+                        int at = 0;
+                        for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
+                            const uint32_t w = __shfl_sync(0xffffffffu, word, x);
+                            if (w == 0u) continue;                   // uniform over the warp
+                            if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
+                            at += __popc(w);
                         }
-                    } else {
-#pragma unroll
-                        for (int m = 0; m < W; ++m) emr[m] = __ldg(a.erel + ikq * W + m);
                     }
-                    unsigned mask = 0;
+                    int base = 0, nleft = 0;
+                    while (true) {
+                        __syncwarp();
+                        const bool fresh = base < npr && nleft < 32;
+                        if (!fresh && nleft == 0) break;
+                        int tt, m = 0;
+                        bool have;
+                        if (fresh) {
+                            tt = base + lane;
+                            have = tt < npr;
+                            base += 32;
+                        } else {
+                            const int take = min(nleft, 32);
+                            nleft -= take;
+                            have = lane < take;
+                            const int e = have ? left[nleft + lane] : 0;
+                            __syncwarp();                            // before the entries are rewritten
+                            tt = e >> 3;
+                            m = e & 7;
+                        }
+                        const bool second = tt >= npa;
+                        const int c = have ? clist[tt] : 0;
+                        const int q = (second ? q1b : q1) * nplane + c_lo + c;
+                        const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
+                        int b2 = k2 + q2, b3 = k3 + q3;
+                        if (b2 >= N2) b2 -= N2;
+                        if (b3 >= N3) b3 -= N3;
+                        const int ikq = ((second ? b1b : b1a) * N2 + b2) * N3 + b3;   // nk W^2 < 2^31 (checked on the host)
+                        if (fresh) {
+                            // final bands within the largest kept mode energy + c eta of e_nk (a superset
+                            // of the bands with a mode inside c eta of either shell; the others add zero)
+                            unsigned mask = 0;
+                            if (have) {
+                                const float lim = __ldg(a.hwmax32 + q) + ceta + 1e-5f;
+                                if constexpr (W % 4 == 0) {
 #pragma unroll
-                    for (int m = 0; m < W; ++m) mask |= (fabsf(en - emr[m]) <= lim ? 1u : 0u) << m;
-                    if (!mask) continue;
-                    const float2 *Ub = Uw + (j - j0) * X;      // form f3 at + f3 JQ X
-                    float c3[NF], wq[NM], nq[NM];
+                                    for (int m4 = 0; m4 < W / 4; ++m4) {
+                                        const float4 e4 = __ldg(reinterpret_cast<const float4 *>(a.erel + ikq * W) + m4);
+                                        mask |= (fabsf(en - e4.x) <= lim ? 1u : 0u) << (4 * m4);
+                                        mask |= (fabsf(en - e4.y) <= lim ? 2u : 0u) << (4 * m4);
+                                        mask |= (fabsf(en - e4.z) <= lim ? 4u : 0u) << (4 * m4);
+                                        mask |= (fabsf(en - e4.w) <= lim ? 8u : 0u) << (4 * m4);
+                                    }
+                                } else {
 #pragma unroll
-                    for (int f = 0; f < NF; ++f) c3[f] = CS3[q3 * NF + f];
-#pragma unroll
-                    for (int nu = 0; nu < NM; ++nu) {
-                        const float2 v = __ldg(a.wn + (int64_t)nu * a.nk + q);
-                        wq[nu] = v.x;
-                        nq[nu] = v.y;
-                    }
-                    int lokq = 0, nwkq = 0;
-                    int64_t grow = 0;                        // this band's row of the pair's Gamma block
-                    if constexpr (GAM) {
-                        lokq = __ldg(a.win_lo + ikq);
-                        nwkq = __ldg(a.win_n + ikq);
-                        grow = a.gent[kp] + a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
-                    }
-                    const float2 *uq = a.uS + q;                     // element e at uq[e * nk]
-                    // small shapes: G (every column) once per pair, shared by its bands
-                    float2 Gp[kPreG ? X : 1];
-                    if constexpr (kPreG) {
-#pragma unroll
-                        for (int x = 0; x < X; ++x) Gp[x] = Ub[x];
-#pragma unroll
-                        for (int f = 1; f < D; ++f) {
-                            const float c = c3[f - 1];
-#pragma unroll
-                            for (int x2 = 0; x2 < X / 2; ++x2) {
-                                const float4 v = reinterpret_cast<const float4 *>(Ub + f * JQ * X)[x2];
-                                Gp[2 * x2].x = fmaf(c, v.x, Gp[2 * x2].x);
-                                Gp[2 * x2].y = fmaf(c, v.y, Gp[2 * x2].y);
-                                Gp[2 * x2 + 1].x = fmaf(c, v.z, Gp[2 * x2 + 1].x);
-                                Gp[2 * x2 + 1].y = fmaf(c, v.w, Gp[2 * x2 + 1].y);
+                                    for (int mm = 0; mm < W; ++mm)
+                                        mask |= (fabsf(en - __ldg(a.erel + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
+                                }
                             }
+                            have = mask != 0;
+                            m = have ? __ffs(mask) - 1 : 0;
+                            mask &= mask - 1;
+                            unsigned more;
+                            while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
+                                if (have && mask) {
+                                    left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
+                                    mask &= mask - 1;
+                                }
+                                nleft += __popc(more);
+                            }
+                            __syncwarp();
                         }
-                    }
-                    while (mask) {
-                        const int m = __ffs(mask) - 1;
-                        mask &= mask - 1;
-                        const float2 emf = __ldg(a.ef + (int64_t)m * a.nk + ikq);
+                        if (!have) continue;
+                        const float2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;   // form f3 at + f3 JQ X
+                        float c3[NF];
+                        load_coef<NF>(CS3 + q3 * NF, c3);
+                        const float2 *uq = a.qt + (int64_t)(q / kTb) * q_block(NM) + q % kTb;   // element e at + e kTb
+                        const float2 *kt = a.kqt + ((int64_t)(ikq / kTb) * W + m) * kq_block(W);
+                        const int x64 = ikq % kTb;
+                        int lokq = 0, nwkq = 0;
+                        int64_t grow = 0;                        // this band's row of the pair's Gamma block
+                        if constexpr (GAM) {
+                            lokq = __ldg(a.win_lo + ikq);
+                            nwkq = __ldg(a.win_n + ikq);
+                            const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
+                            grow = a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq - lokq;
+                        }
+                        const float2 emf = __ldg(kt + kTb * W + x64);
                         const float em = emf.x, fm = emf.y;
                         float2 Vc[W];                        // column m of V(k+q)
-                        const float2 *vp = a.Vb32 + ((int64_t)m * a.nk + ikq) * W;
                         if constexpr (V2) {
 #pragma unroll
                             for (int i = 0; i < W / 2; ++i) {
-                                const float4 v = __ldg(reinterpret_cast<const float4 *>(vp) + i);
+                                const float4 v = __ldg(reinterpret_cast<const float4 *>(kt) + i * kTb + x64);
                                 Vc[2 * i] = make_float2(v.x, v.y);
                                 Vc[2 * i + 1] = make_float2(v.z, v.w);
                             }
                         } else {
 #pragma unroll
-                            for (int i = 0; i < W; ++i) Vc[i] = __ldg(vp + i);
+                            for (int i = 0; i < W; ++i) Vc[i] = __ldg(kt + i * kTb + x64);
                         }
-                        float2 gv[NM];
+                            float2 gv[NM];
 #pragma unroll
-                        for (int nu = 0; nu < NM; ++nu) gv[nu] = make_float2(0.f, 0.f);
+                            for (int nu = 0; nu < NM; ++nu) gv[nu] = make_float2(0.f, 0.f);
 #pragma unroll kMuUnroll
-                        for (int mu = 0; mu < NM; ++mu) {
-                            float2 G[W];
-                            const float2 *u0 = Ub + mu * W;
-                            if constexpr (kPreG) {
-#pragma unroll
-                                for (int i = 0; i < W; ++i) G[i] = Gp[mu * W + i];
-                            } else if constexpr (V2) {
-#pragma unroll
-                                for (int i = 0; i < W / 2; ++i) {
-                                    const float4 v = reinterpret_cast<const float4 *>(u0)[i];
-                                    G[2 * i] = make_float2(v.x, v.y);
-                                    G[2 * i + 1] = make_float2(v.z, v.w);
-                                }
-#pragma unroll
-                                for (int f = 1; f < D; ++f) {
-                                    const float c = c3[f - 1];
-                                    const float4 *uf = reinterpret_cast<const float4 *>(u0 + f * JQ * X);
+                            for (int mu = 0; mu < NM; ++mu) {
+                                float2 G[W];
+                                const float2 *u0 = Ub + mu * W;
+                                if constexpr (V2) {
 #pragma unroll
                                     for (int i = 0; i < W / 2; ++i) {
-                                        const float4 v = uf[i];
-                                        G[2 * i].x = fmaf(c, v.x, G[2 * i].x);
-                                        G[2 * i].y = fmaf(c, v.y, G[2 * i].y);
-                                        G[2 * i + 1].x = fmaf(c, v.z, G[2 * i + 1].x);
-                                        G[2 * i + 1].y = fmaf(c, v.w, G[2 * i + 1].y);
+                                        const float4 v = reinterpret_cast<const float4 *>(u0)[i];
+                                        G[2 * i] = make_float2(v.x, v.y);
+                                        G[2 * i + 1] = make_float2(v.z, v.w);
+                                    }
+#pragma unroll
+                                    for (int f = 1; f < D; ++f) {
+                                        const float c = c3[f - 1];
+                                        const float4 *uf = reinterpret_cast<const float4 *>(u0 + f * JQ * X);
+#pragma unroll
+                                        for (int i = 0; i < W / 2; ++i) {
+                                            const float4 v = uf[i];
+                                            G[2 * i].x = fmaf(c, v.x, G[2 * i].x);
+                                            G[2 * i].y = fmaf(c, v.y, G[2 * i].y);
+                                            G[2 * i + 1].x = fmaf(c, v.z, G[2 * i + 1].x);
+                                            G[2 * i + 1].y = fmaf(c, v.w, G[2 * i + 1].y);
+                                        }
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < W; ++i) G[i] = u0[i];
+#pragma unroll
+                                    for (int f = 1; f < D; ++f) {
+                                        const float c = c3[f - 1];
+#pragma unroll
+                                        for (int i = 0; i < W; ++i) {
+                                            const float2 v = u0[f * JQ * X + i];
+                                            G[i].x = fmaf(c, v.x, G[i].x);
+                                            G[i].y = fmaf(c, v.y, G[i].y);
+                                        }
                                     }
                                 }
-                            } else {
+                                float2 h = make_float2(0.f, 0.f);
 #pragma unroll
-                                for (int i = 0; i < W; ++i) G[i] = u0[i];
+                                for (int i = 0; i < W; ++i) h = cfmacf(Vc[i], G[i], h);
 #pragma unroll
-                                for (int f = 1; f < D; ++f) {
-                                    const float c = c3[f - 1];
+                                for (int nu = 0; nu < NM; ++nu)
+                                    gv[nu] = cfmaf(h, __ldg(uq + (mu * NM + nu) * kTb), gv[nu]);
+                            }
+                            float gm = 0.f;                      // Gamma capture: sum over modes
 #pragma unroll
-                                    for (int i = 0; i < W; ++i) {
-                                        const float2 v = u0[f * JQ * X + i];
-                                        G[i].x = fmaf(c, v.x, G[i].x);
-                                        G[i].y = fmaf(c, v.y, G[i].y);
-                                    }
+                            for (int nu = 0; nu < NM; ++nu) {
+                                const float2 wnv = __ldg(uq + (NM * NM + nu) * kTb);
+                                const float w = wnv.x, nq = wnv.y;
+                                if (w < 0.f) continue;
+                                const float g2 = gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y;
+                                const float x1 = (en + w) - em;
+                                const float x2 = (en - w) - em;
+                                float tt = 0.f;
+                                if (fabsf(x1) <= ceta) {
+                                    const float y = x1 * ieta;
+                                    tt += (nq + fm) * __expf(-y * y);
                                 }
+                                if (fabsf(x2) <= ceta) {
+                                    const float y = x2 * ieta;
+                                    tt += (1.f + nq - fm) * __expf(-y * y);
+                                }
+                                rate = fmaf(g2, tt, rate);
+                                if constexpr (GAM) gm = fmaf(g2, tt, gm);
                             }
-                            float2 h = make_float2(0.f, 0.f);
-#pragma unroll
-                            for (int i = 0; i < W; ++i) h = cfmacf(Vc[i], G[i], h);
-#pragma unroll
-                            for (int nu = 0; nu < NM; ++nu)
-                                gv[nu] = cfmaf(h, __ldg(uq + (int64_t)(mu * NM + nu) * a.nk), gv[nu]);
-                        }
-                        float gm = 0.f;                      // Gamma capture: sum over modes
-#pragma unroll
-                        for (int nu = 0; nu < NM; ++nu) {
-                            const float w = wq[nu];
-                            if (w < 0.f) continue;
-                            const float g2 = gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y;
-                            const float x1 = (en + w) - em;
-                            const float x2 = (en - w) - em;
-                            float tt = 0.f;
-                            if (fabsf(x1) <= ceta) {
-                                const float y = x1 * ieta;
-                                tt += (nq[nu] + fm) * __expf(-y * y);
+                            if constexpr (GAM) {
+                                if (m >= lokq && m < lokq + nwkq) a.gam[grow + m] = gm;
                             }
-                            if (fabsf(x2) <= ceta) {
-                                const float y = x2 * ieta;
-                                tt += (1.f + nq[nu] - fm) * __expf(-y * y);
-                            }
-                            rate = fmaf(g2, tt, rate);
-                            if constexpr (GAM) gm = fmaf(g2, tt, gm);
-                        }
-                        if constexpr (GAM) {
-                            if (m >= lokq && m < lokq + nwkq) a.gam[grow + m] = gm;
-                        }
                     }
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
-                acc += (double)rate;                         // runs of this warp in a fixed order
-                __syncwarp();                                // Uw is rewritten by the next run
+                if (lane == 0) rs[r] = rate;
+                __syncwarp();                                // Uw is rewritten by the next item
             }
-            __syncthreads();                                 // gl, nglist and Y are rewritten next
+            __syncthreads();                                 // gl, nglist, rs and Y are rewritten next
+            if (wid == 0) {
+                for (int r = lane; r < ng; r += 32) acc += (double)rs[r];
+                __syncwarp();                                // before rs is rewritten by this warp's items
+            }
         }
     }
-    if (lane == 0) wsum[wid] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0;
-        for (int w = 0; w < kSfWarps; ++w) t += wsum[w];
-        a.inv_tau[s] = a.pref * t;
+    // rs of the last group was consumed by warp 0: lanes by a fixed tree
+    if (wid == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) a.inv_tau[s] = a.pref * acc;
     }
 }
 
 template <int W, int NM, int RC, bool GAM>
 void launch_sf_t(epwi_ctx *c, const SfArgs &a, int nitems, size_t sm) {
-    EPWI_REQUIRE(sm <= 200 * 1024, EPWI_EUNSUPPORTED,
-                 "fp32 mode: the plane-block tables of this grid do not fit in shared memory");
     EPWI_CUDA(cudaFuncSetAttribute(k_scatter_sf<W, NM, RC, GAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     EPWI_CUDA(cudaFuncSetAttribute(k_scatter_sf<W, NM, RC, GAM>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     if (nitems > 0) {
@@ -670,6 +789,28 @@ void sf_check(const epwi_ctx *c) {
     EPWI_REQUIRE(c->ng[0] * 2 <= 4096 && c->ng[2] <= 0xffff, EPWI_EUNSUPPORTED, "fp32 mode: grid too large");
 }
 
+// cos and sin of theta R, R = 1 .. rc, for every point of the three axes (x R reduced exactly onto
+// the L roots; x st < L): [N1 + N2 + N3][rc] pairs.
+template <typename V2, typename V>
+__global__ void k_sf_coef(GridInfo g, int rc, const V2 *__restrict__ ph, V *__restrict__ coef) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (g.n1 + g.n2 + g.n3) * rc) return;
+    const int R = e % rc + 1, x = e / rc;
+    const int p = x < g.n1 ? x * g.s1 : x < g.n1 + g.n2 ? (x - g.n1) * g.s2 : (x - g.n1 - g.n2) * g.s3;
+    const V2 v = ph[p * R % g.L];
+    coef[2 * e] = v.x;
+    coef[2 * e + 1] = v.y;
+}
+
+template <typename V2, typename V>
+void build_coef(epwi_ctx *c, const V2 *ph) {
+    const GridInfo g = make_grid_info(c);
+    const int nc = (g.n1 + g.n2 + g.n3) * c->sf_r;
+    c->sf_coef.ensure(sizeof(V2) * nc);
+    k_sf_coef<V2, V><<<(unsigned)((nc + 127) / 128), 128, 0, c->stream>>>(g, c->sf_r, ph, c->sf_coef.as<V>());
+    EPWI_CHECK_LAUNCH();
+}
+
 // g' in the recombined cube forms (once per system).
 template <class C2>
 static void build_gsf(epwi_ctx *c, DevBuf &out) {
@@ -687,6 +828,7 @@ static void build_gsf(epwi_ctx *c, DevBuf &out) {
 }
 
 void sf64_prepare(epwi_ctx *c) {
+    build_coef<double2, double>(c, c->ph64.as<double2>());
     if (c->sf_g64_ready) return;
     build_gsf<double2>(c, c->gsf64);
     c->sf_g64_ready = true;
@@ -701,21 +843,15 @@ void sf_prepare(epwi_ctx *c) {
         build_gsf<float2>(c, c->gsf32);
         c->sf_g_ready = true;
     }
-    const int64_t nv = c->nk * W * W, ne = c->nk * W;
-    c->sf_Vt32.ensure(sizeof(float2) * nv);
-    k_band_major_v<<<(unsigned)((nv + 255) / 256), 256, 0, c->stream>>>(c->nk, W, c->V32.as<float2>(),
-                                                                       c->sf_Vt32.as<float2>());
+    build_coef<float2, float>(c, c->ph32.as<float2>());
+    const int64_t nbk = (c->nk + kTb - 1) / kTb;
+    c->sf_kqt.ensure(sizeof(float2) * nbk * W * kq_block(W));
+    k_kq_table<<<(unsigned)((c->nk * W + 255) / 256), 256, 0, c->stream>>>(
+        c->nk, W, c->V32.as<float2>(), c->tc_erel.as<float>(), c->tc_f32.as<float>(), c->sf_kqt.as<float2>());
     EPWI_CHECK_LAUNCH();
-    c->sf_ef.ensure(sizeof(float2) * ne);
-    k_band_major_ef<<<(unsigned)((ne + 255) / 256), 256, 0, c->stream>>>(c->nk, W, c->tc_erel.as<float>(),
-                                                                        c->tc_f32.as<float>(), c->sf_ef.as<float2>());
-    EPWI_CHECK_LAUNCH();
-    const int64_t nu = c->nk * NM * NM;
-    c->sf_uS.ensure(sizeof(float2) * nu);
-    c->sf_wn.ensure(sizeof(float2) * c->nk * NM);
-    k_soa_q<<<(unsigned)((nu + 255) / 256), 256, 0, c->stream>>>(c->nk, NM, c->u32.as<float2>(), c->tc_hw32.as<float>(),
-                                                                c->tc_n32.as<float>(), c->sf_uS.as<float2>(),
-                                                                c->sf_wn.as<float2>());
+    c->sf_qt.ensure(sizeof(float2) * nbk * q_block(NM));
+    k_q_table<<<(unsigned)((c->nk * (NM * NM + NM) + 255) / 256), 256, 0, c->stream>>>(
+        c->nk, NM, c->u32.as<float2>(), c->tc_hw32.as<float>(), c->tc_n32.as<float>(), c->sf_qt.as<float2>());
     EPWI_CHECK_LAUNCH();
 }
 
@@ -750,24 +886,41 @@ void sf_restage(epwi_ctx *c, const RestageArgs &ra_in) {
     else go(k_restage_f32<0, 1>, 1);
 }
 
+// The grids that the mode takes, a fixed rule: at most 8192 (q1, q2 group) runs per plane block and 8192
+// plane blocks, and 200 KB for one run's U per warp, Y, the three axes' coefficients and the
+// run bounds.  The kernel's own layout (sf_smem_layout) of every such grid is within 227 KB.
+static void sf_check_grid(int D, int X, int q2max, const GridInfo &g) {
+    const size_t per_j = sizeof(float2) * D * X;
+    const int jmax = std::max(1, std::min({q2max, (int)(40 * 1024 / (per_j * D)), (int)(36 * 1024 / (per_j * kSfWarps))}));
+    const int64_t njg = (q2max + jmax - 1) / jmax, jq = (q2max + njg - 1) / njg;
+    const int64_t blocks = ((int64_t)g.n2 * g.n3 + kSieveBlock - 1) / kSieveBlock;
+    EPWI_REQUIRE(g.n1 * njg <= 8192 && blocks <= 8192, EPWI_EUNSUPPORTED, "fp32 mode: too many runs or plane blocks");
+    EPWI_REQUIRE(jq * per_j * (D + kSfWarps) + sizeof(float) * ((int64_t)g.n1 + g.n2 + g.n3) * (D - 1) +
+                         sizeof(int) * (kSieveBlock + 2 * g.n1 * njg + g.n1 + blocks + 5) <= 200 * 1024,
+                 EPWI_EUNSUPPORTED, "fp32 mode: the plane-block tables of this grid do not fit in shared memory");
+}
+
 // Rates of the chunk's states: one CTA per (k-point, band), written straight into inv_tau.
-void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off,
-                const std::vector<int64_t> &h_kp_state_chunk) {
+void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off) {
     const int W = c->nw, NM = c->nm, r = c->sf_r;
     const int D = 2 * r + 1, X = NM * W;
     SfArgs a;
     a.g = sa.g;
     a.nplane = sa.g.n2 * sa.g.n3;
-    const SfPlan plan = sf_plan(D, X, sf_q2max(sa.g.n2, sa.g.n3), sa.g.n1, sa.g.n2, sa.g.n3);
-    EPWI_REQUIRE((int64_t)sa.g.n1 * plan.njg <= 8192 && plan.pbmax <= 8192, EPWI_EUNSUPPORTED,
-                 "fp32 mode: too many runs or plane blocks");
+    const int q2max = sf_q2max(sa.g.n2, sa.g.n3);
+    sf_check_grid(D, X, q2max, sa.g);
+    const SfPlan plan = sf_plan(D, X, W, q2max, sa.g.n1, sa.g.n2, sa.g.n3, sizeof(float));
     a.jq = plan.jq;
     a.njg = plan.njg;
     a.pbmax = plan.pbmax;
-    a.fplane = make_fdiv((uint32_t)a.nplane);
-    a.fjq = make_fdiv((uint32_t)plan.jq);
+    a.fn3 = make_fdiv((uint32_t)sa.g.n3);
+    a.fper = make_fdiv((uint32_t)(X % 2 ? plan.jq * X : plan.jq * (X / 2)));
+    a.coef = c->sf_coef.as<float>();
+    a.mask = sa.mask;
+    a.mask_words = sa.mask_words;
+    a.runs = sa.runs;
+    a.run_stride = run_stride(sa.g);
     a.hwmax32 = c->hwmax32.as<float>();
-    a.ph32 = sa.ph32;
     a.ghat = static_cast<const float2 *>(sa.ghat_raw);
     a.kpts = sa.kpts;
     a.win_lo = sa.win_lo;
@@ -776,34 +929,18 @@ void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *
     a.s_base = sa.s_base;
     a.kp_pairs = kp_pairs_local;
     a.p_off = p_off;
-    a.pairs = sa.pairs;
-    a.Vb32 = c->sf_Vt32.as<float2>();
-    a.ef = c->sf_ef.as<float2>();
-    a.uS = c->sf_uS.as<float2>();
-    a.wn = c->sf_wn.as<float2>();
-    a.nk = c->nk;
-    a.u32 = sa.u32;
+    a.kqt = c->sf_kqt.as<float2>();
+    a.qt = c->sf_qt.as<float2>();
     a.erel = c->tc_erel.as<float>();
-    a.f32 = c->tc_f32.as<float>();
-    a.n32 = c->tc_n32.as<float>();
-    a.hw32 = c->tc_hw32.as<float>();
     a.ceta32 = (float)sa.ceta;
     a.inv_eta32 = (float)(1.0 / sa.eta);
     a.pref = 2.0 * epc::kPi / epc::kHbarEVs / (double)c->nk / (sqrt(epc::kPi) * sa.eta);
     a.inv_tau = c->inv_tau.as<double>();
-    // items: (chunk k-point, band), k-point major
-    std::vector<int2> items;
-    for (int64_t p = 0; p < nkp; ++p)
-        for (int64_t n = 0; n < h_kp_state_chunk[p + 1] - h_kp_state_chunk[p]; ++n) items.push_back(make_int2((int)p, (int)n));
-    c->sf_items.ensure(sizeof(int2) * (items.size() + 1));
-    if (!items.empty())
-        EPWI_CUDA(cudaMemcpyAsync(c->sf_items.p, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice,
-                                  c->stream));
-    a.items = c->sf_items.as<int2>();
+    a.nkp = (int)nkp;
     a.gam = sa.gam32;
     a.goff = sa.goff;
     a.gent = sa.gent;
-    const int ni = (int)items.size();
+    const int ni = (int)sa.nstates_chunk;
     const size_t sm = plan.smem;
     if (W == 4 && NM == 3 && r == 1) launch_sf<4, 3, 1>(c, a, ni, sm);
     else if (W == 4 && NM == 3 && r == 2) launch_sf<4, 3, 2>(c, a, ni, sm);
@@ -814,6 +951,4 @@ void sf_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *
     else if (W == 8 && NM == 6 && r == 2) launch_sf<8, 6, 2>(c, a, ni, sm);
     else if (W == 8 && NM == 6 && r == 3) launch_sf<8, 6, 3>(c, a, ni, sm);
     else sf_check(c);
-    // the host vector of items must outlive the copy
-    EPWI_CUDA(cudaStreamSynchronize(c->stream));
 }

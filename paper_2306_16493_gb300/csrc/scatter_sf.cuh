@@ -39,18 +39,22 @@ __device__ __forceinline__ int64_t lower_bound(int64_t lo, int64_t hi, int64_t k
     return lo;
 }
 
-// Shared-memory layout of k_scatter_sf (complex units first, then floats, then ints).
+// Shared-memory layout of the kernels (in units of their real type, then bytes): Y of one q2 group, two
+// runs' U per warp, the axis-3 coefficients, the sums of a group's items; the items, the flags of the
+// groups, and per warp a list of combinations and one of left-over bands.
 struct SfSmem {
-    size_t y, u, cs, ints, bytes;
+    size_t y, u, cs, rs, flags, bytes;           // complex, complex, real, real, words, bytes
 };
-__host__ __device__ inline SfSmem sf_smem_layout(int D, int X, int jq, int N1, int N2, int N3, int njg, int pbmax,
-                                                   size_t real = sizeof(float)) {
+__host__ __device__ inline SfSmem sf_smem_layout(int D, int X, int W, int jq, int N1, int N3, int njg, int pbmax,
+                                                 size_t real) {
     SfSmem s;
-    s.y = (size_t)D * D * jq * X;                          // complex: Y of one q2 group
-    s.u = (size_t)kSfWarps * D * jq * X;                   // complex: U of one run per warp
-    s.cs = (size_t)(N1 + N2 + N3) * (D - 1);               // real: (cos, sin) per R >= 1
-    s.ints = (size_t)kSieveBlock + 2 * (size_t)N1 * njg + (size_t)N1 + (size_t)pbmax + 1 + 4;
-    s.bytes = 2 * real * (s.y + s.u) + real * s.cs + sizeof(int) * s.ints;
+    s.y = ((size_t)D * D * jq * X + 1) & ~size_t(1);       // an even count: what follows stays 16-byte aligned
+    s.u = (size_t)kSfWarps * 2 * D * jq * X;
+    s.cs = ((size_t)N3 * (D - 1) + 3) & ~size_t(3);
+    s.rs = (size_t)(N1 / 2 + 1);
+    s.flags = ((size_t)pbmax * njg + 31) / 32;
+    s.bytes = 2 * real * (s.y + s.u) + real * (s.cs + s.rs) + sizeof(int) * (s.rs + 2 + s.flags) +
+              kSfWarps * ((size_t)kSieveBlock + 64 * (size_t)W);
     return s;
 }
 
@@ -59,17 +63,18 @@ struct SfPlan {
     size_t smem;
 };
 
-// q2 values per group (jq): Y of one group and one run's U per warp within budgets that keep
-// two or more CTAs per SM.
-inline SfPlan sf_plan(int D, int X, int q2max, int N1, int N2, int N3, size_t real = sizeof(float)) {
-    const size_t ybudget = 10240 * real, ubudget = 9216 * real;
+// q2 values per group (jq): Y of one group and two runs' U per warp within budgets that keep two or
+// more CTAs per SM (FP32: three for 12 columns, 70 KB at jq = 7; FP64: two for 12 columns, 101 KB at
+// jq = 5, and one CTA's FP64 instructions run while the other waits at a barrier).
+inline SfPlan sf_plan(int D, int X, int W, int q2max, int N1, int N2, int N3, size_t real) {
+    const size_t ybudget = 10240 * real, ubudget = (real == 8 ? 10240 : 13824) * real;
     SfPlan p;
     const size_t per_j = 2 * real * D * X;
-    const int jmax = std::max(1, std::min({q2max, (int)(ybudget / (per_j * D)), (int)(ubudget / (per_j * kSfWarps))}));
+    const int jmax = std::max(1, std::min({q2max, (int)(ybudget / (per_j * D)), (int)(ubudget / (per_j * kSfWarps * 2))}));
     p.njg = (q2max + jmax - 1) / jmax;             // groups of equal size
     p.jq = (q2max + p.njg - 1) / p.njg;
     p.pbmax = (N2 * N3 + kSieveBlock - 1) / kSieveBlock;
-    p.smem = sf_smem_layout(D, X, p.jq, N1, N2, N3, p.njg, p.pbmax, real).bytes;
+    p.smem = sf_smem_layout(D, X, W, p.jq, N1, N3, p.njg, p.pbmax, real).bytes;
     return p;
 }
 

@@ -5,11 +5,16 @@
 // k_scatter_fp64 by the order of summation only.
 //
 // The FP64 units bind (2 FMA per SM and clock): per (pair, band) the direct sum takes
-// 4 n_Rp N_m W FMA (6000 for 5^3 and W = 4), this one 2 (D - 1) N_m W for the last axis (96), the
-// rotations of the bands within reach (84 each), about 55 for the pair's share of U, and two
-// exponentials per mode inside the Gaussian's support.  Measured on one GB300, Al-like 20^3 (6.6 M
-// pairs): 75 ms with the direct sum, 10.6 ms here.  Per-pair index arithmetic and gathers run
-// in the shadow of the FP64 pipe, so the kernel keeps the plain layouts of the FP64 tables.
+// 4 n_Rp N_m W FMA (6000 for 5^3 and W = 4), this one 2 (D - 1) N_m W for the last axis (96), 84 for
+// the rotations, a share of about 30 of U (the runs q1 and -q1 from one pass over Y), and up to two
+// exponentials per mode (12 operations each from a 64-entry table).  As in the fp32 kernel the pairs
+// of the two runs form one list, and bands beyond a pair's first are worked off together, so that
+// nearly all lanes of an FP64 instruction carry work.  Index arithmetic, gathers and the FP32
+// pre-test of the bands run in the shadow of the FP64 pipe, so the kernel keeps the plain layouts of
+// the FP64 tables.  Two CTAs per SM (plane-block groups sized for that, sf_plan) keep the pipe busy
+// across the barriers: with one, it was 73 % busy.  Measured on one GB300, Al-like 20^3 (6.6 M pairs):
+// direct sum 75 ms; factorised with a run per warp pass, every band of a pair in its lane and CUDA's exp
+// 10.6 ms; paired runs, band list and table exponential 9.1 ms; two CTAs and items from a counter 7.6 ms.
 #include <algorithm>
 
 #include "epwi_internal.cuh"
@@ -22,19 +27,19 @@ namespace {
 struct Sf64Args {
     GridInfo g;
     int nplane;                     // N2 N3
-    FDiv fplane, fjq;
+    FDiv fn3, fper;                 // fper: division by jq X
     int jq, njg, pbmax;
-    const double2 *ph64;
+    const double *coef;             // [N1 + N2 + N3][D - 1] cos, sin of theta R (k_sf_coef)
     const double2 *ghat;            // [state - s_base][D^3 forms][N_m][W]
     const int *kpts, *win_lo, *win_n;
     const int64_t *kp_state;
     int64_t s_base;
-    const int64_t *kp_pairs;        // chunk-local pair offsets, minus p_off
-    int64_t p_off;
-    const int *pairs;
+    const uint32_t *mask;           // sieve decisions of the chunk's k-points (rows of mask_words)
+    int64_t mask_words;
     const double2 *V, *u;           // [k][i][m], [q][mu][nu]
     const double *eps, *hw, *focc, *nocc;
-    const float *hwmax32;
+    const float *hwmax32, *eps32;
+    float lim32;                    // c eta with the FP32 rounding of the pre-test
     double omega_min, eta, ceta;
     double pref;                    // 2 pi / (hbar N_q sqrt(pi) eta)
     double *inv_tau;
@@ -42,30 +47,57 @@ struct Sf64Args {
     double *gam;                    // Gamma capture or nullptr (see scatter_sf.cu)
     const uint32_t *goff;
     const int64_t *gent;
+    const int64_t *kp_pairs;        // with a capture: chunk-local pair offsets, minus p_off, and the
+    int64_t p_off;                  // run tables (sieve.cuh)
+    const int *runs;
+    int64_t run_stride;
 };
 
-// One CTA per (k-point, band): blockIdx.x runs over the chunk's states; the k-point is found in
-// kp_state.  Layout and runs as in k_scatter_sf.
+// e^x for -690 <= x <= 0 by Tang's table-driven method (ACM TOMS 15, 144 (1989)): x = n ln2 / 64 + r,
+// e^x = 2^(n >> 6) T[n & 63] e^r with T[j] = 2^(j/64) and the Taylor polynomial of degree 5 (|r| <=
+// 0.0055: remainder below 4e-17).
+__device__ __forceinline__ double exp_neg(double x, const double *T) {
+    if (x < -690.0) return exp(x);
+    const double big = 6755399441055744.0;                 // 1.5 2^52: rounds to integer
+    const double t = fma(x, 92.332482616893656768, big);   // 64 / ln 2
+    const int n = __double2loint(t);
+    const double nd = t - big;
+    double r = fma(nd, -0x1.62e42fefap-7, x);              // ln2 / 64: 36 bits, then the rest
+    r = fma(nd, -0x1.cf79abc9e3b3ap-46, r);
+    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(r, p, 1.0 / 6.0);
+    p = fma(r, p, 0.5);
+    p = fma(r, p, 1.0);
+    const double tj = T[n & 63];
+    const double v = fma(tj * r, p, tj);
+    return __hiloint2double(__double2hiint(v) + (n >> 6) * (1 << 20), __double2loint(v));
+}
+
+// One CTA per (k-point, band): blockIdx.x runs over the chunk's states.  Groups, items and lists as
+// in k_scatter_sf.
 template <int W, int NM, int RC, bool GAM>
 __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
     constexpr int D = 2 * RC + 1;
     constexpr int NF = D - 1;
     constexpr int X = NM * W;
     extern __shared__ __align__(16) double2 sm64[];
-    const int N1 = a.g.n1, N2 = a.g.n2, N3 = a.g.n3, L = a.g.L;
+    const int N1 = a.g.n1, N2 = a.g.n2, N3 = a.g.n3;
     const int JQ = a.jq, NJG = a.njg;
-    const SfSmem lay = sf_smem_layout(D, X, JQ, N1, N2, N3, NJG, a.pbmax, sizeof(double));
+    const SfSmem lay = sf_smem_layout(D, X, W, JQ, N1, N3, NJG, a.pbmax, sizeof(double));
     double2 *Y = sm64;                           // [D f1][D f3][JQ][X]
-    double *CS = reinterpret_cast<double *>(Y + lay.y + lay.u);   // [N1 + N2 + N3][NF]
-    int *cq = reinterpret_cast<int *>(CS + lay.cs);
-    int *ss = cq + kSieveBlock;
-    int *se = ss + N1 * NJG;
-    int *gl = se + N1 * NJG;
-    int *pbs = gl + N1;
-    int *nglist = pbs + a.pbmax + 1;
-    __shared__ double wsum[kSfWarps];
+    double *CS3 = reinterpret_cast<double *>(Y + lay.y + lay.u);  // [N3][NF]: axis-3 coefficients
+    const int nh = N1 / 2 + 1;
+    double *rs = CS3 + lay.cs;                   // [nh]: sums of the current group's items
+    int *gl = reinterpret_cast<int *>(rs + lay.rs);     // [nh]: the items, (q1, N1 - q1)
+    int *nglist = gl + nh;                       // [2]: items of the group, next one to take
+    uint32_t *flags = reinterpret_cast<uint32_t *>(nglist + 2);      // bit pb NJG + jg: the group has pairs
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    double2 *Uw = Y + lay.y + (size_t)wid * D * JQ * X;
+    uint8_t *clist = reinterpret_cast<uint8_t *>(flags + lay.flags) + wid * kSieveBlock;
+    uint16_t *left = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(flags + lay.flags) + kSfWarps * kSieveBlock) +
+                     wid * 32 * W;
+    __shared__ double T[64];
+    const int ustride = D * JQ * X;
+    double2 *Uw = Y + lay.y + (size_t)wid * 2 * ustride;
     const int64_t s = a.s_base + blockIdx.x;     // global state
     // last k-point whose first state is <= s (every listed k-point has at least one state)
     const int kp = (int)lower_bound(0, a.nkp, s + 1, [&](int64_t p) { return a.kp_state[p + 1]; });
@@ -73,75 +105,96 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
     const int ik = a.kpts[kp];
     const int lo = a.win_lo[ik];
     const double2 *gs = a.ghat + (size_t)blockIdx.x * D * D * D * X;
-    for (int e = tid; e < (N1 + N2 + N3) * RC; e += kSfThreads) {
-        const int R = e % RC + 1, x = e / RC;
-        int xx, st;
-        if (x < N1) { xx = x; st = a.g.s1; }
-        else if (x < N1 + N2) { xx = x - N1; st = a.g.s2; }
-        else { xx = x - N1 - N2; st = a.g.s3; }
-        const double2 v = a.ph64[(int)(((int64_t)xx * st % L) * R % L)];
-        CS[x * NF + 2 * (R - 1)] = v.x;
-        CS[x * NF + 2 * (R - 1) + 1] = v.y;
-    }
-    const double *CS1 = CS, *CS2 = CS + N1 * NF, *CS3 = CS + (N1 + N2) * NF;
+    if (tid < 64) T[tid] = exp2((double)tid / 64.0);
+    const double *CS1 = a.coef, *CS2 = CS1 + N1 * NF;
+    for (int e = tid; e < N3 * NF; e += kSfThreads) CS3[e] = CS2[N2 * NF + e];
     const int nplane = a.nplane;
     const int pb_n = (nplane + kSieveBlock - 1) / kSieveBlock;
-    const int64_t P0 = a.kp_pairs[kp] - a.p_off, P1 = a.kp_pairs[kp + 1] - a.p_off;
-    const int *pl = a.pairs + P0;
-    const int np = (int)(P1 - P0);
-    for (int pb = tid; pb <= pb_n; pb += kSfThreads)
-        pbs[pb] = (int)lower_bound(0, np, pb, [&](int64_t p) {
-            const int q = pl[p];
-            return (int64_t)((q - fdiv(q, a.fplane) * nplane) / kSieveBlock);
-        });
+    const uint32_t *mrow = a.mask + (int64_t)kp * a.mask_words;   // [pb][q1][8 words]
+    // groups with pairs: every thread takes runs (pb, q1) and marks the groups of their set bits
+    for (int e = tid; e < (int)lay.flags; e += kSfThreads) flags[e] = 0u;
+    __syncthreads();
+    for (int r = tid; r < pb_n * N1; r += kSfThreads) {
+        const uint4 *w4 = reinterpret_cast<const uint4 *>(mrow) + 2 * (int64_t)r;
+        const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
+        const uint32_t w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        const int pb = r / N1;
+        if (NJG == 1) {
+            if (w[0] | w[1] | w[2] | w[3] | w[4] | w[5] | w[6] | w[7]) atomicOr(flags + (pb >> 5), 1u << (pb & 31));
+            continue;
+        }
+        const int q2lo = fdiv(pb * kSieveBlock, a.fn3);
+        int seen = -1;                           // last group marked
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            uint32_t b = w[x];
+            while (b) {
+                const int c = x * 32 + __ffs(b) - 1;
+                const int jg = (fdiv(pb * kSieveBlock + c, a.fn3) - q2lo) / JQ;
+                if (jg != seen) {
+                    const int f = pb * NJG + jg;
+                    atomicOr(flags + (f >> 5), 1u << (f & 31));
+                    seen = jg;
+                }
+                // on to the group's end
+                const int end = (q2lo + (jg + 1) * JQ) * N3 - pb * kSieveBlock - x * 32;
+                b = end < 32 ? b & ~((1u << end) - 1u) : 0u;
+            }
+        }
+    }
     int k1, k2, k3;
     grid_coords(a.g, ik, k1, k2, k3);
     const double en = a.eps[(int64_t)ik * W + lo + n];
+    const float en32 = a.eps32[(int64_t)ik * W + lo + n];
     const double ieta = 1.0 / a.eta;
-    double acc = 0;                              // this lane's pairs
+    double acc = 0;                              // warp 0: sums of the items lane, lane + 32, ...
     __syncthreads();
     for (int pb = 0; pb < pb_n; ++pb) {
-        const int seg0 = pbs[pb], nseg = pbs[pb + 1] - seg0;
-        if (nseg == 0) continue;
-        const int *pp = pl + seg0;
         const int c_lo = pb * kSieveBlock, c_hi = min(nplane, c_lo + kSieveBlock) - 1;
-        const int q2lo = c_lo / N3, nq2 = c_hi / N3 - q2lo + 1;
+        const int q2lo = fdiv(c_lo, a.fn3), nq2 = fdiv(c_hi, a.fn3) - q2lo + 1;
         const int njg = (nq2 + JQ - 1) / JQ;
-        for (int t = tid; t < kSieveBlock; t += kSfThreads) {
-            const int c = c_lo + t, q2 = c / N3;
-            cq[t] = ((q2 - q2lo) << 16) | (c - q2 * N3);
-        }
-        for (int t = tid; t < N1 * NJG; t += kSfThreads) ss[t] = -1;
-        __syncthreads();
-        auto keyof = [&](int t) -> int {
-            const int q = pp[t];
-            const int q1 = fdiv(q, a.fplane);
-            return q1 * NJG + fdiv(cq[q - q1 * nplane - c_lo] >> 16, a.fjq);
-        };
-        for (int t = tid; t < nseg; t += kSfThreads) {
-            const int key = keyof(t);
-            if (t == 0 || keyof(t - 1) != key) ss[key] = t;
-            if (t == nseg - 1 || keyof(t + 1) != key) se[key] = t + 1;
-        }
-        __syncthreads();
+        const uint32_t *mpb = mrow + (int64_t)pb * N1 * 8;
         for (int jg = 0; jg < njg; ++jg) {
+            const int fl = pb * NJG + jg;
+            if (!((flags[fl >> 5] >> (fl & 31)) & 1u)) continue;
             const int j0 = jg * JQ, jn = min(JQ, nq2 - j0);
+            // combinations [r0, r1) of the plane block belong to the group
+            const int r0 = max(0, (q2lo + j0) * N3 - c_lo), r1 = min(kSieveBlock, (q2lo + j0 + jn) * N3 - c_lo);
+            // bits of word x (of 8) inside the group
+            auto in_group = [&](int x) -> uint32_t {
+                const int a0 = min(max(r0 - 32 * x, 0), 32), a1 = min(max(r1 - 32 * x, 0), 32);
+                const uint32_t lo_m = a0 < 32 ? ~0u << a0 : 0u, hi_m = a1 < 32 ? ~(~0u << a1) : ~0u;
+                return lo_m & hi_m;
+            };
+            // the group's items {q1, N1 - q1} with pairs (warp 0): the two-run ones first
             if (wid == 0) {
                 int cnt = 0;
-                for (int q0 = 0; q0 < N1; q0 += 32) {
-                    const int q1 = q0 + lane;
-                    const bool on = q1 < N1 && ss[q1 * NJG + jg] >= 0;
+                const int n2 = (N1 - 1) / 2;                     // items with two runs
+                auto filled = [&](int q1) {
+                    const uint4 *w4 = reinterpret_cast<const uint4 *>(mpb) + 2 * q1;
+                    const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
+                    if (NJG == 1) return (u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w) != 0u;
+                    return ((u.x & in_group(0)) | (u.y & in_group(1)) | (u.z & in_group(2)) | (u.w & in_group(3)) |
+                            (v.x & in_group(4)) | (v.y & in_group(5)) | (v.z & in_group(6)) | (v.w & in_group(7))) != 0u;
+                };
+                for (int h0 = 0; h0 < nh; h0 += 32) {
+                    const int h = h0 + lane;                     // 1 .. n2, then 0, then N1 / 2
+                    const int q1 = h < n2 ? h + 1 : h == n2 ? 0 : h;
+                    const bool on = h < nh && (filled(q1) || (h < n2 && filled(N1 - q1)));
                     const unsigned b = __ballot_sync(0xffffffffu, on);
                     if (on) gl[cnt + __popc(b & ((1u << lane) - 1u))] = q1;
                     cnt += __popc(b);
                 }
-                if (lane == 0) *nglist = cnt;
+                if (lane == 0) {
+                    nglist[0] = cnt;
+                    nglist[1] = 0;
+                }
             }
-            const int per = jn * X;
-            for (int e = tid; e < D * D * per; e += kSfThreads) {
-                const int r13 = e / per, e2 = e - r13 * per;
+            for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
+                const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
                 const int jj = e2 / X, col = e2 - jj * X;
-                const int f3 = r13 % D, f1 = r13 / D;
+                if (jj >= jn) continue;
+                const int f1 = r13 / D, f3 = r13 - f1 * D;
                 const double *c2 = CS2 + (q2lo + j0 + jj) * NF;
                 const double2 *src = gs + ((f1 * D) * D + f3) * X + col;
                 double2 v = __ldg(src);
@@ -151,79 +204,136 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
                     v.x = fma(c2[f2 - 1], w.x, v.x);
                     v.y = fma(c2[f2 - 1], w.y, v.y);
                 }
-                Y[(r13 * JQ + jj) * X + col] = v;
+                Y[e] = v;
             }
             __syncthreads();
-            const int ng = *nglist;
-            for (int r = wid; r < ng; r += kSfWarps) {
+            const int ng = nglist[0], per = jn * X;
+            // items are taken from a counter; each writes its own sum, as in k_scatter_sf
+            while (true) {
+                int r = 0;
+                if (lane == 0) r = atomicAdd(nglist + 1, 1);
+                r = __shfl_sync(0xffffffffu, r, 0);
+                if (r >= ng) break;
                 const int q1 = gl[r];
-                const int t0 = ss[q1 * NJG + jg], t1 = se[q1 * NJG + jg];
+                const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
+                // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
+                const int wx = lane & 7;
+                uint32_t word = 0u;
+                if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
+                int skip = 0;                                    // pairs of the run in earlier groups (capture)
+                if (NJG > 1) {
+                    if constexpr (GAM) skip = __popc(word & (r0 > 32 * wx + 31 ? ~0u : r0 > 32 * wx ? ~(~0u << (r0 - 32 * wx)) : 0u));
+                    word &= in_group(wx);
+                }
+                int npc = __popc(word);
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    npc += __shfl_xor_sync(0xffffffffu, npc, o);
+                    if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
+                }
+                const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
+                int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
+                if constexpr (GAM) {
+                    const int *ru = a.runs + (int64_t)kp * a.run_stride + pb * N1;
+                    t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
+                    t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
+                }
+                // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
+                // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
                 double c1[NF];
 #pragma unroll
-                for (int f = 0; f < NF; ++f) c1[f] = CS1[q1 * NF + f];
+                for (int f = 0; f < NF; ++f) c1[f] = __ldg(CS1 + q1 * NF + f);
                 for (int f3 = 0; f3 < D; ++f3)
                     for (int e = lane; e < per; e += 32) {
                         const double2 *src = Y + (size_t)f3 * JQ * X + e;
-                        double2 v = src[0];
+                        double2 v = src[0], o = make_double2(0, 0);
 #pragma unroll
-                        for (int f1 = 1; f1 < D; ++f1) {
-                            const double2 w = src[f1 * D * JQ * X];
-                            v.x = fma(c1[f1 - 1], w.x, v.x);
-                            v.y = fma(c1[f1 - 1], w.y, v.y);
+                        for (int R = 1; R <= RC; ++R) {
+                            const double2 w = src[(2 * R - 1) * D * JQ * X], z = src[2 * R * D * JQ * X];
+                            v.x = fma(c1[2 * R - 2], w.x, v.x);
+                            v.y = fma(c1[2 * R - 2], w.y, v.y);
+                            o.x = fma(c1[2 * R - 1], z.x, o.x);
+                            o.y = fma(c1[2 * R - 1], z.y, o.y);
                         }
-                        Uw[(size_t)f3 * JQ * X + e] = v;
+                        double2 *dst = Uw + (size_t)f3 * JQ * X + e;
+                        dst[0] = make_double2(v.x + o.x, v.y + o.y);
+                        dst[ustride] = make_double2(v.x - o.x, v.y - o.y);
                     }
-                __syncwarp();
-                int b1 = k1 + q1;
-                if (b1 >= N1) b1 -= N1;
-                const int qbase = q1 * nplane + c_lo;
-                for (int t = t0 + lane; t < t1; t += 32) {
-                    const int q = pp[t];
-                    const int jq = cq[q - qbase];
-                    const int j = jq >> 16, q3 = jq & 0xffff;
-                    int b2 = k2 + q2lo + j, b3 = k3 + q3;
-                    if (b2 >= N2) b2 -= N2;
-                    if (b3 >= N3) b3 -= N3;
-                    const int64_t ikq = ((int64_t)b1 * N2 + b2) * N3 + b3;
-                    // final bands within reach of a mode (a superset; the others add zero)
-                    const double lim = (double)__ldg(a.hwmax32 + q) + a.ceta + 1e-6;
-                    unsigned mask = 0;
-#pragma unroll
-                    for (int m = 0; m < W; ++m) mask |= (fabs(en - __ldg(a.eps + ikq * W + m)) <= lim ? 1u : 0u) << m;
-                    if (!mask) continue;
-                    const double2 *Ub = Uw + (j - j0) * X;
-                    double c3[NF];
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) c3[f] = CS3[q3 * NF + f];
-                    int lokq = 0, nwkq = 0;
-                    int64_t grow = 0;
-                    if constexpr (GAM) {
-                        lokq = __ldg(a.win_lo + ikq);
-                        nwkq = __ldg(a.win_n + ikq);
-                        grow = a.gent[kp] + a.goff[P0 + seg0 + t] + (int64_t)n * nwkq - lokq;
-                    }
-                    constexpr bool kPreG = X <= 12;   // G kept for all bands of the pair
-                    auto column = [&](int x) {
-                        double2 v = Ub[x];
-#pragma unroll
-                        for (int f = 1; f < D; ++f) {
-                            const double2 w = Ub[f * JQ * X + x];
-                            v.x = fma(c3[f - 1], w.x, v.x);
-                            v.y = fma(c3[f - 1], w.y, v.y);
+                double rate = 0;
+                int b1a = k1 + q1, b1b = k1 + q1b;
+                if (b1a >= N1) b1a -= N1;
+                if (b1b >= N1) b1b -= N1;
+                const int parts = na + nb <= kSieveBlock ? 1 : 2;
+                for (int part = 0; part < parts; ++part) {
+                    const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
+                    __syncwarp();                                    // Uw is complete, clist is consumed
+                    {
+                        int at = 0;
+                        for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
+                            const uint32_t w = __shfl_sync(0xffffffffu, word, x);
+                            if (w == 0u) continue;                   // uniform over the warp
+                            if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
+                            at += __popc(w);
                         }
-                        return v;
-                    };
-                    double2 Gp[kPreG ? X : 1];
-                    if constexpr (kPreG) {
-#pragma unroll
-                        for (int x = 0; x < X; ++x) Gp[x] = column(x);
                     }
-                    const double2 *uq = a.u + (int64_t)q * NM * NM;
-                    while (mask) {
-                        const int m = __ffs(mask) - 1;
-                        mask &= mask - 1;
+                    int base = 0, nleft = 0;
+                    while (true) {
+                        __syncwarp();
+                        const bool fresh = base < npr && nleft < 32;
+                        if (!fresh && nleft == 0) break;
+                        int tt, m = 0;
+                        bool have;
+                        if (fresh) {
+                            tt = base + lane;
+                            have = tt < npr;
+                            base += 32;
+                        } else {
+                            const int take = min(nleft, 32);
+                            nleft -= take;
+                            have = lane < take;
+                            const int e = have ? left[nleft + lane] : 0;
+                            __syncwarp();                            // before the entries are rewritten
+                            tt = e >> 3;
+                            m = e & 7;
+                        }
+                        const bool second = tt >= npa;
+                        const int c = have ? clist[tt] : 0;
+                        const int q = (second ? q1b : q1) * nplane + c_lo + c;
+                        const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
+                        int b2 = k2 + q2, b3 = k3 + q3;
+                        if (b2 >= N2) b2 -= N2;
+                        if (b3 >= N3) b3 -= N3;
+                        const int64_t ikq = ((int64_t)(second ? b1b : b1a) * N2 + b2) * N3 + b3;
+                        if (fresh) {
+                            // final bands within reach of a mode (a superset, in FP32; the others add zero)
+                            unsigned mask = 0;
+                            if (have) {
+                                const float lim = __ldg(a.hwmax32 + q) + a.lim32;
+#pragma unroll
+                                for (int mm = 0; mm < W; ++mm)
+                                    mask |= (fabsf(en32 - __ldg(a.eps32 + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
+                            }
+                            have = mask != 0;
+                            m = have ? __ffs(mask) - 1 : 0;
+                            mask &= mask - 1;
+                            unsigned more;
+                            while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
+                                if (have && mask) {
+                                    left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
+                                    mask &= mask - 1;
+                                }
+                                nleft += __popc(more);
+                            }
+                            __syncwarp();
+                        }
+                        if (!have) continue;
+                        const double2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;
+                        double c3[NF];
+#pragma unroll
+                        for (int f = 0; f < NF; ++f) c3[f] = CS3[q3 * NF + f];
                         const double em = __ldg(a.eps + ikq * W + m), fm = __ldg(a.focc + ikq * W + m);
                         const double2 *vp = a.V + ikq * W * W + m;
+                        const double2 *uq = a.u + (int64_t)q * NM * NM;
                         double2 Vc[W], gv[NM];
 #pragma unroll
                         for (int i = 0; i < W; ++i) Vc[i] = __ldg(vp + i * W);
@@ -234,10 +344,14 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
                             double2 h = make_double2(0, 0);
 #pragma unroll
                             for (int i = 0; i < W; ++i) {
-                                double2 Gi;
-                                if constexpr (kPreG) Gi = Gp[mu * W + i];
-                                else Gi = column(mu * W + i);
-                                h = cfmac(Vc[i], Gi, h);
+                                double2 G = Ub[mu * W + i];
+#pragma unroll
+                                for (int f = 1; f < D; ++f) {
+                                    const double2 w = Ub[f * JQ * X + mu * W + i];
+                                    G.x = fma(c3[f - 1], w.x, G.x);
+                                    G.y = fma(c3[f - 1], w.y, G.y);
+                                }
+                                h = cfmac(Vc[i], G, h);
                             }
 #pragma unroll
                             for (int nu = 0; nu < NM; ++nu) gv[nu] = cfma(h, __ldg(uq + mu * NM + nu), gv[nu]);
@@ -248,39 +362,44 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
                             const double w = __ldg(a.hw + (int64_t)q * NM + nu);
                             if (!(w >= a.omega_min)) continue;
                             const double x1 = (en + w) - em, x2 = (en - w) - em;
-                            const bool in1 = fabs(x1) <= a.ceta, in2 = fabs(x2) <= a.ceta;
-                            if (!(in1 || in2)) continue;
                             const double N = __ldg(a.nocc + (int64_t)q * NM + nu);
                             double term = 0;
-                            if (in1) {
+                            if (fabs(x1) <= a.ceta) {
                                 const double y = x1 * ieta;
-                                term += (N + fm) * exp(-y * y);
+                                term = (N + fm) * exp_neg(-y * y, T);
                             }
-                            if (in2) {
+                            if (fabs(x2) <= a.ceta) {
                                 const double y = x2 * ieta;
-                                term += (1.0 + N - fm) * exp(-y * y);
+                                term = fma(1.0 + N - fm, exp_neg(-y * y, T), term);
                             }
                             gm = fma(gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y, term, gm);
                         }
-                        acc += gm;
+                        rate += gm;
                         if constexpr (GAM) {
-                            if (m >= lokq && m < lokq + nwkq) a.gam[grow + m] = gm;
+                            const int lokq = __ldg(a.win_lo + ikq), nwkq = __ldg(a.win_n + ikq);
+                            const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
+                            if (m >= lokq && m < lokq + nwkq)
+                                a.gam[a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq + (m - lokq)] = gm;
                         }
                     }
                 }
-                __syncwarp();                                // Uw is rewritten by the next run
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
+                if (lane == 0) rs[r] = rate;
+                __syncwarp();                                // Uw is rewritten by the next item
             }
-            __syncthreads();                                 // gl, nglist and Y are rewritten next
+            __syncthreads();                                 // gl, nglist, rs and Y are rewritten next
+            if (wid == 0) {
+                for (int r = lane; r < ng; r += 32) acc += rs[r];
+                __syncwarp();                                // before rs is rewritten by this warp's items
+            }
         }
     }
-    // lanes by a fixed tree, warps in order: deterministic, independent of the chunking
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) wsum[wid] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0;
-        for (int w = 0; w < kSfWarps; ++w) t += wsum[w];
-        a.inv_tau[s] = a.pref * t;
+    // lanes by a fixed tree: deterministic, independent of the chunking
+    if (wid == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) a.inv_tau[s] = a.pref * acc;
     }
 }
 
@@ -301,7 +420,7 @@ bool sf64_ok(const epwi_ctx *c) {
     const int W = c->nw, NM = c->nm, r = c->sf_r;
     if (!c->keep_g64 || c->rp_twice || c->h_rp_cube.empty() || !sf_shape_built(W, NM, r)) return false;
     if (c->nk >= (int64_t(1) << 31) || c->ng[0] * 2 > 4096 || c->ng[2] > 0xffff) return false;
-    const SfPlan p = sf_plan(2 * r + 1, NM * W, sf_q2max(c->ng[1], c->ng[2]), c->ng[0], c->ng[1], c->ng[2], sizeof(double));
+    const SfPlan p = sf_plan(2 * r + 1, NM * W, W, sf_q2max(c->ng[1], c->ng[2]), c->ng[0], c->ng[1], c->ng[2], sizeof(double));
     return p.smem <= 200 * 1024 && (int64_t)c->ng[0] * p.njg <= 8192 && p.pbmax <= 8192;
 }
 
@@ -309,16 +428,23 @@ size_t sf64_state_bytes(const epwi_ctx *c) { return 2 * sf_state_bytes(c); }
 
 void sf64_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t *kp_pairs_local, int64_t p_off) {
     const int W = c->nw, NM = c->nm, r = c->sf_r;
-    const SfPlan plan = sf_plan(2 * r + 1, NM * W, sf_q2max(sa.g.n2, sa.g.n3), sa.g.n1, sa.g.n2, sa.g.n3, sizeof(double));
+    const SfPlan plan = sf_plan(2 * r + 1, NM * W, W, sf_q2max(sa.g.n2, sa.g.n3), sa.g.n1, sa.g.n2, sa.g.n3, sizeof(double));
     Sf64Args a;
     a.g = sa.g;
     a.nplane = sa.g.n2 * sa.g.n3;
-    a.fplane = make_fdiv((uint32_t)a.nplane);
-    a.fjq = make_fdiv((uint32_t)plan.jq);
+    a.fn3 = make_fdiv((uint32_t)sa.g.n3);
+    a.fper = make_fdiv((uint32_t)(plan.jq * NM * W));
+    a.mask = sa.mask;
+    a.mask_words = sa.mask_words;
+    a.runs = sa.runs;
+    a.run_stride = run_stride(sa.g);
+    a.eps32 = c->eps32.as<float>();
+    // |e| <= E in FP32: each energy and their difference are off by less than 2^-24 (2 E + |x|)
+    a.lim32 = (float)(sa.ceta + 1e-5 + 4e-7 * (2.0 * c->eabs_max + 1.0));
     a.jq = plan.jq;
     a.njg = plan.njg;
     a.pbmax = plan.pbmax;
-    a.ph64 = sa.ph64;
+    a.coef = c->sf_coef.as<double>();
     a.ghat = sa.ghat64;
     a.kpts = sa.kpts;
     a.win_lo = sa.win_lo;
@@ -327,7 +453,6 @@ void sf64_scatter(epwi_ctx *c, const ScatterArgs &sa, int64_t nkp, const int64_t
     a.s_base = sa.s_base;
     a.kp_pairs = kp_pairs_local;
     a.p_off = p_off;
-    a.pairs = sa.pairs;
     a.V = sa.V64;
     a.u = sa.u64;
     a.eps = sa.eps;

@@ -250,7 +250,7 @@ __global__ void k_seg_ranges(int N1, int64_t nplane, int W, int nseg, const floa
 template <int WT, int NMT, bool FILL, int NS>
 __device__ __forceinline__ int64_t sieve_fast_kp(const SieveArgs &a, int nsel, const double *en, const float *en32,
                                                  int ka1, int ka2, int ka3, uint32_t *words, int64_t *sm,
-                                                 uint32_t *mrow, int64_t obase, int *pairs) {
+                                                 uint32_t *mrow, int64_t obase, int *pairs, int *runs) {
     constexpr int kUnr = WT >= 8 ? 2 : 4;        // candidates per step (registers for their energies)
     constexpr int NSX = NS > 0 ? NS : WT;        // window bands held in registers
     constexpr int V4 = WT / 4;                   // 16-byte loads per k+q point
@@ -269,6 +269,7 @@ __device__ __forceinline__ int64_t sieve_fast_kp(const SieveArgs &a, int nsel, c
     const int rowv = nplane * V4;                // float4 per axis-1 row of the energy table
     const float4 *eps4 = reinterpret_cast<const float4 *>(a.eps32);
     uint32_t *mw = words + wid * N1;             // this warp's words of the plane block, by q1
+    const int64_t obase0 = obase;
     int64_t c = 0;
     for (int pb = 0, pbi = 0; pb < nplane; pb += blockDim.x, ++pbi) {
         const int p = pb + threadIdx.x;
@@ -372,6 +373,7 @@ __device__ __forceinline__ int64_t sieve_fast_kp(const SieveArgs &a, int nsel, c
             int64_t tot;
             int64_t o = obase + block_excl_scan((int64_t)pop, sm, tot);
             for (int w = w0; w < w1; ++w) {
+                if (runs && (w & 7) == 0) runs[pbi * N1 + (w >> 3)] = (int)(o - obase0);
                 uint32_t b = words[(w & 7) * N1 + (w >> 3)];
                 const int q0 = (w >> 3) * nplane + pb + (w & 7) * 32;   // (i1, warp) of the word
                 while (b) {
@@ -381,6 +383,7 @@ __device__ __forceinline__ int64_t sieve_fast_kp(const SieveArgs &a, int nsel, c
                 }
             }
             obase += tot;
+            if (runs && threadIdx.x == 0 && pb + (int)blockDim.x >= nplane) runs[(pbi + 1) * N1] = (int)(obase - obase0);
             __syncthreads();                     // the words are cleared next
         } else {
             for (int i1 = lane; i1 < N1; i1 += 32) {
@@ -402,7 +405,7 @@ __global__ void __launch_bounds__(256, 3) k_sieve_count_fast(SieveArgs a, const 
                                                           uint32_t *__restrict__ mask,
                                                           int64_t words_per_kp, int64_t kp0,
                                                           const int64_t *__restrict__ kp_pairs,
-                                                          int *__restrict__ pairs) {
+                                                          int *__restrict__ pairs, int *__restrict__ runs) {
     __shared__ double en[epc::kMaxW];
     __shared__ float en32[epc::kMaxW];
     __shared__ int64_t sm[33];
@@ -415,11 +418,12 @@ __global__ void __launch_bounds__(256, 3) k_sieve_count_fast(SieveArgs a, const 
     grid_coords(a.g, ik, ka1, ka2, ka3);
     uint32_t *mrow = (mask && !FILL) ? mask + (int64_t)blockIdx.x * words_per_kp + (threadIdx.x >> 5) : nullptr;
     const int64_t obase = FILL ? kp_pairs[kp] - kp_pairs[kp0] : 0;   // first output position (FILL)
+    if (FILL && runs) runs += (int64_t)blockIdx.x * run_stride(a.g);
     int64_t c;
     switch (nsel) {                              // the window's band count (uniform over the block)
-    case 1: c = sieve_fast_kp<WT, NMT, FILL, 1>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs); break;
-    case 2: c = sieve_fast_kp<WT, NMT, FILL, 2>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs); break;
-    default: c = sieve_fast_kp<WT, NMT, FILL, 0>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs); break;
+    case 1: c = sieve_fast_kp<WT, NMT, FILL, 1>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs, runs); break;
+    case 2: c = sieve_fast_kp<WT, NMT, FILL, 2>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs, runs); break;
+    default: c = sieve_fast_kp<WT, NMT, FILL, 0>(a, nsel, en, en32, ka1, ka2, ka3, words, sm, mrow, obase, pairs, runs); break;
     }
     if constexpr (FILL) return;
     int64_t tot;
@@ -588,7 +592,7 @@ __global__ void __launch_bounds__(256) k_sieve_fill_mask(GridInfo g, int64_t kp0
                                                          const uint32_t *__restrict__ mask,
                                                          int64_t words_per_kp, int count_block,
                                                          const int64_t *__restrict__ kp_pairs,
-                                                         int *__restrict__ pairs) {
+                                                         int *__restrict__ pairs, int *__restrict__ runs) {
     __shared__ int64_t sm[33];
     __shared__ int buf[256 * 32];
     const int64_t kp = kp0 + blockIdx.x;
@@ -596,11 +600,15 @@ __global__ void __launch_bounds__(256) k_sieve_fill_mask(GridInfo g, int64_t kp0
     const int64_t nplane = (int64_t)g.n2 * g.n3;
     const int wpb = count_block >> 5;
     int *out = pairs + (kp_pairs[kp] - kp_pairs[kp0]);
+    int done = 0;                                        // pairs before this step's words
+    if (runs) runs += (int64_t)blockIdx.x * run_stride(g);
     for (int64_t w0 = 0; w0 < words_per_kp; w0 += blockDim.x) {
         const int64_t w = w0 + threadIdx.x;
         uint32_t bits = w < words_per_kp ? mrow[w] : 0u;
         int64_t tot;
         int o = (int)block_excl_scan((int64_t)__popc(bits), sm, tot);
+        if (runs && w < words_per_kp && w % wpb == 0) runs[w / wpb] = done + o;
+        done += (int)tot;
         if (bits) {
             const int64_t grp = w / wpb;                 // (plane block, i1) group
             const int64_t pbi = grp / g.n1, i1 = grp % g.n1;
@@ -616,6 +624,7 @@ __global__ void __launch_bounds__(256) k_sieve_fill_mask(GridInfo g, int64_t kp0
         out += tot;
         __syncthreads();                                 // buf is refilled next
     }
+    if (runs && threadIdx.x == 0) runs[words_per_kp / wpb] = done;
 }
 
 // Writes the kept q of k-points kp0 + blockIdx.x in the candidate order of k_sieve_count.
@@ -624,7 +633,7 @@ __global__ void __launch_bounds__(256) k_sieve_fill(SieveArgs a, int64_t kp0,
                                                     const int *__restrict__ lo,
                                                     const int *__restrict__ cnt,
                                                     const int64_t *__restrict__ kp_pairs,
-                                                    int *__restrict__ pairs) {
+                                                    int *__restrict__ pairs, int *__restrict__ runs) {
     __shared__ double en[epc::kMaxW];
     __shared__ float en32[epc::kMaxW];
     __shared__ int64_t sm[33];
@@ -637,6 +646,8 @@ __global__ void __launch_bounds__(256) k_sieve_fill(SieveArgs a, int64_t kp0,
     const int64_t nplane = (int64_t)a.g.n2 * a.g.n3;
     int64_t base = kp_pairs[kp] - kp_pairs[kp0];
     const int64_t end = kp_pairs[kp + 1] - kp_pairs[kp0];
+    const int64_t base0 = base;
+    if (runs) runs += (int64_t)blockIdx.x * run_stride(a.g);
     for (int64_t pb = 0; pb < nplane; pb += blockDim.x) {
         const int64_t p = pb + threadIdx.x;
         const bool inb = p < nplane;
@@ -649,6 +660,11 @@ __global__ void __launch_bounds__(256) k_sieve_fill(SieveArgs a, int64_t kp0,
             int64_t tot;
             const int64_t off = block_excl_scan(v, sm, tot);
             if (v && base + off < end) pairs[base + off] = (int)iq;
+            if (runs && threadIdx.x == 0) {
+                int *r = runs + (pb / blockDim.x) * a.g.n1 + i1;
+                r[0] = (int)(base - base0);
+                r[1] = (int)(base - base0 + tot);        // the last one stays: the total
+            }
             base += tot;
             if (++b1 == a.g.n1) b1 = 0;
         }
@@ -805,6 +821,37 @@ void window_lists(epwi_ctx *c, const int *rep) {
     EPWI_CHECK_LAUNCH();
 }
 
+int64_t sieve_words(const epwi_ctx *c) {
+    const int64_t nplane = (int64_t)c->ng[1] * c->ng[2];
+    return ((nplane + kSieveBlock - 1) / kSieveBlock) * c->ng[0] * (kSieveBlock / 32);
+}
+
+// Counts (and decisions, with a mask) of window k-points kp0 .. kp0 + n - 1, one block per k-point.
+static void count_by_kpoint(epwi_ctx *c, const SieveArgs &a, int64_t kp0, int64_t n, int64_t *counts, uint32_t *mk,
+                            int64_t words) {
+    auto fast = (c->nw == 4 && c->nm == 3) ? k_sieve_count_fast<4, 3, false>
+                : (c->nw == 8 && c->nm == 6) ? k_sieve_count_fast<8, 6, false> : nullptr;
+    if (fast && sieve_fast_ok(c)) {
+        fast<<<(unsigned)n, kSieveBlock, sizeof(uint32_t) * 8 * (size_t)c->ng[0], c->stream>>>(
+            a, c->kpts.as<int>() + kp0, c->win_lo.as<int>(), c->win_n.as<int>(), counts, mk, words, 0, nullptr, nullptr,
+            nullptr);
+    } else {
+        auto kern = (c->nw == 4 && c->nm == 3) ? k_sieve_count<4, 3> : k_sieve_count<0, 0>;
+        kern<<<(unsigned)n, kSieveBlock, 0, c->stream>>>(a, n, c->kpts.as<int>() + kp0, c->win_lo.as<int>(),
+                                                         c->win_n.as<int>(), counts, mk, words);
+    }
+    EPWI_CHECK_LAUNCH();
+}
+
+const uint32_t *sieve_mask_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1) {
+    if (c->mask_words) return c->sieve_mask.as<uint32_t>() + kp0 * c->mask_words;
+    const int64_t words = sieve_words(c), n = kp1 - kp0;
+    c->chunk_mask.ensure(sizeof(uint32_t) * words * n);
+    c->chunk_counts.ensure(sizeof(int64_t) * n);
+    count_by_kpoint(c, make_sieve_args(c), kp0, n, c->chunk_counts.as<int64_t>(), c->chunk_mask.as<uint32_t>(), words);
+    return c->chunk_mask.as<uint32_t>();
+}
+
 void sieve_count(epwi_ctx *c) {
     const int64_t nkp = c->nkp;
     seg_ranges(c);
@@ -812,8 +859,7 @@ void sieve_count(epwi_ctx *c) {
     c->kp_pairs.ensure(sizeof(int64_t) * (nkp + 1));
     SieveArgs a = make_sieve_args(c);
     // decision mask for the fill when it fits in 2 GiB (else the fill re-evaluates)
-    const int64_t nplane = (int64_t)c->ng[1] * c->ng[2];
-    const int64_t words = ((nplane + kSieveBlock - 1) / kSieveBlock) * c->ng[0] * (kSieveBlock / 32);
+    const int64_t words = sieve_words(c);
     // EPWI_SIEVE_MASK_MAX_BYTES (default 2 GiB) caps the mask; 0 forces the re-evaluating fill
     int64_t cap = int64_t(1) << 31;
     if (const char *env = std::getenv("EPWI_SIEVE_MASK_MAX_BYTES")) cap = std::strtoll(env, nullptr, 10);
@@ -821,20 +867,9 @@ void sieve_count(epwi_ctx *c) {
     if (c->mask_words) c->sieve_mask.ensure(sizeof(uint32_t) * words * nkp);
     if (nkp > 0) {
         uint32_t *mk = c->mask_words ? c->sieve_mask.as<uint32_t>() : nullptr;
-        auto fast = (c->nw == 4 && c->nm == 3) ? k_sieve_count_fast<4, 3, false>
-                    : (c->nw == 8 && c->nm == 6) ? k_sieve_count_fast<8, 6, false> : nullptr;
-        if (fast && sieve_fast_ok(c) && sieve_count_cols(c, a, mk)) {
-        } else if (fast && sieve_fast_ok(c)) {
-            fast<<<(unsigned)nkp, kSieveBlock, sizeof(uint32_t) * 8 * (size_t)c->ng[0], c->stream>>>(
-                a, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(), c->counts.as<int64_t>(), mk,
-                c->mask_words, 0, nullptr, nullptr);
-        } else {
-            auto kern = (c->nw == 4 && c->nm == 3) ? k_sieve_count<4, 3> : k_sieve_count<0, 0>;
-            kern<<<(unsigned)nkp, kSieveBlock, 0, c->stream>>>(
-                a, nkp, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(), c->counts.as<int64_t>(), mk,
-                c->mask_words);
-        }
-        EPWI_CHECK_LAUNCH();
+        const bool fast = (c->nw == 4 && c->nm == 3) || (c->nw == 8 && c->nm == 6);
+        if (!(fast && sieve_fast_ok(c) && sieve_count_cols(c, a, mk)))
+            count_by_kpoint(c, a, 0, nkp, c->counts.as<int64_t>(), mk, c->mask_words);
     }
     scan_exclusive_i64(c, c->counts.as<int64_t>(), c->kp_pairs.as<int64_t>(), nkp, nullptr);
     c->h_kp_pairs.resize(nkp + 1);
@@ -847,12 +882,12 @@ void sieve_count(epwi_ctx *c) {
     c->npairs = c->h_kp_pairs[nkp];
 }
 
-void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs) {
+void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs, int *runs) {
     if (kp1 <= kp0) return;
     if (c->mask_words) {
         k_sieve_fill_mask<<<(unsigned)(kp1 - kp0), 256, 0, c->stream>>>(
             make_grid_info(c), kp0, c->sieve_mask.as<uint32_t>(), c->mask_words, kSieveBlock,
-            c->kp_pairs.as<int64_t>(), pairs);
+            c->kp_pairs.as<int64_t>(), pairs, runs);
         EPWI_CHECK_LAUNCH();
         return;
     }
@@ -862,12 +897,12 @@ void sieve_fill_chunk(epwi_ctx *c, int64_t kp0, int64_t kp1, int *pairs) {
     if (fast && sieve_fast_ok(c)) {
         fast<<<(unsigned)(kp1 - kp0), kSieveBlock, sizeof(uint32_t) * 8 * (size_t)c->ng[0], c->stream>>>(
             a, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(), nullptr, nullptr, 0, kp0,
-            c->kp_pairs.as<int64_t>(), pairs);
+            c->kp_pairs.as<int64_t>(), pairs, runs);
         EPWI_CHECK_LAUNCH();
         return;
     }
     k_sieve_fill<<<(unsigned)(kp1 - kp0), 256, 0, c->stream>>>(
         a, kp0, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(),
-        c->kp_pairs.as<int64_t>(), pairs);
+        c->kp_pairs.as<int64_t>(), pairs, runs);
     EPWI_CHECK_LAUNCH();
 }

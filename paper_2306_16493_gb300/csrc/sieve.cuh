@@ -9,6 +9,12 @@
 // then q1, then the combination; the sum-factorised interpolation relies on that order.
 constexpr int kSieveBlock = 256;
 
+// Run table of a k-point's pair list (sieve_fill_chunk): first pair, relative to the k-point's own
+// first, of every run (plane block, q1) in list order, and the number of pairs at the end.
+__host__ __device__ __forceinline__ int64_t run_stride(const GridInfo &g) {
+    return ((int64_t)g.n2 * g.n3 + kSieveBlock - 1) / kSieveBlock * g.n1 + 1;
+}
+
 struct SieveArgs {
     GridInfo g;
     int W, Nm;
