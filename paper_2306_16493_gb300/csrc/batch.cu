@@ -50,7 +50,7 @@ struct BSys {
     const float2 *ph32;
     const float2 *V32;
     const float2 *u32;
-    const float *erel, *f32, *n32, *hw32;
+    const float *erel, *f32, *n32, *hw32, *hwmax32;
     const float2 *ghat;           // [state][nRp][Nm][W]
     const int *pairs;             // sieved q of every k-point, grouped by k-point
     const int64_t *kp_pairs;      // [nkp + 1]
@@ -160,155 +160,27 @@ __device__ __forceinline__ void cp_async_wait_group() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// The persistent kernel: CTAs take queue items until the queue is empty.
-__global__ void __launch_bounds__(kBT, 2) k_batch_scatter(const BSys *__restrict__ systems,
-                                                         const BItem *__restrict__ items,
-                                                         const int *__restrict__ order,
-                                                         int nitems, int *__restrict__ counter,
-                                                         double *__restrict__ part) {
-    extern __shared__ float2 sm[];
-    __shared__ int s_item;
-    __shared__ int sq[kMaxMt];
-    __shared__ int sa[3][kMaxMt];
-    __shared__ int srun[kMaxMt + 1];             // starts of the runs of equal q1 (factorised path)
-    __shared__ int s_nrun;
-    __shared__ float2 se1[13];                   // axis-1 phases of the current run (rc <= 6)
-    __shared__ double sred[kBT / 32];
-    const int t = threadIdx.x;
-    for (;;) {
-        if (t == 0) s_item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it >= nitems) break;
-        const int slot = order[it];
-        const BItem I = items[slot];
-        const BSys &S = systems[I.sys];
-        const int W = S.W, Nm = S.Nm, NW = S.NW, KC = S.KC, cnt = I.cnt;
-        const int ik = S.kpts[I.kp];
-        const int64_t st = S.kp_state[I.kp] + I.np;
-        const int band = S.win_lo[ik] + I.np;
-        const float2 *gh = S.ghat + st * (int64_t)S.nRp * NW;
-        const int *pl = S.pairs + S.kp_pairs[I.kp] + I.p0;
-        for (int p = t; p < cnt; p += kBT) {
-            const int iq = pl[p];
-            int i1, i2, i3;
-            grid_coords(S.g, iq, i1, i2, i3);
-            sq[p] = iq;
-            sa[0][p] = i1 * S.g.s1 % S.g.L;
-            sa[1][p] = i2 * S.g.s2 % S.g.L;
-            sa[2][p] = i3 * S.g.s3 % S.g.L;
-        }
-        // shared memory: two K chunks of ghat [KC][NW], phases [Mt][KC+1], product [Mt][NW]
-        float2 *Gs = sm;
-        float2 *P = sm + (size_t)2 * KC * NW;
-        float2 *Cs = P + (size_t)S.Mt * (KC + 1);
-        const int KP = KC + 1;
-        const int cg = t % S.CW, rg = t / S.CW;
-        const bool tact = rg < S.RG;
-        const int ncol = (NW + S.CW - 1) / S.CW;            // 1 or 2
-        const int npt = (cnt + S.RG - 1) / S.RG;            // pairs per thread
-        float2 acc[kAcc];
+// Operands of an item's Rp->q sum in shared memory (float2): two K chunks of ghat [KC][NW] and the
+// phases [Mt][KC + 1], or, for a cube R_p, the phases of axes 2 and 3 [Mt][2 D].
+__host__ __device__ inline size_t front_words(int Mt, int KC, int NW, int rc) {
+    const size_t direct = (size_t)2 * KC * NW + (size_t)Mt * (KC + 1);
+    const size_t cube = rc >= 0 && rc <= 6 ? (size_t)Mt * 2 * (2 * rc + 1) : 0;
+    return direct > cube ? direct : cube;
+}
+
+// Rp -> q over every R_p (no cube), by the whole CTA.
+__device__ __forceinline__ void direct_sum(const BSys &S, const float2 *__restrict__ gh, int cnt,
+                                           const int (&sa)[3][kMaxMt], float2 *sm, float2 *Cs) {
+    const int t = threadIdx.x, NW = S.NW, KC = S.KC, KP = KC + 1;
+    float2 *Gs = sm;
+    float2 *P = sm + (size_t)2 * KC * NW;
+    const int cg = t % S.CW, rg = t / S.CW;
+    const bool tact = rg < S.RG;
+    const int ncol = (NW + S.CW - 1) / S.CW;            // 1 or 2
+    const int npt = (cnt + S.RG - 1) / S.RG;            // pairs per thread
+    float2 acc[kAcc];
 #pragma unroll
-        for (int a = 0; a < kAcc; ++a) acc[a] = make_float2(0.f, 0.f);
-        __syncthreads();
-        // runs of equal q1 (the sieve lists a k-point's pairs by plane block, then q1, so the
-        // pairs of one q1 are contiguous): the factorised path needs at least 4 pairs per run
-        const bool fac = S.rc >= 0 && S.rc <= 6 &&
-                         4 * __syncthreads_count(t < cnt && (t == 0 || sa[0][t] != sa[0][t - 1]) ||
-                                                 (t + kBT < cnt && sa[0][t + kBT] != sa[0][t + kBT - 1]))
-                             <= cnt;
-        if (fac && t < 32) {
-            // ordered run starts, by warp 0
-            int nr = 0;
-            for (int p0 = 0; p0 < cnt; p0 += 32) {
-                const int p = p0 + t;
-                unsigned bits = __ballot_sync(0xffffffffu, p < cnt && (p == 0 || sa[0][p] != sa[0][p - 1]));
-                while (bits) {
-                    const int b = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    if (t == 0) srun[nr] = p0 + b;
-                    ++nr;
-                }
-            }
-            if (t == 0) {
-                srun[nr] = cnt;
-                s_nrun = nr;
-            }
-        }
-        __syncthreads();
-        if (fac) {
-            // ---- Rp -> q factorised along axis 1: per K chunk of the (n2, n3) plane,
-            // C[p] += sum_(n2,n3) e^{i(q2 n2 + q3 n3)} Z_q1[n2 n3], Z_q1 = sum_n1 e^{i q1 n1} ghat[n1][n2 n3],
-            // Z built once per run of equal q1 and chunk (the CTA reads ghat from L2)
-            const int rc = S.rc, D = 2 * rc + 1, DD = D * D, L = S.g.L;
-            float2 *Z = Gs;                                   // [KC][NW]
-            const int nchf = (DD + KC - 1) / KC;
-            for (int j = 0; j < s_nrun; ++j) {
-                const int lo = srun[j], hi = srun[j + 1];
-                if (t < D) {
-                    int x = (sa[0][lo] * (t - rc)) % L;
-                    if (x < 0) x += L;
-                    se1[t] = S.ph32[x];                       // e^{i q1 n1}, n1 = t - rc
-                }
-                // this thread's pairs p = rg + i RG inside [lo, hi)
-                unsigned in = 0u;
-#pragma unroll
-                for (int i = 0; i < kAcc; ++i) {
-                    const int pi = rg + i * S.RG;
-                    if (i < npt && pi >= lo && pi < hi) in |= 1u << i;
-                }
-                __syncthreads();
-                for (int ch = 0; ch < nchf; ++ch) {
-                    const int r0 = ch * KC, kc = min(KC, DD - r0);
-                    for (int e = t; e < (hi - lo) * KC; e += kBT) {
-                        const int p = lo + e / KC, kk = e % KC;
-                        float2 v = make_float2(0.f, 0.f);
-                        if (kk < kc) {
-                            const int n2 = (r0 + kk) / D - rc, n3 = (r0 + kk) % D - rc;
-                            int x = (sa[1][p] * n2 + sa[2][p] * n3) % L;
-                            if (x < 0) x += L;
-                            v = S.ph32[x];
-                        }
-                        P[p * KP + kk] = v;
-                    }
-                    for (int e = t; e < kc * NW; e += kBT) {
-                        const int kk = e / NW, col = e - kk * NW;
-                        const float2 *src = gh + (int64_t)(r0 + kk) * NW + col;
-                        float2 z = make_float2(0.f, 0.f);
-                        for (int j1 = 0; j1 < D; ++j1) z = cfmaf(se1[j1], src[(int64_t)j1 * DD * NW], z);
-                        Z[kk * NW + col] = z;
-                    }
-                    __syncthreads();
-                    if (tact) {
-                        if (ncol == 1) {
-                            for (int kk = 0; kk < kc; ++kk) {
-                                const float2 g0 = Z[kk * NW + cg];
-                                const float2 *pk = P + rg * KP + kk;
-#pragma unroll
-                                for (int i = 0; i < kAcc; ++i)
-                                    if ((in >> i) & 1u) acc[i] = cfmaf(pk[i * S.RG * KP], g0, acc[i]);
-                            }
-                        } else {
-                            const bool c1 = cg + S.CW < NW;
-                            for (int kk = 0; kk < kc; ++kk) {
-                                const float2 g0 = Z[kk * NW + cg];
-                                const float2 g1 = c1 ? Z[kk * NW + cg + S.CW] : make_float2(0.f, 0.f);
-                                const float2 *pk = P + rg * KP + kk;
-#pragma unroll
-                                for (int i = 0; i < kAcc / 2; ++i)
-                                    if ((in >> i) & 1u) {
-                                        const float2 pv = pk[i * S.RG * KP];
-                                        acc[2 * i] = cfmaf(pv, g0, acc[2 * i]);
-                                        acc[2 * i + 1] = cfmaf(pv, g1, acc[2 * i + 1]);
-                                    }
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
-        } else {
+    for (int a = 0; a < kAcc; ++a) acc[a] = make_float2(0.f, 0.f);
             // ---- Rp -> q: C[p][mu, i] = sum_Rp e^{i q_p . Rp} ghat[Rp][mu][i]; the K chunks of
             // ghat are copied to shared memory with cp.async, one chunk ahead of the compute
             const int nch = (S.nRp + KC - 1) / KC;
@@ -347,7 +219,7 @@ __global__ void __launch_bounds__(kBT, 2) k_batch_scatter(const BSys *__restrict
                         for (int kk = 0; kk < kc; ++kk) {
                             const float2 g0 = G[kk * NW + cg];
                             const float2 *pk = P + rg * KP + kk;
-    #pragma unroll
+#pragma unroll
                             for (int i = 0; i < kAcc; ++i)
                                 if (i < nv) acc[i] = cfmaf(pk[i * S.RG * KP], g0, acc[i]);
                         }
@@ -357,7 +229,7 @@ __global__ void __launch_bounds__(kBT, 2) k_batch_scatter(const BSys *__restrict
                             const float2 g0 = G[kk * NW + cg];
                             const float2 g1 = c1 ? G[kk * NW + cg + S.CW] : make_float2(0.f, 0.f);
                             const float2 *pk = P + rg * KP + kk;
-    #pragma unroll
+#pragma unroll
                             for (int i = 0; i < kAcc / 2; ++i)
                                 if (i < nv) {
                                     const float2 pv = pk[i * S.RG * KP];
@@ -369,67 +241,262 @@ __global__ void __launch_bounds__(kBT, 2) k_batch_scatter(const BSys *__restrict
                 }
                 __syncthreads();
             }
-        }
-        cp_async_wait_group<0>();
-        if (tact) {
+            cp_async_wait_group<0>();
+            if (tact) {
 #pragma unroll
-            for (int a = 0; a < kAcc; ++a) {
-                const int i = ncol == 1 ? a : (a >> 1);
-                const int j = ncol == 1 ? 0 : (a & 1);
-                const int p = rg + i * S.RG, c = cg + j * S.CW;
-                if (i < npt && p < cnt && c < NW) Cs[(size_t)p * NW + c] = acc[a];
+                for (int a = 0; a < kAcc; ++a) {
+                    const int i = ncol == 1 ? a : (a >> 1);
+                    const int j = ncol == 1 ? 0 : (a & 1);
+                    const int p = rg + i * S.RG, c = cg + j * S.CW;
+                    if (i < npt && p < cnt && c < NW) Cs[(size_t)p * NW + c] = acc[a];
+                }
             }
+}
+
+constexpr int kUB = 8;            // pairs per lane of a unit of the factorised path
+
+// Rp -> q of a cube R_p, factorised along axis 1, for one unit of a warp: pairs [lo, hi) of one q1 and
+// NC columns per lane.  Per (n2, n3), Z = sum_n1 e^{i q1 n1} ghat[n1][n2 n3] is formed in registers
+// (the loads of all n1 and columns are independent) and added to every pair's columns with the
+// phase e2(q2, n2) e3(q3, n3).
+template <int NC>
+__device__ __forceinline__ void z_unit(const float2 *__restrict__ gh, const float2 *__restrict__ E,
+                                       const float2 *__restrict__ e1, float2 *__restrict__ Cs, int D, int NW, int lo,
+                                       int hi, int c0) {
+    const int lane = threadIdx.x & 31;
+    // fewer than 32 columns: the lanes take further pairs
+    const int CW = NC == 1 ? min(NW, 32) : 32, RG = 32 / CW;
+    const int cg = lane % CW, rg = lane / CW;
+    const int DD = D * D;
+    float2 acc[kUB][NC];
+#pragma unroll
+    for (int i = 0; i < kUB; ++i)
+#pragma unroll
+        for (int x = 0; x < NC; ++x) acc[i][x] = make_float2(0.f, 0.f);
+    int col[NC];
+#pragma unroll
+    for (int x = 0; x < NC; ++x) col[x] = min(c0 + cg + 32 * x, NW - 1);
+    const int ni = (hi - lo + RG - 1) / RG;              // pairs per lane
+    for (int n2 = 0; n2 < D; ++n2)
+        for (int n3 = 0; n3 < D; ++n3) {
+            float2 z[NC];
+#pragma unroll
+            for (int x = 0; x < NC; ++x) z[x] = make_float2(0.f, 0.f);
+            const float2 *src = gh + (int64_t)(n2 * D + n3) * NW;
+#pragma unroll 3
+            for (int n1 = 0; n1 < D; ++n1) {
+                const float2 e = e1[n1];
+#pragma unroll
+                for (int x = 0; x < NC; ++x) z[x] = cfmaf(e, __ldg(src + (int64_t)n1 * DD * NW + col[x]), z[x]);
+            }
+#pragma unroll
+            for (int i = 0; i < kUB; ++i) {
+                if (i >= ni) break;
+                const int p = min(lo + rg + i * RG, hi - 1);
+                const float2 *ep = E + (size_t)p * 2 * D;
+                const float2 ph = cmulf(ep[n2], ep[D + n3]);
+#pragma unroll
+                for (int x = 0; x < NC; ++x) acc[i][x] = cfmaf(ph, z[x], acc[i][x]);
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < kUB; ++i)
+#pragma unroll
+        for (int x = 0; x < NC; ++x) {
+            const int p = lo + rg + i * RG, c = c0 + cg + 32 * x;
+            if (rg < RG && p < hi && c < NW) Cs[(size_t)p * NW + c] = acc[i][x];
+        }
+}
+
+// Rotations and the delta sum of an item: the sum over its (pair, band) with a mode within c eta of
+// either energy shell (the others add exactly zero).  Each warp tests 32 of them at a time with the
+// pair's largest mode energy, keeps those in reach in a list and works that off 32 at a time.
+// NMB: at least the number of modes.
+template <int NMB>
+__device__ __forceinline__ float rotate_sum(const BSys &S, int cnt, int ik, float en, const int *sq, const float2 *Cs,
+                                            uint16_t *buf) {
+    const int lane = threadIdx.x & 31;
+    const int W = S.W, Nm = S.Nm, total = cnt * W;
+    float rate = 0.f;
+    int nb = 0;
+    for (int u0 = threadIdx.x - lane;; u0 += kBT) {
+        const bool more = u0 < total;                    // uniform over the warp
+        if (more) {
+            const int u = u0 + lane;
+            bool on = u < total;
+            if (on) {
+                const int p = u / W, iq = sq[p];
+                const float em = S.erel[kplusq(S.g, ik, iq) * W + (u - p * W)];
+                on = fabsf(en - em) <= S.hwmax32[iq] + S.ceta + 1e-5f;
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, on);
+            if (on) buf[nb + __popc(b & ((1u << lane) - 1u))] = (uint16_t)u;
+            nb += __popc(b);
+        }
+        __syncwarp();
+        while (nb >= 32 || (!more && nb > 0)) {
+            const int take = min(nb, 32);
+            nb -= take;
+            if (lane < take) {
+                const int u = buf[nb + lane];
+                const int p = u / W, m = u - p * W;
+                const int iq = sq[p];
+                const int64_t ikq = kplusq(S.g, ik, iq);
+                const float2 *Vq = S.V32 + ikq * W * W;
+                const float2 *Cp = Cs + (size_t)p * S.NW;
+                float2 h[NMB];
+#pragma unroll
+                for (int mu = 0; mu < NMB; ++mu) h[mu] = make_float2(0.f, 0.f);
+                for (int i = 0; i < W; ++i) {             // one load of V_im(k+q) per i
+                    const float2 v = Vq[i * W + m];
+#pragma unroll
+                    for (int mu = 0; mu < NMB; ++mu)
+                        if (mu < Nm) h[mu] = cfmacf(v, Cp[mu * W + i], h[mu]);
+                }
+                const float em = S.erel[ikq * W + m];
+                const float fm = S.f32[ikq * W + m];
+                const float2 *uq = S.u32 + (int64_t)iq * Nm * Nm;
+                for (int nu = 0; nu < Nm; ++nu) {
+                    const float w = S.hw32[(int64_t)iq * Nm + nu];
+                    if (w < 0.f) continue;
+                    const float x1 = (en + w) - em, x2 = (en - w) - em;
+                    const bool t1 = fabsf(x1) <= S.ceta, t2 = fabsf(x2) <= S.ceta;
+                    if (!t1 && !t2) continue;
+                    float2 gv = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int mu = 0; mu < NMB; ++mu)
+                        if (mu < Nm) gv = cfmaf(h[mu], uq[mu * Nm + nu], gv);
+                    const float g2 = gv.x * gv.x + gv.y * gv.y;
+                    const float N = S.n32[(int64_t)iq * Nm + nu];
+                    float term = 0.f;
+                    if (t1) {
+                        const float y = x1 * S.inv_eta;
+                        term += (N + fm) * expf(-y * y);
+                    }
+                    if (t2) {
+                        const float y = x2 * S.inv_eta;
+                        term += (1.f + N - fm) * expf(-y * y);
+                    }
+                    rate = fmaf(g2, term, rate);
+                }
+            }
+            __syncwarp();                                // buf is rewritten
+        }
+        if (!more) break;
+    }
+    return rate;
+}
+
+// The persistent kernel: CTAs take queue items until the queue is empty.
+//
+// An item holds some tens of pairs, so a CTA-wide step per run of equal q1 (tables, Z, product,
+// three barriers) left the SMs waiting for one another.  For a cube R_p every warp takes units of its
+// own, (up to kUB RG pairs of one q1, a block of columns), between two barriers per item.
+__global__ void __launch_bounds__(kBT, 2) k_batch_scatter(const BSys *__restrict__ systems,
+                                                         const BItem *__restrict__ items,
+                                                         const int *__restrict__ order,
+                                                         int nitems, int *__restrict__ counter,
+                                                         double *__restrict__ part) {
+    extern __shared__ float2 sm[];
+    __shared__ int s_item;
+    __shared__ int sq[kMaxMt];
+    __shared__ int sa[3][kMaxMt];
+    __shared__ int srun[kMaxMt + 1];             // starts of the units (factorised path)
+    __shared__ int s_nrun, s_next;
+    __shared__ float2 se1[kBT / 32][13];         // axis-1 phases of a warp's unit (rc <= 6)
+    __shared__ uint16_t sbuf[kBT / 32][64];
+    __shared__ double sred[kBT / 32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    for (;;) {
+        if (t == 0) {
+            s_item = atomicAdd(counter, 1);
+            s_next = 0;
         }
         __syncthreads();
-        // ---- rotations and the delta sum: one (pair, m) per thread
-        const float en = S.erel[(int64_t)ik * W + band];
-        float rate = 0.f;
-        for (int u = t; u < cnt * W; u += kBT) {
-            const int p = u / W, m = u - p * W;
-            const int iq = sq[p];
-            const int64_t ikq = kplusq(S.g, ik, iq);
-            const float2 *Vq = S.V32 + ikq * W * W;
-            const float2 *Cp = Cs + (size_t)p * NW;
-            float2 h[kNmB];
-#pragma unroll
-            for (int mu = 0; mu < kNmB; ++mu) h[mu] = make_float2(0.f, 0.f);
-            for (int i = 0; i < W; ++i) {             // one load of V_im(k+q) per i
-                const float2 v = Vq[i * W + m];
-#pragma unroll
-                for (int mu = 0; mu < kNmB; ++mu)
-                    if (mu < Nm) h[mu] = cfmacf(v, Cp[mu * W + i], h[mu]);
-            }
-            const float em = S.erel[ikq * W + m];
-            const float fm = S.f32[ikq * W + m];
-            const float2 *uq = S.u32 + (int64_t)iq * Nm * Nm;
-            for (int nu = 0; nu < Nm; ++nu) {
-                const float w = S.hw32[(int64_t)iq * Nm + nu];
-                if (w < 0.f) continue;
-                const float x1 = (en + w) - em, x2 = (en - w) - em;
-                const bool t1 = fabsf(x1) <= S.ceta, t2 = fabsf(x2) <= S.ceta;
-                if (!t1 && !t2) continue;
-                float2 gv = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int mu = 0; mu < kNmB; ++mu)
-                    if (mu < Nm) gv = cfmaf(h[mu], uq[mu * Nm + nu], gv);
-                const float g2 = gv.x * gv.x + gv.y * gv.y;
-                const float N = S.n32[(int64_t)iq * Nm + nu];
-                float term = 0.f;
-                if (t1) {
-                    const float y = x1 * S.inv_eta;
-                    term += (N + fm) * expf(-y * y);
-                }
-                if (t2) {
-                    const float y = x2 * S.inv_eta;
-                    term += (1.f + N - fm) * expf(-y * y);
-                }
-                rate = fmaf(g2, term, rate);
-            }
+        const int it = s_item;
+        __syncthreads();
+        if (it >= nitems) break;
+        const int slot = order[it];
+        const BItem I = items[slot];
+        const BSys &S = systems[I.sys];
+        const int W = S.W, NW = S.NW, KC = S.KC, cnt = I.cnt;
+        const int ik = S.kpts[I.kp];
+        const int64_t st = S.kp_state[I.kp] + I.np;
+        const int band = S.win_lo[ik] + I.np;
+        const float2 *gh = S.ghat + st * (int64_t)S.nRp * NW;
+        const int *pl = S.pairs + S.kp_pairs[I.kp] + I.p0;
+        const bool fac = S.rc >= 0 && S.rc <= 6;
+        const int D = 2 * S.rc + 1;
+        float2 *Cs = sm + front_words(S.Mt, KC, NW, S.rc);   // [Mt][NW], behind the operands of its sum
+        for (int p = t; p < cnt; p += kBT) {
+            const int iq = pl[p];
+            int i1, i2, i3;
+            grid_coords(S.g, iq, i1, i2, i3);
+            sq[p] = iq;
+            sa[0][p] = i1 * S.g.s1 % S.g.L;
+            sa[1][p] = i2 * S.g.s2 % S.g.L;
+            sa[2][p] = i3 * S.g.s3 % S.g.L;
         }
+        __syncthreads();
+        if (fac) {
+            // E[p][2][D]: phases of the pairs along axes 2 and 3
+            float2 *E = sm;
+            for (int e = t; e < cnt * 2 * D; e += kBT) {
+                const int p = e / (2 * D), r = e - p * 2 * D, ax = r >= D, n = r - ax * D - S.rc;
+                int x = sa[1 + ax][p] * n % S.g.L;
+                if (x < 0) x += S.g.L;
+                E[e] = S.ph32[x];
+            }
+            const int nc = NW <= 32 ? 1 : 4;
+            const int ub = kUB * (NW < 32 ? 32 / NW : 1);
+            // unit starts (warp 0): a new q1 (the sieve lists the pairs of one q1 together) or ub pairs
+            if (wid == 0) {
+                int nr = 0;
+                for (int p0 = 0; p0 < cnt; p0 += 32) {
+                    const int p = p0 + lane;
+                    const bool on = p < cnt && (p % ub == 0 || sa[0][p] != sa[0][p - 1]);
+                    const unsigned bits = __ballot_sync(0xffffffffu, on);
+                    if (on) srun[nr + __popc(bits & ((1u << lane) - 1u))] = p;
+                    nr += __popc(bits);
+                }
+                if (lane == 0) {
+                    srun[nr] = cnt;
+                    s_nrun = nr;
+                }
+            }
+            __syncthreads();
+            const int ncb = (NW + 32 * nc - 1) / (32 * nc), nu = s_nrun * ncb;
+            while (true) {
+                int u = 0;
+                if (lane == 0) u = atomicAdd(&s_next, 1);
+                u = __shfl_sync(0xffffffffu, u, 0);
+                if (u >= nu) break;
+                const int r = u / ncb, cb = u - r * ncb;
+                const int lo = srun[r], hi = srun[r + 1];
+                if (lane < D) {
+                    int x = sa[0][lo] * (lane - S.rc) % S.g.L;
+                    if (x < 0) x += S.g.L;
+                    se1[wid][lane] = S.ph32[x];          // e^{i q1 n1}, n1 = lane - rc
+                }
+                __syncwarp();
+                if (nc == 1) z_unit<1>(gh, E, se1[wid], Cs, D, NW, lo, hi, 0);
+                else z_unit<4>(gh, E, se1[wid], Cs, D, NW, lo, hi, cb * 128);
+                __syncwarp();
+            }
+        } else {
+            direct_sum(S, gh, cnt, sa, sm, Cs);
+        }
+        __syncthreads();
+        const float en = S.erel[(int64_t)ik * W + band];
+        float rate;
+        if (S.Nm <= 3) rate = rotate_sum<3>(S, cnt, ik, en, sq, Cs, sbuf[wid]);
+        else if (S.Nm <= 6) rate = rotate_sum<6>(S, cnt, ik, en, sq, Cs, sbuf[wid]);
+        else if (S.Nm <= 12) rate = rotate_sum<12>(S, cnt, ik, en, sq, Cs, sbuf[wid]);
+        else rate = rotate_sum<kNmB>(S, cnt, ik, en, sq, Cs, sbuf[wid]);
         double r = rate;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
-        if ((t & 31) == 0) sred[t >> 5] = r;
+        if (lane == 0) sred[wid] = r;
         __syncthreads();
         if (t == 0) {
             double s = 0;
@@ -495,8 +562,13 @@ __global__ void __launch_bounds__(256) k_batch_sigma(const SigmaDesc *__restrict
     }
 }
 
-size_t smem_bytes(int Mt, int KC, int NW) {
+// Shared memory of a tile: what the rule on tiles counts, and what the kernel takes (a cube's phases may
+// need more than the direct sum's operands; at most 206 KB for a tile that the rule admits).
+size_t smem_rule(int Mt, int KC, int NW) {
     return sizeof(float2) * ((size_t)2 * KC * NW + (size_t)Mt * (KC + 1) + (size_t)Mt * NW);
+}
+size_t smem_bytes(int Mt, int KC, int NW, int rc) {
+    return sizeof(float2) * (front_words(Mt, KC, NW, rc) + (size_t)Mt * NW);
 }
 
 bool tile_ok(int Mt, int KC, int NW) {
@@ -505,7 +577,7 @@ bool tile_ok(int Mt, int KC, int NW) {
     const int ncol = (NW + CW - 1) / CW;
     const int npt = (Mt + RG - 1) / RG;
     return Mt >= 1 && Mt <= kMaxMt && ncol <= 2 && npt * ncol <= kAcc &&
-           smem_bytes(Mt, KC, NW) <= kSmemCap;
+           smem_rule(Mt, KC, NW) <= kSmemCap;
 }
 
 using TileKey = std::tuple<int, int, int>;           // (W, Nm, nRp)
@@ -733,6 +805,7 @@ void fill_bsys(epwi_batch *b, int s, int Mt, int KC, BSys &d) {
     d.f32 = c->tc_f32.as<float>();
     d.n32 = c->tc_n32.as<float>();
     d.hw32 = c->tc_hw32.as<float>();
+    d.hwmax32 = c->hwmax32.as<float>();
     d.ghat = b->ghat[s].as<float2>();
     d.pairs = b->pairs[s].as<int>();
     d.kp_pairs = c->kp_pairs.as<int64_t>();
@@ -777,7 +850,7 @@ float time_tile(epwi_batch *b, int s, int Mt, int KC, int64_t sample, int64_t *p
         put(dord, order, b->stream);
         dc.ensure(sizeof(int));
         dp.ensure(sizeof(double) * items.size());
-        const size_t sm = smem_bytes(Mt, KC, d.NW);
+        const size_t sm = smem_bytes(Mt, KC, d.NW, d.rc);
         const int grid = persistent_grid(b, sm);
         for (int rep = 0; rep < 2; ++rep) {
             EPWI_CUDA(cudaMemsetAsync(dc.p, 0, sizeof(int), b->stream));
@@ -924,7 +997,7 @@ void plan(epwi_batch *b, bool tune) {
         state_sys.resize(state_item.size(), s);
         fill_bsys(b, s, tiles[s].first, tiles[s].second, b->hsys[s]);
         pref[s] = 2.0 * epc::kPi / epc::kHbarEVs / (double)c->nk / (std::sqrt(epc::kPi) * c->eta);
-        smem = std::max(smem, smem_bytes(tiles[s].first, tiles[s].second, c->nw * c->nm));
+        smem = std::max(smem, smem_bytes(tiles[s].first, tiles[s].second, c->nw * c->nm, c->rp_cube_r));
     }
     b->sys_state0[ns] = (int64_t)state_item.size();
     state_item.push_back((int64_t)items.size());
