@@ -578,7 +578,14 @@ static void launch_vel(epwi_ctx *c, const FacDesc &f, const Lattice &lat, const 
     EPWI_CHECK_LAUNCH();
 }
 
-void launch_eigs(epwi_ctx *c) {
+void reserve_phonon_stages(epwi_ctx *c) {
+    if (c->fac_rp_r < 0) return;
+    const int64_t D = 2 * c->fac_rp_r + 1, E = (int64_t)c->nm * c->nm, n2 = c->ng[1], n3 = c->ng[2];
+    c->fac_Tp.ensure(sizeof(double2) * D * D * n3 * E);
+    c->fac_Up.ensure(sizeof(double2) * D * n2 * n3 * E);
+}
+
+void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t join) {
     const int64_t nk = c->nk;
     const int W = c->nw, Nm = c->nm;
     c->eps.ensure(sizeof(double) * nk * W);
@@ -593,6 +600,14 @@ void launch_eigs(epwi_ctx *c) {
     c->u32.ensure(sizeof(float2) * nk * Nm * Nm);
     c->eig_flag.ensure(sizeof(int) * 2);
     EPWI_CUDA(cudaMemsetAsync(c->eig_flag.p, 0, sizeof(int) * 2, c->stream));
+    const bool own = ph != nullptr;               // phonons on their own stream, with their own stage buffers
+    if (own) {
+        reserve_phonon_stages(c);
+        EPWI_CUDA(cudaEventRecord(fork, c->stream));
+        EPWI_CUDA(cudaStreamWaitEvent(ph, fork, 0));
+    } else {
+        ph = c->stream;
+    }
     GridInfo g = make_grid_info(c);
     const int bs = eig_block(nk);
     const unsigned nb = (unsigned)((nk + bs - 1) / bs);
@@ -604,21 +619,21 @@ void launch_eigs(epwi_ctx *c) {
         nT = (int64_t)(vel ? 2 : 1) * D * D * g.n3 * E;
         nU = (int64_t)(vel ? 3 : 1) * D * plane * E;
     };
-    auto fac_stages = [&](const DevBuf &Xc, int rc, int E, bool vel, DevBuf &Uout) {
+    auto fac_stages = [&](const DevBuf &Xc, int rc, int E, bool vel, DevBuf &T, DevBuf &Uout, cudaStream_t st) {
         const int D = 2 * rc + 1;
         const int64_t t3 = (int64_t)D * D * g.n3 * E, t2 = (int64_t)D * plane * E;
         if (vel) {
-            k_fac_axis3<true><<<(unsigned)((t3 + 255) / 256), 256, 0, c->stream>>>(
-                D, rc, g.n3, g.s3, g.L, E, Xc.as<double2>(), c->ph64.as<double2>(), c->fac_T.as<double2>());
+            k_fac_axis3<true><<<(unsigned)((t3 + 255) / 256), 256, 0, st>>>(
+                D, rc, g.n3, g.s3, g.L, E, Xc.as<double2>(), c->ph64.as<double2>(), T.as<double2>());
             EPWI_CHECK_LAUNCH();
-            k_fac_axis2<true><<<(unsigned)((t2 + 255) / 256), 256, 0, c->stream>>>(
-                D, rc, g.n2, g.n3, g.s2, g.L, E, c->fac_T.as<double2>(), c->ph64.as<double2>(), Uout.as<double2>());
+            k_fac_axis2<true><<<(unsigned)((t2 + 255) / 256), 256, 0, st>>>(
+                D, rc, g.n2, g.n3, g.s2, g.L, E, T.as<double2>(), c->ph64.as<double2>(), Uout.as<double2>());
         } else {
-            k_fac_axis3<false><<<(unsigned)((t3 + 255) / 256), 256, 0, c->stream>>>(
-                D, rc, g.n3, g.s3, g.L, E, Xc.as<double2>(), c->ph64.as<double2>(), c->fac_T.as<double2>());
+            k_fac_axis3<false><<<(unsigned)((t3 + 255) / 256), 256, 0, st>>>(
+                D, rc, g.n3, g.s3, g.L, E, Xc.as<double2>(), c->ph64.as<double2>(), T.as<double2>());
             EPWI_CHECK_LAUNCH();
-            k_fac_axis2<false><<<(unsigned)((t2 + 255) / 256), 256, 0, c->stream>>>(
-                D, rc, g.n2, g.n3, g.s2, g.L, E, c->fac_T.as<double2>(), c->ph64.as<double2>(), Uout.as<double2>());
+            k_fac_axis2<false><<<(unsigned)((t2 + 255) / 256), 256, 0, st>>>(
+                D, rc, g.n2, g.n3, g.s2, g.L, E, T.as<double2>(), c->ph64.as<double2>(), Uout.as<double2>());
         }
         EPWI_CHECK_LAUNCH();
         FacDesc f;
@@ -632,7 +647,7 @@ void launch_eigs(epwi_ctx *c) {
     for (int i = 0; i < 9; ++i) lat.a[i / 3][i % 3] = c->lattice[i];
     const bool fac_el = c->fac_re_r >= 0, fac_ph = c->fac_rp_r >= 0;
     {
-        // both builds share the stage buffers: size them once, before any launch
+        // on one stream both builds share the stage buffers: size them once, before any launch
         int64_t nT = 1, nU = 1, t, u;
         if (fac_el) {
             fac_sizes(c->fac_re_r, W * W, true, t, u);
@@ -641,8 +656,10 @@ void launch_eigs(epwi_ctx *c) {
         }
         if (fac_ph) {
             fac_sizes(c->fac_rp_r, Nm * Nm, false, t, u);
-            nT = std::max(nT, t);
-            nU = std::max(nU, u);
+            if (!own) {
+                nT = std::max(nT, t);
+                nU = std::max(nU, u);
+            }
         }
         if (fac_el || fac_ph) {
             c->fac_T.ensure(sizeof(double2) * nT);
@@ -658,7 +675,7 @@ void launch_eigs(epwi_ctx *c) {
         c->fac_Uel.ensure(sizeof(double2) * u);
     }
     FacDesc fe{}, fp{};
-    if (fac_el) fe = fac_stages(c->fac_Hc, c->fac_re_r, W * W, true, defer ? c->fac_Uel : c->fac_U);
+    if (fac_el) fe = fac_stages(c->fac_Hc, c->fac_re_r, W * W, true, c->fac_T, defer ? c->fac_Uel : c->fac_U, c->stream);
     c->vel_state = defer ? 0 : 2;
 #define EL_ARGS                                                                              \
     g, nk, W, c->nRe, c->Re.as<int>(), c->Rcart.as<double>(), c->Hw.as<double2>(),            \
@@ -698,24 +715,29 @@ void launch_eigs(epwi_ctx *c) {
         c->ph64.as<double2>(), c->opt.omega_min_eV, c->hw.as<double>(), c->hwmax32.as<float>(), \
         c->hw32.as<float>(),                                                                   \
         c->u.as<double2>(), c->u32.as<float2>(), c->eig_flag.as<int>() + 1
-    // the electron kernel above has read fac_U; the phonon stages reuse the buffers (same stream)
-    if (fac_ph) fp = fac_stages(c->fac_Pc, c->fac_rp_r, Nm * Nm, false, c->fac_U);
+    // on one stream the electron kernel above has read fac_U: the phonon stages reuse the buffers
+    if (fac_ph)
+        fp = fac_stages(c->fac_Pc, c->fac_rp_r, Nm * Nm, false, own ? c->fac_Tp : c->fac_T, own ? c->fac_Up : c->fac_U, ph);
     if (Nm == 3) {
-        k_eig_ph<3, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
+        k_eig_ph<3, true><<<nb, bs, 0, ph>>>(PH_ARGS, fp);
     } else if (Nm == 6) {
-        k_eig_ph<6, true><<<nb, bs, 0, c->stream>>>(PH_ARGS, fp);
+        k_eig_ph<6, true><<<nb, bs, 0, ph>>>(PH_ARGS, fp);
     } else {
         const size_t sm = warp_scratch_bytes(Nm);
         if (fac_ph) {
             set_smem_once(k_eig_ph_warp<true>, sm);
-            k_eig_ph_warp<true><<<nbw, 32 * kWarpsPerBlock, sm, c->stream>>>(PH_ARGS, fp);
+            k_eig_ph_warp<true><<<nbw, 32 * kWarpsPerBlock, sm, ph>>>(PH_ARGS, fp);
         } else {
             set_smem_once(k_eig_ph_warp<false>, sm);
-            k_eig_ph_warp<false><<<nbw, 32 * kWarpsPerBlock, sm, c->stream>>>(PH_ARGS, fp);
+            k_eig_ph_warp<false><<<nbw, 32 * kWarpsPerBlock, sm, ph>>>(PH_ARGS, fp);
         }
     }
 #undef PH_ARGS
     EPWI_CHECK_LAUNCH();
+    if (own) {
+        EPWI_CUDA(cudaEventRecord(join, ph));
+        EPWI_CUDA(cudaStreamWaitEvent(c->stream, join, 0));
+    }
 }
 
 void ensure_velocities(epwi_ctx *c, bool all) {

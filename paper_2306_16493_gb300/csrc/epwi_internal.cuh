@@ -180,6 +180,7 @@ struct epwi_ctx {
     int fac_re_r = -1, fac_rp_r = -1;
     DevBuf fac_Hc, fac_Pc;         // double2 [Dc^3][W W], [Dc^3][Nm Nm]
     DevBuf fac_T, fac_U;           // stage outputs (see eigs.cu)
+    DevBuf fac_Tp, fac_Up;         // the phonons' own, where they run on their own stream
     // factorised Re->k sum (kstage.cuh)
     bool re_cube_ok = false;       // re_cube is valid (R_e within |n| <= 6, no vector twice)
     DevBuf re_cube;                // int [Dc^3]: R_e index of each bounding-cube point, -1 if absent
@@ -240,7 +241,7 @@ struct epwi_ctx {
                          &tc_n32, &tc_hw32, &tc_err, &tc_meta, &is_pairs, &is_w,
                          &is_kp_pairs, &sieve_mask, &tc_arows, &ib_pairs, &ib_goff, &ib_gam,
                          &ib_pt, &ib_F0, &ib_F, &ib_Fn, &ib_red, &ib_F32, &ib_Fn32, &ib_col, &ib_ent, &sym_rep, &seg_ranges,
-                         &gsf32, &sf_kqt, &sf_qt, &sf_coef, &chunk_mask, &chunk_counts, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel,
+                         &gsf32, &sf_kqt, &sf_qt, &sf_coef, &chunk_mask, &chunk_counts, &gcube32, &fac_Hc, &fac_Pc, &fac_T, &fac_U, &fac_Uel, &fac_Tp, &fac_Up,
                          &re_cube, &ks_T, &col_buf, &gsf64};
         for (DevBuf *b : all) b->release();
         for (DevBuf &b : is_ws) b.release();
@@ -328,7 +329,10 @@ __host__ __device__ __forceinline__ int phase_index(int a1, int a2, int a3, int 
 // ----------------------------------------------------------------------------- launches
 GridInfo make_grid_info(const epwi_ctx *c);
 void launch_phase_tables(epwi_ctx *c);
-void launch_eigs(epwi_ctx *c);
+// ph, with the events fork and join: the phonon solves on that stream, beside the electrons', with
+// stage buffers of their own (reserve_phonon_stages allocates them).
+void reserve_phonon_stages(epwi_ctx *c);
+void launch_eigs(epwi_ctx *c, cudaStream_t ph = nullptr, cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
 // Band velocities of the window's k-points (all = false; needs win_n) or of every grid point,
 // where the eigensolve deferred them; a no-op otherwise.  Every builder of a rates window calls
 // it (all = false) after build_window.
