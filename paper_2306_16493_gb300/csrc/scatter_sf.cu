@@ -33,7 +33,9 @@
 // lists (4 bytes per pair written and read twice) and no search for the runs in them.  Measured on
 // one GB300, Al-like 48^3 (1.26 G pairs), list fill and this kernel together: 57.1 ms with a run per
 // warp pass, 50.7 ms with both runs from one pass and the runs' bounds from a table, 49.3 ms from the
-// mask; 20 x 27 x 45 (61 M pairs) 4.6, 3.4 and 3.3 ms.
+// mask, 47.9 ms with packed multiply-adds (__ffma2_rn: two FP32 FMAs per issue slot) and a group's
+// items listed while the group before is worked off; 20 x 27 x 45 (61 M pairs) 4.6, 3.4, 3.3 and 3.0 ms;
+// Si-like 100^3 14.6 -> 13.4 ms by the last.
 #include <algorithm>
 
 #include "epwi_internal.cuh"
@@ -302,6 +304,14 @@ __device__ __forceinline__ void load_coef_g(const float *__restrict__ p, float (
     }
 }
 
+// v += c w, two packed multiply-adds (one issue slot for two FP32 FMAs)
+__device__ __forceinline__ void ffma4(float c, const float4 &w, float4 &v) {
+    const float2 cc = make_float2(c, c);
+    const float2 lo = __ffma2_rn(cc, make_float2(w.x, w.y), make_float2(v.x, v.y));
+    const float2 hi = __ffma2_rn(cc, make_float2(w.z, w.w), make_float2(v.z, v.w));
+    v = make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
 template <int W, int NM, int RC, bool GAM>
 __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfArgs a) {
     constexpr int D = 2 * RC + 1;
@@ -317,9 +327,9 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
     float *CS3 = reinterpret_cast<float *>(Y + lay.y + lay.u);  // [N3][NF]: axis-3 coefficients
     const int nh = N1 / 2 + 1;
     float *rs = CS3 + lay.cs;                           // [nh]: sums of the current group's items
-    int *gl = reinterpret_cast<int *>(rs + lay.rs);     // [nh]: the items, (q1, N1 - q1)
-    int *nglist = gl + nh;                              // [2]: items of the group, next one to take
-    uint32_t *flags = reinterpret_cast<uint32_t *>(nglist + 2);      // bit pb NJG + jg: the group has pairs
+    // two lists, of the current group and the next: [nh] items (q1, N1 - q1), their number, next one to take
+    int *lists = reinterpret_cast<int *>(rs + lay.rs);
+    uint32_t *flags = reinterpret_cast<uint32_t *>(lists + 2 * (nh + 2));   // bit pb NJG + jg: the group has pairs
     uint8_t *clist = reinterpret_cast<uint8_t *>(flags + lay.flags) + (threadIdx.x >> 5) * kSieveBlock;
     uint16_t *left = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(flags + lay.flags) + kSfWarps * kSieveBlock) +
                      (threadIdx.x >> 5) * 32 * W;       // see below
@@ -336,417 +346,347 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
     const float *CS1 = a.coef, *CS2 = CS1 + N1 * NF;
     for (int e = tid; e < N3 * NF; e += kSfThreads) CS3[e] = CS2[N2 * NF + e];
     const int nplane = a.nplane;
-    const int pb_n = (nplane + kSieveBlock - 1) / kSieveBlock;
     const uint32_t *mrow = a.mask + (int64_t)kp * a.mask_words;   // [pb][q1][8 words]
-    // groups with pairs: every thread takes runs (pb, q1) and marks the groups of their set bits
-    for (int e = tid; e < (int)lay.flags; e += kSfThreads) flags[e] = 0u;
-    __syncthreads();
-    for (int r = tid; r < pb_n * N1; r += kSfThreads) {
-        const uint4 *w4 = reinterpret_cast<const uint4 *>(mrow) + 2 * (int64_t)r;
-        const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
-        const uint32_t w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-        const int pb = r / N1;
-        if (NJG == 1) {
-            if (w[0] | w[1] | w[2] | w[3] | w[4] | w[5] | w[6] | w[7]) atomicOr(flags + (pb >> 5), 1u << (pb & 31));
-            continue;
-        }
-        const int q2lo = fdiv(pb * kSieveBlock, a.fn3);
-        int seen = -1;                           // last group marked
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            uint32_t b = w[x];
-            while (b) {
-                const int c = x * 32 + __ffs(b) - 1;
-                const int jg = (fdiv(pb * kSieveBlock + c, a.fn3) - q2lo) / JQ;
-                if (jg != seen) {
-                    const int f = pb * NJG + jg;
-                    atomicOr(flags + (f >> 5), 1u << (f & 31));
-                    seen = jg;
-                }
-                // on to the group's end
-                const int end = (q2lo + (jg + 1) * JQ) * N3 - pb * kSieveBlock - x * 32;
-                b = end < 32 ? b & ~((1u << end) - 1u) : 0u;
-            }
-        }
-    }
+    const SfGroups groups{mrow, flags, a.fn3, N1, N3, nplane, JQ, NJG};
+    mark_groups(groups, (int)lay.flags);
     int k1, k2, k3;
     grid_coords(a.g, ik, k1, k2, k3);
     const float en = a.erel[(int64_t)ik * W + lo + n];
     const float ceta = a.ceta32, ieta = a.inv_eta32;
     double acc = 0;                              // warp 0: sums of the items lane, lane + 32, ...
-    __syncthreads();
-    for (int pb = 0; pb < pb_n; ++pb) {
-        const int c_lo = pb * kSieveBlock, c_hi = min(nplane, c_lo + kSieveBlock) - 1;
-        const int q2lo = fdiv(c_lo, a.fn3), nq2 = fdiv(c_hi, a.fn3) - q2lo + 1;
-        const int njg = (nq2 + JQ - 1) / JQ;
-        const uint32_t *mpb = mrow + (int64_t)pb * N1 * 8;
-        for (int jg = 0; jg < njg; ++jg) {
-            const int fl = pb * NJG + jg;
-            if (!((flags[fl >> 5] >> (fl & 31)) & 1u)) continue;
-            const int j0 = jg * JQ, jn = min(JQ, nq2 - j0);
-            // combinations [r0, r1) of the plane block belong to the group
-            const int r0 = max(0, (q2lo + j0) * N3 - c_lo), r1 = min(kSieveBlock, (q2lo + j0 + jn) * N3 - c_lo);
-            // bits of word x (of 8) inside the group
-            auto in_group = [&](int x) -> uint32_t {
-                const int a0 = min(max(r0 - 32 * x, 0), 32), a1 = min(max(r1 - 32 * x, 0), 32);
-                const uint32_t lo_m = a0 < 32 ? ~0u << a0 : 0u, hi_m = a1 < 32 ? ~(~0u << a1) : ~0u;
-                return lo_m & hi_m;
-            };
-            // the group's items {q1, N1 - q1} with pairs (warp 0): the two-run ones first
-            if (wid == 0) {
-                int cnt = 0;
-                const int n2 = (N1 - 1) / 2;                     // items with two runs
-                auto filled = [&](int q1) {
-                    const uint4 *w4 = reinterpret_cast<const uint4 *>(mpb) + 2 * q1;
-                    const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
-                    if (NJG == 1) return (u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w) != 0u;
-                    return ((u.x & in_group(0)) | (u.y & in_group(1)) | (u.z & in_group(2)) | (u.w & in_group(3)) |
-                            (v.x & in_group(4)) | (v.y & in_group(5)) | (v.z & in_group(6)) | (v.w & in_group(7))) != 0u;
-                };
-                for (int h0 = 0; h0 < nh; h0 += 32) {
-                    const int h = h0 + lane;                     // 1 .. n2, then 0, then N1 / 2
-                    const int q1 = h < n2 ? h + 1 : h == n2 ? 0 : h;
-                    const bool on = h < nh && (filled(q1) || (h < n2 && filled(N1 - q1)));
-                    const unsigned b = __ballot_sync(0xffffffffu, on);
-                    if (on) gl[cnt + __popc(b & ((1u << lane) - 1u))] = q1;
-                    cnt += __popc(b);
+    __syncthreads();                             // flags and CS3 are complete
+    int f = groups.next(-1), buf = 0;
+    if (wid == 0 && f >= 0) list_items(groups.group(f), N1, lists);
+    for (; f >= 0; buf ^= 1) {
+        const SfGroup grp = groups.group(f);
+        const int c_lo = grp.c_lo, q2lo = grp.q2lo, j0 = grp.j0, jn = grp.jn;
+        int *gl = lists + buf * (nh + 2);
+        const int fnext = groups.next(f);
+        // Y of this group's q2 values (all threads), read from ghat' (L1 / L2): two columns per
+        // thread and step; the index is taken apart by a launch constant and compile-time ones
+        if constexpr (X % 2 == 0) {
+            const int per4 = JQ * (X / 2);
+            for (int e = tid; e < D * D * per4; e += kSfThreads) {
+                const int r13 = fdiv(e, a.fper), e2 = e - r13 * per4;
+                const int jj = e2 / (X / 2), col2 = e2 - jj * (X / 2);
+                if (jj >= jn) continue;
+                const int f1 = r13 / D, f3 = r13 - f1 * D;
+                float c2[NF];
+                load_coef_g<NF>(CS2 + (q2lo + j0 + jj) * NF, c2);
+                const float4 *src = reinterpret_cast<const float4 *>(gs + ((f1 * D) * D + f3) * X) + col2;
+                float4 v = __ldg(src);                   // form f2 = 0
+#pragma unroll
+                for (int f2 = 1; f2 < D; ++f2) {
+                    ffma4(c2[f2 - 1], __ldg(src + f2 * D * X / 2), v);
                 }
-                if (lane == 0) {
-                    nglist[0] = cnt;
-                    nglist[1] = 0;
-                }
+                reinterpret_cast<float4 *>(Y)[e] = v;    // [r13][jj][col], rows of JQ X
             }
-            // Y of this group's q2 values (all threads), read from ghat' (L1 / L2): two columns per
-            // thread and step; the index is taken apart by a launch constant and compile-time ones
-            if constexpr (X % 2 == 0) {
-                const int per4 = JQ * (X / 2);
-                for (int e = tid; e < D * D * per4; e += kSfThreads) {
-                    const int r13 = fdiv(e, a.fper), e2 = e - r13 * per4;
-                    const int jj = e2 / (X / 2), col2 = e2 - jj * (X / 2);
-                    if (jj >= jn) continue;
-                    const int f1 = r13 / D, f3 = r13 - f1 * D;
-                    float c2[NF];
-                    load_coef_g<NF>(CS2 + (q2lo + j0 + jj) * NF, c2);
-                    const float4 *src = reinterpret_cast<const float4 *>(gs + ((f1 * D) * D + f3) * X) + col2;
-                    float4 v = __ldg(src);                   // form f2 = 0
+        } else {
+            for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
+                const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
+                const int jj = e2 / X, col = e2 - jj * X;
+                if (jj >= jn) continue;
+                const int f1 = r13 / D, f3 = r13 - f1 * D;
+                const float *c2 = CS2 + (q2lo + j0 + jj) * NF;
+                const float2 *src = gs + ((f1 * D) * D + f3) * X + col;
+                float2 v = __ldg(src);
 #pragma unroll
-                    for (int f2 = 1; f2 < D; ++f2) {
-                        const float c = c2[f2 - 1];
-                        const float4 w = __ldg(src + f2 * D * X / 2);
-                        v.x = fmaf(c, w.x, v.x);
-                        v.y = fmaf(c, w.y, v.y);
-                        v.z = fmaf(c, w.z, v.z);
-                        v.w = fmaf(c, w.w, v.w);
-                    }
-                    reinterpret_cast<float4 *>(Y)[e] = v;    // [r13][jj][col], rows of JQ X
+                for (int f2 = 1; f2 < D; ++f2) {
+                    const float c = c2[f2 - 1];
+                    const float2 w = __ldg(src + f2 * D * X);
+                    v.x = fmaf(c, w.x, v.x);
+                    v.y = fmaf(c, w.y, v.y);
                 }
-            } else {
-                for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
-                    const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
-                    const int jj = e2 / X, col = e2 - jj * X;
-                    if (jj >= jn) continue;
-                    const int f1 = r13 / D, f3 = r13 - f1 * D;
-                    const float *c2 = CS2 + (q2lo + j0 + jj) * NF;
-                    const float2 *src = gs + ((f1 * D) * D + f3) * X + col;
-                    float2 v = __ldg(src);
-#pragma unroll
-                    for (int f2 = 1; f2 < D; ++f2) {
-                        const float c = c2[f2 - 1];
-                        const float2 w = __ldg(src + f2 * D * X);
-                        v.x = fmaf(c, w.x, v.x);
-                        v.y = fmaf(c, w.y, v.y);
-                    }
-                    Y[e] = v;
-                }
-            }
-            __syncthreads();
-            const int ng = nglist[0];
-            // items are taken from a counter; each writes its own sum, so the result does not
-            // depend on which warp takes it
-            while (true) {
-                int r = 0;
-                if (lane == 0) r = atomicAdd(nglist + 1, 1);
-                r = __shfl_sync(0xffffffffu, r, 0);
-                if (r >= ng) break;
-                const int q1 = gl[r];
-                const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
-                // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
-                const int wx = lane & 7;
-                uint32_t word = 0u;
-                if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
-                int skip = 0;                                    // pairs of the run in earlier groups (capture)
-                if (NJG > 1) {
-                    if constexpr (GAM) skip = __popc(word & (r0 > 32 * wx + 31 ? ~0u : r0 > 32 * wx ? ~(~0u << (r0 - 32 * wx)) : 0u));
-                    word &= in_group(wx);
-                }
-                int npc = __popc(word);
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
-                    npc += __shfl_xor_sync(0xffffffffu, npc, o);
-                    if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
-                }
-                const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
-                int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
-                if constexpr (GAM) {
-                    const int *ru = a.runs + (int64_t)kp * a.run_stride + pb * N1;
-                    t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
-                    t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
-                }
-                // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
-                // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
-                {
-                    float c1[NF];
-                    load_coef_g<NF>(CS1 + q1 * NF, c1);
-                    if constexpr (X % 2 == 0) {
-                        // (f3, e2) over D rows of per4 float4, walked as one list by the lanes
-                        const int per4 = jn * X / 2;
-                        int f3 = 0, e2 = lane;
-                        while (true) {
-                            while (e2 >= per4 && f3 < D) {
-                                e2 -= per4;
-                                ++f3;
-                            }
-                            if (f3 >= D) break;
-                            const float4 *src = reinterpret_cast<const float4 *>(Y + (size_t)f3 * JQ * X) + e2;
-                            float4 v = src[0], o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                            for (int R = 1; R <= RC; ++R) {
-                                const float cc = c1[2 * R - 2], cs = c1[2 * R - 1];
-                                const float4 w = src[(2 * R - 1) * D * JQ * X / 2], z = src[2 * R * D * JQ * X / 2];
-                                v.x = fmaf(cc, w.x, v.x);
-                                v.y = fmaf(cc, w.y, v.y);
-                                v.z = fmaf(cc, w.z, v.z);
-                                v.w = fmaf(cc, w.w, v.w);
-                                o.x = fmaf(cs, z.x, o.x);
-                                o.y = fmaf(cs, z.y, o.y);
-                                o.z = fmaf(cs, z.z, o.z);
-                                o.w = fmaf(cs, z.w, o.w);
-                            }
-                            float4 *dst = reinterpret_cast<float4 *>(Uw + (size_t)f3 * JQ * X) + e2;
-                            dst[0] = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
-                            dst[ustride / 2] = make_float4(v.x - o.x, v.y - o.y, v.z - o.z, v.w - o.w);
-                            e2 += 32;
-                        }
-                    } else {
-                        const int per = jn * X;
-#pragma unroll
-                        for (int f3 = 0; f3 < D; ++f3) {
-                            const float2 *src = Y + (size_t)f3 * JQ * X;
-                            float2 *dst = Uw + (size_t)f3 * JQ * X;
-                            for (int e = lane; e < per; e += 32) {
-                                float2 v = src[e], o = make_float2(0.f, 0.f);
-#pragma unroll
-                                for (int R = 1; R <= RC; ++R) {
-                                    const float2 w = src[e + (2 * R - 1) * D * JQ * X], z = src[e + 2 * R * D * JQ * X];
-                                    v.x = fmaf(c1[2 * R - 2], w.x, v.x);
-                                    v.y = fmaf(c1[2 * R - 2], w.y, v.y);
-                                    o.x = fmaf(c1[2 * R - 1], z.x, o.x);
-                                    o.y = fmaf(c1[2 * R - 1], z.y, o.y);
-                                }
-                                dst[e] = make_float2(v.x + o.x, v.y + o.y);
-                                dst[e + ustride] = make_float2(v.x - o.x, v.y - o.y);
-                            }
-                        }
-                    }
-                }
-                float rate = 0.f;
-                int b1a = k1 + q1, b1b = k1 + q1b;
-                if (b1a >= N1) b1a -= N1;
-                if (b1b >= N1) b1b -= N1;
-                // The pairs of both runs as one list of combinations (one run at a time where both hold
-                // more than a plane block's worth), 32 at a time, each lane with the first final band
-                // within reach of its pair.  The few further bands are kept in a list of the
-                // warp, (pair, band), and worked off 32 at a time as well: one lane with two bands
-                // would otherwise hold up the other 31 for a second pass over the band.
-                const int parts = na + nb <= kSieveBlock ? 1 : 2;
-                for (int part = 0; part < parts; ++part) {
-                    const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
-                    __syncwarp();                                    // Uw is complete, clist is consumed
-                    {
-                        int at = 0;
-                        for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
-                            const uint32_t w = __shfl_sync(0xffffffffu, word, x);
-                            if (w == 0u) continue;                   // uniform over the warp
-                            if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
-                            at += __popc(w);
-                        }
-                    }
-                    int base = 0, nleft = 0;
-                    while (true) {
-                        __syncwarp();
-                        const bool fresh = base < npr && nleft < 32;
-                        if (!fresh && nleft == 0) break;
-                        int tt, m = 0;
-                        bool have;
-                        if (fresh) {
-                            tt = base + lane;
-                            have = tt < npr;
-                            base += 32;
-                        } else {
-                            const int take = min(nleft, 32);
-                            nleft -= take;
-                            have = lane < take;
-                            const int e = have ? left[nleft + lane] : 0;
-                            __syncwarp();                            // before the entries are rewritten
-                            tt = e >> 3;
-                            m = e & 7;
-                        }
-                        const bool second = tt >= npa;
-                        const int c = have ? clist[tt] : 0;
-                        const int q = (second ? q1b : q1) * nplane + c_lo + c;
-                        const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
-                        int b2 = k2 + q2, b3 = k3 + q3;
-                        if (b2 >= N2) b2 -= N2;
-                        if (b3 >= N3) b3 -= N3;
-                        const int ikq = ((second ? b1b : b1a) * N2 + b2) * N3 + b3;   // nk W^2 < 2^31 (checked on the host)
-                        if (fresh) {
-                            // final bands within the largest kept mode energy + c eta of e_nk (a superset
-                            // of the bands with a mode inside c eta of either shell; the others add zero)
-                            unsigned mask = 0;
-                            if (have) {
-                                const float lim = __ldg(a.hwmax32 + q) + ceta + 1e-5f;
-                                if constexpr (W % 4 == 0) {
-#pragma unroll
-                                    for (int m4 = 0; m4 < W / 4; ++m4) {
-                                        const float4 e4 = __ldg(reinterpret_cast<const float4 *>(a.erel + ikq * W) + m4);
-                                        mask |= (fabsf(en - e4.x) <= lim ? 1u : 0u) << (4 * m4);
-                                        mask |= (fabsf(en - e4.y) <= lim ? 2u : 0u) << (4 * m4);
-                                        mask |= (fabsf(en - e4.z) <= lim ? 4u : 0u) << (4 * m4);
-                                        mask |= (fabsf(en - e4.w) <= lim ? 8u : 0u) << (4 * m4);
-                                    }
-                                } else {
-#pragma unroll
-                                    for (int mm = 0; mm < W; ++mm)
-                                        mask |= (fabsf(en - __ldg(a.erel + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
-                                }
-                            }
-                            have = mask != 0;
-                            m = have ? __ffs(mask) - 1 : 0;
-                            mask &= mask - 1;
-                            unsigned more;
-                            while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
-                                if (have && mask) {
-                                    left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
-                                    mask &= mask - 1;
-                                }
-                                nleft += __popc(more);
-                            }
-                            __syncwarp();
-                        }
-                        if (!have) continue;
-                        const float2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;   // form f3 at + f3 JQ X
-                        float c3[NF];
-                        load_coef<NF>(CS3 + q3 * NF, c3);
-                        const float2 *uq = a.qt + (int64_t)(q / kTb) * q_block(NM) + q % kTb;   // element e at + e kTb
-                        const float2 *kt = a.kqt + ((int64_t)(ikq / kTb) * W + m) * kq_block(W);
-                        const int x64 = ikq % kTb;
-                        int lokq = 0, nwkq = 0;
-                        int64_t grow = 0;                        // this band's row of the pair's Gamma block
-                        if constexpr (GAM) {
-                            lokq = __ldg(a.win_lo + ikq);
-                            nwkq = __ldg(a.win_n + ikq);
-                            const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
-                            grow = a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq - lokq;
-                        }
-                        const float2 emf = __ldg(kt + kTb * W + x64);
-                        const float em = emf.x, fm = emf.y;
-                        float2 Vc[W];                        // column m of V(k+q)
-                        if constexpr (V2) {
-#pragma unroll
-                            for (int i = 0; i < W / 2; ++i) {
-                                const float4 v = __ldg(reinterpret_cast<const float4 *>(kt) + i * kTb + x64);
-                                Vc[2 * i] = make_float2(v.x, v.y);
-                                Vc[2 * i + 1] = make_float2(v.z, v.w);
-                            }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < W; ++i) Vc[i] = __ldg(kt + i * kTb + x64);
-                        }
-                            float2 gv[NM];
-#pragma unroll
-                            for (int nu = 0; nu < NM; ++nu) gv[nu] = make_float2(0.f, 0.f);
-#pragma unroll kMuUnroll
-                            for (int mu = 0; mu < NM; ++mu) {
-                                float2 G[W];
-                                const float2 *u0 = Ub + mu * W;
-                                if constexpr (V2) {
-#pragma unroll
-                                    for (int i = 0; i < W / 2; ++i) {
-                                        const float4 v = reinterpret_cast<const float4 *>(u0)[i];
-                                        G[2 * i] = make_float2(v.x, v.y);
-                                        G[2 * i + 1] = make_float2(v.z, v.w);
-                                    }
-#pragma unroll
-                                    for (int f = 1; f < D; ++f) {
-                                        const float c = c3[f - 1];
-                                        const float4 *uf = reinterpret_cast<const float4 *>(u0 + f * JQ * X);
-#pragma unroll
-                                        for (int i = 0; i < W / 2; ++i) {
-                                            const float4 v = uf[i];
-                                            G[2 * i].x = fmaf(c, v.x, G[2 * i].x);
-                                            G[2 * i].y = fmaf(c, v.y, G[2 * i].y);
-                                            G[2 * i + 1].x = fmaf(c, v.z, G[2 * i + 1].x);
-                                            G[2 * i + 1].y = fmaf(c, v.w, G[2 * i + 1].y);
-                                        }
-                                    }
-                                } else {
-#pragma unroll
-                                    for (int i = 0; i < W; ++i) G[i] = u0[i];
-#pragma unroll
-                                    for (int f = 1; f < D; ++f) {
-                                        const float c = c3[f - 1];
-#pragma unroll
-                                        for (int i = 0; i < W; ++i) {
-                                            const float2 v = u0[f * JQ * X + i];
-                                            G[i].x = fmaf(c, v.x, G[i].x);
-                                            G[i].y = fmaf(c, v.y, G[i].y);
-                                        }
-                                    }
-                                }
-                                float2 h = make_float2(0.f, 0.f);
-#pragma unroll
-                                for (int i = 0; i < W; ++i) h = cfmacf(Vc[i], G[i], h);
-#pragma unroll
-                                for (int nu = 0; nu < NM; ++nu)
-                                    gv[nu] = cfmaf(h, __ldg(uq + (mu * NM + nu) * kTb), gv[nu]);
-                            }
-                            float gm = 0.f;                      // Gamma capture: sum over modes
-#pragma unroll
-                            for (int nu = 0; nu < NM; ++nu) {
-                                const float2 wnv = __ldg(uq + (NM * NM + nu) * kTb);
-                                const float w = wnv.x, nq = wnv.y;
-                                if (w < 0.f) continue;
-                                const float g2 = gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y;
-                                const float x1 = (en + w) - em;
-                                const float x2 = (en - w) - em;
-                                float tt = 0.f;
-                                if (fabsf(x1) <= ceta) {
-                                    const float y = x1 * ieta;
-                                    tt += (nq + fm) * __expf(-y * y);
-                                }
-                                if (fabsf(x2) <= ceta) {
-                                    const float y = x2 * ieta;
-                                    tt += (1.f + nq - fm) * __expf(-y * y);
-                                }
-                                rate = fmaf(g2, tt, rate);
-                                if constexpr (GAM) gm = fmaf(g2, tt, gm);
-                            }
-                            if constexpr (GAM) {
-                                if (m >= lokq && m < lokq + nwkq) a.gam[grow + m] = gm;
-                            }
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
-                if (lane == 0) rs[r] = rate;
-                __syncwarp();                                // Uw is rewritten by the next item
-            }
-            __syncthreads();                                 // gl, nglist, rs and Y are rewritten next
-            if (wid == 0) {
-                for (int r = lane; r < ng; r += 32) acc += (double)rs[r];
-                __syncwarp();                                // before rs is rewritten by this warp's items
+                Y[e] = v;
             }
         }
+        __syncthreads();
+        const int ng = gl[nh];
+        // items are taken from a counter; each writes its own sum, so the result does not
+        // depend on which warp takes it
+        int r = 0;
+        while (true) {
+            if (lane == 0) r = atomicAdd(gl + nh + 1, 1);
+            r = __shfl_sync(0xffffffffu, r, 0);
+            if (r >= ng) break;
+            const int q1 = gl[r];
+            const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
+            // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
+            const int wx = lane & 7;
+            uint32_t word = 0u;
+            if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(grp.mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
+            int skip = 0;                                    // pairs of the run in earlier groups (capture)
+            if (NJG > 1) {
+                if constexpr (GAM) skip = __popc(word & (grp.r0 > 32 * wx + 31 ? ~0u : grp.r0 > 32 * wx ? ~(~0u << (grp.r0 - 32 * wx)) : 0u));
+                word &= grp.bits(wx);
+            }
+            int npc = __popc(word);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                npc += __shfl_xor_sync(0xffffffffu, npc, o);
+                if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
+            }
+            const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
+            int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
+            if constexpr (GAM) {
+                const int *ru = a.runs + (int64_t)kp * a.run_stride + c_lo / kSieveBlock * N1;
+                t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
+                t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
+            }
+            // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
+            // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
+            {
+                float c1[NF];
+                load_coef_g<NF>(CS1 + q1 * NF, c1);
+                if constexpr (X % 2 == 0) {
+                    // (f3, e2) over D rows of per4 float4, walked as one list by the lanes
+                    const int per4 = jn * X / 2;
+                    int f3 = 0, e2 = lane;
+                    while (true) {
+                        while (e2 >= per4 && f3 < D) {
+                            e2 -= per4;
+                            ++f3;
+                        }
+                        if (f3 >= D) break;
+                        const float4 *src = reinterpret_cast<const float4 *>(Y + (size_t)f3 * JQ * X) + e2;
+                        float4 v = src[0], o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int R = 1; R <= RC; ++R) {
+                            const float4 w = src[(2 * R - 1) * D * JQ * X / 2], z = src[2 * R * D * JQ * X / 2];
+                            ffma4(c1[2 * R - 2], w, v);
+                            ffma4(c1[2 * R - 1], z, o);
+                        }
+                        float4 *dst = reinterpret_cast<float4 *>(Uw + (size_t)f3 * JQ * X) + e2;
+                        dst[0] = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+                        dst[ustride / 2] = make_float4(v.x - o.x, v.y - o.y, v.z - o.z, v.w - o.w);
+                        e2 += 32;
+                    }
+                } else {
+                    const int per = jn * X;
+#pragma unroll
+                    for (int f3 = 0; f3 < D; ++f3) {
+                        const float2 *src = Y + (size_t)f3 * JQ * X;
+                        float2 *dst = Uw + (size_t)f3 * JQ * X;
+                        for (int e = lane; e < per; e += 32) {
+                            float2 v = src[e], o = make_float2(0.f, 0.f);
+#pragma unroll
+                            for (int R = 1; R <= RC; ++R) {
+                                const float2 w = src[e + (2 * R - 1) * D * JQ * X], z = src[e + 2 * R * D * JQ * X];
+                                v.x = fmaf(c1[2 * R - 2], w.x, v.x);
+                                v.y = fmaf(c1[2 * R - 2], w.y, v.y);
+                                o.x = fmaf(c1[2 * R - 1], z.x, o.x);
+                                o.y = fmaf(c1[2 * R - 1], z.y, o.y);
+                            }
+                            dst[e] = make_float2(v.x + o.x, v.y + o.y);
+                            dst[e + ustride] = make_float2(v.x - o.x, v.y - o.y);
+                        }
+                    }
+                }
+            }
+            float rate = 0.f;
+            int b1a = k1 + q1, b1b = k1 + q1b;
+            if (b1a >= N1) b1a -= N1;
+            if (b1b >= N1) b1b -= N1;
+            // The pairs of both runs as one list of combinations (one run at a time where both hold
+            // more than a plane block's worth), 32 at a time, each lane with the first final band
+            // within reach of its pair.  The few further bands are kept in a list of the
+            // warp, (pair, band), and worked off 32 at a time as well: one lane with two bands
+            // would otherwise hold up the other 31 for a second pass over the band.
+            const int parts = na + nb <= kSieveBlock ? 1 : 2;
+            for (int part = 0; part < parts; ++part) {
+                const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
+                __syncwarp();                                    // Uw is complete, clist is consumed
+                {
+                    int at = 0;
+                    for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
+                        const uint32_t w = __shfl_sync(0xffffffffu, word, x);
+                        if (w == 0u) continue;                   // uniform over the warp
+                        if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
+                        at += __popc(w);
+                    }
+                }
+                int base = 0, nleft = 0;
+                while (true) {
+                    __syncwarp();
+                    const bool fresh = base < npr && nleft < 32;
+                    if (!fresh && nleft == 0) break;
+                    int tt, m = 0;
+                    bool have;
+                    if (fresh) {
+                        tt = base + lane;
+                        have = tt < npr;
+                        base += 32;
+                    } else {
+                        const int take = min(nleft, 32);
+                        nleft -= take;
+                        have = lane < take;
+                        const int e = have ? left[nleft + lane] : 0;
+                        __syncwarp();                            // before the entries are rewritten
+                        tt = e >> 3;
+                        m = e & 7;
+                    }
+                    const bool second = tt >= npa;
+                    const int c = have ? clist[tt] : 0;
+                    const int q = (second ? q1b : q1) * nplane + c_lo + c;
+                    const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
+                    int b2 = k2 + q2, b3 = k3 + q3;
+                    if (b2 >= N2) b2 -= N2;
+                    if (b3 >= N3) b3 -= N3;
+                    const int ikq = ((second ? b1b : b1a) * N2 + b2) * N3 + b3;   // nk W^2 < 2^31 (checked on the host)
+                    if (fresh) {
+                        // final bands within the largest kept mode energy + c eta of e_nk (a superset
+                        // of the bands with a mode inside c eta of either shell; the others add zero)
+                        unsigned mask = 0;
+                        if (have) {
+                            const float lim = __ldg(a.hwmax32 + q) + ceta + 1e-5f;
+                            if constexpr (W % 4 == 0) {
+#pragma unroll
+                                for (int m4 = 0; m4 < W / 4; ++m4) {
+                                    const float4 e4 = __ldg(reinterpret_cast<const float4 *>(a.erel + ikq * W) + m4);
+                                    mask |= (fabsf(en - e4.x) <= lim ? 1u : 0u) << (4 * m4);
+                                    mask |= (fabsf(en - e4.y) <= lim ? 2u : 0u) << (4 * m4);
+                                    mask |= (fabsf(en - e4.z) <= lim ? 4u : 0u) << (4 * m4);
+                                    mask |= (fabsf(en - e4.w) <= lim ? 8u : 0u) << (4 * m4);
+                                }
+                            } else {
+#pragma unroll
+                                for (int mm = 0; mm < W; ++mm)
+                                    mask |= (fabsf(en - __ldg(a.erel + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
+                            }
+                        }
+                        have = mask != 0;
+                        m = have ? __ffs(mask) - 1 : 0;
+                        mask &= mask - 1;
+                        unsigned more;
+                        while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
+                            if (have && mask) {
+                                left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
+                                mask &= mask - 1;
+                            }
+                            nleft += __popc(more);
+                        }
+                        __syncwarp();
+                    }
+                    if (!have) continue;
+                    const float2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;   // form f3 at + f3 JQ X
+                    float c3[NF];
+                    load_coef<NF>(CS3 + q3 * NF, c3);
+                    const float2 *uq = a.qt + (int64_t)(q / kTb) * q_block(NM) + q % kTb;   // element e at + e kTb
+                    const float2 *kt = a.kqt + ((int64_t)(ikq / kTb) * W + m) * kq_block(W);
+                    const int x64 = ikq % kTb;
+                    int lokq = 0, nwkq = 0;
+                    int64_t grow = 0;                        // this band's row of the pair's Gamma block
+                    if constexpr (GAM) {
+                        lokq = __ldg(a.win_lo + ikq);
+                        nwkq = __ldg(a.win_n + ikq);
+                        const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
+                        grow = a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq - lokq;
+                    }
+                    const float2 emf = __ldg(kt + kTb * W + x64);
+                    const float em = emf.x, fm = emf.y;
+                    float2 Vc[W];                        // column m of V(k+q)
+                    if constexpr (V2) {
+#pragma unroll
+                        for (int i = 0; i < W / 2; ++i) {
+                            const float4 v = __ldg(reinterpret_cast<const float4 *>(kt) + i * kTb + x64);
+                            Vc[2 * i] = make_float2(v.x, v.y);
+                            Vc[2 * i + 1] = make_float2(v.z, v.w);
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < W; ++i) Vc[i] = __ldg(kt + i * kTb + x64);
+                    }
+                        float2 gr[NM], gi[NM];
+#pragma unroll
+                        for (int nu = 0; nu < NM; ++nu) gr[nu] = gi[nu] = make_float2(0.f, 0.f);
+#pragma unroll kMuUnroll
+                        for (int mu = 0; mu < NM; ++mu) {
+                            float2 G[W];
+                            const float2 *u0 = Ub + mu * W;
+                            if constexpr (V2) {
+#pragma unroll
+                                for (int i = 0; i < W / 2; ++i) {
+                                    const float4 v = reinterpret_cast<const float4 *>(u0)[i];
+                                    G[2 * i] = make_float2(v.x, v.y);
+                                    G[2 * i + 1] = make_float2(v.z, v.w);
+                                }
+#pragma unroll
+                                for (int f = 1; f < D; ++f) {
+                                    const float2 c = make_float2(c3[f - 1], c3[f - 1]);
+                                    const float4 *uf = reinterpret_cast<const float4 *>(u0 + f * JQ * X);
+#pragma unroll
+                                    for (int i = 0; i < W / 2; ++i) {
+                                        const float4 v = uf[i];
+                                        G[2 * i] = __ffma2_rn(c, make_float2(v.x, v.y), G[2 * i]);
+                                        G[2 * i + 1] = __ffma2_rn(c, make_float2(v.z, v.w), G[2 * i + 1]);
+                                    }
+                                }
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < W; ++i) G[i] = u0[i];
+#pragma unroll
+                                for (int f = 1; f < D; ++f) {
+                                    const float2 c = make_float2(c3[f - 1], c3[f - 1]);
+#pragma unroll
+                                    for (int i = 0; i < W; ++i) G[i] = __ffma2_rn(c, u0[f * JQ * X + i], G[i]);
+                                }
+                            }
+                            // h = sum_i conj(V_i) G_i and g_nu += h u as real and imaginary factor
+                            // times (x, y), put together at the end
+                            float2 hr = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
+#pragma unroll
+                            for (int i = 0; i < W; ++i) {
+                                hr = __ffma2_rn(make_float2(Vc[i].x, Vc[i].x), G[i], hr);
+                                hi = __ffma2_rn(make_float2(Vc[i].y, Vc[i].y), G[i], hi);
+                            }
+                            const float hx = hr.x + hi.y, hy = hr.y - hi.x;
+#pragma unroll
+                            for (int nu = 0; nu < NM; ++nu) {
+                                const float2 u = __ldg(uq + (mu * NM + nu) * kTb);
+                                gr[nu] = __ffma2_rn(make_float2(hx, hx), u, gr[nu]);
+                                gi[nu] = __ffma2_rn(make_float2(hy, hy), u, gi[nu]);
+                            }
+                        }
+                        float gm = 0.f;                      // Gamma capture: sum over modes
+#pragma unroll
+                        for (int nu = 0; nu < NM; ++nu) {
+                            const float2 wnv = __ldg(uq + (NM * NM + nu) * kTb);
+                            const float w = wnv.x, nq = wnv.y;
+                            if (w < 0.f) continue;
+                            const float gx = gr[nu].x - gi[nu].y, gy = gr[nu].y + gi[nu].x;
+                            const float g2 = gx * gx + gy * gy;
+                            const float x1 = (en + w) - em;
+                            const float x2 = (en - w) - em;
+                            float tt = 0.f;
+                            if (fabsf(x1) <= ceta) {
+                                const float y = x1 * ieta;
+                                tt += (nq + fm) * __expf(-y * y);
+                            }
+                            if (fabsf(x2) <= ceta) {
+                                const float y = x2 * ieta;
+                                tt += (1.f + nq - fm) * __expf(-y * y);
+                            }
+                            rate = fmaf(g2, tt, rate);
+                            if constexpr (GAM) gm = fmaf(g2, tt, gm);
+                        }
+                        if constexpr (GAM) {
+                            if (m >= lokq && m < lokq + nwkq) a.gam[grow + m] = gm;
+                        }
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
+            if (lane == 0) rs[r] = rate;
+            __syncwarp();                                // Uw is rewritten by the next item
+        }
+        // the first warp without an item lists the next group's
+        if (r == ng && fnext >= 0) list_items(groups.group(fnext), N1, lists + (buf ^ 1) * (nh + 2));
+        __syncthreads();                                 // the list, rs and Y are rewritten next
+        if (wid == 0) {
+            for (int r = lane; r < ng; r += 32) acc += (double)rs[r];
+            __syncwarp();                                // before rs is rewritten by this warp's items
+        }
+        f = fnext;
     }
     // rs of the last group was consumed by warp 0: lanes by a fixed tree
     if (wid == 0) {

@@ -88,9 +88,8 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
     double *CS3 = reinterpret_cast<double *>(Y + lay.y + lay.u);  // [N3][NF]: axis-3 coefficients
     const int nh = N1 / 2 + 1;
     double *rs = CS3 + lay.cs;                   // [nh]: sums of the current group's items
-    int *gl = reinterpret_cast<int *>(rs + lay.rs);     // [nh]: the items, (q1, N1 - q1)
-    int *nglist = gl + nh;                       // [2]: items of the group, next one to take
-    uint32_t *flags = reinterpret_cast<uint32_t *>(nglist + 2);      // bit pb NJG + jg: the group has pairs
+    int *lists = reinterpret_cast<int *>(rs + lay.rs);  // two item lists (list_items)
+    uint32_t *flags = reinterpret_cast<uint32_t *>(lists + 2 * (nh + 2));
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     uint8_t *clist = reinterpret_cast<uint8_t *>(flags + lay.flags) + wid * kSieveBlock;
     uint16_t *left = reinterpret_cast<uint16_t *>(reinterpret_cast<uint8_t *>(flags + lay.flags) + kSfWarps * kSieveBlock) +
@@ -109,39 +108,9 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
     const double *CS1 = a.coef, *CS2 = CS1 + N1 * NF;
     for (int e = tid; e < N3 * NF; e += kSfThreads) CS3[e] = CS2[N2 * NF + e];
     const int nplane = a.nplane;
-    const int pb_n = (nplane + kSieveBlock - 1) / kSieveBlock;
     const uint32_t *mrow = a.mask + (int64_t)kp * a.mask_words;   // [pb][q1][8 words]
-    // groups with pairs: every thread takes runs (pb, q1) and marks the groups of their set bits
-    for (int e = tid; e < (int)lay.flags; e += kSfThreads) flags[e] = 0u;
-    __syncthreads();
-    for (int r = tid; r < pb_n * N1; r += kSfThreads) {
-        const uint4 *w4 = reinterpret_cast<const uint4 *>(mrow) + 2 * (int64_t)r;
-        const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
-        const uint32_t w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-        const int pb = r / N1;
-        if (NJG == 1) {
-            if (w[0] | w[1] | w[2] | w[3] | w[4] | w[5] | w[6] | w[7]) atomicOr(flags + (pb >> 5), 1u << (pb & 31));
-            continue;
-        }
-        const int q2lo = fdiv(pb * kSieveBlock, a.fn3);
-        int seen = -1;                           // last group marked
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            uint32_t b = w[x];
-            while (b) {
-                const int c = x * 32 + __ffs(b) - 1;
-                const int jg = (fdiv(pb * kSieveBlock + c, a.fn3) - q2lo) / JQ;
-                if (jg != seen) {
-                    const int f = pb * NJG + jg;
-                    atomicOr(flags + (f >> 5), 1u << (f & 31));
-                    seen = jg;
-                }
-                // on to the group's end
-                const int end = (q2lo + (jg + 1) * JQ) * N3 - pb * kSieveBlock - x * 32;
-                b = end < 32 ? b & ~((1u << end) - 1u) : 0u;
-            }
-        }
-    }
+    const SfGroups groups{mrow, flags, a.fn3, N1, N3, nplane, JQ, NJG};
+    mark_groups(groups, (int)lay.flags);
     int k1, k2, k3;
     grid_coords(a.g, ik, k1, k2, k3);
     const double en = a.eps[(int64_t)ik * W + lo + n];
@@ -149,251 +118,219 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
     const double ieta = 1.0 / a.eta;
     double acc = 0;                              // warp 0: sums of the items lane, lane + 32, ...
     __syncthreads();
-    for (int pb = 0; pb < pb_n; ++pb) {
-        const int c_lo = pb * kSieveBlock, c_hi = min(nplane, c_lo + kSieveBlock) - 1;
-        const int q2lo = fdiv(c_lo, a.fn3), nq2 = fdiv(c_hi, a.fn3) - q2lo + 1;
-        const int njg = (nq2 + JQ - 1) / JQ;
-        const uint32_t *mpb = mrow + (int64_t)pb * N1 * 8;
-        for (int jg = 0; jg < njg; ++jg) {
-            const int fl = pb * NJG + jg;
-            if (!((flags[fl >> 5] >> (fl & 31)) & 1u)) continue;
-            const int j0 = jg * JQ, jn = min(JQ, nq2 - j0);
-            // combinations [r0, r1) of the plane block belong to the group
-            const int r0 = max(0, (q2lo + j0) * N3 - c_lo), r1 = min(kSieveBlock, (q2lo + j0 + jn) * N3 - c_lo);
-            // bits of word x (of 8) inside the group
-            auto in_group = [&](int x) -> uint32_t {
-                const int a0 = min(max(r0 - 32 * x, 0), 32), a1 = min(max(r1 - 32 * x, 0), 32);
-                const uint32_t lo_m = a0 < 32 ? ~0u << a0 : 0u, hi_m = a1 < 32 ? ~(~0u << a1) : ~0u;
-                return lo_m & hi_m;
-            };
-            // the group's items {q1, N1 - q1} with pairs (warp 0): the two-run ones first
-            if (wid == 0) {
-                int cnt = 0;
-                const int n2 = (N1 - 1) / 2;                     // items with two runs
-                auto filled = [&](int q1) {
-                    const uint4 *w4 = reinterpret_cast<const uint4 *>(mpb) + 2 * q1;
-                    const uint4 u = __ldg(w4), v = __ldg(w4 + 1);
-                    if (NJG == 1) return (u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w) != 0u;
-                    return ((u.x & in_group(0)) | (u.y & in_group(1)) | (u.z & in_group(2)) | (u.w & in_group(3)) |
-                            (v.x & in_group(4)) | (v.y & in_group(5)) | (v.z & in_group(6)) | (v.w & in_group(7))) != 0u;
-                };
-                for (int h0 = 0; h0 < nh; h0 += 32) {
-                    const int h = h0 + lane;                     // 1 .. n2, then 0, then N1 / 2
-                    const int q1 = h < n2 ? h + 1 : h == n2 ? 0 : h;
-                    const bool on = h < nh && (filled(q1) || (h < n2 && filled(N1 - q1)));
-                    const unsigned b = __ballot_sync(0xffffffffu, on);
-                    if (on) gl[cnt + __popc(b & ((1u << lane) - 1u))] = q1;
-                    cnt += __popc(b);
-                }
-                if (lane == 0) {
-                    nglist[0] = cnt;
-                    nglist[1] = 0;
-                }
+    int f = groups.next(-1), buf = 0;
+    if (wid == 0 && f >= 0) list_items(groups.group(f), N1, lists);
+    for (; f >= 0; buf ^= 1) {
+        const SfGroup grp = groups.group(f);
+        const int c_lo = grp.c_lo, q2lo = grp.q2lo, j0 = grp.j0, jn = grp.jn;
+        int *gl = lists + buf * (nh + 2);
+        const int fnext = groups.next(f);
+        for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
+            const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
+            const int jj = e2 / X, col = e2 - jj * X;
+            if (jj >= jn) continue;
+            const int f1 = r13 / D, f3 = r13 - f1 * D;
+            const double *c2 = CS2 + (q2lo + j0 + jj) * NF;
+            const double2 *src = gs + ((f1 * D) * D + f3) * X + col;
+            double2 v = __ldg(src);
+#pragma unroll
+            for (int f2 = 1; f2 < D; ++f2) {
+                const double2 w = __ldg(src + f2 * D * X);
+                v.x = fma(c2[f2 - 1], w.x, v.x);
+                v.y = fma(c2[f2 - 1], w.y, v.y);
             }
-            for (int e = tid; e < D * D * JQ * X; e += kSfThreads) {
-                const int r13 = fdiv(e, a.fper), e2 = e - r13 * JQ * X;
-                const int jj = e2 / X, col = e2 - jj * X;
-                if (jj >= jn) continue;
-                const int f1 = r13 / D, f3 = r13 - f1 * D;
-                const double *c2 = CS2 + (q2lo + j0 + jj) * NF;
-                const double2 *src = gs + ((f1 * D) * D + f3) * X + col;
-                double2 v = __ldg(src);
-#pragma unroll
-                for (int f2 = 1; f2 < D; ++f2) {
-                    const double2 w = __ldg(src + f2 * D * X);
-                    v.x = fma(c2[f2 - 1], w.x, v.x);
-                    v.y = fma(c2[f2 - 1], w.y, v.y);
-                }
-                Y[e] = v;
-            }
-            __syncthreads();
-            const int ng = nglist[0], per = jn * X;
-            // items are taken from a counter; each writes its own sum, as in k_scatter_sf
-            while (true) {
-                int r = 0;
-                if (lane == 0) r = atomicAdd(nglist + 1, 1);
-                r = __shfl_sync(0xffffffffu, r, 0);
-                if (r >= ng) break;
-                const int q1 = gl[r];
-                const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
-                // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
-                const int wx = lane & 7;
-                uint32_t word = 0u;
-                if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
-                int skip = 0;                                    // pairs of the run in earlier groups (capture)
-                if (NJG > 1) {
-                    if constexpr (GAM) skip = __popc(word & (r0 > 32 * wx + 31 ? ~0u : r0 > 32 * wx ? ~(~0u << (r0 - 32 * wx)) : 0u));
-                    word &= in_group(wx);
-                }
-                int npc = __popc(word);
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
-                    npc += __shfl_xor_sync(0xffffffffu, npc, o);
-                    if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
-                }
-                const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
-                int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
-                if constexpr (GAM) {
-                    const int *ru = a.runs + (int64_t)kp * a.run_stride + pb * N1;
-                    t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
-                    t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
-                }
-                // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
-                // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
-                double c1[NF];
-#pragma unroll
-                for (int f = 0; f < NF; ++f) c1[f] = __ldg(CS1 + q1 * NF + f);
-                for (int f3 = 0; f3 < D; ++f3)
-                    for (int e = lane; e < per; e += 32) {
-                        const double2 *src = Y + (size_t)f3 * JQ * X + e;
-                        double2 v = src[0], o = make_double2(0, 0);
-#pragma unroll
-                        for (int R = 1; R <= RC; ++R) {
-                            const double2 w = src[(2 * R - 1) * D * JQ * X], z = src[2 * R * D * JQ * X];
-                            v.x = fma(c1[2 * R - 2], w.x, v.x);
-                            v.y = fma(c1[2 * R - 2], w.y, v.y);
-                            o.x = fma(c1[2 * R - 1], z.x, o.x);
-                            o.y = fma(c1[2 * R - 1], z.y, o.y);
-                        }
-                        double2 *dst = Uw + (size_t)f3 * JQ * X + e;
-                        dst[0] = make_double2(v.x + o.x, v.y + o.y);
-                        dst[ustride] = make_double2(v.x - o.x, v.y - o.y);
-                    }
-                double rate = 0;
-                int b1a = k1 + q1, b1b = k1 + q1b;
-                if (b1a >= N1) b1a -= N1;
-                if (b1b >= N1) b1b -= N1;
-                const int parts = na + nb <= kSieveBlock ? 1 : 2;
-                for (int part = 0; part < parts; ++part) {
-                    const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
-                    __syncwarp();                                    // Uw is complete, clist is consumed
-                    {
-                        int at = 0;
-                        for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
-                            const uint32_t w = __shfl_sync(0xffffffffu, word, x);
-                            if (w == 0u) continue;                   // uniform over the warp
-                            if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
-                            at += __popc(w);
-                        }
-                    }
-                    int base = 0, nleft = 0;
-                    while (true) {
-                        __syncwarp();
-                        const bool fresh = base < npr && nleft < 32;
-                        if (!fresh && nleft == 0) break;
-                        int tt, m = 0;
-                        bool have;
-                        if (fresh) {
-                            tt = base + lane;
-                            have = tt < npr;
-                            base += 32;
-                        } else {
-                            const int take = min(nleft, 32);
-                            nleft -= take;
-                            have = lane < take;
-                            const int e = have ? left[nleft + lane] : 0;
-                            __syncwarp();                            // before the entries are rewritten
-                            tt = e >> 3;
-                            m = e & 7;
-                        }
-                        const bool second = tt >= npa;
-                        const int c = have ? clist[tt] : 0;
-                        const int q = (second ? q1b : q1) * nplane + c_lo + c;
-                        const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
-                        int b2 = k2 + q2, b3 = k3 + q3;
-                        if (b2 >= N2) b2 -= N2;
-                        if (b3 >= N3) b3 -= N3;
-                        const int64_t ikq = ((int64_t)(second ? b1b : b1a) * N2 + b2) * N3 + b3;
-                        if (fresh) {
-                            // final bands within reach of a mode (a superset, in FP32; the others add zero)
-                            unsigned mask = 0;
-                            if (have) {
-                                const float lim = __ldg(a.hwmax32 + q) + a.lim32;
-#pragma unroll
-                                for (int mm = 0; mm < W; ++mm)
-                                    mask |= (fabsf(en32 - __ldg(a.eps32 + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
-                            }
-                            have = mask != 0;
-                            m = have ? __ffs(mask) - 1 : 0;
-                            mask &= mask - 1;
-                            unsigned more;
-                            while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
-                                if (have && mask) {
-                                    left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
-                                    mask &= mask - 1;
-                                }
-                                nleft += __popc(more);
-                            }
-                            __syncwarp();
-                        }
-                        if (!have) continue;
-                        const double2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;
-                        double c3[NF];
-#pragma unroll
-                        for (int f = 0; f < NF; ++f) c3[f] = CS3[q3 * NF + f];
-                        const double em = __ldg(a.eps + ikq * W + m), fm = __ldg(a.focc + ikq * W + m);
-                        const double2 *vp = a.V + ikq * W * W + m;
-                        const double2 *uq = a.u + (int64_t)q * NM * NM;
-                        double2 Vc[W], gv[NM];
-#pragma unroll
-                        for (int i = 0; i < W; ++i) Vc[i] = __ldg(vp + i * W);
-#pragma unroll
-                        for (int nu = 0; nu < NM; ++nu) gv[nu] = make_double2(0, 0);
-#pragma unroll
-                        for (int mu = 0; mu < NM; ++mu) {
-                            double2 h = make_double2(0, 0);
-#pragma unroll
-                            for (int i = 0; i < W; ++i) {
-                                double2 G = Ub[mu * W + i];
-#pragma unroll
-                                for (int f = 1; f < D; ++f) {
-                                    const double2 w = Ub[f * JQ * X + mu * W + i];
-                                    G.x = fma(c3[f - 1], w.x, G.x);
-                                    G.y = fma(c3[f - 1], w.y, G.y);
-                                }
-                                h = cfmac(Vc[i], G, h);
-                            }
-#pragma unroll
-                            for (int nu = 0; nu < NM; ++nu) gv[nu] = cfma(h, __ldg(uq + mu * NM + nu), gv[nu]);
-                        }
-                        double gm = 0;
-#pragma unroll
-                        for (int nu = 0; nu < NM; ++nu) {
-                            const double w = __ldg(a.hw + (int64_t)q * NM + nu);
-                            if (!(w >= a.omega_min)) continue;
-                            const double x1 = (en + w) - em, x2 = (en - w) - em;
-                            const double N = __ldg(a.nocc + (int64_t)q * NM + nu);
-                            double term = 0;
-                            if (fabs(x1) <= a.ceta) {
-                                const double y = x1 * ieta;
-                                term = (N + fm) * exp_neg(-y * y, T);
-                            }
-                            if (fabs(x2) <= a.ceta) {
-                                const double y = x2 * ieta;
-                                term = fma(1.0 + N - fm, exp_neg(-y * y, T), term);
-                            }
-                            gm = fma(gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y, term, gm);
-                        }
-                        rate += gm;
-                        if constexpr (GAM) {
-                            const int lokq = __ldg(a.win_lo + ikq), nwkq = __ldg(a.win_n + ikq);
-                            const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
-                            if (m >= lokq && m < lokq + nwkq)
-                                a.gam[a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq + (m - lokq)] = gm;
-                        }
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
-                if (lane == 0) rs[r] = rate;
-                __syncwarp();                                // Uw is rewritten by the next item
-            }
-            __syncthreads();                                 // gl, nglist, rs and Y are rewritten next
-            if (wid == 0) {
-                for (int r = lane; r < ng; r += 32) acc += rs[r];
-                __syncwarp();                                // before rs is rewritten by this warp's items
-            }
+            Y[e] = v;
         }
+        __syncthreads();
+        const int ng = gl[nh], per = jn * X;
+        int r = 0;
+        // items are taken from a counter; each writes its own sum, as in k_scatter_sf
+        while (true) {
+            if (lane == 0) r = atomicAdd(gl + nh + 1, 1);
+            r = __shfl_sync(0xffffffffu, r, 0);
+            if (r >= ng) break;
+            const int q1 = gl[r];
+            const int q1b = q1 == 0 || 2 * q1 == N1 ? q1 : N1 - q1;
+            // lanes 0-7 and 8-15: the words of the two runs; na, nb: their pairs
+            const int wx = lane & 7;
+            uint32_t word = 0u;
+            if (lane < 8 || (lane < 16 && q1b != q1)) word = __ldg(grp.mpb + (lane < 8 ? q1 : q1b) * 8 + wx);
+            int skip = 0;                                    // pairs of the run in earlier groups (capture)
+            if (NJG > 1) {
+                if constexpr (GAM) skip = __popc(word & (grp.r0 > 32 * wx + 31 ? ~0u : grp.r0 > 32 * wx ? ~(~0u << (grp.r0 - 32 * wx)) : 0u));
+                word &= grp.bits(wx);
+            }
+            int npc = __popc(word);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                npc += __shfl_xor_sync(0xffffffffu, npc, o);
+                if constexpr (GAM) skip += __shfl_xor_sync(0xffffffffu, skip, o);
+            }
+            const int na = __shfl_sync(0xffffffffu, npc, 0), nb = __shfl_sync(0xffffffffu, npc, 8);
+            int t0 = 0, t0b = 0;                             // capture: list positions of the runs' pairs
+            if constexpr (GAM) {
+                const int *ru = a.runs + (int64_t)kp * a.run_stride + c_lo / kSieveBlock * N1;
+                t0 = ru[q1] + __shfl_sync(0xffffffffu, skip, 0);
+                t0b = ru[q1b] + __shfl_sync(0xffffffffu, skip, 8);
+            }
+            // U of the runs q1 and -q1 from one pass over Y: with E the even part (form 0 and
+            // the cosine forms) and O the odd part (the sine forms), U(+-q1) = E +- O
+            double c1[NF];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) c1[f] = __ldg(CS1 + q1 * NF + f);
+            for (int f3 = 0; f3 < D; ++f3)
+                for (int e = lane; e < per; e += 32) {
+                    const double2 *src = Y + (size_t)f3 * JQ * X + e;
+                    double2 v = src[0], o = make_double2(0, 0);
+#pragma unroll
+                    for (int R = 1; R <= RC; ++R) {
+                        const double2 w = src[(2 * R - 1) * D * JQ * X], z = src[2 * R * D * JQ * X];
+                        v.x = fma(c1[2 * R - 2], w.x, v.x);
+                        v.y = fma(c1[2 * R - 2], w.y, v.y);
+                        o.x = fma(c1[2 * R - 1], z.x, o.x);
+                        o.y = fma(c1[2 * R - 1], z.y, o.y);
+                    }
+                    double2 *dst = Uw + (size_t)f3 * JQ * X + e;
+                    dst[0] = make_double2(v.x + o.x, v.y + o.y);
+                    dst[ustride] = make_double2(v.x - o.x, v.y - o.y);
+                }
+            double rate = 0;
+            int b1a = k1 + q1, b1b = k1 + q1b;
+            if (b1a >= N1) b1a -= N1;
+            if (b1b >= N1) b1b -= N1;
+            const int parts = na + nb <= kSieveBlock ? 1 : 2;
+            for (int part = 0; part < parts; ++part) {
+                const int npa = part == 0 ? na : 0, npr = parts == 1 ? na + nb : part == 0 ? na : nb;
+                __syncwarp();                                    // Uw is complete, clist is consumed
+                {
+                    int at = 0;
+                    for (int x = part * 8; x < (parts == 1 || part == 1 ? 16 : 8); ++x) {
+                        const uint32_t w = __shfl_sync(0xffffffffu, word, x);
+                        if (w == 0u) continue;                   // uniform over the warp
+                        if ((w >> lane) & 1u) clist[at + __popc(w & ((1u << lane) - 1u))] = (uint8_t)((x & 7) * 32 + lane);
+                        at += __popc(w);
+                    }
+                }
+                int base = 0, nleft = 0;
+                while (true) {
+                    __syncwarp();
+                    const bool fresh = base < npr && nleft < 32;
+                    if (!fresh && nleft == 0) break;
+                    int tt, m = 0;
+                    bool have;
+                    if (fresh) {
+                        tt = base + lane;
+                        have = tt < npr;
+                        base += 32;
+                    } else {
+                        const int take = min(nleft, 32);
+                        nleft -= take;
+                        have = lane < take;
+                        const int e = have ? left[nleft + lane] : 0;
+                        __syncwarp();                            // before the entries are rewritten
+                        tt = e >> 3;
+                        m = e & 7;
+                    }
+                    const bool second = tt >= npa;
+                    const int c = have ? clist[tt] : 0;
+                    const int q = (second ? q1b : q1) * nplane + c_lo + c;
+                    const int q2 = fdiv(c_lo + c, a.fn3), q3 = c_lo + c - q2 * N3, j = q2 - q2lo;
+                    int b2 = k2 + q2, b3 = k3 + q3;
+                    if (b2 >= N2) b2 -= N2;
+                    if (b3 >= N3) b3 -= N3;
+                    const int64_t ikq = ((int64_t)(second ? b1b : b1a) * N2 + b2) * N3 + b3;
+                    if (fresh) {
+                        // final bands within reach of a mode (a superset, in FP32; the others add zero)
+                        unsigned mask = 0;
+                        if (have) {
+                            const float lim = __ldg(a.hwmax32 + q) + a.lim32;
+#pragma unroll
+                            for (int mm = 0; mm < W; ++mm)
+                                mask |= (fabsf(en32 - __ldg(a.eps32 + ikq * W + mm)) <= lim ? 1u : 0u) << mm;
+                        }
+                        have = mask != 0;
+                        m = have ? __ffs(mask) - 1 : 0;
+                        mask &= mask - 1;
+                        unsigned more;
+                        while ((more = __ballot_sync(0xffffffffu, have && mask)) != 0) {
+                            if (have && mask) {
+                                left[nleft + __popc(more & ((1u << lane) - 1u))] = (uint16_t)(tt << 3 | (__ffs(mask) - 1));
+                                mask &= mask - 1;
+                            }
+                            nleft += __popc(more);
+                        }
+                        __syncwarp();
+                    }
+                    if (!have) continue;
+                    const double2 *Ub = Uw + (second ? ustride : 0) + (j - j0) * X;
+                    double c3[NF];
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) c3[f] = CS3[q3 * NF + f];
+                    const double em = __ldg(a.eps + ikq * W + m), fm = __ldg(a.focc + ikq * W + m);
+                    const double2 *vp = a.V + ikq * W * W + m;
+                    const double2 *uq = a.u + (int64_t)q * NM * NM;
+                    double2 Vc[W], gv[NM];
+#pragma unroll
+                    for (int i = 0; i < W; ++i) Vc[i] = __ldg(vp + i * W);
+#pragma unroll
+                    for (int nu = 0; nu < NM; ++nu) gv[nu] = make_double2(0, 0);
+#pragma unroll
+                    for (int mu = 0; mu < NM; ++mu) {
+                        double2 h = make_double2(0, 0);
+#pragma unroll
+                        for (int i = 0; i < W; ++i) {
+                            double2 G = Ub[mu * W + i];
+#pragma unroll
+                            for (int f = 1; f < D; ++f) {
+                                const double2 w = Ub[f * JQ * X + mu * W + i];
+                                G.x = fma(c3[f - 1], w.x, G.x);
+                                G.y = fma(c3[f - 1], w.y, G.y);
+                            }
+                            h = cfmac(Vc[i], G, h);
+                        }
+#pragma unroll
+                        for (int nu = 0; nu < NM; ++nu) gv[nu] = cfma(h, __ldg(uq + mu * NM + nu), gv[nu]);
+                    }
+                    double gm = 0;
+#pragma unroll
+                    for (int nu = 0; nu < NM; ++nu) {
+                        const double w = __ldg(a.hw + (int64_t)q * NM + nu);
+                        if (!(w >= a.omega_min)) continue;
+                        const double x1 = (en + w) - em, x2 = (en - w) - em;
+                        const double N = __ldg(a.nocc + (int64_t)q * NM + nu);
+                        double term = 0;
+                        if (fabs(x1) <= a.ceta) {
+                            const double y = x1 * ieta;
+                            term = (N + fm) * exp_neg(-y * y, T);
+                        }
+                        if (fabs(x2) <= a.ceta) {
+                            const double y = x2 * ieta;
+                            term = fma(1.0 + N - fm, exp_neg(-y * y, T), term);
+                        }
+                        gm = fma(gv[nu].x * gv[nu].x + gv[nu].y * gv[nu].y, term, gm);
+                    }
+                    rate += gm;
+                    if constexpr (GAM) {
+                        const int lokq = __ldg(a.win_lo + ikq), nwkq = __ldg(a.win_n + ikq);
+                        const int t = second ? t0b + tt - npa : t0 + tt;    // the pair's place in the k-point's list
+                        if (m >= lokq && m < lokq + nwkq)
+                            a.gam[a.gent[kp] + a.goff[a.kp_pairs[kp] - a.p_off + t] + (int64_t)n * nwkq + (m - lokq)] = gm;
+                    }
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rate += __shfl_xor_sync(0xffffffffu, rate, o);
+            if (lane == 0) rs[r] = rate;
+            __syncwarp();                                // Uw is rewritten by the next item
+        }
+        // the first warp without an item lists the next group's
+        if (r == ng && fnext >= 0) list_items(groups.group(fnext), N1, lists + (buf ^ 1) * (nh + 2));
+        __syncthreads();                                 // the list, rs and Y are rewritten next
+        if (wid == 0) {
+            for (int x = lane; x < ng; x += 32) acc += rs[x];
+            __syncwarp();                                // before rs is rewritten by this warp's items
+        }
+        f = fnext;
     }
     // lanes by a fixed tree: deterministic, independent of the chunking
     if (wid == 0) {
