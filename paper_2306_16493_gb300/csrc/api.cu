@@ -460,29 +460,38 @@ epwi_status epwi_find_mu(epwi_ctx *c, double T, double n_c, int32_t nv, double *
         const double emin = device_reduce_minmax(c, e, c->nk, c->nw, nv, false);
         double lo = emin - 3.0;
         double hi = device_reduce_minmax(c, e, c->nk, c->nw, c->nw - 1, true) + 3.0;
-        // n(mu) is increasing and nearly exponential below the band edge, so the root of
-        // h(mu) = ln n(mu) - ln n_c is bracketed and found by regula falsi with the Illinois
-        // modification (a retained end's h is halved), falling back to bisection where h is not
-        // finite (n underflowed); stop at the same residual as a bisection: |n - n_c| <= 1e-13 n_c.
+        // n(mu) is increasing and nearly exponential below the band edge, and d ln n / d mu <= 1 / kT
+        // everywhere, so from a point lo below the root of h(mu) = ln n(mu) - ln n_c the tangent of that
+        // slope leads to a point still below it, and secants through the last two such points to
+        // one close to it; no point far above, where every band counts, is needed.  Once a point above
+        // is known, regula falsi with the Illinois modification (a retained end's h is halved);
+        // bisection where h is not finite (n underflowed) or a step leaves the bracket.  Stop at the
+        // same residual as a bisection: |n - n_c| <= 1e-13 n_c.
         auto h = [&](double mu, double &n) {
             n = carrier_density(c, T, mu, nv, emin);
             return n > 0 ? std::log(n / n_c) : -HUGE_VAL;
         };
-        double nlo, nhi;
-        double hlo = h(lo, nlo), hhi = h(hi, nhi);
+        const double kT = epc::kKbEVK * T;
+        double n;
+        double hlo = h(lo, n), hhi = HUGE_VAL;
+        double plo = lo, phlo = -HUGE_VAL;       // the point below before lo
         double mid = 0.5 * (lo + hi);
         int side = 0;
         for (int it = 0; it < 400; ++it) {
-            if (std::isfinite(hlo) && std::isfinite(hhi) && hhi > hlo) {
-                mid = hi - hhi * (hi - lo) / (hhi - hlo);
-                if (!(mid > lo && mid < hi)) mid = 0.5 * (lo + hi);
-            } else {
-                mid = 0.5 * (lo + hi);
+            mid = 0.5 * (lo + hi);
+            double x = mid;
+            if (std::isfinite(hlo) && std::isfinite(hhi)) {
+                if (hhi > hlo) x = hi - hhi * (hi - lo) / (hhi - hlo);
+            } else if (std::isfinite(hlo) && hlo < 0 && it < 20) {   // (n_c above what the bands hold: bisect)
+                x = lo - kT * hlo;
+                if (std::isfinite(phlo) && hlo > phlo) x = std::max(x, lo - hlo * (lo - plo) / (hlo - phlo));
             }
-            double n;
+            if (x > lo && x < hi) mid = x;
             const double hm = h(mid, n);
             if (std::fabs(n - n_c) <= 1e-13 * n_c || hi - lo <= 1e-15) break;
             if (n < n_c) {
+                plo = lo;
+                phlo = hlo;
                 lo = mid;
                 hlo = hm;
                 if (side == -1 && std::isfinite(hhi)) hhi *= 0.5;
