@@ -112,8 +112,11 @@ struct Lattice {
 // Electrons: eps (ascending), V (columns), velocities, FP32 copies.
 // fac.U given: H(k) from the factorised stages (and no velocities); otherwise direct sums, with the
 // velocities of every point when do_vel is set.
+// Above four bands the matrices live in local memory (4.5 KB a thread): 48 registers and ten blocks per
+// SM cover its latency better than 226 registers and two, and the FP64 pipe binds (Si-like 100^3, 8
+// bands and 6 modes: 35.1 -> 28.3 ms).
 template <int WMAX, bool FIXED>
-__global__ void __launch_bounds__(128) k_eig_el(GridInfo g, int64_t nk, int W_, int nR,
+__global__ void __launch_bounds__(128, WMAX > 4 ? 10 : 1) k_eig_el(GridInfo g, int64_t nk, int W_, int nR,
                                                 const int *__restrict__ R,
                                                 const double *__restrict__ Rcart,
                                                 const double2 *__restrict__ Hw,
@@ -266,7 +269,7 @@ __device__ __forceinline__ int64_t minus_q(const GridInfo &g, int i1, int i2, in
 // Phonons: hbar*omega, u = e (hbar^2 / (2 m hbar omega))^{1/2}, FP32 copies; D(q) from the
 // factorised stages when fac.U is given.
 template <int NMAX, bool FIXED>
-__global__ void __launch_bounds__(128) k_eig_ph(GridInfo g, int64_t nq, int Nm_, int nR,
+__global__ void __launch_bounds__(128, NMAX > 4 ? 10 : 1) k_eig_ph(GridInfo g, int64_t nq, int Nm_, int nR,
                                                 const int *__restrict__ R,
                                                 const double *__restrict__ Phiw,
                                                 const double *__restrict__ mode_mass,
