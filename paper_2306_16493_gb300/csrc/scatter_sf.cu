@@ -35,7 +35,8 @@
 // warp pass, 50.7 ms with both runs from one pass and the runs' bounds from a table, 49.3 ms from the
 // mask, 47.9 ms with packed multiply-adds (__ffma2_rn: two FP32 FMAs per issue slot) and a group's
 // items listed while the group before is worked off; 20 x 27 x 45 (61 M pairs) 4.6, 3.4, 3.3 and 3.0 ms;
-// Si-like 100^3 14.6 -> 13.4 ms by the last.
+// Si-like 100^3 14.6 -> 13.4 ms by the last.  With the mode energies loaded ahead of the rotation 45.4
+// (48^3), 2.8 (20 x 27 x 45) and 11.9 ms (Si-like).
 #include <algorithm>
 
 #include "epwi_internal.cuh"
@@ -596,6 +597,39 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
 #pragma unroll
                         for (int i = 0; i < W; ++i) Vc[i] = __ldg(kt + i * kTb + x64);
                     }
+                    // (hbar omega, N) of the modes, loaded ahead of the rotation.  Wide systems form the
+                    // occupation x delta factors ahead as well, while V and u travel, and pass over a band
+                    // without any (Si-like 100^3 12.8 -> 11.9 ms; for W = 4 the registers are missed: 48^3
+                    // 45.4 -> 46.3 ms).
+                    constexpr bool kEarly = W > 4;
+                    float2 wn[NM];
+#pragma unroll
+                    for (int nu = 0; nu < NM; ++nu) wn[nu] = __ldg(uq + (NM * NM + nu) * kTb);
+                    auto factor = [&](int nu) -> float {
+                        const float w = wn[nu].x, nq = wn[nu].y;
+                        const float x1 = (en + w) - em;
+                        const float x2 = (en - w) - em;
+                        float tt = 0.f;
+                        if (fabsf(x1) <= ceta) {
+                            const float y = x1 * ieta;
+                            tt += (nq + fm) * __expf(-y * y);
+                        }
+                        if (fabsf(x2) <= ceta) {
+                            const float y = x2 * ieta;
+                            tt += (1.f + nq - fm) * __expf(-y * y);
+                        }
+                        return tt;
+                    };
+                    float td[kEarly ? NM : 1];
+                    if constexpr (kEarly) {
+                        bool any = GAM;
+#pragma unroll
+                        for (int nu = 0; nu < NM; ++nu) {
+                            td[nu] = wn[nu].x < 0.f ? 0.f : factor(nu);
+                            any |= td[nu] != 0.f;
+                        }
+                        if (!any) continue;
+                    }
                         float2 gr[NM], gi[NM];
 #pragma unroll
                         for (int nu = 0; nu < NM; ++nu) gr[nu] = gi[nu] = make_float2(0.f, 0.f);
@@ -650,22 +684,10 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
                         float gm = 0.f;                      // Gamma capture: sum over modes
 #pragma unroll
                         for (int nu = 0; nu < NM; ++nu) {
-                            const float2 wnv = __ldg(uq + (NM * NM + nu) * kTb);
-                            const float w = wnv.x, nq = wnv.y;
-                            if (w < 0.f) continue;
+                            if (!kEarly && wn[nu].x < 0.f) continue;
                             const float gx = gr[nu].x - gi[nu].y, gy = gr[nu].y + gi[nu].x;
                             const float g2 = gx * gx + gy * gy;
-                            const float x1 = (en + w) - em;
-                            const float x2 = (en - w) - em;
-                            float tt = 0.f;
-                            if (fabsf(x1) <= ceta) {
-                                const float y = x1 * ieta;
-                                tt += (nq + fm) * __expf(-y * y);
-                            }
-                            if (fabsf(x2) <= ceta) {
-                                const float y = x2 * ieta;
-                                tt += (1.f + nq - fm) * __expf(-y * y);
-                            }
+                            const float tt = kEarly ? td[kEarly ? nu : 0] : factor(nu);
                             rate = fmaf(g2, tt, rate);
                             if constexpr (GAM) gm = fmaf(g2, tt, gm);
                         }
