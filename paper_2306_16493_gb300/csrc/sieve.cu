@@ -439,7 +439,9 @@ __global__ void __launch_bounds__(256, 3) k_sieve_count_fast(SieveArgs a, const 
 // L2 once (20 bytes per candidate), which bound the per-k-point kernel; here the arithmetic
 // does.  A whole b1 is passed over when no lane of the warp has a band within the largest reach
 // of any window energy of the column.  Candidates inside the FP32 margin are collected per b1
-// and decided exactly (pair_valid_tail) after the others.
+// and decided exactly (pair_valid_tail) after the others.  The compare and select half of the pipes binds
+// (76 % busy), so a candidate's test is one difference against two constants, and the test of its
+// mode energy against hm_fast is left out where no lane of the warp can fail it (48^3: 7.3 -> 6.4 ms).
 constexpr int kColSlots = 16;                    // k-points of a column per pass
 
 __host__ __device__ constexpr size_t sieve_cols_smem(int N1, int TB) {
@@ -473,8 +475,10 @@ __global__ void __launch_bounds__(TB) k_sieve_count_cols(SieveArgs a, ColumnSet 
         hms[q1 * TB + tid] = h;                  // read back by this thread only
         hmx = fmaxf(hmx, h);
     }
-    const float rej = a.ceta32 + a.delta32, acc = a.ceta32 - a.delta32;
+    // s = d - hm against c eta +- delta, half a delta wider either way for the rounding of s
+    const float rej = a.ceta32 + 1.5f * a.delta32, acc = a.ceta32 - 1.5f * a.delta32;
     const float hm_fast = a.ceta32 - 2.f * a.delta32;
+    const bool all_fast = __all_sync(0xffffffffu, hmx <= hm_fast);
     const float4 *eq = reinterpret_cast<const float4 *>(a.eps32) + (size_t)kqp * V4;
     const size_t rowv = (size_t)nplane * V4;
     const int p0 = cs.start[col], p1 = cs.start[col + 1];
@@ -492,7 +496,7 @@ __global__ void __launch_bounds__(TB) k_sieve_count_cols(SieveArgs a, ColumnSet 
                     en[tid][n] = a.eps[(int64_t)ik * WT + lo[ik] + n];
                     en32[tid][n] = a.eps32[(int64_t)ik * WT + lo[ik] + n];
                 }
-                r = make_float4(en32[tid][0], ns > 1 ? en32[tid][1] : 3.0e38f, __int_as_float(ik / nplane),
+                r = make_float4(en32[tid][0], ns > 1 ? en32[tid][1] : 3.0e38f, __int_as_float(ik / nplane * TB),
                                 __int_as_float(ns));
             }
             rec[tid] = r;
@@ -526,36 +530,42 @@ __global__ void __launch_bounds__(TB) k_sieve_count_cols(SieveArgs a, ColumnSet 
             for (int m = 0; m < WT; ++m) in |= (em[m] >= elo) & (em[m] <= ehi);
             uint32_t mine = 0u, amb = 0u;
             if (__any_sync(0xffffffffu, in)) {
+                // PLAIN: no mode energy of the warp's columns exceeds hm_fast
+                auto candidates = [&](auto plain) {
 #pragma unroll 4
-                for (int x = 0; x < nbp; ++x) {
-                    const float4 r = rec[x];
-                    int q1 = b1 - __float_as_int(r.z);
-                    if (q1 < 0) q1 += N1;
-                    const float hm = hms[q1 * TB + tid];
-                    float d = fabsf(r.x - em[0]);
+                    for (int x = 0; x < nbp; ++x) {
+                        const float4 r = rec[x];
+                        // (b1 - k1) mod N1, times TB: the smaller of the two as unsigned
+                        const unsigned q0 = (unsigned)(b1 * TB) - __float_as_uint(r.z);
+                        const float hm = hms[min(q0, q0 + (unsigned)(N1 * TB)) + tid];
+                        float d = fabsf(r.x - em[0]);
 #pragma unroll
-                    for (int m = 1; m < WT; ++m) d = fminf(d, fabsf(r.x - em[m]));
-                    const int ns = __float_as_int(r.w);
-                    if (ns > 1) {                // uniform over the block
+                        for (int m = 1; m < WT; ++m) d = fminf(d, fabsf(r.x - em[m]));
+                        const int ns = __float_as_int(r.w);
+                        if (ns > 1) {                // uniform over the block
 #pragma unroll
-                        for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(r.y - em[m]));
-                        for (int n = 2; n < ns; ++n) {
-                            const float e = en32[x][n];
+                            for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(r.y - em[m]));
+                            for (int n = 2; n < ns; ++n) {
+                                const float e = en32[x][n];
 #pragma unroll
-                            for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(e - em[m]));
+                                for (int m = 0; m < WT; ++m) d = fminf(d, fabsf(e - em[m]));
+                            }
                         }
+                        const float s = d - hm;
+                        const bool near = s <= rej;
+                        const bool sure = (decltype(plain)::value || hm <= hm_fast) & (s <= acc);
+                        const uint32_t bits = __ballot_sync(0xffffffffu, sure);
+                        if (lane == x) mine = bits;
+                        amb |= (near & !sure ? 1u : 0u) << x;
                     }
-                    const bool near = d <= hm + rej;
-                    const bool sure = (hm <= hm_fast) & (d <= hm + acc);
-                    const uint32_t bits = __ballot_sync(0xffffffffu, near & sure);
-                    if (lane == x) mine = bits;
-                    amb |= (near & !sure ? 1u : 0u) << x;
-                }
+                };
+                if (all_fast) candidates(std::true_type{});
+                else candidates(std::false_type{});
                 uint32_t any = __reduce_or_sync(0xffffffffu, amb);
                 while (any) {
                     const int x = __ffs(any) - 1;
                     any &= any - 1;
-                    int q1 = b1 - __float_as_int(rec[x].z);
+                    int q1 = b1 - __float_as_int(rec[x].z) / TB;
                     if (q1 < 0) q1 += N1;
                     bool v = false;
                     if ((amb >> x) & 1u)
@@ -567,7 +577,7 @@ __global__ void __launch_bounds__(TB) k_sieve_count_cols(SieveArgs a, ColumnSet 
                 }
             }
             if (lane < nb) {
-                int q1 = b1 - __float_as_int(rec[lane].z);
+                int q1 = b1 - __float_as_int(rec[lane].z) / TB;
                 if (q1 < 0) q1 += N1;
                 mst[lane * MS + q1 * NWB + wid] = mine;
                 c += __popc(mine);
