@@ -358,30 +358,31 @@ constexpr int kWarpsPerBlock = 4;
 
 struct WarpScratch {
     double2 *A, *V;
+    float2 *f;
     double *w;
     int *perm;
     JRot *rot;
 };
 
+__host__ __device__ inline size_t warp_scratch_per(int n) {
+    const size_t per = (sizeof(double2) * 2 + sizeof(float2)) * n * (n + 1) + sizeof(double) * 32 + sizeof(int) * 32 +
+                       sizeof(JRot) * 16;
+    return (per + 15) & ~size_t(15);
+}
+
 __device__ inline WarpScratch warp_scratch(uint8_t *base, int n) {
     const int ld = n + 1;
-    const size_t per = sizeof(double2) * 2 * n * ld + sizeof(double) * 32 + sizeof(int) * 32 +
-                       sizeof(JRot) * 16;
-    uint8_t *b = base + (threadIdx.x >> 5) * ((per + 15) & ~size_t(15));
     WarpScratch ws;
-    ws.A = reinterpret_cast<double2 *>(b);
+    ws.A = reinterpret_cast<double2 *>(base + (threadIdx.x >> 5) * warp_scratch_per(n));
     ws.V = ws.A + n * ld;
-    ws.w = reinterpret_cast<double *>(ws.V + n * ld);
+    ws.f = reinterpret_cast<float2 *>(ws.V + n * ld);
+    ws.w = reinterpret_cast<double *>(ws.f + n * ld);
     ws.perm = reinterpret_cast<int *>(ws.w + 32);
     ws.rot = reinterpret_cast<JRot *>(ws.perm + 32);
     return ws;
 }
 
-size_t warp_scratch_bytes(int n) {
-    const size_t per = sizeof(double2) * 2 * n * (n + 1) + sizeof(double) * 32 + sizeof(int) * 32 +
-                       sizeof(JRot) * 16;
-    return kWarpsPerBlock * ((per + 15) & ~size_t(15));
-}
+size_t warp_scratch_bytes(int n) { return kWarpsPerBlock * warp_scratch_per(n); }
 
 // FAC: H(k) and dH/dk from the factorised stages (as in k_eig_el), each lane building its row.
 template <bool FAC>
@@ -419,7 +420,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_eig_el_warp(
         }
     }
     __syncwarp();
-    const int ok = eig_hermitian_warp(S.A, S.V, W, ld, S.w, S.rot, S.perm);
+    const int ok = eig_hermitian_warp(S.A, S.V, S.f, W, ld, S.w, S.rot, S.perm);
     if (lane == 0 && !ok) atomicAdd(flag, 1);
     if (lane < W) {
         eps[ik * W + lane] = S.w[lane];
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_eig_ph_warp(
         }
     }
     __syncwarp();
-    const int ok = eig_hermitian_warp(S.A, S.V, Nm, ld, S.w, S.rot, S.perm);
+    const int ok = eig_hermitian_warp(S.A, S.V, S.f, Nm, ld, S.w, S.rot, S.perm);
     if (lane == 0 && !ok) atomicAdd(flag, im == iq ? 1 : 2);
     // lane = mode nu
     float wmax = -1.f;

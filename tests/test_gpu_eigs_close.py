@@ -34,8 +34,12 @@ def _check(s, grid):
 
 
 @pytest.mark.parametrize("split", [0.0, 1e-12, 1e-9, 1e-6, 1e-4])
-def test_split_degeneracies(split):
+@pytest.mark.parametrize("copies", [1, 2, 4])          # 4, 8 and 16 bands (the warp solver)
+def test_split_degeneracies(split, copies):
     s = synth.al_like_sym_system()
+    if copies > 1:                                    # every level copies-fold degenerate
+        s = dataclasses.replace(s, nw=copies * s.nw, H=np.kron(np.eye(copies), s.H),
+                                g=np.kron(np.eye(copies), s.g))
     rng = np.random.default_rng(3)
     h = rng.normal(size=(s.nw, s.nw)) + 1j * rng.normal(size=(s.nw, s.nw))
     H = s.H.copy()
