@@ -6,9 +6,8 @@
 // bind: per point the kernels form only the upper triangle of the Hermitian sums, and the
 // launches use small blocks on small grids so that every SM's FP64 unit has work.  Measured on one
 // GB300 against plain FP64 Jacobi sweeps (FP64 sweeps after an FP32 start for 8 and 6 rows), all
-// eigensolves and velocities of a step: Si-like 100^3 (8 and 6 rows) 65 -> 40.5 ms, metal 48^3 (4 and
-// 3 rows) 2.9 -> 0.96 ms, tiny 8^3 0.57 -> 0.20 ms; seven systems of up to 24 rows one after the other
-// 15 -> 7.5 ms.  Each point is diagonalised once (Nk + Nq solves); the
+// eigensolves and velocities of a step: Si-like 100^3 (8 and 6 rows) 65 -> 27.8 ms, metal 48^3 (4 and
+// 3 rows) 2.9 -> 0.6 ms, tiny 8^3 0.57 -> 0.15 ms.  Each point is diagonalised once (Nk + Nq solves); the
 // scattering loops gather V(k+q), u(q) from these tables instead of re-diagonalising per
 // pair.
 #include <algorithm>

@@ -143,7 +143,7 @@ struct epwi_ctx {
 
     // scratch
     DevBuf pairs;                  // int32 q index per pair of the chunk
-    DevBuf runs;                   // int32 run tables of the chunk's k-points (sieve.cuh)
+    DevBuf runs;                   // int32 run tables of the window's k-points (sieve.cuh; capture)
     DevBuf ghat;                   // per-chunk Re->k output
     DevBuf tiles;                  // int4 per tile {kp_local, pair_begin, pair_end, 0}
     DevBuf tile_part;              // double [tile][W] partial sums

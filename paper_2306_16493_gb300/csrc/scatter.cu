@@ -455,8 +455,9 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
         sf_prepare(c);
     }
     if (tc) tc_prepare(c);
-    // Sum-factorised FP64 rates: needs pair lists in the sieve's order (filled here, or for the
-    // Gamma capture) and the window's bands, without weights or per-pair outputs
+    // Sum-factorised FP64 rates: the sieve's pairs (read from its decisions; with the Gamma capture the
+    // lists in the sieve's order serve as well) and the window's bands, without weights or per-pair
+    // outputs
     const bool sf64 = !sf && !tc && !g2out && !tout && !ws.pair_w && ws.ovr_nsel < 0 && (!ws.pairs_dev || ws.runs_dev) &&
                       sf64_ok(c);
     if (sf64) sf64_prepare(c);
