@@ -18,57 +18,67 @@ namespace {
 constexpr int kScanBlock = 1024;
 constexpr int kScanItems = 4;
 
-__device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
+// The scans take 64-bit words or the two counts of a window (sieve.cuh).
+__device__ __forceinline__ int64_t lane_up(int64_t v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ WindowCount lane_up(WindowCount v, int o) {
+    return {__shfl_up_sync(0xffffffffu, v.kpoints, o), __shfl_up_sync(0xffffffffu, v.states, o)};
+}
+
+template <class T>
+__device__ __forceinline__ T warp_incl_scan(T v) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int64_t t = __shfl_up_sync(0xffffffffu, v, o);
+        T t = lane_up(v, o);
         if (lane >= o) v += t;
     }
     return v;
 }
 
 // Exclusive scan of v across the block (blockDim.x multiple of 32, <= 1024).
-__device__ int64_t block_excl_scan(int64_t v, int64_t *sm, int64_t &total) {
+template <class T>
+__device__ T block_excl_scan(T v, T *sm, T &total) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int64_t inc = warp_incl_scan(v);
+    T inc = warp_incl_scan(v);
     if (lane == 31) sm[wid] = inc;
     __syncthreads();
     if (wid == 0) {
-        int64_t s = lane < nw ? sm[lane] : 0;
-        int64_t si = warp_incl_scan(s);
+        T s = lane < nw ? sm[lane] : T{};
+        T si = warp_incl_scan(s);
         if (lane < nw) sm[lane] = si - s;
         if (lane == nw - 1) sm[32] = si;
     }
     __syncthreads();
-    int64_t r = inc - v + sm[wid];
+    T r = inc - v + sm[wid];
     total = sm[32];
     __syncthreads();
     return r;
 }
 
-__global__ void k_scan_blocks(const int64_t *in, int64_t n, int64_t *bsum) {
-    __shared__ int64_t sm[33];
+template <class T>
+__global__ void __launch_bounds__(kScanBlock) k_scan_blocks(const T *in, int64_t n, T *bsum) {
+    __shared__ T sm[33];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock * kScanItems + threadIdx.x * kScanItems;
-    int64_t s = 0;
+    T s{};
     for (int i = 0; i < kScanItems; ++i)
         if (base + i < n) s += in[base + i];
-    int64_t tot;
+    T tot;
     block_excl_scan(s, sm, tot);
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
-__global__ void k_scan_apply(const int64_t *in, int64_t n, const int64_t *boff, int64_t *out) {
-    __shared__ int64_t sm[33];
+template <class T>
+__global__ void __launch_bounds__(kScanBlock) k_scan_apply(const T *in, int64_t n, const T *boff, T *out) {
+    __shared__ T sm[33];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock * kScanItems + threadIdx.x * kScanItems;
-    int64_t v[kScanItems];
-    int64_t s = 0;
+    T v[kScanItems];
+    T s{};
     for (int i = 0; i < kScanItems; ++i) {
-        v[i] = base + i < n ? in[base + i] : 0;
+        v[i] = base + i < n ? in[base + i] : T{};
         s += v[i];
     }
-    int64_t tot;
-    int64_t run = block_excl_scan(s, sm, tot) + boff[blockIdx.x];
+    T tot;
+    T run = block_excl_scan(s, sm, tot) + boff[blockIdx.x];
     for (int i = 0; i < kScanItems; ++i) {
         if (base + i < n) out[base + i] = run;
         run += v[i];
@@ -77,18 +87,19 @@ __global__ void k_scan_apply(const int64_t *in, int64_t n, const int64_t *boff, 
 }
 
 // The whole scan in one block (short inputs: one launch instead of four).
-__global__ void __launch_bounds__(kScanBlock) k_scan_one(const int64_t *in, int64_t n, int64_t *out) {
-    __shared__ int64_t sm[33];
-    int64_t carry = 0;
+template <class T>
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(const T *in, int64_t n, T *out) {
+    __shared__ T sm[33];
+    T carry{};
     for (int64_t base = 0; base < n; base += kScanBlock * kScanItems) {
         const int64_t i0 = base + threadIdx.x * kScanItems;
-        int64_t v[kScanItems], s = 0;
+        T v[kScanItems], s{};
         for (int i = 0; i < kScanItems; ++i) {
-            v[i] = i0 + i < n ? in[i0 + i] : 0;
+            v[i] = i0 + i < n ? in[i0 + i] : T{};
             s += v[i];
         }
-        int64_t tot;
-        int64_t run = carry + block_excl_scan(s, sm, tot);
+        T tot;
+        T run = carry + block_excl_scan(s, sm, tot);
         for (int i = 0; i < kScanItems; ++i) {
             if (i0 + i < n) out[i0 + i] = run;
             run += v[i];
@@ -116,24 +127,21 @@ __device__ __forceinline__ bool window_kpoint(int64_t k, const int *cnt, const i
     return cnt[k] > 0 && (!rep || rep[k] == (int)k);
 }
 
-// k-points and states of each grid point, packed in one word (k-points above bit 36: a grid has
-// fewer than 2^31 points of at most 24 bands), so that one scan places both.
-constexpr int kStateBits = 36;
+// k-points and states of each grid point; one scan places both.
 __global__ void k_window_flags(int64_t nk, const int *__restrict__ cnt, const int *__restrict__ rep,
-                               int64_t *__restrict__ flag) {
+                               WindowCount *__restrict__ flag) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nk) flag[k] = window_kpoint(k, cnt, rep) ? ((int64_t)1 << kStateBits) + cnt[k] : 0;
+    if (k < nk) flag[k] = window_kpoint(k, cnt, rep) ? WindowCount{1, cnt[k]} : WindowCount{};
 }
 
 // The k-point list, first states (with the total at the end) and states of the window.
-__global__ void k_compact_kpts(int64_t nk, const int64_t *__restrict__ pos, const int *__restrict__ cnt,
+__global__ void k_compact_kpts(int64_t nk, const WindowCount *__restrict__ pos, const int *__restrict__ cnt,
                                const int *__restrict__ rep, const int *__restrict__ lo, int *__restrict__ kpts,
                                int64_t *__restrict__ kp_state, int *__restrict__ st_k, int *__restrict__ st_n) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t low = ((int64_t)1 << kStateBits) - 1;
-    if (k == 0) kp_state[pos[nk] >> kStateBits] = pos[nk] & low;
+    if (k == 0) kp_state[pos[nk].kpoints] = pos[nk].states;
     if (k >= nk || !window_kpoint(k, cnt, rep)) return;
-    const int64_t p = pos[k] >> kStateBits, s0 = pos[k] & low;
+    const int64_t p = pos[k].kpoints, s0 = pos[k].states;
     kpts[p] = (int)k;
     kp_state[p] = s0;
     for (int n = 0; n < cnt[k]; ++n) {
@@ -756,42 +764,48 @@ static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
     return true;
 }
 
-static void scan_levels(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int level, int64_t level_off) {
+template <class T>
+static void scan_levels(epwi_ctx *c, const T *in, T *out, int64_t n, int level, int64_t level_off) {
     const int64_t per = (int64_t)kScanBlock * kScanItems;
     const int64_t nb = (n + per - 1) / per;
     // up to 16 blocks' worth in one block; the block sums of longer inputs go to the context's
     // workspace, level by level (nb + 1 sums and offsets each)
     if (nb <= 16) {
-        k_scan_one<<<1, kScanBlock, 0, c->stream>>>(in, n, out);
+        k_scan_one<T><<<1, kScanBlock, 0, c->stream>>>(in, n, out);
         EPWI_CHECK_LAUNCH();
     } else {
         if (level == 0) {
             int64_t need = 0;
             for (int64_t m = nb; m > 16; m = (m + per - 1) / per) need += 2 * (m + 1);
-            c->scan_ws.ensure(sizeof(int64_t) * (need + 2 * 17 + 2));
+            c->scan_ws.ensure(sizeof(T) * (need + 2 * 17 + 2));
             level_off = 0;
         }
-        int64_t *bs = c->scan_ws.as<int64_t>() + level_off, *bo = bs + nb + 1;
-        k_scan_blocks<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bs);
+        T *bs = c->scan_ws.as<T>() + level_off, *bo = bs + nb + 1;
+        k_scan_blocks<T><<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bs);
         EPWI_CHECK_LAUNCH();
-        scan_levels(c, bs, bo, nb, level + 1, level_off + 2 * (nb + 1));
-        k_scan_apply<<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bo, out);
+        scan_levels<T>(c, bs, bo, nb, level + 1, level_off + 2 * (nb + 1));
+        k_scan_apply<T><<<(unsigned)nb, kScanBlock, 0, c->stream>>>(in, n, bo, out);
         EPWI_CHECK_LAUNCH();
     }
 }
 
-void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
-    // out has n + 1 entries; out[n] = sum
+// out has n + 1 entries; out[n] = sum
+template <class T>
+static void scan_exclusive(epwi_ctx *c, const T *in, T *out, int64_t n, T *total) {
     if (n == 0) {
-        EPWI_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), c->stream));
-        if (total) *total = 0;
+        EPWI_CUDA(cudaMemsetAsync(out, 0, sizeof(T), c->stream));
+        if (total) *total = T{};
         return;
     }
-    scan_levels(c, in, out, n, 0, 0);
+    scan_levels<T>(c, in, out, n, 0, 0);
     if (total) {
-        EPWI_CUDA(cudaMemcpyAsync(total, out + n, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+        EPWI_CUDA(cudaMemcpyAsync(total, out + n, sizeof(T), cudaMemcpyDeviceToHost, c->stream));
         EPWI_CUDA(cudaStreamSynchronize(c->stream));
     }
+}
+
+void scan_exclusive_i64(epwi_ctx *c, const int64_t *in, int64_t *out, int64_t n, int64_t *total) {
+    scan_exclusive<int64_t>(c, in, out, n, total);
 }
 
 void build_window(epwi_ctx *c, const int *rep) {
@@ -809,14 +823,14 @@ void build_window(epwi_ctx *c, const int *rep) {
 
 void window_lists(epwi_ctx *c, const int *rep) {
     const int64_t nk = c->nk;
-    c->counts.ensure(sizeof(int64_t) * (nk + 1));
-    c->scan_tmp.ensure(sizeof(int64_t) * (nk + 1));
+    c->counts.ensure(sizeof(WindowCount) * (nk + 1));
+    c->scan_tmp.ensure(sizeof(WindowCount) * (nk + 1));
     const unsigned nb = (unsigned)((nk + 255) / 256);
-    k_window_flags<<<nb, 256, 0, c->stream>>>(nk, c->win_n.as<int>(), rep, c->counts.as<int64_t>());
+    k_window_flags<<<nb, 256, 0, c->stream>>>(nk, c->win_n.as<int>(), rep, c->counts.as<WindowCount>());
     EPWI_CHECK_LAUNCH();
-    int64_t tot = 0;
-    scan_exclusive_i64(c, c->counts.as<int64_t>(), c->scan_tmp.as<int64_t>(), nk, &tot);
-    const int64_t nkp = tot >> kStateBits, nst = tot & (((int64_t)1 << kStateBits) - 1);
+    WindowCount tot;
+    scan_exclusive<WindowCount>(c, c->counts.as<WindowCount>(), c->scan_tmp.as<WindowCount>(), nk, &tot);
+    const int64_t nkp = tot.kpoints, nst = tot.states;
     c->nkp = nkp;
     c->nstates = nst;
     c->win_ncol = c->win_nk3 = 0;
@@ -825,7 +839,7 @@ void window_lists(epwi_ctx *c, const int *rep) {
     c->st_k.ensure(sizeof(int) * (nst + 1));
     c->st_n.ensure(sizeof(int) * (nst + 1));
     c->inv_tau.ensure(sizeof(double) * (nst + 1));
-    k_compact_kpts<<<nb, 256, 0, c->stream>>>(nk, c->scan_tmp.as<int64_t>(), c->win_n.as<int>(), rep, c->win_lo.as<int>(),
+    k_compact_kpts<<<nb, 256, 0, c->stream>>>(nk, c->scan_tmp.as<WindowCount>(), c->win_n.as<int>(), rep, c->win_lo.as<int>(),
                                              c->kpts.as<int>(), c->kp_state.as<int64_t>(), c->st_k.as<int>(),
                                              c->st_n.as<int>());
     EPWI_CHECK_LAUNCH();

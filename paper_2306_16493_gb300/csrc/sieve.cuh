@@ -15,6 +15,21 @@ __host__ __device__ __forceinline__ int64_t run_stride(const GridInfo &g) {
     return ((int64_t)g.n2 * g.n3 + kSieveBlock - 1) / kSieveBlock * g.n1 + 1;
 }
 
+// k-points and states of a window, counted together.  A grid has up to 2^31 - 1 points of up to 24
+// bands: 31 and 36 bits, more than one 64-bit word holds.
+struct WindowCount {
+    int64_t kpoints, states;
+    __host__ __device__ WindowCount &operator+=(const WindowCount &o) {
+        kpoints += o.kpoints;
+        states += o.states;
+        return *this;
+    }
+};
+__host__ __device__ inline WindowCount operator+(WindowCount a, const WindowCount &b) { return a += b; }
+__host__ __device__ inline WindowCount operator-(const WindowCount &a, const WindowCount &b) {
+    return {a.kpoints - b.kpoints, a.states - b.states};
+}
+
 struct SieveArgs {
     GridInfo g;
     int W, Nm;
