@@ -291,7 +291,11 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
                 out.assign((size_t)Dc * Dc * Dc * ne, make_double2(0, 0));
                 for (int k = 0; k < n; ++k) {
                     const size_t cf = ((size_t)(R[3 * k] + r) * Dc + (R[3 * k + 1] + r)) * Dc + (R[3 * k + 2] + r);
-                    for (size_t e = 0; e < ne; ++e) out[cf * ne + e] = value(k, e);
+                    for (size_t e = 0; e < ne; ++e) {        // += : a set can list a vector twice
+                        const double2 v = value(k, e);
+                        out[cf * ne + e].x += v.x;
+                        out[cf * ne + e].y += v.y;
+                    }
                 }
                 rout = r;
             };
