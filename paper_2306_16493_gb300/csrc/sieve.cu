@@ -7,6 +7,7 @@
 // Each candidate is first evaluated in FP32 with a rigorous bound delta on the rounding
 // error; only candidates whose nearest |x| lies within delta of c eta are re-evaluated in
 // FP64 in the oracle's rounding order, so every decision equals the FP64 one.
+#include <algorithm>
 #include <cstdlib>
 
 #include "epwi_internal.cuh"
@@ -709,7 +710,10 @@ SieveArgs make_sieve_args(epwi_ctx *c) {
     a.hwmax32 = c->hwmax32.as<float>();
     a.omega_min = c->opt.omega_min_eV;
     a.ceta = c->opt.sieve_c * c->eta;
-    a.ceta32 = (float)a.ceta;
+    // A cut-off beyond FP32 (an infinite sieve_c keeps every pair with a mode) stays below the 3e38 that
+    // stands for "no mode" and for points outside the plane in k_sieve_count_cols; every energy
+    // difference is far below both.
+    a.ceta32 = (float)std::min(a.ceta, 1e30);
     // FP32 rounding of |e| <= E and of the two operations is < 2^-24 (3E + |w| + |x|) < 4e-7 E'
     a.delta32 = (float)(1e-6 + 4e-7 * (2.0 * c->eabs_max + 1.0));
     a.lim_extra = (float)(a.ceta + a.delta32 + 1e-5);
