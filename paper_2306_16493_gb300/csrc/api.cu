@@ -318,14 +318,17 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
             c->gcube_ready = false;
             c->gcube32.release();
             c->h_rp_cube.clear();
+            c->h_rp_next.clear();
             c->rp_twice = false;
             if (r <= 6) {
                 const int Dc = 2 * r + 1;
                 c->h_rp_cube.assign((size_t)Dc * Dc * Dc, -1);
+                c->h_rp_next.assign(nRp, -1);
                 for (int k = 0; k < nRp; ++k) {
                     int &at = c->h_rp_cube[((size_t)(s->Rp[3 * k] + r) * Dc + (s->Rp[3 * k + 1] + r)) * Dc +
                                            (s->Rp[3 * k + 2] + r)];
                     c->rp_twice |= at >= 0;
+                    c->h_rp_next[k] = at;
                     at = k;
                 }
             }
@@ -366,7 +369,12 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
             }
         });
         double gbound = 0;
-        for (double v : rp_bound) gbound = std::max(gbound, v);
+        for (int rp = 0; rp < nRp; ++rp) {        // (the entries of one vector add up)
+            double v = rp_bound[rp];
+            if (c->rp_twice)
+                for (int x = c->h_rp_next[rp]; x >= 0; x = c->h_rp_next[x]) v += rp_bound[x];
+            gbound = std::max(gbound, v);
+        }
         c->tc_scale_exp = gbound > 0 ? 14 - (int)std::ceil(std::log2(gbound)) : 0;
         c->tc_ptab_key = -1;
         c->tc_arows_key = -1;

@@ -166,6 +166,7 @@ struct epwi_ctx {
     DevBuf tc_arows;               // gathered-A mode: split phase rows of every grid point
     int sf_r = 0;                  // fp32 mode: half-width of the bounding cube of R_p
     std::vector<int> h_rp_cube;    // fp32 mode: R_p index of each bounding-cube point, -1 if absent
+    std::vector<int> h_rp_next;    // next R_p index with the same vector, -1 if there is none
     DevBuf gsf32;                  // fp32 mode: g' [Re][cube forms][Nm][W][W] (+-R recombined)
     bool sf_g_ready = false;       // gsf32 built for the current system
     DevBuf gsf64;                  // FP64 mode: the same in FP64
@@ -262,6 +263,15 @@ inline void upload_ints(epwi_ctx *c, DevBuf &b, const std::vector<int> &h) {
     b.ensure(sizeof(int) * (h.size() + 1));
     if (!h.empty())
         EPWI_CUDA(cudaMemcpyAsync(b.p, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, c->stream));
+}
+
+// R_p indices of the bounding cube's points followed by the chain of equal vectors (h_rp_next): entry rp
+// of a point is followed by entry map[points + rp].
+inline void upload_rp_map(epwi_ctx *c, DevBuf &b) {
+    std::vector<int> m(c->h_rp_cube);
+    m.insert(m.end(), c->h_rp_next.begin(), c->h_rp_next.end());
+    upload_ints(c, b, m);
+    EPWI_CUDA(cudaStreamSynchronize(c->stream));   // m is freed on return
 }
 
 // ----------------------------------------------------------------------------- complex

@@ -167,8 +167,8 @@ struct SfStore {
 };
 
 // g'(Re, f1 f2 f3) = (T x T x T) g(Re, cube): along each axis, form 0 is R = 0, form 2R-1 is
-// v[R] + v[-R] and form 2R is i (v[R] - v[-R]).  cube[c] is the index of the R_p vector at
-// cube point c, or -1 (zero weight).  One thread per output element; FP64 sums, output in FP32
+// v[R] + v[-R] and form 2R is i (v[R] - v[-R]).  cube: upload_rp_map (points without a vector have
+// zero weight).  One thread per output element; FP64 sums, output in FP32
 // or FP64.
 template <class C2>
 __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, const int *__restrict__ cube,
@@ -196,10 +196,11 @@ __global__ void k_sf_transform(int64_t n, int nRp, int Dc, int rc, int rowlen, c
         for (int y = 0; y < nt[1]; ++y)
             for (int z = 0; z < nt[2]; ++z) {
                 const int c = ((Rv[0][x] + rc) * Dc + (Rv[1][y] + rc)) * Dc + (Rv[2][z] + rc);
-                const int rp = cube[c];
-                if (rp < 0) continue;
-                const size_t gi = ((size_t)re * nRp + rp) * rowlen + e;
-                const double2 v = g64 ? g64[gi] : make_double2(g32[gi].x, g32[gi].y);
+                double2 v = make_double2(0, 0);
+                for (int rp = cube[c]; rp >= 0; rp = cube[D3 + rp]) {
+                    const size_t gi = ((size_t)re * nRp + rp) * rowlen + e;
+                    v = cadd(v, g64 ? g64[gi] : make_double2(g32[gi].x, g32[gi].y));
+                }
                 const int p = (pw[0][x] + pw[1][y] + pw[2][z]) & 3;     // s += i^p v
                 const double px = p & 1 ? v.y : v.x, py = p & 1 ? v.x : v.y;
                 s.x += p == 1 || p == 2 ? -px : px;
@@ -779,7 +780,7 @@ static void build_gsf(epwi_ctx *c, DevBuf &out) {
     const int Dc = 2 * c->sf_r + 1, rowlen = c->nm * c->nw * c->nw;
     const int64_t n = (int64_t)c->nRe * Dc * Dc * Dc * rowlen;
     DevBuf cube;
-    upload_ints(c, cube, c->h_rp_cube);
+    upload_rp_map(c, cube);
     out.ensure(sizeof(C2) * n);
     k_sf_transform<C2><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
         n, c->nRp, Dc, c->sf_r, rowlen, cube.as<int>(), c->keep_g64 ? c->gw64.as<double2>() : nullptr,

@@ -1187,7 +1187,7 @@ void tc_restage(epwi_ctx *c, const RestageArgs &ra) {
 }
 
 // A non-cube R_p set embedded in its bounding cube: gcube32[Re][cube point][mu][i][j] = the
-// weighted g of the R_p vector at that point, or 0.
+// weighted g of the R_p vector at that point, or 0 (cube: upload_rp_map).
 __global__ void k_cube_embed(int64_t n, int nRp, int D3, int rowlen, const int *__restrict__ cube,
                              const float2 *__restrict__ g32, float2 *__restrict__ out) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1196,8 +1196,12 @@ __global__ void k_cube_embed(int64_t n, int nRp, int D3, int rowlen, const int *
     const int64_t t = idx / rowlen;
     const int cf = (int)(t % D3);
     const int64_t re = t / D3;
-    const int rp = cube[cf];
-    out[idx] = rp < 0 ? make_float2(0.f, 0.f) : g32[((size_t)re * nRp + rp) * rowlen + e];
+    float2 v = make_float2(0.f, 0.f);
+    for (int rp = cube[cf]; rp >= 0; rp = cube[D3 + rp]) {
+        const float2 x = g32[((size_t)re * nRp + rp) * rowlen + e];
+        v = make_float2(v.x + x.x, v.y + x.y);
+    }
+    out[idx] = v;
 }
 
 // The split-precision view of the R_p set (tc_rp_r, tc_rp_count): for a set that is not a full
@@ -1210,7 +1214,7 @@ void tc_prepare(epwi_ctx *c) {
     const int D = 2 * c->sf_r + 1, D3 = D * D * D, rowlen = c->nm * c->nw * c->nw;
     const int64_t n = (int64_t)c->nRe * D3 * rowlen;
     DevBuf cube;
-    upload_ints(c, cube, c->h_rp_cube);
+    upload_rp_map(c, cube);
     c->gcube32.ensure(sizeof(float2) * n);
     k_cube_embed<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, c->nRp, D3, rowlen, cube.as<int>(),
                                                                     c->gw32.as<float2>(), c->gcube32.as<float2>());

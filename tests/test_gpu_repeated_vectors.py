@@ -41,3 +41,23 @@ def test_bands_and_phonons(name, grid, copies):
     # summed over the bands: that is the trace of dH/dk, whatever the basis of degenerate bands
     for x, y in zip(*out):
         assert np.abs(x - y).max() <= 1e-12 * np.abs(x).max()
+
+
+# nw = 4, 3 modes, R_p within |n| <= 2; twice the bounds of the modes' parity with the oracle
+@pytest.mark.parametrize("precision,tol", [("fp64", 2e-10), ("fp32", 2e-5), ("fp16x3", 2e-4), ("bf16x3", 2e-4),
+                                           ("tf32x3", 2e-4)])
+@pytest.mark.parametrize("copies", [2, 8])
+def test_rates(precision, tol, copies):
+    s = synth.al_like_system()
+    out = []
+    for x in (s, repeated(s, copies)):
+        ctx = epwi.Context(precision=precision)
+        ctx.setup(x)
+        ctx.eigs((10, 9, 8))
+        mu = 0.5 * sum(ctx.band_range())
+        ctx.scatter_rates(300.0, mu, 0.05, mu - 0.4, mu + 0.4)
+        out.append(ctx.rates())
+        ctx.close()
+    (k, n, r), (k2, n2, r2) = out
+    assert np.array_equal(k, k2) and np.array_equal(n, n2)
+    assert np.abs(r2 - r).max() <= tol * r.max()
