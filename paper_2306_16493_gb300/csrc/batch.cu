@@ -826,8 +826,7 @@ void fill_bsys(epwi_batch *b, int s, int Mt, int KC, BSys &d) {
 int persistent_grid(epwi_batch *b, size_t smem) {
     int nsm = 0, per = 0;
     EPWI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
-    EPWI_CUDA(cudaFuncSetAttribute(k_batch_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)std::max<size_t>(smem, 1)));
+    allow_smem(k_batch_scatter);
     EPWI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_scatter, kBT, smem));
     EPWI_REQUIRE(per >= 1, EPWI_EUNSUPPORTED, "persistent kernel does not fit on an SM");
     return nsm * per;

@@ -11,8 +11,6 @@
 // scattering loops gather V(k+q), u(q) from these tables instead of re-diagonalising per
 // pair.
 #include <algorithm>
-#include <utility>
-#include <vector>
 
 #include "epwi_internal.cuh"
 #include "jacobi.cuh"
@@ -564,26 +562,6 @@ void launch_phase_tables(epwi_ctx *c) {
     EPWI_CHECK_LAUNCH();
 }
 
-// Raises a kernel's dynamic shared-memory limit the first time a larger size is needed
-// (the first launch of each size happens outside any stream capture).  The limit set so far is
-// kept per kernel: kernels of one signature share the template instance.
-template <class K>
-void set_smem_once(K kern, size_t bytes) {
-    static std::vector<std::pair<const void *, size_t>> set;
-    const void *key = reinterpret_cast<const void *>(kern);
-    size_t *have = nullptr;
-    for (auto &e : set)
-        if (e.first == key) have = &e.second;
-    if (!have) {
-        set.emplace_back(key, size_t(48 * 1024));
-        have = &set.back().second;
-    }
-    if (bytes > *have) {
-        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-        *have = bytes;
-    }
-}
-
 // Threads per block of the thread-per-point kernels: an SM's FP64 unit takes 16 clocks per warp
 // instruction, so a grid's points are spread over all SMs first (32-thread blocks up to 128 points
 // per SM, 64 up to 256).
@@ -726,10 +704,10 @@ void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t joi
     } else {
         const size_t sm = warp_scratch_bytes(W);
         if (fac_el) {
-            set_smem_once(k_eig_el_warp<true>, sm);
+            allow_smem(k_eig_el_warp<true>);
             k_eig_el_warp<true><<<nbw, 32 * kWarpsPerBlock, sm, c->stream>>>(EL_ARGS, fe, lat);
         } else {
-            set_smem_once(k_eig_el_warp<false>, sm);
+            allow_smem(k_eig_el_warp<false>);
             k_eig_el_warp<false><<<nbw, 32 * kWarpsPerBlock, sm, c->stream>>>(EL_ARGS, fe, lat);
         }
     }
@@ -755,10 +733,10 @@ void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t joi
     } else {
         const size_t sm = warp_scratch_bytes(Nm);
         if (fac_ph) {
-            set_smem_once(k_eig_ph_warp<true>, sm);
+            allow_smem(k_eig_ph_warp<true>);
             k_eig_ph_warp<true><<<nbhw, 32 * kWarpsPerBlock, sm, ph>>>(PH_ARGS, fp);
         } else {
-            set_smem_once(k_eig_ph_warp<false>, sm);
+            allow_smem(k_eig_ph_warp<false>);
             k_eig_ph_warp<false><<<nbhw, 32 * kWarpsPerBlock, sm, ph>>>(PH_ARGS, fp);
         }
     }

@@ -50,6 +50,18 @@ extern int64_t g_epwi_launches;
         EPWI_CUDA(cudaGetLastError());                                                     \
     } while (0)
 
+// Lets a kernel take all of an SM's shared memory beside its static part (227 KB a CTA).  The limit
+// belongs to the kernel, not to a call: one that a call set to its own size could be lowered by another
+// thread's before the launch, so every call asks for the same.
+template <class K>
+inline void allow_smem(K kern) {
+    cudaFuncAttributes fa;
+    EPWI_CUDA(cudaFuncGetAttributes(&fa, kern));
+    const int most = 227 * 1024 - (int)fa.sharedSizeBytes;
+    if (fa.maxDynamicSharedSizeBytes < most)
+        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+}
+
 #define EPWI_REQUIRE(cond, st, m)                                                          \
     do {                                                                                   \
         if (!(cond)) throw EpwiError{st, m};                                               \

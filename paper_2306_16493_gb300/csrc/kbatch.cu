@@ -201,7 +201,7 @@ void launch_restage(const KbArgs &a, cudaStream_t st) {
     constexpr int KG = 8;
     const size_t sm = sizeof(double2) * KG * a.nRp;
     if (sm > 48 * 1024)
-        EPWI_CUDA(cudaFuncSetAttribute(k_kb_restage<NMT, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(k_kb_restage<NMT, KG>);
     dim3 grid((unsigned)((a.nRe * a.W * a.W + 127) / 128), (unsigned)((a.nq + KG - 1) / KG));
     k_kb_restage<NMT, KG><<<grid, 128, sm, st>>>(a);
     EPWI_CHECK_LAUNCH();

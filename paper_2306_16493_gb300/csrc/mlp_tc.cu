@@ -251,7 +251,7 @@ size_t infer_smem() {
 template <bool PROP>
 void launch_infer(epwi_ctx *c, const MlpTcArgs &a) {
     const size_t sm = infer_smem();
-    EPWI_CUDA(cudaFuncSetAttribute(k_mlp_infer_tc<PROP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem(k_mlp_infer_tc<PROP>);
     int nsm = 0;
     EPWI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
     // one CTA per SM; few tiles spread over the SMs first

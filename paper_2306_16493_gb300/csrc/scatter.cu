@@ -214,9 +214,7 @@ void launch_fp64_pair(const RestageArgs &ra, const ScatterArgs &sa, int64_t ntil
     constexpr int KG = WT ? (WT >= 16 ? 1 : (WT >= 8 ? 4 : 8)) : 1;
     dim3 grid((ra.nrow + 127) / 128, (unsigned)((ra.nkp + KG - 1) / KG));
     const size_t sm = sizeof(double2) * KG * ra.nRe;
-    if (sm > 48 * 1024)
-        EPWI_CUDA(cudaFuncSetAttribute(k_restage_fp64<WT, KG>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) allow_smem(k_restage_fp64<WT, KG>);
     k_restage_fp64<WT, KG><<<grid, 128, sm, st>>>(ra);
     EPWI_CHECK_LAUNCH();
     (void)sa;

@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(kSfThreads, (W <= 4 ? 3 : 2)) k_scatter_sf(SfA
 
 template <int W, int NM, int RC, bool GAM>
 void launch_sf_t(epwi_ctx *c, const SfArgs &a, int nitems, size_t sm) {
-    EPWI_CUDA(cudaFuncSetAttribute(k_scatter_sf<W, NM, RC, GAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem(k_scatter_sf<W, NM, RC, GAM>);
     EPWI_CUDA(cudaFuncSetAttribute(k_scatter_sf<W, NM, RC, GAM>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     if (nitems > 0) {
         k_scatter_sf<W, NM, RC, GAM><<<(unsigned)nitems, kSfThreads, sm, c->stream>>>(a);
@@ -832,7 +832,7 @@ void sf_restage(epwi_ctx *c, const RestageArgs &ra_in) {
     auto go = [&](auto kern, int KG) {
         dim3 grid((ra.nrow + 127) / 128, (unsigned)((ra.nkp + KG - 1) / KG));
         const size_t sm = sizeof(float2) * KG * ra.nRe;
-        if (sm > 48 * 1024) EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        if (sm > 48 * 1024) allow_smem(kern);
         kern<<<grid, 128, sm, c->stream>>>(ra, out);
         EPWI_CHECK_LAUNCH();
     };

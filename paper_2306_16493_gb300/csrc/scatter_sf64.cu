@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kSfThreads) k_scatter_sf64(Sf64Args a) {
 template <int W, int NM, int RC>
 void launch(epwi_ctx *c, const Sf64Args &a, int64_t nstates, size_t sm) {
     auto go = [&](auto kern) {
-        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(kern);
         kern<<<(unsigned)nstates, kSfThreads, sm, c->stream>>>(a);
         EPWI_CHECK_LAUNCH();
     };

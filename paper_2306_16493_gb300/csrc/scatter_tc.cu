@@ -1056,8 +1056,8 @@ void launch_tc(epwi_ctx *c, const ScatterArgs &sa, int64_t ntiles) {
     EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     // keep (resident CTAs per SM) x (TMEM columns) <= 512 so that tcgen05.alloc never waits
     int per_sm = 0;
+    allow_smem(kern);
     for (;;) {
-        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         EPWI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 288, smem));
         EPWI_REQUIRE(per_sm >= 1, EPWI_EUNSUPPORTED, "tensor-core kernel does not fit on an SM");
         if ((uint32_t)per_sm * cols <= 512) break;
@@ -1162,8 +1162,7 @@ void restage_tc_launch(epwi_ctx *c, const RestageArgs &ra) {
     dim3 grid((ra.nrow + 127) / 128, (unsigned)((ra.nkp + KG - 1) / KG));
     const size_t sm = sizeof(float2) * KG * ra.nRe;
     auto kern = k_restage_tc<Op, W, NM, KG>;
-    if (sm > 48 * 1024)
-        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) allow_smem(kern);
     kern<<<grid, 128, sm, c->stream>>>(ra, store);
     EPWI_CHECK_LAUNCH();
 }

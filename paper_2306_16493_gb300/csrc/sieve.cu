@@ -756,7 +756,7 @@ static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
     EPWI_CUDA(cudaMemsetAsync(c->counts.p, 0, sizeof(int64_t) * c->nkp, c->stream));
     auto go = [&](auto kern, int TB) {
         const size_t sm = sieve_cols_smem(N1, TB);
-        EPWI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_smem(kern);
         const dim3 grid((unsigned)cs.ncol, (unsigned)((nplane + kSieveBlock - 1) / kSieveBlock * (kSieveBlock / TB)));
         kern<<<grid, TB, sm, c->stream>>>(a, cs, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(),
                                           c->counts.as<unsigned long long>(), mk, c->mask_words);
