@@ -230,16 +230,6 @@ bool kstage_pays(const epwi_ctx *c, int64_t nkp, int64_t nrow, bool fp64) {
     return 2.0 * fac < direct && macs > (fp64 ? 1e7 : 2e8);
 }
 
-int64_t kstage_rows(const epwi_ctx *c, const ColumnSet &cs, int64_t nrow, int W, size_t elem) {
-    const int64_t D = 2 * c->fac_re_r + 1;
-    const double per_row = (double)(D * D * cs.nk3 + D * cs.ncol) * W * elem;
-    const int64_t fit = (int64_t)((double)(int64_t(1) << 30) / per_row);
-    if (fit >= nrow) return nrow;
-    const int64_t blocks = (nrow + std::max<int64_t>(fit, kKsThreads) - 1) / std::max<int64_t>(fit, kKsThreads);
-    const int64_t rows = (nrow + blocks - 1) / blocks;            // equal blocks, whole CTAs of rows
-    return (rows + kKsThreads - 1) / kKsThreads * kKsThreads;
-}
-
 template <class C2>
 void kstage_axes32(epwi_ctx *c, const ColumnSet &cs, const C2 *g, const C2 *ph, int64_t nrow, int W, int row0, int nrows,
                    C2 *T1, C2 *T2) {

@@ -31,6 +31,19 @@ ColumnSet build_columns(epwi_ctx *c, const int *kpts, int64_t nkp);
 // Whether the factorised sum is the faster one for a work set of nkp k-points of the current grid.
 bool kstage_pays(const epwi_ctx *c, int64_t nkp, int64_t nrow, bool fp64);
 
+// Rows per block so that the workspaces T1 [D D][nk3] and T2 [D][ncol] (times rows times W) stay within
+// 1 GiB.  Fewer than one CTA's rows leave lanes idle, so a block has at least that many up to 4 GiB; beyond (wide
+// planes with hundreds of thousands of columns) it has what 4 GiB hold.
+inline int64_t ks_block_rows(int64_t D, int64_t nk3, int64_t ncol, int64_t nrow, int W, size_t elem, int cta) {
+    const double per_row = ((double)D * D * nk3 + (double)D * ncol) * W * elem;
+    const int64_t fit = (int64_t)((double)(int64_t(1) << 30) / per_row), most = (int64_t)((double)(int64_t(1) << 32) / per_row);
+    if (fit >= nrow) return nrow;
+    const int64_t cap = fit >= cta ? fit : most >= cta ? cta : most > 1 ? most : 1;
+    const int64_t blocks = (nrow + cap - 1) / cap, rows = (nrow + blocks - 1) / blocks;      // equal blocks,
+    const int64_t whole = cap >= cta ? (rows + cta - 1) / cta * cta : rows;                 // whole CTAs of rows
+    return whole < nrow ? whole : nrow;
+}
+
 constexpr int kKsThreads = 128;    // rows per block of the last stage
 constexpr int kKsBatch = 16;       // k-points staged at once
 
@@ -126,15 +139,12 @@ template <class C2>
 void kstage_axes32(epwi_ctx *c, const ColumnSet &cs, const C2 *g, const C2 *ph, int64_t nrow, int W, int row0,
                    int nrows, C2 *T1, C2 *T2);
 
-// Rows per block so that T1 and T2 stay within the workspace budget.
-int64_t kstage_rows(const epwi_ctx *c, const ColumnSet &cs, int64_t nrow, int W, size_t elem);
-
 template <class C2, class Epi>
 void kstage_run(epwi_ctx *c, const RestageArgs &ra, const C2 *g, const C2 *ph, const C2 *V, const Epi &epi) {
     const ColumnSet cs = build_columns(c, ra.kpts, ra.nkp);
     if (cs.ncol == 0) return;
     const int W = ra.W, D = 2 * c->fac_re_r + 1;
-    const int64_t rows = kstage_rows(c, cs, ra.nrow, W, sizeof(C2));
+    const int64_t rows = ks_block_rows(D, cs.nk3, cs.ncol, ra.nrow, W, sizeof(C2), kKsThreads);
     const int64_t n1 = (int64_t)D * D * cs.nk3 * rows * W, n2 = (int64_t)D * cs.ncol * rows * W;
     c->ks_T.ensure(sizeof(C2) * (n1 + n2));
     KStageArgs<C2> a;
