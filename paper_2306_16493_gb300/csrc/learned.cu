@@ -653,11 +653,9 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
                 logit.ensure(sizeof(float) * nsc * ncell);
                 cdf.ensure(sizeof(double) * nsc * ncell);
                 tot.ensure(sizeof(double) * (nsc + 1));
-                const int64_t per_state = ncell * c->nm, rows = nsc * per_state;
-                // whole states per launch, at most 2^28 rows (1 GiB of outputs)
-                const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(nsc, (int64_t(1) << 28) / per_state));
-                EPWI_REQUIRE(per_state < (int64_t(1) << 31), EPWI_EUNSUPPORTED, "too many cells and modes");
-                yb.ensure(sizeof(float) * batch * per_state);
+                const int64_t rows = nsc * ncell * c->nm;
+                const PropBlock blk = prop_block(nsc, ncell, c->nm);
+                yb.ensure(sizeof(float) * blk.states * blk.cells * c->nm);
                 fs.ensure(sizeof(float) * 5 * nsc);
                 tab.ensure(sizeof(float) * (c1 + c2 + c3 + c->nm));
                 k_prop_states<<<(unsigned)((nsc + 127) / 128), 128, 0, st>>>(nsc, g, c->nw, c->nm, s0, c->st_k.as<int>(),
@@ -669,19 +667,21 @@ void run_is(epwi_ctx *c, double T, double mu, double eta, double emin, double em
                 EPWI_CHECK_LAUNCH();
                 PropRows pr;
                 pr.Nm = c->nm;
-                pr.ncell = (int)ncell;
                 pr.c1 = c1;
                 pr.c2 = c2;
                 pr.c3 = c3;
                 pr.tab = tab.as<float>();
-                for (int64_t b0 = 0; b0 < nsc; b0 += batch) {
-                    const int64_t nb = std::min(batch, nsc - b0), ng = nb * ncell;
-                    pr.state = fs.as<float>() + 5 * b0;
-                    mlp_forward_fast(c, nb * per_state, nullptr, yb.as<float>(), &pr);
-                    k_prop_lse<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(
-                        ng, c->nm, (float)c->mlp->out_scale, yb.as<float>(), logit.as<float>() + b0 * ncell);
-                    EPWI_CHECK_LAUNCH();
-                }
+                for (int64_t b0 = 0; b0 < nsc; b0 += blk.states)
+                    for (int64_t x0 = 0; x0 < ncell; x0 += blk.cells) {
+                        const int64_t nx = std::min(blk.cells, ncell - x0), ng = std::min(blk.states, nsc - b0) * nx;
+                        pr.state = fs.as<float>() + 5 * b0;
+                        pr.cell0 = (int)x0;
+                        pr.ncell = (int)nx;
+                        mlp_forward_fast(c, ng * c->nm, nullptr, yb.as<float>(), &pr);
+                        k_prop_lse<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(
+                            ng, c->nm, (float)c->mlp->out_scale, yb.as<float>(), logit.as<float>() + b0 * ncell + x0);
+                        EPWI_CHECK_LAUNCH();
+                    }
                 flops += 2.0 * (double)rows * (kIn * kHid + 2.0 * kHid * kHid + kHid);
                 k_state_cdf<<<(unsigned)nsc, 1024, 0, st>>>(ncell, logit.as<float>(), cdf.as<double>(),
                                                            tot.as<double>());

@@ -70,10 +70,22 @@ double mlp_dataset_loss(epwi_ctx *c);
 void mlp_train_graph(epwi_ctx *c, const std::vector<StepParams> &steps, int64_t B);
 // Rows (state, cell, mode) of the proposal, mode fastest: inputs put together in the kernel.
 struct PropRows {
-    int Nm = 1, ncell = 1, c1 = 1, c2 = 1, c3 = 1;   // modes, cells, cells per axis
+    int Nm = 1, c1 = 1, c2 = 1, c3 = 1;   // modes, cells per axis
+    int cell0 = 0, ncell = 1;         // cells of the launch
     const float *state = nullptr;     // [state][5]: k coordinates, energy, band inputs
     const float *tab = nullptr;       // [c1 + c2 + c3 + Nm]: q coordinate of each cell index, mode input
 };
+
+// States and cells of one proposal launch: whole states of at most 2^28 rows (1 GiB of outputs), or
+// part of the cells of one state that has more.
+struct PropBlock {
+    int64_t states, cells;
+};
+inline PropBlock prop_block(int64_t nstates, int64_t ncell, int Nm) {
+    const int64_t most = int64_t(1) << 28, per_state = ncell * Nm;
+    if (per_state > most) return {1, most / Nm};
+    return {nstates < most / per_state ? nstates : most / per_state, ncell};
+}
 
 // mlp_tc.cu: the same forward pass on the tensor cores (BF16 activations between layers)
 void mlp_forward_tc(epwi_ctx *c, int64_t n, const float *X, float *y, int *err_dev);

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kRows * kGroups, 1) k_mlp_infer_tc(MlpTcArgs a
         if constexpr (PROP) {
             const uint32_t r = (uint32_t)min(row, a.n - 1);          // n < 2^31
             const uint32_t sc = r / (uint32_t)a.pr.Nm, nu = r - sc * a.pr.Nm;
-            const uint32_t st = sc / (uint32_t)a.pr.ncell, cell = sc - st * a.pr.ncell;
+            const uint32_t st = sc / (uint32_t)a.pr.ncell, cell = a.pr.cell0 + (sc - st * a.pr.ncell);
             const uint32_t c12 = cell / (uint32_t)a.pr.c3, c3 = cell - c12 * a.pr.c3;
             const uint32_t c1 = c12 / (uint32_t)a.pr.c2, c2 = c12 - c1 * a.pr.c2;
             const float *fs = a.pr.state + (size_t)st * 5, *ft = a.pr.tab;
