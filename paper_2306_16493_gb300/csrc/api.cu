@@ -221,6 +221,7 @@ epwi_status epwi_setup(epwi_ctx *c, const epwi_system *s) {
         EPWI_REQUIRE(asr <= 1e-8 * std::max(pmax, 1e-300), EPWI_EINVAL, "acoustic sum rule violated");
 
         c->have_sys = c->have_eigs = c->have_rates = c->have_sigma = false;
+        c->give_back(epwi_ctx::kAllKept);
         c->nat = s->nat;
         c->nw = W;
         c->nm = Nm;
@@ -408,6 +409,7 @@ epwi_status epwi_eigs(epwi_ctx *c, const int32_t kgrid[3], const int32_t qgrid[3
         c->tc_ptab_key = -1;
         c->tc_arows_key = -1;
         c->seg_ready = false;
+        if (!std::equal(kgrid, kgrid + 3, c->ng)) c->give_back(epwi_ctx::kAllKept);
         for (int a = 0; a < 3; ++a) c->ng[a] = kgrid[a];
         c->nk = nk;
         c->L = (int)L;
@@ -630,6 +632,7 @@ epwi_status epwi_scatter_rates(epwi_ctx *c, double T, double mu, double eta, dou
         EPWI_REQUIRE(c->opt.ordering == 0 || c->opt.ordering == 1, EPWI_EINVAL, "ordering must be 0 or 1");
         EPWI_REQUIRE(c->opt.ordering == 0 || c->opt.precision == EPWI_FP64, EPWI_EUNSUPPORTED,
                      "the k-batch ordering is FP64 only");
+        c->give_back(epwi_ctx::kDraws | epwi_ctx::kCapture);
         const bool sym = !c->sym_ops.empty();
         WorkSet ws = begin_rates(c, T, mu, eta, emin, emax, sym);
         if (c->opt.ordering == 1) process_kbatch(c);
@@ -658,6 +661,7 @@ epwi_status epwi_ibte(epwi_ctx *c, double T, double mu, double eta, double emin,
                      "need max_iter >= 0 and a finite tol >= 0");
         EPWI_REQUIRE(c->sym_ops.empty(), EPWI_EUNSUPPORTED,
                      "the iterative BTE couples every k-point: clear the symmetry operations first");
+        c->give_back(epwi_ctx::kDraws);
         cudaEvent_t e0, e1;
         EPWI_CUDA(cudaEventCreate(&e0));
         EPWI_CUDA(cudaEventCreate(&e1));
@@ -926,6 +930,7 @@ epwi_status epwi_mlp_train(epwi_ctx *c, double T, double mu, double eta, double 
         EPWI_REQUIRE(o.epochs >= 0 && o.batch >= 1 && o.batch <= mlp::kMaxBatch && o.lr > 0 &&
                          o.background >= 0 && o.floor_rel > 0,
                      EPWI_EINVAL, "bad training options");
+        c->give_back(epwi_ctx::kAllKept);
         mlp_train(c, T, mu, eta, emin, emax, o, final_loss);
     });
 }
@@ -1059,6 +1064,7 @@ epwi_status epwi_scatter_rates_is(epwi_ctx *c, double T, double mu, double eta, 
                              c->ng[2] % stride == 0,
                          EPWI_EINVAL, "cell_stride must divide every grid dimension");
         }
+        c->give_back(epwi_ctx::kCapture | epwi_ctx::kChunk);
         run_is(c, T, mu, eta, emin, emax, S, alpha, stride, proposal, seed);
         if (n_states) *n_states = c->nstates;
         if (n_pairs) *n_pairs = c->npairs;

@@ -246,6 +246,20 @@ struct epwi_ctx {
     epwi_ibte_stats ib_stats{};
 
     ~epwi_ctx() {
+    // Workspaces that one kind of call keeps for its next one: the draws of the importance sampling (up to
+    // 4 GiB), the pair lists of the iterative BTE's capture (up to 4 GiB and their run tables) and the decisions
+    // of a chunk of k-points (up to 2 GiB).  A call of another kind, another grid or another system
+    // gives them back: it may need the memory itself.
+    enum { kDraws = 1, kCapture = 2, kChunk = 4, kAllKept = 7 };
+    void give_back(int which) {
+        if (which & kDraws)
+            for (DevBuf &b : is_ws) b.release();
+        if (which & kCapture)
+            for (DevBuf *b : {&ib_pairs, &ib_goff, &runs}) b->release();
+        if (which & kChunk)
+            for (DevBuf *b : {&chunk_mask, &chunk_counts}) b->release();
+    }
+
         DevBuf *all[] = {&Re, &Rp, &Rcart, &Hw, &Phiw, &mode_mass, &gw64, &gw32, &ph64, &ph32,
                          &eps, &eps32, &V, &V32, &vel, &hw, &hwmax32, &hw32, &u, &u32, &eig_flag,
                          &kpts, &win_lo, &win_n, &kp_state, &kp_pairs, &inv_tau, &st_k,
