@@ -347,10 +347,14 @@ void ibte_prepare(epwi_ctx *c, WorkSet &ws) {
     const int64_t nkp = c->nkp, npairs = c->npairs;
     const bool fp64 = c->opt.precision == EPWI_FP64;
     c->ib_pairs.ensure(sizeof(int) * (npairs + 1));
-    const int64_t rstride = run_stride(make_grid_info(c));
-    c->runs.ensure(sizeof(int) * (nkp * rstride + 1));
-    sieve_fill_chunk(c, 0, nkp, c->ib_pairs.as<int>(), c->runs.as<int>());
-    ws.runs_dev = c->runs.as<int>();
+    // the sum-factorised kernels find a pair's place in the list by the runs' first pairs
+    int *runs = nullptr;
+    if (c->opt.precision == EPWI_FP32 || (fp64 && sf64_ok(c))) {
+        c->runs.ensure(sizeof(int) * (nkp * run_stride(make_grid_info(c)) + 1));
+        runs = c->runs.as<int>();
+    }
+    sieve_fill_chunk(c, 0, nkp, c->ib_pairs.as<int>(), runs);
+    ws.runs_dev = runs;
     EPWI_REQUIRE(c->nstates < (int64_t(1) << 27), EPWI_EUNSUPPORTED, "iterative BTE needs fewer than 2^27 states");
     c->ib_pt.ensure(sizeof(unsigned) * c->nk);
     EPWI_CUDA(cudaMemsetAsync(c->ib_pt.p, 0, sizeof(unsigned) * c->nk, c->stream));

@@ -64,3 +64,21 @@ def test_decisions_of_a_chunk(monkeypatch):
     ctx.eigs((6, 5, 4))
     assert _free() - f0 >= mask - (2 << 20)
     ctx.close()
+
+
+def test_split_modes_hold_no_run_tables():
+    """The run tables (one word per plane block, q1 and k-point) serve the sum-factorised kernels only."""
+    s = synth.al_like_system()
+    ctx = epwi.Context(precision="fp16x3")
+    ctx.setup(s)
+    ctx.eigs((1000, 3, 2))
+    mu = 0.5 * sum(ctx.band_range())
+    args = (300.0, mu, 0.05, mu - 0.4, mu + 0.4)
+    _, npairs = ctx.scatter_rates(*args)
+    runs = 4 * 1001 * ctx.stats()["n_kpoints"]
+    assert runs > 12 << 20
+    ctx.ibte(*args, max_iter=2)
+    f0 = _free()
+    ctx.scatter_rates(*args)                      # gives the capture's lists back
+    assert abs(_free() - f0 - 8 * npairs) <= 6 << 20
+    ctx.close()
