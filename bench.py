@@ -67,6 +67,14 @@ def fma_peaks(device=0, stream=None):
     return out
 
 
+def scatter_kernel(precision, stats):
+    """The Rp->q kernel of a rates call: the sum-factorised ones process no 128-pair tiles."""
+    if precision == "fp32" or (precision == "fp64" and stats.get("n_tiles") == 0):
+        name = "k_scatter_sf" if precision == "fp32" else "k_scatter_sf64"
+        return f"{name} (sum-factorised Rp->q + rotations + delta sum)"
+    return f"{'k_scatter_fp64' if precision == 'fp64' else 'k_scatter_tc'} (fused Rp->q GEMM + rotations + delta sum)"
+
+
 def roofline_for(precision, stats, per_launch_traffic=None, simt_peaks=None):
     """Dominant kernel: the fused Rp->q + rotation + delta kernel (one launch per chunk)."""
     mp, src = peaks()
@@ -87,8 +95,7 @@ def roofline_for(precision, stats, per_launch_traffic=None, simt_peaks=None):
         note = f"{src} bf16 burst peak x {ratio}"
     return {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
             "frac": achieved / peak, "traffic": per_launch_traffic, "traffic_unit": "bytes per launch",
-            "kernel": ("k_scatter_sf (sum-factorised Rp->q + rotations + delta sum)" if precision == "fp32"
-                       else "k_scatter (fused Rp->q GEMM + rotations + delta sum)"),
+            "kernel": scatter_kernel(precision, stats),
             "launches_per_step": stats["n_chunks"], "peak_source": note}
 
 
@@ -607,8 +614,8 @@ def run_ibte(args):
             ev[k][0].record(stream)
             st, sig, mu = step()
             ev[k][1].record(stream)
-            sts.append(dict(st, ms_scatter=ctx.stats()["ms_scatter"], scatter_flops=ctx.stats()["scatter_flops"],
-                            n_chunks=ctx.stats()["n_chunks"]))
+            rs = ctx.stats()
+            sts.append(dict(st, **{x: rs[x] for x in ("ms_scatter", "scatter_flops", "n_chunks", "n_tiles")}))
         torch.cuda.synchronize()
     launches = (epwi.epwi_kernel_launches() - launches0) // args.steps
     ms = sum(a.elapsed_time(b) for a, b in ev) / args.steps
@@ -623,7 +630,8 @@ def run_ibte(args):
                  "launches_per_step": st["iters"], "peak_source": f"{src} HBM copy bandwidth"}
     roof_sc = roofline_for(precision, dict(scatter_flops=statistics.mean(x["scatter_flops"] for x in sts),
                                            ms_scatter=statistics.mean(x["ms_scatter"] for x in sts),
-                                           n_chunks=st["n_chunks"]), simt_peaks=fma_peaks(0, stream.cuda_stream))
+                                           n_chunks=st["n_chunks"], n_tiles=st["n_tiles"]),
+                           simt_peaks=fma_peaks(0, stream.cuda_stream))
     it_ms = statistics.mean(x["ms_step"] * x["iters"] for x in sts)
     sc_ms = statistics.mean(x["ms_scatter"] for x in sts)
     roof, roof_other = (roof_sc, roof_step) if sc_ms >= it_ms else (roof_step, roof_sc)

@@ -111,11 +111,15 @@ typedef struct {
     int64_t n_kpoints;          /* k-points with at least one state in the window */
     int64_t n_states;           /* states (n,k) in the window */
     int64_t n_pairs;            /* (k,q) pairs kept by the sieve */
-    int64_t n_tiles;            /* 128-pair work tiles processed */
+    int64_t n_tiles;            /* 128-pair work tiles processed (0 where the sum-factorised kernels ran,
+                                   which have none: fp32, and FP64 rates on the shapes of scatter_flops) */
     int64_t n_chunks;           /* on-the-fly k-point chunks */
     double ms_eigs, ms_sieve, ms_restage, ms_scatter, ms_reduce;   /* device time per stage */
     int64_t restage_bytes;      /* algorithmic bytes of the Re->k stage (g read once per chunk) */
-    double scatter_flops;       /* algorithmic flops of the Rp->q GEMM (one pass, no padding) */
+    double scatter_flops;       /* algorithmic flops of the Rp->q GEMM (one pass, no padding); where the
+                                   R_p sum ran factorised (fp32; FP64 rates with (nw, modes) in {(4,3), (8,6)}
+                                   and R_p within |n| <= 3, or (1,3) and <= 2, no vector listed
+                                   twice), per pair and band its last axis and the rotations */
     int32_t precision;
     int32_t sm_count;           /* multiprocessors of the device */
     int64_t tc_grid;            /* CTAs of the last tensor-core launch (0 in FP64 mode) */

@@ -532,7 +532,7 @@ WorkSet begin_rates(epwi_ctx *c, double T, double mu, double eta, double emin, d
     require_eigs(c);
     EPWI_REQUIRE(T > 0 && eta > 0 && std::isfinite(mu) && !(emin > emax), EPWI_EINVAL,
                  "need T > 0, smear > 0, finite mu and emin <= emax");
-    c->have_rates = c->have_sigma = c->have_is = c->have_ibte = false;
+    c->have_rates = c->have_sigma = c->have_is = c->have_ibte = c->sf64_used = false;
     c->T = T;
     c->mu = mu;
     c->eta = eta;
@@ -583,7 +583,7 @@ void end_rates(epwi_ctx *c) {
                              c->nw * (c->opt.precision == EPWI_FP64 ? 16 : 8);
     const double nbar = (double)c->nstates / std::max<int64_t>(1, c->nkp);
     c->stats.scatter_flops = 8.0 * c->nRp * c->nm * c->nw * (double)c->npairs * nbar;
-    if (c->opt.precision == EPWI_FP32) {
+    if (c->opt.precision == EPWI_FP32 || c->sf64_used) {
         // per (pair, band): the last factor of the R_p sum (real coefficients on 2r recombined
         // forms, 4 flop each per column) and the rotations of one final band, the least any
         // pair needs (the per-block and per-run sums are shared, bands out of range are

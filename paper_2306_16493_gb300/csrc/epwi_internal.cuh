@@ -182,6 +182,7 @@ struct epwi_ctx {
     DevBuf gsf32;                  // fp32 mode: g' [Re][cube forms][Nm][W][W] (+-R recombined)
     bool sf_g_ready = false;       // gsf32 built for the current system
     DevBuf gsf64;                  // FP64 mode: the same in FP64
+    bool sf64_used = false;        // the last rates call ran the FP64 sum-factorised kernel
     bool sf_g64_ready = false;
     bool rp_twice = false;         // R_p holds a vector twice (no FP64 cube form)
     DevBuf sf_kqt, sf_qt;          // fp32 mode: gather tables of the k+q and q sides (scatter_sf.cu)
@@ -245,7 +246,6 @@ struct epwi_ctx {
     DevBuf ib_red;                 // uint64 [2]: bit patterns of max |dF| and max |F|
     epwi_ibte_stats ib_stats{};
 
-    ~epwi_ctx() {
     // Workspaces that one kind of call keeps for its next one: the draws of the importance sampling (up to
     // 4 GiB), the pair lists of the iterative BTE's capture (up to 4 GiB and their run tables) and the decisions
     // of a chunk of k-points (up to 2 GiB).  A call of another kind, another grid or another system
@@ -260,6 +260,7 @@ struct epwi_ctx {
             for (DevBuf *b : {&chunk_mask, &chunk_counts}) b->release();
     }
 
+    ~epwi_ctx() {
         DevBuf *all[] = {&Re, &Rp, &Rcart, &Hw, &Phiw, &mode_mass, &gw64, &gw32, &ph64, &ph32,
                          &eps, &eps32, &V, &V32, &vel, &hw, &hwmax32, &hw32, &u, &u32, &eig_flag,
                          &kpts, &win_lo, &win_n, &kp_state, &kp_pairs, &inv_tau, &st_k,

@@ -458,6 +458,7 @@ void process_workset(epwi_ctx *c, const WorkSet &ws, double *g2out, double *tout
     // outputs
     const bool sf64 = !sf && !tc && !g2out && !tout && !ws.pair_w && ws.ovr_nsel < 0 && (!ws.pairs_dev || ws.runs_dev) &&
                       sf64_ok(c);
+    c->sf64_used = sf64;
     if (sf64) sf64_prepare(c);
     // chunk limits: Re->k output size, and the pair lists (2^27 q indices) or, in the sum-factorised
     // kernels, the decision mask where it is evaluated per chunk (2 GiB)
