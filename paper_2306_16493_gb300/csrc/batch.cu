@@ -18,7 +18,7 @@
 //
 // Each system has its own tile shape: the pairs per item M_t and the K chunk of the Rp sum.
 // An autotuner picks it by timing the persistent kernel on a sample of each class
-// (W, N_m, n_Rp) and caches the choice per class for the process.
+// (W, N_m, n_Rp and whether R_p is a cube) and caches the choice per class for the process.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -581,7 +581,9 @@ bool tile_ok(int Mt, int KC, int NW) {
            smem_rule(Mt, KC, NW) <= kSmemCap;
 }
 
-using TileKey = std::tuple<int, int, int>;           // (W, Nm, nRp)
+// (W, Nm, nRp), the half-width of an R_p cube that the product factorises over (else -1: the direct sum,
+// which another tile suits) and the device
+using TileKey = std::tuple<int, int, int, int, int>;
 std::map<TileKey, std::pair<int, int>> g_tile_cache;  // autotuned (Mt, KC) per class
 
 }  // namespace
@@ -891,7 +893,7 @@ std::pair<int, int> default_tile(int NW) {
 
 std::pair<int, int> autotune(epwi_batch *b, int s, int &src) {
     epwi_ctx *c = b->sys[s];
-    const TileKey key{c->nw, c->nm, c->nRp};
+    const TileKey key{c->nw, c->nm, c->nRp, c->rp_cube_r <= 6 ? c->rp_cube_r : -1, b->device};
     auto it = g_tile_cache.find(key);
     if (it != g_tile_cache.end()) {
         src = 2;
