@@ -24,6 +24,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <tuple>
@@ -585,6 +586,7 @@ bool tile_ok(int Mt, int KC, int NW) {
 // which another tile suits) and the device
 using TileKey = std::tuple<int, int, int, int, int>;
 std::map<TileKey, std::pair<int, int>> g_tile_cache;  // autotuned (Mt, KC) per class
+std::mutex g_tile_mutex;                              // guards it: batches of several host threads
 
 }  // namespace
 
@@ -894,10 +896,13 @@ std::pair<int, int> default_tile(int NW) {
 std::pair<int, int> autotune(epwi_batch *b, int s, int &src) {
     epwi_ctx *c = b->sys[s];
     const TileKey key{c->nw, c->nm, c->nRp, c->rp_cube_r <= 6 ? c->rp_cube_r : -1, b->device};
-    auto it = g_tile_cache.find(key);
-    if (it != g_tile_cache.end()) {
-        src = 2;
-        return it->second;
+    {
+        const std::lock_guard<std::mutex> lock(g_tile_mutex);
+        const auto it = g_tile_cache.find(key);
+        if (it != g_tile_cache.end()) {
+            src = 2;
+            return it->second;
+        }
     }
     const int NW = c->nw * c->nm;
     std::pair<int, int> best = default_tile(NW);
@@ -916,7 +921,10 @@ std::pair<int, int> autotune(epwi_batch *b, int s, int &src) {
         }
     }
     src = 1;
-    if (best_t < 1e300) g_tile_cache[key] = best;
+    if (best_t < 1e300) {
+        const std::lock_guard<std::mutex> lock(g_tile_mutex);
+        g_tile_cache[key] = best;
+    }
     return best;
 }
 
