@@ -565,7 +565,9 @@ void launch_phase_tables(epwi_ctx *c) {
 // Threads per block of the thread-per-point kernels: an SM's FP64 unit takes 16 clocks per warp
 // instruction, so a grid's points are spread over all SMs first (32-thread blocks up to 128 points
 // per SM, 64 up to 256).
-static int eig_block(int64_t nk) { return nk <= 152 * 128 ? 32 : nk <= 152 * 256 ? 64 : 128; }
+static int eig_block(const epwi_ctx *c, int64_t nk) {
+    return nk <= c->sm_count * int64_t(128) ? 32 : nk <= c->sm_count * int64_t(256) ? 64 : 128;
+}
 
 // Velocities of the n listed points (NULL: all) from the electron stage output f.
 static void launch_vel(epwi_ctx *c, const FacDesc &f, const Lattice &lat, const int *list, int64_t n) {
@@ -614,7 +616,7 @@ void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t joi
         ph = c->stream;
     }
     GridInfo g = make_grid_info(c);
-    const int bs = eig_block(nk);
+    const int bs = eig_block(c, nk);
     const unsigned nb = (unsigned)((nk + bs - 1) / bs);
     const int64_t plane = (int64_t)g.n2 * g.n3;
     // factorised build: axis-3 and axis-2 stages into fac_U (sources 0..nsrc-1), axis 1 in the
@@ -716,7 +718,7 @@ void launch_eigs(epwi_ctx *c, cudaStream_t ph, cudaEvent_t fork, cudaEvent_t joi
     EPWI_CHECK_LAUNCH();
     if (fac_el && W <= 8 && !defer) launch_vel(c, fe, lat, nullptr, nk);   // before the phonon stages reuse fac_U
     const int64_t nh = (g.n1 / 2 + 1) * plane;    // see minus_q
-    const int bsh = eig_block(nh);
+    const int bsh = eig_block(c, nh);
     const unsigned nbh = (unsigned)((nh + bsh - 1) / bsh), nbhw = (unsigned)((nh + kWarpsPerBlock - 1) / kWarpsPerBlock);
 #define PH_ARGS                                                                             \
     g, nh, Nm, c->nRp, c->Rp.as<int>(), c->Phiw.as<double>(), c->mode_mass.as<double>(),     \

@@ -211,23 +211,17 @@ ColumnSet build_columns(epwi_ctx *c, const int *kpts, int64_t nkp) {
     return cs;
 }
 
-// Multiply-adds of both forms per column of g, the factorised one with the window's counts of k3 and
-// columns or the largest the list can have, and twice over for its extra passes through T1 and T2; below the
-// work that the column lists' launches and one synchronisation (about 40 us) are worth, the direct
-// sum stays (tiny 8^3: 25 us).
+// The rule (ks_pays) with the window's counts of k3 and columns, or the largest the list can have.
 bool kstage_pays(const epwi_ctx *c, int64_t nkp, int64_t nrow, bool fp64) {
     // one block scans the columns: leave planes of over 2^20 columns to the direct sum
     if (!c->re_cube_ok || nkp <= 0 || (int64_t)c->ng[1] * c->ng[2] > (1 << 20)) return false;
-    const double D = 2.0 * c->fac_re_r + 1;
     double nk3 = (double)std::min<int64_t>(c->ng[2], nkp);
     double ncol = (double)std::min<int64_t>((int64_t)c->ng[1] * c->ng[2], nkp);
     if (c->win_ncol > 0 && nkp == c->nkp) {       // the window's own counts, where the sieve took them
         nk3 = c->win_nk3;
         ncol = c->win_ncol;
     }
-    const double direct = (double)c->nRe * nkp, fac = D * D * (D * nk3 + ncol) + D * nkp;
-    const double macs = direct * (double)nrow * c->nw;
-    return 2.0 * fac < direct && macs > (fp64 ? 1e7 : 2e8);
+    return ks_pays(2 * c->fac_re_r + 1, c->nRe, nkp, nk3, ncol, nrow, c->nw, fp64);
 }
 
 template <class C2>

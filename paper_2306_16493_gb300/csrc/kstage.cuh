@@ -28,6 +28,13 @@ struct ColumnSet {
 // Builds the columns of kpts[0 .. nkp-1] in c->col_buf (synchronises the stream for the counts).
 ColumnSet build_columns(epwi_ctx *c, const int *kpts, int64_t nkp);
 
+// Multiply-adds of both forms per column of g, the factorised one twice over for its extra passes
+// through T1 and T2; below the work that the column lists' launches and one synchronisation (about
+// 40 us) are worth, the direct sum stays (tiny 8^3: 25 us).
+inline bool ks_pays(int D, int nRe, int64_t nkp, double nk3, double ncol, int64_t nrow, int nw, bool fp64) {
+    const double direct = (double)nRe * nkp, fac = (double)D * D * (D * nk3 + ncol) + (double)D * nkp;
+    return 2.0 * fac < direct && direct * (double)nrow * nw > (fp64 ? 1e7 : 2e8);
+}
 // Whether the factorised sum is the faster one for a work set of nkp k-points of the current grid.
 bool kstage_pays(const epwi_ctx *c, int64_t nkp, int64_t nrow, bool fp64);
 
