@@ -36,11 +36,11 @@ DTYPE = {"fp64": "f64", "tf32x3": "tf32x3 (f32 acc, f64 sums)", "bf16x3": "bf16x
          "fp16x3": "fp16x3 (f32 acc, f64 sums)", "fp32": "f32 (sum-factorised, f64 sums)"}
 L2_BYTES = 129 * 2 ** 20
 # DRAM bytes (read + write) per (k,q) pair of the dominant kernel, from one ncu capture each:
-# k_scatter_tc (fp16x3) at 24^3, 255 MB / 19.6 M pairs (ncu --set full); k_scatter_sf (fp32,
-# pairs from the decision mask) at 20 x 27 x 45, 170.7 + 3.8 MB / 60.7 M pairs.  Traffic grows
-# with the pairs processed, so a launch's traffic is this times its pairs.  Valid for the kernel
-# versions of those captures.
-TRAFFIC_BYTES_PER_PAIR = {"fp16x3": 13.0, "fp32": 2.87}
+# k_scatter_sf (fp32) at the benchmark's own 48^3, 1297 + 5 MB / 1.2576e9 pairs; k_scatter_tc
+# (fp16x3) at 24^3, 255 MB / 19.6 M pairs (ncu --set full).  The decision mask, the tables and the Re->k
+# output do not grow with the pairs alone (fp32 at 20 x 27 x 45: 2.87 bytes per pair), so at other
+# sizes this times a launch's pairs is an extrapolation.
+TRAFFIC_BYTES_PER_PAIR = {"fp16x3": 13.0, "fp32": 1.04}
 
 
 def peaks():

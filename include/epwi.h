@@ -50,10 +50,13 @@ typedef enum {
 } epwi_status;
 
 /* Arithmetic of the g(k,q) interpolation (steps Re->k, Rp->q and the rotations).
- * Eigensolves, delta functions, occupations and the 1/tau and sigma sums are FP64 in
- * every mode.  EPWI_FP64 is the reference path. */
+ * Energies, eigenvectors, occupations and the sieve's decisions have FP64 accuracy in every mode, and
+ * 1/tau per state and sigma are FP64 sums; the delta terms are FP64 in EPWI_FP64 and FP32 otherwise.  (The
+ * eigensolver starts in FP32 and finishes in FP64: sweeps where levels are close, otherwise a
+ * perturbation series whose terms of second and higher order, below 2e-9, are formed in FP32.)
+ * EPWI_FP64 is the reference path. */
 typedef enum {
-    EPWI_FP64 = 0,   /* FP64 throughout */
+    EPWI_FP64 = 0,   /* FP64 throughout, but for the eigensolver's start and small terms (above) */
     EPWI_TF32X3 = 1, /* Rp->q GEMM on tcgen05 kind::tf32, 3-term hi/lo split, FP32 accumulate */
     EPWI_BF16X3 = 2, /* Rp->q GEMM on tcgen05 kind::f16 with bf16 operands, 3-term split */
     EPWI_FP16X3 = 3, /* Rp->q GEMM on tcgen05 kind::f16 with fp16 operands, 3-term split */
@@ -145,7 +148,8 @@ typedef struct {
     double change;              /* max |F^i - F^(i-1)| / max |F^i| after the last iteration */
     double ms_rates;            /* window, sieve, interpolation, 1/tau and the Gamma capture */
     double ms_iterate;          /* every iteration: step kernels and convergence reads */
-    double ms_step;             /* mean device time of one step kernel */
+    double ms_step;             /* mean device time per step done (up to seven launches queued behind
+                                   the last step, which do nothing, are part of it) */
     double bytes_per_step;      /* algorithmic bytes of one step: the index, Gamma, F0, tau,
                                    F read and written once */
     int64_t index_bytes;        /* the step's index: a 4-byte column word per Gamma entry and
@@ -181,7 +185,7 @@ epwi_status epwi_setup(epwi_ctx *ctx, const epwi_system *sys);
 /* Interpolates and diagonalises H(k) and D(q) on the full grids (Sec. II B, Eqs. 4-6):
  * eps_nk (ascending), V(k) (columns), v_nk = (1/hbar) Re[V^dag dH/dk V]_nn, hbar*omega_qnu
  * and u_{mu nu}(q) = (hbar / 2 m_mu omega_nu)^{1/2} e_{mu nu}(q) (FP64 Jacobi, one matrix per
- * grid point).  qgrid must equal kgrid (k+q is a grid point, Sec. III E).  The least
+ * grid point, started in FP32).  qgrid must equal kgrid (k+q is a grid point, Sec. III E).  The least
  * common multiple of the three grid sizes must be <= 4096.  Errors: ESTATE (no setup),
  * EINVAL, ENUMERIC (Jacobi did not converge). */
 epwi_status epwi_eigs(epwi_ctx *ctx, const int32_t kgrid[3], const int32_t qgrid[3]);
@@ -211,8 +215,13 @@ epwi_status epwi_carrier_density(epwi_ctx *ctx, double T_K, double mu_eV, int32_
  * (either may be NULL) receive the state and sieved-pair counts.  Synchronises.
  * Memory: the sieve keeps its decisions as a bit mask (one bit per (k-point, q) candidate)
  * when that mask fits in EPWI_SIEVE_MASK_MAX_BYTES (environment variable, bytes, default
- * 2 GiB); otherwise each chunk's pair lists are rebuilt by evaluating the sieve again.  Both
- * give the same pair lists and rates. */
+ * 2 GiB); otherwise the sieve is evaluated again for each chunk of k-points: its pair lists in the
+ * split modes and the direct FP64 sum, its decisions (up to 2 GiB) in the sum-factorised
+ * modes.  Both give the same pairs and rates.
+ * Between calls a context keeps its largest workspaces for the next call of the same kind: the
+ * decisions of a chunk (up to 2 GiB), the draws of epwi_scatter_rates_is (up to 4 GiB), and the pair
+ * lists of epwi_ibte (up to 4 GiB and a word per 256 (q2, q3), q1 and k-point).  A call of
+ * another kind, another grid and another system give them back. */
 epwi_status epwi_scatter_rates(epwi_ctx *ctx, double T_K, double mu_eV, double smear_eV,
                                double emin_eV, double emax_eV,
                                int64_t *n_states, int64_t *n_pairs);
@@ -393,8 +402,8 @@ epwi_status epwi_get_is_pairs(epwi_ctx *ctx, int64_t capacity, int32_t *ik, int3
  *
  * epwi_batch_plan runs each system's eigensolves, window and sieve count, then picks a tile
  * shape per system: the pairs per work item M_t and the K chunk of the Rp sum.  The
- * autotuner chooses it by timing candidates on a sample of each class (nw, 3 nat, n_Rp) and
- * caches the choice per class for the process.  The plan then captures one CUDA graph.  In
+ * autotuner chooses it by timing candidates on a sample of each class (nw, 3 nat, n_Rp, whether
+ * R_p is a cube) and caches the choice per class and device for the process.  The plan then captures one CUDA graph.  In
  * the graph, each system gets its eigensolves, sieve fill and FP32 Re->k stage.  Then ONE
  * persistent kernel works through a queue of (system, k-point, band, block of q) items
  * covering every system.  Per item it runs the Rp->q product, the rotations and the delta

@@ -432,7 +432,7 @@ void ibte_iterate(epwi_ctx *c, int max_iter, double tol) {
     // once the stop rule is met, so the host reads the maxima only once per kQueue steps.
     constexpr int kQueue = 8;
     c->ib_red.ensure(sizeof(unsigned long long) * 2 * (kQueue + 1));
-    unsigned long long *red = c->ib_red.as<unsigned long long>();   // slot 0: last step of the queue before
+    unsigned long long *red = c->ib_red.as<unsigned long long>();   // maxima of step i in slot i + 1
     cudaEvent_t e0, e1;
     EPWI_CUDA(cudaEventCreate(&e0));
     EPWI_CUDA(cudaEventCreate(&e1));

@@ -64,7 +64,7 @@ struct SfPlan {
 };
 
 // q2 values per group (jq): Y of one group and two runs' U per warp within budgets that keep two or
-// more CTAs per SM (FP32: three for 12 columns, 70 KB at jq = 7; FP64: two for 12 columns, 101 KB at
+// more CTAs per SM (FP32: three for 12 columns, 74 KiB at jq = 7; FP64: two for 12 columns, 103 KiB at
 // jq = 5, and one CTA's FP64 instructions run while the other waits at a barrier).
 inline SfPlan sf_plan(int D, int X, int W, int q2max, int N1, int N2, int N3, size_t real) {
     const size_t ybudget = 10240 * real, ubudget = (real == 8 ? 10240 : 13824) * real;

@@ -781,8 +781,8 @@ static bool sieve_count_cols(epwi_ctx *c, const SieveArgs &a, uint32_t *mk) {
         kern<<<grid, TB, sm, c->stream>>>(a, cs, c->kpts.as<int>(), c->win_lo.as<int>(), c->win_n.as<int>(),
                                           c->counts.as<unsigned long long>(), mk, c->mask_words);
     };
-    // 256 combinations keep three CTAs per SM up to 64 axis-1 points (1.5 KB each), 128 two or
-    // more beyond
+    // 256 combinations take 1.5 KiB per axis-1 point: three CTAs per SM up to 49 points, two up to 64;
+    // 128 combinations beyond keep two or more
     if (c->nw == 4) N1 <= 64 ? go(k_sieve_count_cols<4, 3, 256>, 256) : go(k_sieve_count_cols<4, 3, 128>, 128);
     else N1 <= 64 ? go(k_sieve_count_cols<8, 6, 256>, 256) : go(k_sieve_count_cols<8, 6, 128>, 128);
     return true;
