@@ -1,10 +1,17 @@
 """Workspaces that a context keeps between calls of one kind (draws, the capture's pair lists, decisions
 of a chunk) are given back by the first call of another kind, and by another grid."""
+import gc
+
 import pytest
 
 from paper_2306_16493_gb300 import epwi, synth
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _no_garbage():
+    gc.collect()                                  # contexts of other tests are gone before the first reading
 
 
 def _free():
